@@ -208,6 +208,60 @@ def run(state):
     return [np.array(kept, dtype=np.int64)] + [L.decode() for L in net.layers]
 
 
+# ------------------------------------------------------------------------------------------------ the results in 64 bits
+
+def _pruned64(case, g, rows, k):
+    """The pruned weight matrix of _layer(case, g, rows, k), from the definition of the pattern, as float64 [rows, k]."""
+    w = _weight(g, rows, k)
+    s = _saliency(g, w).double()
+    bm, bk, n, m = case["block_rows"], case["block_k"], case["n"], case["m"]
+    nrt, nblk, kkeep = _blocks(case, rows, k)
+    s = torch.nn.functional.pad(s, (0, nblk * bk - k, 0, nrt * bm - rows))
+    # the n largest of every m consecutive elements, the lower index first among equals
+    groups = s.view(-1, m)
+    order = torch.sort(groups, dim=1, descending=True, stable=True).indices[:, :n]
+    kept = torch.zeros_like(groups).scatter_(1, order, 1.0)
+    # the kkeep blocks of every row tile with the largest sums of what is left
+    score = (groups * kept).view(nrt, bm, nblk, bk).sum(dim=(1, 3))
+    best = torch.sort(score, dim=1, descending=True, stable=True).indices[:, :kkeep]
+    blocks = torch.zeros_like(score).scatter_(1, best, 1.0)
+    kept = kept.view(nrt, bm, nblk, bk) * blocks[:, None, :, None]
+    return w.double() * kept.view(nrt * bm, nblk * bk)[:rows, :k]
+
+
+def exact(case, seed):
+    """What run returns for these inputs in float64; None where the outputs are bytes and integers."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    if case["kind"] == "product":
+        w = _pruned64(case, g, case["rows"], case["k"])
+        bias = _normal(g, (case["rows"],), 0.1).double() if case["bias"] else None
+        y = w @ _activation(g, (case["k"], case["ncols"])).double()
+        if bias is not None:
+            y += bias[:, None]
+        return y.clamp_(min=0) if case["relu"] else y
+    if case["kind"] == "conv":
+        kn, rows, c, layers = case["kernel"], case["rows"], case["channels"], []
+        for _ in range(case["layers"]):
+            w = _pruned64(case, g, rows, kn * kn * c)
+            layers.append((w.view(rows, kn, kn, c), _normal(g, (rows,), 0.1).double()))
+            c = rows
+        x, outs = _activation(g, (case["batch"], case["side"], case["side"], case["channels"])), []
+        for w, bias in layers:
+            out = torch.empty(x.shape[:3] + (rows,), dtype=torch.float64, device="cuda")
+            for b in range(x.shape[0]):                       # one image at a time, filter tap by filter tap
+                p = torch.nn.functional.pad(x[b].double(), (0, 0, kn // 2, kn // 2, kn // 2, kn // 2))
+                acc = bias.expand(x.shape[1], x.shape[2], rows).clone()
+                for i in range(kn):
+                    for j in range(kn):
+                        acc += p[i:i + x.shape[1], j:j + x.shape[2]] @ w[:, i, j].t()
+                out[b] = acc.clamp_(min=0)
+            outs.append(out)
+            x = out
+        return outs if case["nhwc_out"] else [o.reshape(-1, rows).t().contiguous() for o in outs]
+    return None
+
+
 # ------------------------------------------------------------------------------------------------ work and tolerance
 
 def _shapes(case):
