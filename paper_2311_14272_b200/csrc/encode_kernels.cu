@@ -270,28 +270,91 @@ encode_block_m4_kernel(const uint16_t *__restrict__ w, int64_t ld, Geometry g, c
     }
 }
 
+// Dense weights from the canonical format, pruned positions as zero, in one pass over the output (which is what has to
+// be written: 2 bytes an element).  A CTA takes 32 rows x 256 elements, a warp four of the rows, a lane eight consecutive
+// elements of each: one 16-byte store, 512 consecutive bytes per row and warp.  The values of a lane's eight elements are
+// V = 8 N / M consecutive ones of their block and their offsets V consecutive fields, so a lane reads both with a load or
+// two and shifts every value to its place in registers.  Which slot of the row tile holds a block column is looked up once
+// per CTA.  Measured (4096 x 4096, 2:4, keep 0.5; 33 MB out, 19 MB in): 12.4 us, against 25 us + 6 us for a memset
+// and a kernel that scattered 2-byte values one by one with three integer divisions each.
+constexpr int kDecodeRows = 32, kDecodeCols = 256;
+
+template <int M, int N>
 __global__ void __launch_bounds__(256)
-decode_block_kernel(Geometry g, const int32_t *__restrict__ blk_col,
-                    const uint16_t *__restrict__ vals, const uint32_t *__restrict__ idx,
-                    uint16_t *__restrict__ w, int64_t ld) {
-    const int blk = blockIdx.x;
-    const int rt = blk / g.kkeep;
-    const int jb = blk_col[blk];
-    const int groups = g.groups();
-    const int64_t vpb = g.vals_per_block();
-    const uint16_t *vin = vals + (int64_t)blk * vpb;
-    const uint32_t *iin = idx + (int64_t)blk * (vpb * g.idx_bits / 32);
-    const uint32_t field = (1u << g.idx_bits) - 1u;
-    for (int o = threadIdx.x; o < (int)vpb; o += blockDim.x) {
-        const int item = o / g.n;
-        const int r = item / groups, gi = item - r * groups;
-        const int bit = o * g.idx_bits;
-        uint32_t t = iin[bit >> 5] >> (bit & 31);
-        if ((bit & 31) + g.idx_bits > 32) t |= iin[(bit >> 5) + 1] << (32 - (bit & 31));
-        t &= field;
-        const int64_t row = (int64_t)rt * g.bm + r;
-        const int64_t col = (int64_t)jb * g.bk + (int64_t)gi * g.m + t;
-        if (row < g.rows && col < g.k) w[row * ld + col] = vin[o];
+decode_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *__restrict__ vals,
+              const uint32_t *__restrict__ idx, uint16_t *__restrict__ w, int64_t ld, bool vec_ok, int chunks) {
+    constexpr int V = 8 / M * N, kBits = M == 4 ? 2 : 3, kRows = kDecodeRows / 8;
+    __shared__ int s_slot[kDecodeCols / 32];
+    const int rg = blockIdx.x / chunks, chunk = blockIdx.x - rg * chunks;
+    const int row0 = rg * kDecodeRows, rt = row0 / g.bm;
+    const int jb0 = chunk * kDecodeCols / g.bk;
+    if (threadIdx.x < kDecodeCols / 32) s_slot[threadIdx.x] = -1;
+    __syncthreads();
+    for (int i = threadIdx.x; i < g.kkeep; i += blockDim.x) {
+        const int d = __ldg(blk_col + (int64_t)rt * g.kkeep + i) - jb0;
+        if (d >= 0 && d < kDecodeCols / 32) s_slot[d] = i;          // (block columns beyond the chunk do no harm)
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k0 = chunk * kDecodeCols + lane * 8;
+    if (k0 >= g.k) return;
+    const int jb = k0 / g.bk, slot = s_slot[jb - jb0];
+    const int first = row0 + warp * kRows;
+    uint16_t v[kRows][V];
+    uint32_t f[kRows];
+    if (slot >= 0) {
+        const int vpb = (int)g.vals_per_block(), groups = g.groups();
+        const int64_t blk = (int64_t)rt * g.kkeep + slot;
+        const uint16_t *vin = vals + blk * vpb;
+        const uint32_t *iin = idx + blk * (vpb * kBits / 32);
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const int o = ((first + i - rt * g.bm) * groups + (k0 - jb * g.bk) / M) * N;     // (rows of padding are stored too)
+            if constexpr (V == 8) {
+                const uint4 t = __ldg(reinterpret_cast<const uint4 *>(vin + o));
+                v[i][0] = (uint16_t)t.x; v[i][1] = (uint16_t)(t.x >> 16); v[i][2] = (uint16_t)t.y; v[i][3] = (uint16_t)(t.y >> 16);
+                v[i][4] = (uint16_t)t.z; v[i][5] = (uint16_t)(t.z >> 16); v[i][6] = (uint16_t)t.w; v[i][7] = (uint16_t)(t.w >> 16);
+            } else if constexpr (V == 4) {
+                const uint2 t = __ldg(reinterpret_cast<const uint2 *>(vin + o));
+                v[i][0] = (uint16_t)t.x; v[i][1] = (uint16_t)(t.x >> 16); v[i][2] = (uint16_t)t.y; v[i][3] = (uint16_t)(t.y >> 16);
+            } else if constexpr (V % 2 == 0) {
+#pragma unroll
+                for (int j = 0; j < V; j += 2) {
+                    const uint32_t t = __ldg(reinterpret_cast<const uint32_t *>(vin + o + j));
+                    v[i][j] = (uint16_t)t; v[i][j + 1] = (uint16_t)(t >> 16);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < V; ++j) v[i][j] = __ldg(vin + o + j);
+            }
+            const int bit = o * kBits;
+            uint32_t t = __ldg(iin + (bit >> 5)) >> (bit & 31);
+            if (32 % (V * kBits) != 0 && (bit & 31) + V * kBits > 32) t |= __ldg(iin + (bit >> 5) + 1) << (32 - (bit & 31));
+            f[i] = t;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+        const int row = first + i;
+        if (row >= g.rows) break;
+        unsigned long long half[2] = {0ull, 0ull};                   // elements 0..3 and 4..7
+        if (slot >= 0) {
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const uint32_t t = (f[i] >> (j * kBits)) & ((1u << kBits) - 1u);
+                const unsigned long long at = (unsigned long long)v[i][j] << (16 * (t & 3u));
+                if constexpr (M == 4) half[j / N] |= at;
+                else { half[0] |= t < 4u ? at : 0ull; half[1] |= t < 4u ? 0ull : at; }
+            }
+        }
+        uint16_t *dst = w + (int64_t)row * ld + k0;
+        if (vec_ok && k0 + 8 <= g.k) {
+            *reinterpret_cast<uint4 *>(dst) = make_uint4((uint32_t)half[0], (uint32_t)(half[0] >> 32), (uint32_t)half[1], (uint32_t)(half[1] >> 32));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (k0 + j < g.k) dst[j] = (uint16_t)(half[j >> 2] >> (16 * (j & 3)));
+        }
     }
 }
 
@@ -353,11 +416,22 @@ cudaError_t launch_encode_canonical(const uint16_t *d_w, int64_t ld, const Geome
 
 cudaError_t launch_decode(const Geometry &g, const int32_t *d_blk_col, const uint16_t *d_vals,
                           const uint32_t *d_idx, uint16_t *d_w, int64_t ld, cudaStream_t st) {
-    cudaError_t e = cudaMemset2DAsync(d_w, (size_t)ld * 2, 0, (size_t)g.k * 2, (size_t)g.rows, st);
-    if (e != cudaSuccess) return e;
-    const int nblocks = g.nrt * g.kkeep;
-    if (nblocks == 0) return cudaSuccess;
-    decode_block_kernel<<<nblocks, 256, 0, st>>>(g, d_blk_col, d_vals, d_idx, d_w, ld);
+    const int chunks = (g.k + kDecodeCols - 1) / kDecodeCols;
+    const int64_t ctas = (int64_t)((g.rows + kDecodeRows - 1) / kDecodeRows) * chunks;
+    if (ctas > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+    const bool vec_ok = reinterpret_cast<uintptr_t>(d_w) % 16 == 0 && ld % 8 == 0;
+#define CRISP_DECODE(MV, NV)                                                                                        \
+    case NV: decode_kernel<MV, NV><<<(unsigned)ctas, 256, 0, st>>>(g, d_blk_col, d_vals, d_idx, d_w, ld, vec_ok, chunks); break
+    if (g.m == 4) {
+        switch (g.n) { CRISP_DECODE(4, 1); CRISP_DECODE(4, 2); CRISP_DECODE(4, 3); CRISP_DECODE(4, 4); default: return cudaErrorInvalidValue; }
+    } else {
+        switch (g.n) {
+            CRISP_DECODE(8, 1); CRISP_DECODE(8, 2); CRISP_DECODE(8, 3); CRISP_DECODE(8, 4);
+            CRISP_DECODE(8, 5); CRISP_DECODE(8, 6); CRISP_DECODE(8, 7); CRISP_DECODE(8, 8);
+            default: return cudaErrorInvalidValue;
+        }
+    }
+#undef CRISP_DECODE
     return cudaGetLastError();
 }
 
