@@ -287,6 +287,37 @@ CRISP_API crisp_status_t crisp_global_rank(int32_t n_layers, const crisp_rank_la
                                            double prune_fraction, void *d_workspace, int32_t *d_kkeep,
                                            void *stream);
 
+/* A pruning iteration over all layers of a network in a handful of launches instead of a dozen per layer:
+ *
+ *   crisp_prune_score        = per layer crisp_saliency_accumulate for every sample, crisp_saliency_finish_max,
+ *                              and the N:M step and block scores of crisp_build_mask_ex(MAX_KNOWN), keep ratio 1
+ *   (crisp_global_rank on the workspaces' scores gives the kept counts)
+ *   crisp_prune_encode       = per layer the selection of `kkeep` blocks (crisp_mask_reselect) and crisp_encode
+ *
+ * with the same results, bit for bit.  All layers have the same n and m; keep_ratio of the descriptors is not read.
+ * Buffers are the caller's: the mask buffer and workspace of crisp_mask_sizes with keep ratio 1; `d_saliency` [rows, k]
+ * fp32 receives S; canonical and execution buffers of crisp_prune_encode_sizes (which reads desc and kkeep).
+ * crisp_prune_score reads desc .. d_workspace, crisp_prune_encode reads desc, d_w, ld_w, the mask buffer, the workspace and
+ * the fields after them, and returns masks and handles as crisp_build_mask and crisp_encode do (all of them or none). */
+typedef struct {
+    crisp_layer_desc_t desc;
+    const uint16_t *d_w_bf16; int64_t ld_w;
+    const void *const *d_grads;       /* host array of `samples` device tensors [rows, k]                     */
+    const int64_t *ld_grads;          /* host array: their leading dimensions, in elements                    */
+    const int32_t *grad_dtypes;       /* host array: 0 bf16, 1 fp32                                           */
+    int32_t samples;
+    float *d_saliency; int64_t ld_s;
+    void *d_mask_buf, *d_workspace;
+    int32_t kkeep;                    /* blocks to keep per row tile, 0 .. nblk                               */
+    void *d_canonical_buf, *d_exec_buf;
+} crisp_prune_layer_t;
+
+CRISP_API crisp_status_t crisp_prune_score(int32_t n_layers, const crisp_prune_layer_t *layers, void *stream);
+CRISP_API crisp_status_t crisp_prune_encode_sizes(int32_t n_layers, const crisp_prune_layer_t *layers,
+                                                  size_t *canonical_bytes, size_t *exec_bytes);
+CRISP_API crisp_status_t crisp_prune_encode(int32_t n_layers, const crisp_prune_layer_t *layers, void *stream,
+                                            crisp_mask_t *masks, crisp_handle_t *handles);
+
 /* Copy the mask to host: h_blk_col [nrt*kkeep] int32, h_nm_bits [nrt*block_rows *
  * nblk*block_k/32] uint32.  Either may be NULL.  Synchronises `stream`. */
 CRISP_API crisp_status_t crisp_mask_export(crisp_mask_t mask, int32_t *h_blk_col, uint32_t *h_nm_bits,

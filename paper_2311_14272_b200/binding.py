@@ -29,6 +29,13 @@ class RankLayer(C.Structure):
                 ("block_elems", C.c_int64), ("min_keep", C.c_int32), ("reserved", C.c_int32)]
 
 
+class PruneLayer(C.Structure):
+    _fields_ = [("desc", LayerDesc), ("d_w_bf16", C.c_void_p), ("ld_w", C.c_int64), ("d_grads", C.c_void_p),
+                ("ld_grads", C.c_void_p), ("grad_dtypes", C.c_void_p), ("samples", C.c_int32), ("d_saliency", C.c_void_p),
+                ("ld_s", C.c_int64), ("d_mask_buf", C.c_void_p), ("d_workspace", C.c_void_p), ("kkeep", C.c_int32),
+                ("d_canonical_buf", C.c_void_p), ("d_exec_buf", C.c_void_p)]
+
+
 class ConvDesc(C.Structure):
     _fields_ = [("batch", C.c_int32), ("height", C.c_int32), ("width", C.c_int32), ("channels", C.c_int32),
                 ("kernel_h", C.c_int32), ("kernel_w", C.c_int32), ("pad", C.c_int32), ("y_layout", C.c_int32)]
@@ -106,6 +113,9 @@ def load(path: Optional[str] = None):
         "crisp_bytes_model": [vp, i64, i32, P(BytesModel)],
         "crisp_mask_scores": [P(LayerDesc), vp, P(vp), P(vp)],
         "crisp_global_rank_sizes": [i32, P(RankLayer), P(sz)],
+        "crisp_prune_score": [i32, P(PruneLayer), vp],
+        "crisp_prune_encode_sizes": [i32, P(PruneLayer), P(sz), P(sz)],
+        "crisp_prune_encode": [i32, P(PruneLayer), vp, P(vp), P(vp)],
         "crisp_global_rank": [i32, P(RankLayer), C.c_double, vp, vp, vp],
     }
     for name, args in sig.items():
@@ -242,6 +252,25 @@ def crisp_global_rank_sizes(rank_layers) -> int:
 def crisp_global_rank(rank_layers, prune_fraction: float, d_workspace, d_kkeep, stream=None):
     _check(load().crisp_global_rank(len(rank_layers), rank_layers, float(prune_fraction), _ptr(d_workspace),
                                     _ptr(d_kkeep), _stream(stream)), "crisp_global_rank")
+
+
+def crisp_prune_score(layers, stream=None):
+    """layers: ctypes array of PruneLayer."""
+    _check(load().crisp_prune_score(len(layers), layers, _stream(stream)), "crisp_prune_score")
+
+
+def crisp_prune_encode_sizes(layers):
+    """-> (canonical bytes, execution bytes) of every layer, for the kept counts in the array."""
+    a, b = (C.c_size_t * len(layers))(), (C.c_size_t * len(layers))()
+    _check(load().crisp_prune_encode_sizes(len(layers), layers, a, b), "crisp_prune_encode_sizes")
+    return list(a), list(b)
+
+
+def crisp_prune_encode(layers, stream=None):
+    """-> (masks, handles)"""
+    m, h = (C.c_void_p * len(layers))(), (C.c_void_p * len(layers))()
+    _check(load().crisp_prune_encode(len(layers), layers, _stream(stream), m, h), "crisp_prune_encode")
+    return list(m), list(h)
 
 
 def crisp_build_mask(d_saliency, ld_s: int, desc: LayerDesc, d_mask_buf, d_workspace, stream=None) -> int:
@@ -431,15 +460,24 @@ class HybridLayer:
 
     def encode(self, w, stream=None):
         assert w.is_cuda and w.element_size() == 2 and w.stride(1) == 1
-        torch = self.torch
-        cbytes, ebytes = crisp_encode_sizes(self.mask)
-        if self.canonical_buf is None or self.canonical_buf.numel() < cbytes:
-            self.canonical_buf = torch.empty(cbytes, dtype=torch.uint8, device=self.device)
-        if self.exec_buf is None or self.exec_buf.numel() < ebytes:
-            self.exec_buf = torch.empty(ebytes, dtype=torch.uint8, device=self.device)
+        self._reserve(*crisp_encode_sizes(self.mask))
         crisp_destroy(self.handle)
         self.handle = crisp_encode(w, w.stride(0), self.mask, self.canonical_buf, self.exec_buf, stream)
         return self
+
+    def _reserve(self, canonical_bytes, exec_bytes):
+        if self.canonical_buf is None or self.canonical_buf.numel() < canonical_bytes:
+            self.canonical_buf = self.torch.empty(canonical_bytes, dtype=self.torch.uint8, device=self.device)
+        if self.exec_buf is None or self.exec_buf.numel() < exec_bytes:
+            self.exec_buf = self.torch.empty(exec_bytes, dtype=self.torch.uint8, device=self.device)
+
+    def _adopt(self, kkeep, mask, handle):
+        """Take over a mask and a handle that a batched call made in this layer's buffers."""
+        crisp_mask_destroy(self.mask)
+        crisp_destroy(self.handle)
+        self.mask, self.handle = mask, handle
+        self.desc.keep_ratio = crisp_keep_ratio_for_count(self.desc, kkeep)
+        self.kkeep = kkeep
 
     def export(self, stream=None):
         import numpy as np
@@ -529,11 +567,9 @@ class HybridLayer:
 class PruningNetwork:
     """One pruning iteration of Algorithm 1 over all layers of a network, without the fine-tuning that follows it:
 
-        per layer   saliency of Eq. 1 from the caller's gradients   crisp_saliency_accumulate / _finish_max
-        per layer   N:M step and block scores (keep ratio 1)        crisp_build_mask_ex(MAX_KNOWN)
-        network     rank-column sums, global order, selection       crisp_global_rank
-        per layer   keep the selected number of blocks              crisp_mask_reselect
-        per layer   compress                                        crisp_encode
+        network     saliency of Eq. 1 from the caller's gradients, N:M step, block scores   crisp_prune_score
+        network     rank-column sums, global order, selection                              crisp_global_rank
+        network     keep the selected number of blocks per layer, compress                 crisp_prune_encode
 
     This class only owns buffers and issues those calls in that order; every number is computed by the library.
     `shapes` is a list of (rows, k); the pattern (n:m, block shape) is shared by the layers.
@@ -546,7 +582,6 @@ class PruningNetwork:
         self.n, self.m = n, m
         self.min_keep = min_keep
         self.layers = [HybridLayer(r, k, n, m, block_rows, block_k, 1.0, device=device) for (r, k) in shapes]
-        self.acc = [torch.empty((r, k), dtype=torch.float32, device=self.device) for (r, k) in shapes]
         self.sal = [torch.empty((r, k), dtype=torch.float32, device=self.device) for (r, k) in shapes]
         self.rank_arr = make_rank_layers([L.rank_layer(min_keep) for L in self.layers])
         self.rank_ws = torch.empty(crisp_global_rank_sizes(self.rank_arr), dtype=torch.uint8, device=self.device)
@@ -557,24 +592,37 @@ class PruningNetwork:
         kappa: overall sparsity target of this iteration.  Returns the kept-block count of every layer; the layers'
         masks and handles (self.layers[l]) hold the result."""
         torch = self.torch
-        for L, w, gs, acc, s in zip(self.layers, weights, grads, self.acc, self.sal):
-            rows, k = L.desc.rows, L.desc.k
-            for i, g in enumerate(gs):
-                crisp_saliency_accumulate(g, 0 if g.dtype == torch.bfloat16 else 1, g.stride(0), rows, k, acc, k, i == 0,
-                                          stream)
-            crisp_saliency_finish_max(acc, k, w, w.stride(0), rows, k, len(gs), s, k, L.workspace, stream)
-            L.desc.keep_ratio = 1.0
-            L.nblk, L.kkeep = crisp_keep_count(L.desc)
-            L.build_mask_max_known(s, stream)
+        bf16 = torch.bfloat16
+        arr = (PruneLayer * len(self.layers))()
+        host = []                                            # the arrays that the table points into
+        for P, L, w, gs, s in zip(arr, self.layers, weights, grads, self.sal):
+            assert w.is_cuda and w.element_size() == 2 and w.stride(1) == 1
+            h = len(gs)
+            ptrs = (C.c_void_p * h)(*[g.data_ptr() for g in gs])
+            lds = (C.c_int64 * h)(*[g.stride(0) for g in gs])
+            dts = (C.c_int32 * h)(*[0 if g.dtype == bf16 else 1 for g in gs])
+            host.append((ptrs, lds, dts))
+            P.desc = L.desc
+            P.d_w_bf16, P.ld_w = w.data_ptr(), w.stride(0)
+            P.d_grads, P.ld_grads, P.grad_dtypes = C.addressof(ptrs), C.addressof(lds), C.addressof(dts)
+            P.samples = h
+            P.d_saliency, P.ld_s = s.data_ptr(), L.desc.k
+            P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
+        crisp_prune_score(arr, stream)
         crisp_global_rank(self.rank_arr, crisp_prune_fraction(kappa, self.n, self.m), self.rank_ws, self.d_kkeep, stream)
         if stream is None:
             kk = self.d_kkeep.cpu().tolist()
         else:
             with torch.cuda.stream(stream):
                 kk = self.d_kkeep.cpu().tolist()
-        for L, w, c in zip(self.layers, weights, kk):
-            L.reselect(c, stream)
-            L.encode(w, stream)
+        for P, c in zip(arr, kk):
+            P.kkeep = c
+        for P, L, cb, eb in zip(arr, self.layers, *crisp_prune_encode_sizes(arr)):
+            L._reserve(cb, eb)
+            P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
+        masks, handles = crisp_prune_encode(arr, stream)
+        for L, c, mask, handle in zip(self.layers, kk, masks, handles):
+            L._adopt(c, mask, handle)
         return kk
 
     def close(self):

@@ -2,11 +2,11 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
 #include "crisp_internal.h"
-#include "walks.cuh"
 
 using crisp::align_up;
 using crisp::Geometry;
@@ -45,6 +45,14 @@ void fill_desc(const Geometry &g, double keep_ratio, crisp_layer_desc_t *d) {
     d->block_rows = g.bm; d->block_k = g.bk; d->keep_ratio = keep_ratio; d->score_mode = g.score_mode;
 }
 
+// Geometry with every block kept: how the buffers of a pruning iteration are laid out before the counts are known.
+crisp_status_t full_geometry(const crisp_layer_desc_t *d, Geometry *g) {
+    if (!d) return CRISP_INVALID_ARG;
+    crisp_layer_desc_t full = *d;
+    full.keep_ratio = 1.0;
+    return make_geometry(&full, g);
+}
+
 // Which execution image crisp_encode lays out.  Default: the 2:4 sparse-MMA image when every aligned
 // 4-group keeps at most two values (n <= 2), the zero-expanded dense-tile image otherwise.  The
 // environment variable CRISP_EXEC_IMAGE = dense | none overrides it (for measurements).  Evaluated once
@@ -66,6 +74,49 @@ size_t blk_col_bytes(const Geometry &g) { return align_up((size_t)g.nrt * g.kkee
 size_t nm_bits_bytes(const Geometry &g) { return align_up((size_t)g.mp() * g.wpr * sizeof(uint32_t)); }
 size_t vals_bytes(const Geometry &g) { return align_up((size_t)g.nnz() * sizeof(uint16_t) + 4); }
 size_t idx_bytes(const Geometry &g) { return align_up((size_t)g.idx_words() * sizeof(uint32_t) + 4); }
+
+// The handle of an encoded layer and what the encode kernel has to know to fill its buffers (all arguments checked).
+crisp_handle_s *new_handle(const uint16_t *d_w_bf16, int64_t ld_w, const crisp_mask_s *mask, void *d_canonical_buf,
+                           void *d_exec_buf, crisp::EncodeLayer *L) {
+    crisp_handle_s *h = new (std::nothrow) crisp_handle_s;
+    if (!h) return nullptr;
+    const Geometry &g = mask->g;
+    uint8_t *p = reinterpret_cast<uint8_t *>(d_canonical_buf);
+    h->g = g;
+    h->d_blk_col = reinterpret_cast<int32_t *>(p); p += blk_col_bytes(g);
+    h->d_vals = reinterpret_cast<uint16_t *>(p); p += vals_bytes(g);
+    h->d_idx = reinterpret_cast<uint32_t *>(p);
+    h->d_status = reinterpret_cast<int32_t *>(d_exec_buf);
+    h->d_exec = reinterpret_cast<uint8_t *>(d_exec_buf) + kAlign;
+    h->exec_kind = mask->image_kind;
+    h->exec_payload_bytes = exec_payload_bytes(g, h->exec_kind);
+    h->forced_path = -1;
+    h->epilogue = crisp::Epilogue{nullptr, 0};
+    const char *nt_env = std::getenv("CRISP_TC_NT");          // 64-column boxes per CTA tile, tuning only; read once
+    h->nt_override = nt_env ? std::atoi(nt_env) : 0;
+    h->group_override = 0;
+    h->wait_limit_cycles = 0;
+    h->debug_skip_stage = -1;
+    h->plan = nullptr;
+    h->last = crisp_launch_info_t{-1, 0, 0, 1, 0, 0, 0, 0, 1};
+    *L = crisp::EncodeLayer{};
+    L->g = g;
+    L->w = d_w_bf16; L->ld = ld_w;
+    L->mask_blk_col = mask->d_blk_col; L->nm_bits = mask->d_nm_bits;
+    L->blk_col = h->d_blk_col; L->vals = h->d_vals; L->idx = h->d_idx;
+    L->kind = h->exec_kind;
+    L->stack = 1;
+    if (h->exec_kind != CRISP_PATH_DIRECT && (int64_t)g.nrt * g.kkeep > 0) {
+        const crisp::TcImageLayout T = crisp::tc_image_layout(g, h->exec_kind);
+        L->image = h->d_exec + T.image_off;
+        L->walk_col = reinterpret_cast<int32_t *>(h->d_exec + T.walk_col_off);
+        L->walk_len = reinterpret_cast<int32_t *>(h->d_exec + T.walk_len_off);
+        L->header = reinterpret_cast<uint32_t *>(d_exec_buf);
+        L->nst = T.nst; L->wcap = T.wcap; L->stack = T.stack;
+        L->a_bytes = T.a_bytes; L->entry_bytes = T.entry_bytes;
+    }
+    return h;
+}
 
 }  // namespace
 
@@ -199,50 +250,119 @@ crisp_status_t crisp_encode(const uint16_t *d_w_bf16, int64_t ld_w, crisp_mask_t
         return CRISP_INVALID_ARG;
     const Geometry &g = mask->g;
     if (ld_w < g.k) return CRISP_BAD_SHAPE;
-    crisp_handle_s *h = new (std::nothrow) crisp_handle_s;
-    if (!h) return CRISP_CUDA_ERROR;
-    uint8_t *p = reinterpret_cast<uint8_t *>(d_canonical_buf);
-    h->g = g;
-    h->d_blk_col = reinterpret_cast<int32_t *>(p); p += blk_col_bytes(g);
-    h->d_vals = reinterpret_cast<uint16_t *>(p); p += vals_bytes(g);
-    h->d_idx = reinterpret_cast<uint32_t *>(p);
-    h->d_status = reinterpret_cast<int32_t *>(d_exec_buf);
-    h->d_exec = reinterpret_cast<uint8_t *>(d_exec_buf) + kAlign;
-    h->exec_kind = mask->image_kind;
-    h->exec_payload_bytes = exec_payload_bytes(g, h->exec_kind);
-    h->forced_path = -1;
-    h->epilogue = crisp::Epilogue{nullptr, 0};
-    const char *nt_env = std::getenv("CRISP_TC_NT");          // 64-column boxes per CTA tile, tuning only; read once
-    h->nt_override = nt_env ? std::atoi(nt_env) : 0;
-    h->group_override = 0;
-    h->wait_limit_cycles = 0;
-    h->debug_skip_stage = -1;
-    h->plan = nullptr;
-    h->last = crisp_launch_info_t{-1, 0, 0, 1, 0, 0, 0, 0, 1};
     cudaStream_t st = (cudaStream_t)stream;
-    // the status block is cleared by the encode kernel where one is launched with walk lists, else by a memset
-    const bool clear_in_kernel = h->exec_kind != CRISP_PATH_DIRECT && (int64_t)g.nrt * g.kkeep > 0;
-    cudaError_t e = clear_in_kernel ? cudaSuccess : cudaMemsetAsync(d_exec_buf, 0, kAlign, st);
-    // 128-row blocks: one kept block is one tensor-core tile, so the encode kernel writes it directly
-    const bool fuse_tiles = (h->exec_kind == CRISP_PATH_DENSE || h->exec_kind == CRISP_PATH_SPARSE) && g.bm == 128;
-    crisp::TcImageLayout L = {};
-    if (h->exec_kind != CRISP_PATH_DIRECT) L = crisp::tc_image_layout(g, h->exec_kind);
-    // the walk lists of the tensor-core kernel depend on the mask only: CTAs of the encode kernel build them
-    const bool tc = h->exec_kind != CRISP_PATH_DIRECT;
-    crisp::WalkArgs walks = {};
-    if (tc) walks = crisp::tc_walk_args(g, h->exec_kind, mask->d_blk_col, h->d_exec);
-    walks.header = clear_in_kernel ? reinterpret_cast<uint32_t *>(d_exec_buf) : nullptr;
-    if (e == cudaSuccess)
-        e = crisp::launch_encode_canonical(d_w_bf16, ld_w, g, mask->d_blk_col, mask->d_nm_bits,
-                                           h->d_blk_col, h->d_vals, h->d_idx, fuse_tiles ? h->exec_kind : 0,
-                                           fuse_tiles ? h->d_exec + L.image_off : nullptr, L.a_bytes, L.entry_bytes,
-                                           tc ? &walks : nullptr, st);
-    if (e == cudaSuccess && tc)
-        e = crisp::launch_build_image(g, h->exec_kind, h->d_blk_col, h->d_vals, h->d_idx,
-                                      h->d_exec, fuse_tiles, /*walks_done=*/true, st);
+    crisp::EncodeLayer L;
+    crisp_handle_s *h = new_handle(d_w_bf16, ld_w, mask, d_canonical_buf, d_exec_buf, &L);
+    if (!h) return CRISP_CUDA_ERROR;
+    // the status block is cleared by the encode kernel where it writes an image, else by a memset
+    cudaError_t e = L.header ? cudaSuccess : cudaMemsetAsync(d_exec_buf, 0, kAlign, st);
+    if (e == cudaSuccess) e = crisp::launch_encode(&L, 1, st);
     if (e != cudaSuccess) { delete h; return CRISP_CUDA_ERROR; }
     *out = h;
     return CRISP_OK;
+}
+
+crisp_status_t crisp_prune_score(int32_t n_layers, const crisp_prune_layer_t *layers, void *stream) {
+    if (n_layers <= 0 || !layers) return CRISP_INVALID_ARG;
+    std::unique_ptr<crisp::ScoreLayer[]> sc(new (std::nothrow) crisp::ScoreLayer[(size_t)n_layers]);
+    if (!sc) return CRISP_CUDA_ERROR;
+    for (int l = 0; l < n_layers; ++l) {
+        const crisp_prune_layer_t &P = layers[l];
+        Geometry g;
+        crisp_status_t s = full_geometry(&P.desc, &g);
+        if (s != CRISP_OK) return s;
+        if (g.n != layers[0].desc.n || g.m != layers[0].desc.m) return CRISP_UNSUPPORTED;
+        if (!P.d_w_bf16 || !P.d_grads || !P.ld_grads || !P.grad_dtypes || !P.d_saliency || !P.d_mask_buf || !P.d_workspace ||
+            P.samples <= 0)
+            return CRISP_INVALID_ARG;
+        if (!aligned(P.d_w_bf16, 2) || !aligned(P.d_saliency, 4) || !aligned(P.d_mask_buf, kAlign) || !aligned(P.d_workspace, kAlign))
+            return CRISP_INVALID_ARG;
+        if (P.ld_w < g.k || P.ld_s < g.k) return CRISP_BAD_SHAPE;
+        for (int h = 0; h < P.samples; ++h) {
+            if (!P.d_grads[h] || (P.grad_dtypes[h] != 0 && P.grad_dtypes[h] != 1)) return CRISP_INVALID_ARG;
+            if (P.ld_grads[h] < g.k) return CRISP_BAD_SHAPE;
+            if (!aligned(P.d_grads[h], P.grad_dtypes[h] ? 4 : 2)) return CRISP_INVALID_ARG;
+        }
+        crisp::ScoreLayer &S = sc[l];
+        S.g = g;
+        S.s = P.d_saliency; S.ld = P.ld_s;
+        S.max_key = reinterpret_cast<const uint32_t *>(P.d_workspace);
+        S.score = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(P.d_workspace) + kAlign);
+        S.blk_col = reinterpret_cast<int32_t *>(P.d_mask_buf);
+        S.nm_bits = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(P.d_mask_buf) + blk_col_bytes(g));
+    }
+    cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t e = crisp::launch_clear_scores(sc.get(), n_layers, st);
+    if (e == cudaSuccess) e = crisp::launch_saliency_bits(layers, sc.get(), n_layers, st);
+    if (e == cudaSuccess) e = crisp::launch_block_scores(sc.get(), n_layers, st);
+    return e == cudaSuccess ? CRISP_OK : CRISP_CUDA_ERROR;
+}
+
+crisp_status_t crisp_prune_encode_sizes(int32_t n_layers, const crisp_prune_layer_t *layers, size_t *canonical_bytes,
+                                        size_t *exec_bytes) {
+    if (n_layers <= 0 || !layers || !canonical_bytes || !exec_bytes) return CRISP_INVALID_ARG;
+    for (int l = 0; l < n_layers; ++l) {
+        Geometry g;
+        crisp_status_t s = full_geometry(&layers[l].desc, &g);
+        if (s != CRISP_OK) return s;
+        if (layers[l].kkeep < 0 || layers[l].kkeep > g.nblk) return CRISP_INVALID_ARG;
+        const int kind = image_kind(g);
+        g.kkeep = layers[l].kkeep;
+        canonical_bytes[l] = blk_col_bytes(g) + vals_bytes(g) + idx_bytes(g);
+        exec_bytes[l] = kAlign + exec_payload_bytes(g, kind);
+    }
+    return CRISP_OK;
+}
+
+crisp_status_t crisp_prune_encode(int32_t n_layers, const crisp_prune_layer_t *layers, void *stream, crisp_mask_t *masks,
+                                  crisp_handle_t *handles) {
+    if (n_layers <= 0 || !layers || !masks || !handles) return CRISP_INVALID_ARG;
+    std::unique_ptr<crisp::ScoreLayer[]> sc(new (std::nothrow) crisp::ScoreLayer[(size_t)n_layers]);
+    std::unique_ptr<crisp::EncodeLayer[]> en(new (std::nothrow) crisp::EncodeLayer[(size_t)n_layers]);
+    if (!sc || !en) return CRISP_CUDA_ERROR;
+    for (int l = 0; l < n_layers; ++l) { masks[l] = nullptr; handles[l] = nullptr; }
+    cudaStream_t st = (cudaStream_t)stream;
+    crisp_status_t s = CRISP_OK;
+    for (int l = 0; l < n_layers && s == CRISP_OK; ++l) {
+        const crisp_prune_layer_t &P = layers[l];
+        Geometry g;
+        s = full_geometry(&P.desc, &g);
+        if (s != CRISP_OK) break;
+        if (g.n != layers[0].desc.n || g.m != layers[0].desc.m) { s = CRISP_UNSUPPORTED; break; }
+        if (P.kkeep < 0 || P.kkeep > g.nblk || !P.d_w_bf16 || !P.d_mask_buf || !P.d_workspace || !P.d_canonical_buf || !P.d_exec_buf ||
+            !aligned(P.d_w_bf16, 2) || !aligned(P.d_mask_buf, kAlign) || !aligned(P.d_workspace, kAlign) ||
+            !aligned(P.d_canonical_buf, kAlign) || !aligned(P.d_exec_buf, kAlign)) {
+            s = CRISP_INVALID_ARG;
+            break;
+        }
+        if (P.ld_w < g.k) { s = CRISP_BAD_SHAPE; break; }
+        masks[l] = new (std::nothrow) crisp_mask_s;
+        if (!masks[l]) { s = CRISP_CUDA_ERROR; break; }
+        masks[l]->d_blk_col = reinterpret_cast<int32_t *>(P.d_mask_buf);
+        masks[l]->d_nm_bits = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(P.d_mask_buf) + blk_col_bytes(g));
+        masks[l]->image_kind = image_kind(g);
+        g.kkeep = P.kkeep;                                   // the buffer is laid out for every block, the mask keeps these
+        masks[l]->g = g;
+        handles[l] = new_handle(P.d_w_bf16, P.ld_w, masks[l], P.d_canonical_buf, P.d_exec_buf, &en[l]);
+        if (!handles[l]) { s = CRISP_CUDA_ERROR; break; }
+        if (!en[l].header && cudaMemsetAsync(P.d_exec_buf, 0, kAlign, st) != cudaSuccess) { s = CRISP_CUDA_ERROR; break; }
+        crisp::ScoreLayer &S = sc[l];
+        S = crisp::ScoreLayer{};
+        S.g = g;
+        S.score = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(P.d_workspace) + kAlign);
+        S.blk_col = masks[l]->d_blk_col; S.nm_bits = masks[l]->d_nm_bits;
+    }
+    if (s == CRISP_OK) {
+        cudaError_t e = crisp::launch_block_selects(sc.get(), n_layers, st);
+        if (e == cudaSuccess) e = crisp::launch_encode(en.get(), n_layers, st);
+        if (e != cudaSuccess) s = CRISP_CUDA_ERROR;
+    }
+    if (s != CRISP_OK)
+        for (int l = 0; l < n_layers; ++l) {
+            delete masks[l]; delete handles[l];
+            masks[l] = nullptr; handles[l] = nullptr;
+        }
+    return s;
 }
 
 crisp_status_t crisp_encoded_counts(crisp_handle_t h, int64_t *n_blk_col, int64_t *n_vals, int64_t *n_idx_words) {

@@ -31,6 +31,27 @@ struct Geometry {
     __host__ __device__ int64_t idx_words() const { return (nnz() * idx_bits + 31) / 32; }
 };
 
+// One launch over several layers: work units (items, CTAs) are numbered through, layer l owning first[l] .. first[l + 1] - 1.
+// The table travels as a kernel parameter (no copy, nothing to keep alive).  CAP = 1 is the single-layer call.
+constexpr int kBatchLayers = 64;
+template <typename L, int CAP>
+struct Batch {
+    int n;
+    int64_t first[CAP + 1];
+    L layer[CAP];
+#ifdef __CUDACC__
+    __device__ __forceinline__ int find(int64_t unit) const {       // the layer that owns `unit`
+        if constexpr (CAP == 1) return 0;
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (first[mid] <= unit) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    }
+#endif
+};
+
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 
@@ -74,23 +95,54 @@ struct crisp_handle_s {
 
 namespace crisp {
 
-struct WalkArgs;
-
 // mask_kernels.cu
 cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, int32_t *d_blk_col,
                               uint32_t *d_nm_bits, void *d_workspace, size_t workspace_bytes, bool max_known,
                               cudaStream_t st);
+// One layer of a batched launch: the saliency that is scored, the group bits and scores (in the mask workspace) and where
+// the selection writes its block list.
+struct ScoreLayer {
+    Geometry g;
+    const float *s;
+    int64_t ld;
+    const uint32_t *max_key;
+    uint32_t *nm_bits;
+    unsigned long long *score;
+    int32_t *blk_col;
+    int chunks, vec_ok;                  // (filled in by the launchers)
+};
+cudaError_t launch_clear_scores(const ScoreLayer *layers, int n, cudaStream_t st);     // scores and max_key
+cudaError_t launch_block_scores(const ScoreLayer *layers, int n, cudaStream_t st);
+cudaError_t launch_block_selects(const ScoreLayer *layers, int n, cudaStream_t st);
 // per-row-tile selection alone, on the scores and group bits an earlier launch_build_mask left behind
 cudaError_t launch_block_select(const Geometry &g, const void *d_workspace, int32_t *d_blk_col, uint32_t *d_nm_bits,
                                 cudaStream_t st);
 size_t mask_workspace_bytes(const Geometry &g);
 
+// saliency_kernels.cu: saliency, group bits and layer maxima of a network in one launch (max_key cleared before)
+cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreLayer *scores, int n, cudaStream_t st);
+
 // encode_kernels.cu
-cudaError_t launch_encode_canonical(const uint16_t *d_w, int64_t ld, const Geometry &g,
-                                    const int32_t *d_mask_blk_col, const uint32_t *d_nm_bits,
-                                    int32_t *d_blk_col, uint16_t *d_vals, uint32_t *d_idx,
-                                    int tile_kind, uint8_t *d_image, uint32_t a_bytes, uint32_t entry_bytes,
-                                    const struct WalkArgs *walks, cudaStream_t st);
+constexpr int kMaxBlockWords = 128;      // nblk <= 4096
+// One layer of an encode launch: canonical blocks, and the execution image of `kind` with its walk lists (kind DIRECT:
+// canonical blocks only, walk_col = nullptr).  The layers of one launch share n and m.
+struct EncodeLayer {
+    Geometry g;
+    const uint16_t *w;
+    int64_t ld;
+    const int32_t *mask_blk_col;
+    const uint32_t *nm_bits;
+    int32_t *blk_col;
+    uint16_t *vals;
+    uint32_t *idx;
+    uint8_t *image;
+    int32_t *walk_col, *walk_len;
+    uint32_t *header;                    // 64 words cleared by the kernel (the handle's status block), or nullptr
+    int kind, nst, wcap, stack;
+    uint32_t a_bytes, entry_bytes;
+    int vec_ok;                          // (filled in by the launcher)
+};
+cudaError_t launch_encode(const EncodeLayer *layers, int n, cudaStream_t st);
 cudaError_t launch_decode(const Geometry &g, const int32_t *d_blk_col, const uint16_t *d_vals,
                           const uint32_t *d_idx, uint16_t *d_w, int64_t ld, cudaStream_t st);
 
@@ -107,12 +159,6 @@ struct TcImageLayout {
 };
 bool tc_pattern_is_sparse(const Geometry &g);
 TcImageLayout tc_image_layout(const Geometry &g, int kind);      // kind: CRISP_PATH_DENSE / SPARSE / SPARSE2
-// walk lists of the tensor-core kernel (walks.cuh): built by CTAs of the encode kernel (walks != nullptr in
-// launch_encode_canonical, then walks_done below) or by a kernel of their own
-struct WalkArgs tc_walk_args(const Geometry &g, int kind, const int32_t *d_mask_blk_col, uint8_t *d_exec);
-cudaError_t launch_build_image(const Geometry &g, int kind, const int32_t *d_blk_col, const uint16_t *d_vals,
-                               const uint32_t *d_idx, uint8_t *d_exec, bool tiles_done, bool walks_done,
-                               cudaStream_t st);
 bool tc_operands_ok(const void *x, int64_t ldx, const void *y, int64_t ldy, int y_dtype, int64_t ncols);
 // Convolution geometry for the implicit-GEMM mode (stride 1): NHWC activation, ho x wo output pixels.
 struct ConvGeom { int batch, height, width, channels, kh, kw, pad, ho, wo, nhwc_out; };

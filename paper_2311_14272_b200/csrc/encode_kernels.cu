@@ -1,272 +1,280 @@
 // Canonical compressed format of Sec. III-A: kept-block column list (Blocked-ELLPACK) plus,
 // per kept value, its bf16 payload and a log2(M)-bit zero-based offset inside its M-vector.
 #include "crisp_internal.h"
-#include "walks.cuh"
 
 namespace crisp {
 
 namespace {
 
-// The M weights of one group as 16-bit patterns; one vector load when the layout allows it.
-template <int M>
-__device__ __forceinline__ void load_group(const uint16_t *__restrict__ w, int64_t ld, int rows, int k,
-                                           int64_t row, int64_t col0, bool vec_ok, uint16_t v[M]) {
-    if (row >= rows || col0 >= k) {
+// One CTA per entry of the walk list of a 128-row CTA tile of the tensor-core kernel: it writes the canonical blocks
+// (values, offsets) of the tile's row tiles that keep the entry's column and, from the same registers, the entry of the
+// execution image: the weight tile and the 2:4 metadata of all 128 rows, with zeros (and valid padding metadata) for row
+// tiles that do not keep it.  The walk list of a CTA tile is the ascending union of its row tiles' lists: with 128-row
+// blocks the list itself, else every CTA marks the union in a bitmap and takes the column at its own position.
+//
+// A thread takes eight consecutive elements of a row: one 16-byte load and one byte of the mask.  Everything a 4-group
+// needs follows from its four mask bits and is looked up in a 16-entry table: byte-permute selectors that move the kept
+// values to the front, offset fields, the slot pair of the 2:4 image and its metadata nibble.  Values go straight to
+// global memory (consecutive lanes write consecutive bytes), the tile and the offset fields through shared memory;
+// every metadata byte belongs to one thread, so there are no atomics on it.  What bounds the kernel is the chain of
+// dependent round trips of a CTA (block list, weights, stores), hidden by the five CTAs an SM holds (48 registers; 40 spill
+// and take 20 us where this takes 14).  A thread keeps its chunk column and goes down the rows: with the row and column of
+// every chunk computed anew, and the image chosen at run time, the same work took 22 us.
+// Measured: 4096 x 4096, 2:4, keep 0.5, 128 x 64 blocks 14.0 us (36 MB moved); the 13 layers of VGG-16 with 64 x 64 blocks in
+// one launch 15.9 us, where a canonical pass and an image pass over it per layer took 62 + 165 us.
+// Shared-memory planes of the tile are padded (2064 or 2080 instead of 2048 bytes), which spreads the eight lanes of a row
+// over the banks.
+// Image layouts: see the tensor-core SpMM.  Stacked thin layers: copy q of the image holds the rows shifted by
+// q * 128 / stack; the copies are written from one staged tile.
+constexpr int kTileRows = 128, kMetaTileBytes = 2048;
+
+// What a 4-group needs, by its four mask bits:
+//   x  byte-permute selectors that move the kept values to the front in ascending order: 1st and 2nd | 3rd and 4th << 16
+//   y  byte-permute selector of the 2:4 slot pair | metadata nibble << 16 | kept count << 24
+//   z  2-bit positions of the kept values, ascending | 3-bit positions << 16
+//   w  0xFFFF in the slots that carry a value
+__device__ __forceinline__ uint4 nibble_entry(uint32_t nib) {
+    uint32_t front = 0u, f2 = 0u, f3 = 0u;
+    int cnt = 0;
 #pragma unroll
-        for (int i = 0; i < M; ++i) v[i] = 0;
-        return;
-    }
-    const uint16_t *p = w + row * ld + col0;
-    if (vec_ok && col0 + M <= k) {
-        if constexpr (M == 4) {
-            const uint2 q = __ldg(reinterpret_cast<const uint2 *>(p));
-            v[0] = (uint16_t)q.x; v[1] = (uint16_t)(q.x >> 16); v[2] = (uint16_t)q.y; v[3] = (uint16_t)(q.y >> 16);
-        } else {
-            const uint4 q = __ldg(reinterpret_cast<const uint4 *>(p));
-            v[0] = (uint16_t)q.x; v[1] = (uint16_t)(q.x >> 16); v[2] = (uint16_t)q.y; v[3] = (uint16_t)(q.y >> 16);
-            v[4] = (uint16_t)q.z; v[5] = (uint16_t)(q.z >> 16); v[6] = (uint16_t)q.w; v[7] = (uint16_t)(q.w >> 16);
+    for (int p = 0; p < 4; ++p)
+        if ((nib >> p) & 1u) {
+            front |= (uint32_t)((2 * p) | ((2 * p + 1) << 4)) << (8 * cnt);
+            f2 |= (uint32_t)p << (2 * cnt);
+            f3 |= (uint32_t)p << (3 * cnt);
+            ++cnt;
         }
+    int a = 0, b = 1, va = 0, vb = 0;                        // 2:4 slots: ascending positions, an empty slot padded
+    if (nib) {
+        const int first = __ffs(nib) - 1;
+        const uint32_t rest = nib & (nib - 1);
+        if (rest) { a = first; va = 1; b = __ffs(rest) - 1; vb = 1; }
+        else if (first == 3) { a = 0; b = 3; vb = 1; }
+        else { a = first; va = 1; b = 3; }
+    }
+    return make_uint4(front,
+                      (uint32_t)(2 * a) | ((uint32_t)(2 * a + 1) << 4) | ((uint32_t)(2 * b) << 8) | ((uint32_t)(2 * b + 1) << 12) |
+                          ((uint32_t)(a | (b << 2)) << 16) | ((uint32_t)cnt << 24),
+                      f2 | (f3 << 16), (va ? 0x0000FFFFu : 0u) | (vb ? 0xFFFF0000u : 0u));
+}
+// 0xFFFF in the halves whose bit is set
+__device__ __forceinline__ uint32_t half_mask(uint32_t two_bits) {
+    return ((two_bits & 1u) ? 0x0000FFFFu : 0u) | ((two_bits & 2u) ? 0xFFFF0000u : 0u);
+}
+
+// IMAGE: the image the layers of the launch have (CRISP_PATH_DENSE also for layers without one).
+template <int M, int N, int IMAGE, int CAP>
+__global__ void __launch_bounds__(256, 5)
+encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
+    constexpr int V = 8 / M * N, kIdxBits = M == 4 ? 2 : 3, kFieldBits = V * kIdxBits;
+    constexpr int kUnroll = 4;
+    constexpr bool kSparse = IMAGE == CRISP_PATH_SPARSE;
+    extern __shared__ uint4 s_raw4[];
+    __shared__ uint4 s_lut[16];
+    __shared__ uint32_t s_map[kMaxBlockWords];               // kept columns of the tile (the union)
+    __shared__ int s_slot[4];                                // where row tile i keeps this column, or -1
+    const int l = batch.find(blockIdx.x);
+    const EncodeLayer &L = batch.layer[l];
+    const Geometry &g = L.g;
+    const int cta = (int)(blockIdx.x - batch.first[l]);
+    const int r = kTileRows / g.bm;
+    const int per_tile = r == 1 ? g.kkeep : min(r * g.kkeep, g.nblk);     // most entries of a walk list
+    const int st = cta / per_tile, entry = cta - st * per_tile;
+    const int first_rt = st * r, n_rt = min(r, g.nrt - first_rt);
+    if (cta == 0 && L.header != nullptr && threadIdx.x < 64) L.header[threadIdx.x] = 0u;     // the handle's status block
+    const bool lists = L.walk_col != nullptr;
+    int jb;
+    if (r == 1) {                                            // the walk list is the row tile's kept list
+        jb = __ldg(L.mask_blk_col + (int64_t)st * g.kkeep + entry);
+        if (threadIdx.x < 4) s_slot[threadIdx.x] = threadIdx.x == 0 ? entry : -1;
+        if (threadIdx.x >= 32 && threadIdx.x < 48) s_lut[threadIdx.x - 32] = nibble_entry(threadIdx.x - 32);
+        if (lists && entry == 0 && threadIdx.x == 0) L.walk_len[st] = g.kkeep;
+        __syncthreads();
     } else {
-#pragma unroll
-        for (int i = 0; i < M; ++i) v[i] = (col0 + i < k) ? __ldg(p + i) : (uint16_t)0;
+        const int map_words = (g.nblk + 31) / 32, listed = n_rt * g.kkeep;
+        const int c = threadIdx.x < listed ? __ldg(L.mask_blk_col + (int64_t)first_rt * g.kkeep + threadIdx.x) : 0;
+        for (int i = threadIdx.x; i < map_words; i += blockDim.x) s_map[i] = 0u;
+        if (threadIdx.x < 4) s_slot[threadIdx.x] = -1;
+        if (threadIdx.x >= 32 && threadIdx.x < 48) s_lut[threadIdx.x - 32] = nibble_entry(threadIdx.x - 32);
+        __syncthreads();
+        if (threadIdx.x < listed) atomicOr(&s_map[c >> 5], 1u << (c & 31));
+        for (int i = threadIdx.x + blockDim.x; i < listed; i += blockDim.x) {
+            const int d = __ldg(L.mask_blk_col + (int64_t)first_rt * g.kkeep + i);
+            atomicOr(&s_map[d >> 5], 1u << (d & 31));
+        }
+        __syncthreads();
+        // the column with `entry` kept columns of the union below it
+        int word = 0, below = 0, cnt = 0;
+        for (; word < map_words; ++word, below += cnt) {
+            cnt = __popc(s_map[word]);
+            if (below + cnt > entry) break;
+        }
+        if (lists && entry == 0 && threadIdx.x == 0) {
+            int n = 0;
+            for (int i = 0; i < map_words; ++i) n += __popc(s_map[i]);
+            L.walk_len[st] = n;
+        }
+        if (word == map_words) return;                       // a shorter list
+        uint32_t left = s_map[word];
+        for (int i = below; i < entry; ++i) left &= left - 1;
+        jb = word * 32 + __ffs(left) - 1;
+        if (threadIdx.x < listed && c == jb) { const int q = threadIdx.x / g.kkeep; s_slot[q] = threadIdx.x - q * g.kkeep; }
+        for (int i = threadIdx.x + blockDim.x; i < listed; i += blockDim.x)
+            if (__ldg(L.mask_blk_col + (int64_t)first_rt * g.kkeep + i) == jb) { const int q = i / g.kkeep; s_slot[q] = i - q * g.kkeep; }
+        __syncthreads();
     }
-}
+    if (lists && threadIdx.x == 0) L.walk_col[(int64_t)st * L.wcap + entry] = jb;
+    if (threadIdx.x < n_rt && s_slot[threadIdx.x] >= 0)
+        L.blk_col[(int64_t)(first_rt + threadIdx.x) * g.kkeep + s_slot[threadIdx.x]] = jb;
 
-// One CTA per kept block.  A thread takes whole groups of M elements (one vector load), so that the
-// N values of a group land contiguously; values and offsets are staged in shared memory and written
-// out with coalesced 16-byte stores.  Offsets go through a bit stream because a field may straddle
-// two words (3-bit fields for M = 8).
-// TILE selects what else the CTA emits for 128-row blocks (one kept block = one tensor-core tile):
-// 0 nothing, CRISP_PATH_DENSE the zero-expanded tile, CRISP_PATH_SPARSE the 2:4 compressed tile with
-// its metadata (layouts: see the execution-image kernels of the tensor-core SpMM).
-template <int M, int TILE>
-__global__ void __launch_bounds__(256, 8)
-encode_block_kernel(const uint16_t *__restrict__ w, int64_t ld, Geometry g, bool vec_ok,
-                    const int32_t *__restrict__ mask_blk_col, const uint32_t *__restrict__ nm_bits,
-                    int32_t *__restrict__ blk_col, uint16_t *__restrict__ vals,
-                    uint32_t *__restrict__ idx, uint8_t *__restrict__ image, uint32_t a_bytes,
-                    uint32_t entry_bytes, WalkArgs walks) {
-    extern __shared__ uint32_t s_buf[];
-    // The first walks.nctas CTAs build the walk lists of the tensor-core kernel instead of encoding a block:
-    // that needs only the mask's block list, so it overlaps the encoding instead of following it.
-    clear_header(walks);
-    if ((int)blockIdx.x < walks.nctas) {
-        __shared__ WalkShared s_walks;
-        build_walks_body(g, walks, blockIdx.x, s_walks);
-        return;
+    const int c8n = g.bk / 8;                                // a chunk: eight elements of a row
+    const bool image = kSparse || L.kind == CRISP_PATH_DENSE;
+    // staged tile: planes of 8 columns (one per 16-byte chunk of a row) with 128 rows of 16 bytes
+    constexpr uint32_t kPlane = kSparse ? 2080u : 2064u;
+    const int planes = kSparse ? c8n / 2 : c8n;
+    const uint32_t meta_at = (uint32_t)planes * kPlane, addend_bytes = meta_at + (kSparse ? kMetaTileBytes : 0);
+    const int addends = kSparse && N > 2 ? 2 : 1;
+    uint8_t *tile = reinterpret_cast<uint8_t *>(s_raw4);
+    uint32_t *s_field = reinterpret_cast<uint32_t *>(tile + (image ? addends * addend_bytes : 0u));    // [128 * c8n]
+    if (kSparse && g.bk < 128) {                             // metadata words beyond block_k / 32 per row are zero
+        for (int i = threadIdx.x; i < addends * kMetaTileBytes / 16; i += blockDim.x) {
+            const int a = i / (kMetaTileBytes / 16);
+            reinterpret_cast<uint4 *>(tile + a * addend_bytes + meta_at)[i - a * (kMetaTileBytes / 16)] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncthreads();
     }
-    const int blk = (int)blockIdx.x - walks.nctas;   // rt * kkeep + slot
-    const int rt = blk / g.kkeep;
-    const int jb = mask_blk_col[blk];
-    const int groups = g.bk / M;
-    const int vpb = g.bm * groups * g.n;
-    const int idx_words = vpb * g.idx_bits / 32;
-    const int val_words = (vpb + 1) / 2;
-    uint32_t *s_idx = s_buf;                          // [idx_words]
-    uint16_t *s_val = reinterpret_cast<uint16_t *>(s_buf + idx_words);   // [vpb]
-    uint8_t *tile = reinterpret_cast<uint8_t *>(s_buf + idx_words + (vpb + 7) / 8 * 4);   // [entry_bytes], 16-byte aligned
-    for (int i = threadIdx.x; i < idx_words; i += blockDim.x) s_idx[i] = 0u;
-    if constexpr (TILE != 0)
-        for (uint32_t i = threadIdx.x; i < entry_bytes / 16; i += blockDim.x)
-            reinterpret_cast<uint4 *>(tile)[i] = make_uint4(0, 0, 0, 0);
-    if (threadIdx.x == 0) blk_col[blk] = jb;
-    __syncthreads();
-
-    // a thread takes eight consecutive elements of a row (one 16-byte load: two groups of 4 or one of 8)
-    constexpr int kGroupsPerLoad = 8 / M;
-    const int loads_per_row = g.bk / 8;
-    for (int li = threadIdx.x; li < g.bm * loads_per_row; li += blockDim.x) {
-      const int r = li / loads_per_row, c8 = li - r * loads_per_row;
-      const int64_t row = (int64_t)rt * g.bm + r;
-      const int64_t col8 = (int64_t)jb * g.bk + (int64_t)c8 * 8;
-      uint16_t v8[8];
-      load_group<8>(w, ld, g.rows, g.k, row, col8, vec_ok, v8);
-      const uint32_t bits8 = (nm_bits[row * g.wpr + (col8 >> 5)] >> (col8 & 31)) & 0xFFu;
+    const int groups = g.bk / M, vpb = g.bm * groups * N, bm_log2 = 31 - __clz(g.bm);
+    // a thread keeps its chunk column and goes down the rows, so that all addresses advance by constants
+    const int step = blockDim.x / c8n, c8 = threadIdx.x % c8n, row_first = threadIdx.x / c8n;
+    const int64_t col = (int64_t)jb * g.bk + 8 * c8;
+    const bool wide = L.vec_ok && col + 8 <= g.k;
+    const int64_t grow = (int64_t)st * kTileRows;
+    const uint8_t *bits_col = reinterpret_cast<const uint8_t *>(L.nm_bits + grow * g.wpr) + (col >> 3);
+    const uint16_t *w_col = L.w + grow * L.ld + col;
+    uint8_t *const tile_col = tile + (kSparse ? (c8 >> 1) * kPlane + (c8 & 1) * 8 : c8 * kPlane);
+    const uint32_t meta_col = meta_at + (8 * ((c8 >> 1) & 1) * 4 + (c8 >> 2)) * 4 + (c8 & 1);
+    for (int row0 = row_first < step ? row_first : kTileRows; row0 < kTileRows; row0 += kUnroll * step) {
+        uint4 wv[kUnroll];
+        uint32_t bits[kUnroll];
 #pragma unroll
-      for (int sub = 0; sub < kGroupsPerLoad; ++sub) {
-        const int gi = c8 * kGroupsPerLoad + sub;
-        const int item = r * groups + gi;
-        const uint16_t *v = v8 + sub * M;
-        const uint32_t bits = (bits8 >> (sub * M)) & ((1u << M) - 1u);
-        if constexpr (TILE == CRISP_PATH_DENSE) {
+        for (int u = 0; u < kUnroll; ++u) {
+            const int row = row0 + u * step;
+            wv[u] = make_uint4(0u, 0u, 0u, 0u);
+            bits[u] = 0u;
+            if (row < kTileRows && s_slot[row >> bm_log2] >= 0) {
+                bits[u] = bits_col[(int64_t)row * g.wpr * 4];
+                if (grow + row < g.rows) {
+                    const uint16_t *p = w_col + row * L.ld;
+                    if (wide) {
+                        wv[u] = __ldg(reinterpret_cast<const uint4 *>(p));
+                    } else {
+                        uint32_t e[8];
 #pragma unroll
-            for (int t = 0; t < M; ++t)
-                if ((bits >> t) & 1u) {
-                    const int k = gi * M + t;
-                    *reinterpret_cast<uint16_t *>(tile + (k >> 3) * 2048 + r * 16 + (k & 7) * 2) = v[t];
+                        for (int t = 0; t < 8; ++t) e[t] = col + t < g.k ? (uint32_t)__ldg(p + t) : 0u;
+                        wv[u] = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+                    }
                 }
-        } else if constexpr (TILE == CRISP_PATH_SPARSE) {
-            uint32_t *meta = reinterpret_cast<uint32_t *>(tile + a_bytes);
+            }
+        }
 #pragma unroll
-            for (int q = 0; q < M / 4; ++q) {                // aligned 4-groups: at most two kept values each
-                const uint32_t qb = (bits >> (4 * q)) & 0xFu;
-                int p0 = 0, p1 = 1;
-                uint16_t v0 = 0, v1 = 0;
-                if (qb) {
-                    const int first = __ffs(qb) - 1;
-                    const uint32_t rest = qb & (qb - 1);
-                    if (rest) { p0 = first; v0 = v[4 * q + first]; p1 = __ffs(rest) - 1; v1 = v[4 * q + p1]; }
-                    else if (first == 3) { p0 = 0; p1 = 3; v1 = v[4 * q + 3]; }
-                    else { p0 = first; v0 = v[4 * q + first]; p1 = 3; }
+        for (int u = 0; u < kUnroll; ++u) {
+            const int row = row0 + u * step;
+            if (row >= kTileRows) break;
+            const uint32_t n0 = bits[u] & 15u, n1 = bits[u] >> 4;
+            const uint4 t0 = s_lut[n0], t1 = s_lut[n1];
+            const int sub = row >> bm_log2, slot = s_slot[sub];
+            if (slot >= 0) {
+                // canonical: V values and V offset fields, in ascending position
+                unsigned long long lo = (unsigned long long)__byte_perm(wv[u].x, wv[u].y, t0.x & 0xFFFFu) |
+                                        ((unsigned long long)__byte_perm(wv[u].x, wv[u].y, t0.x >> 16) << 32);
+                const unsigned long long q = (unsigned long long)__byte_perm(wv[u].z, wv[u].w, t1.x & 0xFFFFu) |
+                                             ((unsigned long long)__byte_perm(wv[u].z, wv[u].w, t1.x >> 16) << 32);
+                const int n_lo = M == 4 ? N : (int)(t0.y >> 24);                        // values of the first 4-group
+                unsigned long long hi = q;
+                if (n_lo != 4) {
+                    const int sh = 16 * (n_lo & 3);
+                    lo = (lo & ((1ull << sh) - 1ull)) | (q << sh);
+                    hi = q >> 1 >> (63 - sh);
                 }
-                const int k0 = gi * M + 4 * q, c0 = k0 >> 1;  // compressed column of the first slot (even)
-                *reinterpret_cast<uint32_t *>(tile + (c0 >> 3) * 2048 + r * 16 + (c0 & 7) * 2) =
-                    (uint32_t)v0 | ((uint32_t)v1 << 16);
-                const int lrow = (r & 7) + 8 * ((k0 >> 4) & 1) + 16 * (r >> 4);
-                atomicOr(&meta[lrow * 4 + (k0 >> 5)], ((uint32_t)p0 | ((uint32_t)p1 << 2)) << ((k0 & 15) + 16 * ((r >> 3) & 1)));
-            }
-        }
-        // values in ascending position; the group's offsets are gathered in a register and merged into
-        // the shared bit stream with one atomic (two if the field straddles a word)
-        constexpr int kIdxBits = M == 4 ? 2 : 3;
-        int o = item * g.n;
-        const int bit0 = o * kIdxBits;
-        uint32_t field = 0u;
-        int cnt = 0;
+                uint16_t *vout = L.vals + (int64_t)((first_rt + sub) * g.kkeep + slot) * vpb + ((row & (g.bm - 1)) * c8n + c8) * V;
+                if constexpr (V == 8) {
+                    *reinterpret_cast<uint4 *>(vout) = make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+                } else if constexpr (V == 4) {
+                    *reinterpret_cast<uint2 *>(vout) = make_uint2((uint32_t)lo, (uint32_t)(lo >> 32));
+                } else if constexpr (V % 2 == 0) {
 #pragma unroll
-        for (int t = 0; t < M; ++t) {
-            if ((bits >> t) & 1u) {
-                s_val[o + cnt] = v[t];
-                field |= (uint32_t)t << (kIdxBits * cnt);
-                ++cnt;
-            }
-        }
-        if (field) {
-            const int sh = bit0 & 31;
-            atomicOr(&s_idx[bit0 >> 5], field << sh);
-            if (sh + kIdxBits * cnt > 32) atomicOr(&s_idx[(bit0 >> 5) + 1], field >> (32 - sh));
-        }
-      }
-    }
-    __syncthreads();
-    // vals_per_block is a multiple of 32 values = 64 bytes, the block's slice starts 64-byte aligned
-    uint32_t *vout = reinterpret_cast<uint32_t *>(vals + (int64_t)blk * vpb);
-    const uint32_t *s_val32 = reinterpret_cast<const uint32_t *>(s_val);
-    for (int i = threadIdx.x; i < val_words; i += blockDim.x) vout[i] = s_val32[i];
-    uint32_t *iout = idx + (int64_t)blk * idx_words;
-    for (int i = threadIdx.x; i < idx_words; i += blockDim.x) iout[i] = s_idx[i];
-    if constexpr (TILE != 0) {
-        // with 128-row blocks the walk list of a CTA tile is its row tile's kept list: entry = blk
-        uint4 *out = reinterpret_cast<uint4 *>(image + (int64_t)blk * entry_bytes);
-        for (uint32_t i = threadIdx.x; i < entry_bytes / 16; i += blockDim.x) out[i] = reinterpret_cast<uint4 *>(tile)[i];
-    }
-}
-
-// Fast path of encode_block_kernel for groups of 4 with one or two kept values (1:4, 2:4) and blocks 64 or 128
-// elements deep, which is what the large layers use.  Everything a 4-group needs follows from its four mask
-// bits, so it is looked up: a 16-entry table (built per CTA) gives, per nibble, the byte-permute selector that
-// picks the two kept bf16 values out of the group's two registers, which of the two slots carry a value, the 2:4
-// metadata nibble and the offset field.  Values, offsets, tile slots and metadata are then assembled in
-// registers, combined across the lanes that share a 32-bit word with shuffles, and stored once: no shared-memory
-// atomics, no zero-filling, a fraction of the instructions of the general kernel (which was bound by instruction
-// issue).  Rows are visited so that rows r and r + 8 (whose metadata shares words) sit in the same warp.
-// Output identical to encode_block_kernel's.  TILE: 0 or CRISP_PATH_SPARSE (128-row blocks).
-template <int N, int TILE>
-__global__ void __launch_bounds__(256, 8)
-encode_block_m4_kernel(const uint16_t *__restrict__ w, int64_t ld, Geometry g, const int32_t *__restrict__ mask_blk_col,
-                       const uint32_t *__restrict__ nm_bits, int32_t *__restrict__ blk_col, uint16_t *__restrict__ vals,
-                       uint32_t *__restrict__ idx, uint8_t *__restrict__ image, uint32_t a_bytes, uint32_t entry_bytes,
-                       WalkArgs walks) {
-    extern __shared__ uint32_t s_buf[];
-    __shared__ uint32_t s_lut[16], s_lut_mask[16];
-    clear_header(walks);
-    if ((int)blockIdx.x < walks.nctas) {
-        __shared__ WalkShared s_walks;
-        build_walks_body(g, walks, blockIdx.x, s_walks);
-        return;
-    }
-    if (threadIdx.x < 16) {
-        // nibble -> slots (a, b), their validity, metadata nibble, first kept position
-        const uint32_t nib = threadIdx.x;
-        int a = 0, b = 1, va = 0, vb = 0, first = 0;
-        if (nib) {
-            first = __ffs(nib) - 1;
-            const uint32_t rest = nib & (nib - 1);
-            if (rest) { a = first; va = 1; b = __ffs(rest) - 1; vb = 1; }
-            else if (first == 3) { a = 0; b = 3; vb = 1; }
-            else { a = first; va = 1; b = 3; }
-        }
-        const uint32_t sel = (uint32_t)(2 * a) | ((uint32_t)(2 * a + 1) << 4) | ((uint32_t)(2 * b) << 8) | ((uint32_t)(2 * b + 1) << 12);
-        s_lut[nib] = sel | ((uint32_t)(a | (b << 2)) << 16) | ((uint32_t)first << 20);
-        s_lut_mask[nib] = (va ? 0x0000FFFFu : 0u) | (vb ? 0xFFFF0000u : 0u);
-    }
-    const int blk = (int)blockIdx.x - walks.nctas;    // rt * kkeep + slot
-    const int rt = blk / g.kkeep;
-    const int jb = mask_blk_col[blk];
-    const int groups = g.bk / 4;
-    const int vpb = g.bm * groups * N;
-    const int idx_words = vpb * 2 / 32;
-    const int val_words = vpb / 2;
-    uint32_t *s_idx = s_buf;                                                        // [idx_words]
-    uint32_t *s_val32 = s_buf + idx_words;                                          // [vpb / 2]
-    uint8_t *tile = reinterpret_cast<uint8_t *>(s_buf + idx_words + (vpb + 7) / 8 * 4);   // [entry_bytes], 16-byte aligned
-    if (threadIdx.x == 0) blk_col[blk] = jb;
-    if constexpr (TILE == CRISP_PATH_SPARSE)           // metadata words beyond block_k / 32 per row are never written
-        for (uint32_t i = threadIdx.x; i < (entry_bytes - a_bytes) / 16; i += blockDim.x)
-            reinterpret_cast<uint4 *>(tile + a_bytes)[i] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-
-    const int L = g.bk / 8;                            // 16-byte loads per row: 8 or 16
-    const int lshift = L == 8 ? 3 : 4;
-    for (int li = threadIdx.x; li < g.bm * L; li += blockDim.x) {
-        const int q = li >> lshift, c8 = li & (L - 1);
-        const int r = ((q & 1) << 3) | ((q >> 1) & 7) | (q & ~15);      // rows q, q ^ 1 of the walk are r, r ^ 8
-        const int64_t row = (int64_t)rt * g.bm + r;
-        const int64_t col8 = (int64_t)jb * g.bk + (int64_t)c8 * 8;
-        uint32_t wv[4] = {0u, 0u, 0u, 0u};
-        if (row < g.rows && col8 + 8 <= g.k) {
-            const uint4 t = __ldg(reinterpret_cast<const uint4 *>(w + row * ld + col8));
-            wv[0] = t.x; wv[1] = t.y; wv[2] = t.z; wv[3] = t.w;
-        } else if (row < g.rows && col8 < g.k) {
-            uint16_t v8[8];
-            load_group<8>(w, ld, g.rows, g.k, row, col8, false, v8);
+                    for (int j = 0; j < V; j += 2)
+                        *reinterpret_cast<uint32_t *>(vout + j) = (uint32_t)((j < 4 ? lo : hi) >> (16 * (j & 3)));
+                } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) wv[i] = (uint32_t)v8[2 * i] | ((uint32_t)v8[2 * i + 1] << 16);
-        }
-        const uint32_t bits8 = (nm_bits[row * g.wpr + (col8 >> 5)] >> (col8 & 31)) & 0xFFu;
-        const uint32_t e0 = s_lut[bits8 & 15u], e1 = s_lut[bits8 >> 4];
-        const uint32_t p0 = __byte_perm(wv[0], wv[1], e0 & 0xFFFFu) & s_lut_mask[bits8 & 15u];
-        const uint32_t p1 = __byte_perm(wv[2], wv[3], e1 & 0xFFFFu) & s_lut_mask[bits8 >> 4];
-        const int item0 = r * groups + 2 * c8;                          // the thread's two groups: item0, item0 + 1
-        if constexpr (TILE == CRISP_PATH_SPARSE) {
-            // slot pairs of the two 4-groups: compressed columns 4 * c8 .. 4 * c8 + 3, one 8-byte store
-            *reinterpret_cast<uint2 *>(tile + (c8 >> 1) * 2048 + r * 16 + (c8 & 1) * 8) = make_uint2(p0, p1);
-            // metadata: this thread's two nibbles, the neighbour's (other half of the 16-element chunk) and those
-            // of row r ^ 8 make one 32-bit word
-            uint32_t mv = (((e0 >> 16) & 15u) | (((e1 >> 16) & 15u) << 4)) << (8 * (c8 & 1) + 16 * (q & 1));
-            mv |= __shfl_xor_sync(0xFFFFFFFFu, mv, 1);
-            mv |= __shfl_xor_sync(0xFFFFFFFFu, mv, L);
-            if (((c8 | q) & 1) == 0) {
-                const int lrow = (r & 7) + 8 * ((c8 >> 1) & 1) + 16 * (r >> 4);
-                reinterpret_cast<uint32_t *>(tile + a_bytes)[lrow * 4 + (c8 >> 2)] = mv;
+                    for (int j = 0; j < V; ++j) vout[j] = (uint16_t)((j < 4 ? lo : hi) >> (16 * (j & 3)));
+                }
+                uint32_t field;
+                if constexpr (M == 4) field = (t0.z & 0xFFu) | ((t1.z & 0xFFu) << (2 * N));
+                else                                         // bit 2 of every field of the second 4-group: + 4 each
+                    field = (t0.z >> 16) | (((t1.z >> 16) | (0x924u & ((1u << (3 * (t1.y >> 24))) - 1u))) << (3 * n_lo));
+                s_field[row * c8n + c8] = field;
             }
-        }
-        if constexpr (N == 2) {
-            // both values of a group are kept values in ascending position: the slot pair is the canonical pair
-            *reinterpret_cast<uint2 *>(s_val32 + item0) = make_uint2(p0, p1);
-            uint32_t f = (((e0 >> 16) & 15u) | (((e1 >> 16) & 15u) << 4)) << (8 * (c8 & 3));
-            f |= __shfl_xor_sync(0xFFFFFFFFu, f, 1);
-            f |= __shfl_xor_sync(0xFFFFFFFFu, f, 2);
-            if ((c8 & 3) == 0) s_idx[(item0 >> 3)] = f;                  // 4 bits per group: 8 groups per word
-        } else {
-            // one kept value per group: it sits in slot 0, or in slot 1 when it is the group's last element
-            const uint32_t v0 = (p0 & 0xFFFFu) | (p0 >> 16), v1 = (p1 & 0xFFFFu) | (p1 >> 16);
-            s_val32[item0 >> 1] = v0 | (v1 << 16);
-            uint32_t f = (((e0 >> 20) & 3u) | (((e1 >> 20) & 3u) << 2)) << (4 * (c8 & 7));
-            f |= __shfl_xor_sync(0xFFFFFFFFu, f, 1);
-            f |= __shfl_xor_sync(0xFFFFFFFFu, f, 2);
-            f |= __shfl_xor_sync(0xFFFFFFFFu, f, 4);
-            if ((c8 & 7) == 0) s_idx[(item0 >> 4)] = f;                  // 2 bits per group: 16 groups per word
+            if constexpr (!kSparse) {
+                if (image)
+                    *reinterpret_cast<uint4 *>(tile_col + row * 16) =
+                        make_uint4(wv[u].x & half_mask(n0), wv[u].y & half_mask(n0 >> 2), wv[u].z & half_mask(n1), wv[u].w & half_mask(n1 >> 2));
+            } else {
+                const uint32_t meta_row = ((row & 7) + 16 * (row >> 4)) * 16 + 2 * ((row >> 3) & 1);
+                auto slots = [&](int a, const uint4 &e0, const uint4 &e1) {
+                    const uint32_t p0 = __byte_perm(wv[u].x, wv[u].y, e0.y & 0xFFFFu) & e0.w;
+                    const uint32_t p1 = __byte_perm(wv[u].z, wv[u].w, e1.y & 0xFFFFu) & e1.w;
+                    *reinterpret_cast<uint2 *>(tile_col + a * addend_bytes + row * 16) = make_uint2(p0, p1);
+                    tile[a * addend_bytes + meta_col + meta_row] = (uint8_t)(((e0.y >> 16) & 15u) | (((e1.y >> 16) & 15u) << 4));
+                };
+                if constexpr (N <= 2) slots(0, t0, t1);
+                else {                                       // the first two values of a 4-group, then the rest
+                    const uint32_t r0 = n0 & (n0 - 1), r1 = n1 & (n1 - 1);
+                    const uint32_t s0 = r0 & (r0 - 1), s1 = r1 & (r1 - 1);
+                    slots(0, s_lut[n0 ^ s0], s_lut[n1 ^ s1]);
+                    slots(1, s_lut[s0], s_lut[s1]);
+                }
+            }
         }
     }
     __syncthreads();
-    uint32_t *vout = reinterpret_cast<uint32_t *>(vals + (int64_t)blk * vpb);
-    for (int i = threadIdx.x; i < val_words; i += blockDim.x) vout[i] = s_val32[i];
-    uint32_t *iout = idx + (int64_t)blk * idx_words;
-    for (int i = threadIdx.x; i < idx_words; i += blockDim.x) iout[i] = s_idx[i];
-    if constexpr (TILE != 0) {
-        uint4 *out = reinterpret_cast<uint4 *>(image + (int64_t)blk * entry_bytes);
-        for (uint32_t i = threadIdx.x; i < entry_bytes / 16; i += blockDim.x) out[i] = reinterpret_cast<uint4 *>(tile)[i];
+    // offsets: word w of a block's bit stream holds the fields of chunks from 32 w / kFieldBits on
+    const int words = vpb * kIdxBits / 32, block_chunks = g.bm * c8n;
+    for (int sub = 0; sub < n_rt; ++sub) {
+        if (s_slot[sub] < 0) continue;
+        uint32_t *iout = L.idx + ((int64_t)(first_rt + sub) * g.kkeep + s_slot[sub]) * words;
+        const uint32_t *f = s_field + sub * block_chunks;
+        for (int w = threadIdx.x; w < words; w += blockDim.x) {
+            int c = 32 * w / kFieldBits, at = c * kFieldBits - 32 * w;
+            uint32_t v = 0u;
+#pragma unroll
+            for (int j = 0; j < (31 + kFieldBits - 1) / kFieldBits + 1; ++j, ++c, at += kFieldBits)
+                if (at < 32 && c < block_chunks) v |= at >= 0 ? f[c] << at : f[c] >> -at;
+            iout[w] = v;
+        }
+    }
+    if (!image) return;
+    const int window = kTileRows / L.stack;                  // rows a copy of a stacked image carries
+    for (int q = 0; q < L.stack; ++q) {
+        const int shift = q * window;
+        for (int a = 0; a < addends; ++a) {
+            const uint8_t *ta = tile + a * addend_bytes;
+            uint4 *out = reinterpret_cast<uint4 *>(L.image + ((int64_t)(q * L.nst + st) * L.wcap + entry) * L.entry_bytes +
+                                                   (int64_t)a * (L.a_bytes + kMetaTileBytes));
+            for (int i = threadIdx.x; i < planes * kTileRows; i += blockDim.x) {
+                const int src = (i & (kTileRows - 1)) - shift;
+                out[i] = src >= 0 && src < window ? *reinterpret_cast<const uint4 *>(ta + (i >> 7) * kPlane + src * 16) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            if constexpr (kSparse) {
+                const uint32_t pad = 0x44444444u;
+                for (int i = threadIdx.x; i < kMetaTileBytes / 16; i += blockDim.x) {
+                    const int src = i - shift;
+                    out[planes * kTileRows + i] = src >= 0 && src < window
+                        ? *reinterpret_cast<const uint4 *>(ta + meta_at + src * 16)
+                        : make_uint4(pad, g.bk > 32 ? pad : 0u, g.bk > 64 ? pad : 0u, g.bk > 96 ? pad : 0u);
+                }
+            }
+        }
     }
 }
 
@@ -360,58 +368,93 @@ decode_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *_
 
 }  // namespace
 
-cudaError_t launch_encode_canonical(const uint16_t *d_w, int64_t ld, const Geometry &g,
-                                    const int32_t *d_mask_blk_col, const uint32_t *d_nm_bits,
-                                    int32_t *d_blk_col, uint16_t *d_vals, uint32_t *d_idx,
-                                    int tile_kind, uint8_t *d_image, uint32_t a_bytes, uint32_t entry_bytes,
-                                    const WalkArgs *walks, cudaStream_t st) {
-    const int nblocks = g.nrt * g.kkeep;
-    if (nblocks == 0) return cudaSuccess;
-    WalkArgs wa = {};
-    if (walks) wa = *walks;
-    const size_t vpb = (size_t)g.vals_per_block();
-    size_t smem = (vpb * g.idx_bits / 32) * sizeof(uint32_t) + (vpb + 7) / 8 * 16 + 16;
-    if (tile_kind != 0) smem += entry_bytes;
-    // the 16-byte loads of eight elements need every row to start 16-byte aligned (block columns are multiples of 32)
-    const size_t gbytes = 16;
-    const bool vec_ok = (reinterpret_cast<uintptr_t>(d_w) % gbytes == 0) && ((size_t)ld * 2 % gbytes == 0);
-#define CRISP_ENCODE_LAUNCH(MV, TV)                                                                          \
-    do {                                                                                                     \
-        auto kern = encode_block_kernel<MV, TV>;                                                             \
-        if (smem > 48 * 1024) {                                                                              \
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-            if (e != cudaSuccess) return e;                                                                  \
-        }                                                                                                    \
-        kern<<<nblocks + wa.nctas, 256, smem, st>>>(d_w, ld, g, vec_ok, d_mask_blk_col, d_nm_bits, d_blk_col, \
-                                                     d_vals, d_idx, d_image, a_bytes, entry_bytes, wa);      \
-    } while (0)
-    // groups of 4 with one or two kept values, 64- or 128-deep blocks, 16-byte aligned rows: the table-driven kernel
-    const bool fast = g.m == 4 && g.n <= 2 && (g.bk == 64 || g.bk == 128) && vec_ok && tile_kind != CRISP_PATH_DENSE;
-#define CRISP_ENCODE_FAST(NV, TV)                                                                            \
-    do {                                                                                                     \
-        auto kern = encode_block_m4_kernel<NV, TV>;                                                          \
-        if (smem > 48 * 1024) {                                                                              \
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-            if (e != cudaSuccess) return e;                                                                  \
-        }                                                                                                    \
-        kern<<<nblocks + wa.nctas, 256, smem, st>>>(d_w, ld, g, d_mask_blk_col, d_nm_bits, d_blk_col, d_vals,  \
-                                                    d_idx, d_image, a_bytes, entry_bytes, wa);               \
-    } while (0)
-    if (fast) {
-        if (g.n == 2) { if (tile_kind == CRISP_PATH_SPARSE) CRISP_ENCODE_FAST(2, CRISP_PATH_SPARSE); else CRISP_ENCODE_FAST(2, 0); }
-        else { if (tile_kind == CRISP_PATH_SPARSE) CRISP_ENCODE_FAST(1, CRISP_PATH_SPARSE); else CRISP_ENCODE_FAST(1, 0); }
-    } else if (g.m == 4) {
-        if (tile_kind == CRISP_PATH_SPARSE) CRISP_ENCODE_LAUNCH(4, CRISP_PATH_SPARSE);
-        else if (tile_kind == CRISP_PATH_DENSE) CRISP_ENCODE_LAUNCH(4, CRISP_PATH_DENSE);
-        else CRISP_ENCODE_LAUNCH(4, 0);
-    } else {
-        if (tile_kind == CRISP_PATH_SPARSE) CRISP_ENCODE_LAUNCH(8, CRISP_PATH_SPARSE);
-        else if (tile_kind == CRISP_PATH_DENSE) CRISP_ENCODE_LAUNCH(8, CRISP_PATH_DENSE);
-        else CRISP_ENCODE_LAUNCH(8, 0);
+namespace {
+
+size_t encode_smem(const EncodeLayer &L) {
+    const size_t c8n = (size_t)L.g.bk / 8, fields = kTileRows * c8n * 4;
+    switch (L.kind) {
+        case CRISP_PATH_DENSE: return c8n * 2064 + fields;
+        case CRISP_PATH_SPARSE: return c8n / 2 * 2080 + kMetaTileBytes + fields;
+        case CRISP_PATH_SPARSE2: return 2 * (c8n / 2 * 2080 + kMetaTileBytes) + fields;
+        default: return fields;
     }
-#undef CRISP_ENCODE_LAUNCH
-#undef CRISP_ENCODE_FAST
+}
+
+template <int M, int N, int IMAGE, int CAP>
+cudaError_t run_encode_image(const Batch<EncodeLayer, CAP> &b, cudaStream_t st) {
+    size_t smem = 0;
+    for (int i = 0; i < b.n; ++i) smem = encode_smem(b.layer[i]) > smem ? encode_smem(b.layer[i]) : smem;
+    if (smem > 40 * 1024) {          // (the kernel's own arrays take some of the default 48 KB)
+        cudaError_t e = cudaFuncSetAttribute(encode_kernel<M, N, IMAGE, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    if (b.first[b.n] == 0) return cudaSuccess;
+    if (b.first[b.n] > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+    encode_kernel<M, N, IMAGE, CAP><<<(unsigned)b.first[b.n], 256, smem, st>>>(b);
     return cudaGetLastError();
+}
+template <int M, int N, int CAP>
+cudaError_t run_encode(const Batch<EncodeLayer, CAP> &b, cudaStream_t st) {
+    // (one addend for n <= 2, two beyond: the kind follows from n, or is dense or none for all layers)
+    if (b.layer[0].kind == CRISP_PATH_SPARSE || b.layer[0].kind == CRISP_PATH_SPARSE2)
+        return run_encode_image<M, N, CRISP_PATH_SPARSE, CAP>(b, st);
+    return run_encode_image<M, N, CRISP_PATH_DENSE, CAP>(b, st);
+}
+
+template <int CAP>
+cudaError_t run_encode_any(const Batch<EncodeLayer, CAP> &b, cudaStream_t st) {
+    const int n = b.layer[0].g.n;
+    if (b.layer[0].g.m == 4) {
+        switch (n) {
+            case 1: return run_encode<4, 1, CAP>(b, st);
+            case 2: return run_encode<4, 2, CAP>(b, st);
+            case 3: return run_encode<4, 3, CAP>(b, st);
+            case 4: return run_encode<4, 4, CAP>(b, st);
+        }
+    } else {
+        switch (n) {
+            case 1: return run_encode<8, 1, CAP>(b, st);
+            case 2: return run_encode<8, 2, CAP>(b, st);
+            case 3: return run_encode<8, 3, CAP>(b, st);
+            case 4: return run_encode<8, 4, CAP>(b, st);
+            case 5: return run_encode<8, 5, CAP>(b, st);
+            case 6: return run_encode<8, 6, CAP>(b, st);
+            case 7: return run_encode<8, 7, CAP>(b, st);
+            case 8: return run_encode<8, 8, CAP>(b, st);
+        }
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <int CAP>
+cudaError_t encode_batch(const EncodeLayer *layers, int n, cudaStream_t st) {
+    Batch<EncodeLayer, CAP> b;
+    b.n = 0;
+    b.first[0] = 0;
+    for (int i = 0; i < n; ++i) {
+        const Geometry &g = layers[i].g;
+        if (g.nrt * g.kkeep == 0) continue;                  // nothing kept: nothing to write
+        EncodeLayer &L = b.layer[b.n];
+        L = layers[i];
+        // the 16-byte loads of eight elements need every row to start 16-byte aligned (block columns are multiples of 32)
+        L.vec_ok = reinterpret_cast<uintptr_t>(L.w) % 16 == 0 && L.ld % 8 == 0;
+        const int64_t tiles = (g.mp() + kTileRows - 1) / kTileRows;
+        const int64_t entries = (int64_t)(kTileRows / g.bm) * g.kkeep;
+        b.first[b.n + 1] = b.first[b.n] + tiles * (entries < g.nblk ? entries : g.nblk);
+        ++b.n;
+    }
+    return b.n ? run_encode_any<CAP>(b, st) : cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t launch_encode(const EncodeLayer *layers, int n, cudaStream_t st) {
+    if (n == 1) return encode_batch<1>(layers, 1, st);
+    for (int at = 0; at < n; at += kBatchLayers) {
+        cudaError_t e = encode_batch<kBatchLayers>(layers + at, n - at < kBatchLayers ? n - at : kBatchLayers, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_decode(const Geometry &g, const int32_t *d_blk_col, const uint16_t *d_vals,

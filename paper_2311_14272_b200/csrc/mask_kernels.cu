@@ -9,22 +9,13 @@
 //         bits of the pruned ones (blocks keep their positions)
 // Coalesced 32-byte-per-lane accesses; K-M1a is bound by HBM bandwidth.
 #include "crisp_internal.h"
+#include "mask_common.cuh"
 
 namespace crisp {
 
 namespace {
 
 constexpr int kScoreFractionBits = 40;
-constexpr int kM1Threads = 256;
-constexpr int kM1ChunkK = 256;           // k-elements covered by one warp pass (32 lanes x 8)
-
-// |s| as an order-preserving uint32 key: NaN -> 0, Inf -> FLT_MAX.
-__device__ __forceinline__ uint32_t canonical_key(float s) {
-    uint32_t u = __float_as_uint(s) & 0x7FFFFFFFu;
-    if (u > 0x7F800000u) return 0u;
-    if (u == 0x7F800000u) return 0x7F7FFFFFu;
-    return u;
-}
 
 // Raw bits of eight consecutive saliency values; the caller guarantees row < rows, k0 + 8 <= k and
 // 16-byte alignment.  Kept free of branches so that several of these can be in flight per lane.
@@ -35,12 +26,6 @@ __device__ __forceinline__ void load8_raw(const float *__restrict__ s, int64_t l
     key[0] = a.x; key[1] = a.y; key[2] = a.z; key[3] = a.w;
     key[4] = b.x; key[5] = b.y; key[6] = b.z; key[7] = b.w;
 }
-// |s| with NaN -> 0 and Inf -> FLT_MAX in two instructions: max(|s|, 0) drops a NaN (the maximum of a NaN and a
-// number is the number), min(., FLT_MAX) caps infinity; -0 becomes +0, denormals pass unchanged.
-__device__ __forceinline__ uint32_t canonical_bits(uint32_t u) {
-    return __float_as_uint(fminf(fmaxf(fabsf(__uint_as_float(u)), 0.f), 3.402823466e+38f));
-}
-
 // Eight consecutive saliency values of one row, zero beyond the matrix.
 __device__ __forceinline__ void load8(const float *__restrict__ s, int64_t ld, int rows, int k,
                                       int64_t row, int64_t k0, bool vec_ok, uint32_t key[8]) {
@@ -78,62 +63,6 @@ __device__ __forceinline__ unsigned long long fixed_point_score(uint32_t key, in
     const uint32_t down = mant >> min(max(-sh, 0), 31);                          // mant < 2^24: shifts >= 24 give 0
     const int up = max(sh, 0);                                                   // only one of the two shifts is non-zero
     return ((unsigned long long)__funnelshift_l(down, 0u, up) << 32) | (unsigned long long)(down << up);
-}
-
-// Bit i of the result is set iff element i is among the N largest of its group of M
-// (ties to the lower index).  M is 4 or 8; the 8 keys hold two groups or one.
-// For i < j, element i beats element j iff key[i] >= key[j].
-template <int M>
-__device__ __forceinline__ uint32_t top_n_bits(const uint32_t key[8], int n) {
-    uint32_t bits = 0u;
-#pragma unroll
-    for (int g = 0; g < 8 / M; ++g) {
-        int rank[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) rank[i] = 0;
-#pragma unroll
-        for (int i = 0; i < M; ++i)
-#pragma unroll
-            for (int j = i + 1; j < M; ++j) {
-                const int i_wins = key[g * M + i] >= key[g * M + j];
-                rank[j] += i_wins;
-                rank[i] += 1 - i_wins;
-            }
-#pragma unroll
-        for (int i = 0; i < M; ++i) bits |= (rank[i] < n ? 1u : 0u) << (g * M + i);
-    }
-    return bits;
-}
-
-// Groups of 4: the six pairwise outcomes index a 64-entry table of keep masks (built per CTA for
-// the layer's n by keep_mask_of_outcomes), which replaces the rank arithmetic.
-__device__ __forceinline__ uint32_t outcomes4(const uint32_t *k) {
-    return (uint32_t)(k[0] >= k[1]) | ((uint32_t)(k[0] >= k[2]) << 1) | ((uint32_t)(k[0] >= k[3]) << 2) |
-           ((uint32_t)(k[1] >= k[2]) << 3) | ((uint32_t)(k[1] >= k[3]) << 4) | ((uint32_t)(k[2] >= k[3]) << 5);
-}
-__device__ __forceinline__ uint32_t keep_mask_of_outcomes(uint32_t o, int n) {
-    const int w01 = o & 1, w02 = (o >> 1) & 1, w03 = (o >> 2) & 1, w12 = (o >> 3) & 1, w13 = (o >> 4) & 1,
-              w23 = (o >> 5) & 1;
-    const int r0 = (1 - w01) + (1 - w02) + (1 - w03);
-    const int r1 = w01 + (1 - w12) + (1 - w13);
-    const int r2 = w02 + w12 + (1 - w23);
-    const int r3 = w03 + w13 + w23;
-    return (uint32_t)(r0 < n) | ((uint32_t)(r1 < n) << 1) | ((uint32_t)(r2 < n) << 2) | ((uint32_t)(r3 < n) << 3);
-}
-
-constexpr int kM1Rows = 32;              // rows per work item of K-M1a / K-M1b (divides every block height)
-constexpr int kM1RowsPerWarp = kM1Rows / (kM1Threads / 32);
-
-// One work item = 32 rows x 256 k-elements.  Warp w takes rows 4w..4w+3 (all loads issued first); lane l owns
-// the 8 elements at k = chunk*256 + 8*l of each row, so a lane stays inside one block column.  Items are dealt
-// out to a grid of resident CTAs (grid-stride), chunk fastest, so that a CTA streams along rows.
-struct M1Item { int64_t row0; int chunk; };
-__device__ __forceinline__ M1Item m1_item(int64_t it, int chunks) {
-    M1Item x;
-    const int64_t rg = it / chunks;
-    x.chunk = (int)(it - rg * chunks);
-    x.row0 = rg * kM1Rows;
-    return x;
 }
 
 // The 8 canonical keys of the lane's elements of row `row` (zero beyond the matrix).
@@ -236,25 +165,30 @@ __device__ __forceinline__ void floor_parts2(uint64_t v, uint64_t &r, uint64_t &
 // byte K-M1a stored, or all of them) over its warp's four rows, the four lanes of a 32-element word add up
 // (a mask word never straddles a block: block_k is a multiple of 32), and one lane per word adds the partial
 // score to the block's 64-bit total with an atomic (integer addition: any order gives the same sum).
+template <int CAP>
 __global__ void __launch_bounds__(kM1Threads)
-block_score_kernel(const float *__restrict__ s, int64_t ld, Geometry g, bool vec_ok, int64_t items, int chunks,
-                   const uint32_t *__restrict__ max_key, const uint32_t *__restrict__ nm_bits,
-                   unsigned long long *__restrict__ score) {
+block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t mk = *max_key;
-    if (!mk) return;                                         // an all-zero layer: every score stays 0
+    for (int64_t unit = blockIdx.x; unit < batch.first[batch.n]; unit += gridDim.x) {
+    const int l = batch.find(unit);
+    const ScoreLayer &L = batch.layer[l];
+    const Geometry &g = L.g;
+    const float *__restrict__ s = L.s;
+    const int64_t ld = L.ld;
+    const uint32_t *__restrict__ nm_bits = L.nm_bits;
+    const uint32_t mk = *L.max_key;
+    if (!mk) continue;                                       // an all-zero layer: every score stays 0
     const int e_max = key_exponent(mk);
     // floor(value * 2^(40 - e_max)): when that power of two is an fp32 number, the product is exact
     // (value <= layer maximum, so it stays below 2^41)
     const int scale_exp = kScoreFractionBits - e_max;
     const bool float_scale = scale_exp >= -126 && scale_exp <= 127;
     const float scale = float_scale ? __uint_as_float((uint32_t)(127 + scale_exp) << 23) : 0.f;
-    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-        const M1Item x = m1_item(it, chunks);
+        const M1Item x = m1_item(unit - batch.first[l], L.chunks);
         const int64_t k0 = (int64_t)x.chunk * kM1ChunkK + lane * 8;
         const int rt = (int)(x.row0 / g.bm);
         uint32_t key[kM1RowsPerWarp][8];
-        m1_load_rows(s, ld, g, vec_ok, x, warp, k0, key);
+        m1_load_rows(s, ld, g, L.vec_ok != 0, x, warp, k0, key);
         const bool in_kp = k0 < g.kp();
         unsigned long long acc = 0ull;
         if (float_scale) {
@@ -296,23 +230,30 @@ block_score_kernel(const float *__restrict__ s, int64_t ld, Geometry g, bool vec
         const int grp = g.bk % 128 == 0 ? 15 : (g.bk % 64 == 0 ? 7 : 3);
         if ((lane & grp) == 0 && in_kp && acc) {
             const int jb = (int)(k0 / g.bk);
-            if (jb < g.nblk) atomicAdd(&score[(int64_t)rt * g.nblk + jb], acc);
+            if (jb < g.nblk) atomicAdd(&L.score[(int64_t)rt * g.nblk + jb], acc);
         }
     }
 }
 
-// K-M2.  grid = (row tiles, block_rows / 32).  Every CTA ranks its row tile's block scores (cheap)
-// and clears the mask words of pruned blocks in its own 32 rows; the CTA with blockIdx.y == 0 also
+// K-M2.  One CTA per 32 rows of a row tile.  Every CTA ranks its row tile's block scores (cheap)
+// and clears the mask words of pruned blocks in its own 32 rows; the first CTA of a row tile also
 // emits the kept columns in ascending order.
+template <int CAP>
 __global__ void __launch_bounds__(256)
-block_select_kernel(Geometry g, const unsigned long long *__restrict__ score,
-                    int32_t *__restrict__ blk_col, uint32_t *__restrict__ nm_bits) {
+block_select_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     extern __shared__ unsigned long long sm[];
+    const int l = batch.find(blockIdx.x);
+    const ScoreLayer &L = batch.layer[l];
+    const Geometry &g = L.g;
+    const unsigned long long *__restrict__ score = L.score;
+    int32_t *__restrict__ blk_col = L.blk_col;
+    uint32_t *__restrict__ nm_bits = L.nm_bits;
     unsigned long long *sc = sm;                                   // [nblk]
     int *kept = reinterpret_cast<int *>(sm + g.nblk);              // [nblk]
     __shared__ int s_warp_tot[8];
     __shared__ int s_base;
-    const int rt = blockIdx.x;
+    const int cta = (int)(blockIdx.x - batch.first[l]), slabs = g.bm / 32;
+    const int rt = cta / slabs, slab = cta - rt * slabs;
     for (int j = threadIdx.x; j < g.nblk; j += blockDim.x) sc[j] = score[(int64_t)rt * g.nblk + j];
     if (threadIdx.x == 0) s_base = 0;
     __syncthreads();
@@ -327,7 +268,7 @@ block_select_kernel(Geometry g, const unsigned long long *__restrict__ score,
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (blockIdx.y == 0) {
+    if (slab == 0) {
         // ascending compaction: block-wide exclusive scan over chunks of blockDim.x flags
         for (int j0 = 0; j0 < g.nblk; j0 += blockDim.x) {
             const int j = j0 + threadIdx.x;
@@ -350,10 +291,78 @@ block_select_kernel(Geometry g, const unsigned long long *__restrict__ score,
     // final mask = group bits AND block kept: one warp per row, lanes stride over the row's words
     const int wpb = g.bk / 32;
     for (int r = warp; r < 32; r += 8) {
-        uint32_t *row_words = nm_bits + ((int64_t)rt * g.bm + blockIdx.y * 32 + r) * g.wpr;
+        uint32_t *row_words = nm_bits + ((int64_t)rt * g.bm + slab * 32 + r) * g.wpr;
         for (int wc = lane; wc < g.wpr; wc += 32)
             if (!kept[wc / wpb]) row_words[wc] = 0u;
     }
+}
+
+// Scores and maxima of a batch, cleared (one CTA per layer; a memset per layer costs a launch each).
+template <int CAP>
+__global__ void __launch_bounds__(256)
+clear_scores_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
+    const ScoreLayer &L = batch.layer[blockIdx.x];
+    if (threadIdx.x == 0) *const_cast<uint32_t *>(L.max_key) = 0u;
+    const int64_t n = (int64_t)L.g.nrt * L.g.nblk;
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) L.score[i] = 0ull;
+}
+
+// Grids of resident CTAs: every CTA is on an SM from the start and takes its share of the items.
+int resident_grid(const void *kern, int64_t items) {
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        sms = 148;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kM1Threads, 0) != cudaSuccess || per_sm <= 0) per_sm = 4;
+    const int64_t cap = (int64_t)sms * per_sm;
+    return (int)(items < cap ? items : cap);
+}
+
+bool saliency_vec_ok(const float *s, int64_t ld) { return (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(s) & 15u) == 0); }
+int saliency_chunks(const Geometry &g) { return (int)((g.kp() + kM1ChunkK - 1) / kM1ChunkK); }
+
+// Layers [0, n) in launches of up to kBatchLayers; units(layer) = work units of a layer, launch(batch, units of the batch).
+template <typename Units, typename Launch>
+cudaError_t for_batches(const ScoreLayer *layers, int n, Units units, Launch launch) {
+    for (int at = 0; at < n; at += kBatchLayers) {
+        Batch<ScoreLayer, kBatchLayers> b;
+        b.n = n - at < kBatchLayers ? n - at : kBatchLayers;
+        b.first[0] = 0;
+        for (int i = 0; i < b.n; ++i) {
+            b.layer[i] = layers[at + i];
+            b.layer[i].chunks = saliency_chunks(b.layer[i].g);
+            b.layer[i].vec_ok = saliency_vec_ok(b.layer[i].s, b.layer[i].ld);
+            b.first[i + 1] = b.first[i] + units(b.layer[i].g);
+        }
+        if (b.first[b.n] > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+        cudaError_t e = launch(b);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+Batch<ScoreLayer, 1> batch_of_one(const ScoreLayer &L, int64_t units) {
+    Batch<ScoreLayer, 1> b;
+    b.n = 1; b.first[0] = 0; b.first[1] = units;
+    b.layer[0] = L;
+    b.layer[0].chunks = saliency_chunks(L.g);
+    b.layer[0].vec_ok = saliency_vec_ok(L.s, L.ld);
+    return b;
+}
+
+size_t select_smem(const Geometry &g) { return (size_t)g.nblk * (sizeof(unsigned long long) + sizeof(int)); }
+int64_t select_ctas(const Geometry &g) { return (int64_t)g.nrt * (g.bm / 32); }
+
+template <int CAP>
+cudaError_t run_block_select(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
+    size_t smem = 0;
+    for (int i = 0; i < b.n; ++i) smem = select_smem(b.layer[i].g) > smem ? select_smem(b.layer[i].g) : smem;
+    if (smem + 64 > 48 * 1024) {     // the longest rows (nblk near 4096) need the opt-in shared-memory size
+        cudaError_t e = cudaFuncSetAttribute(block_select_kernel<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    if (b.first[b.n] == 0) return cudaSuccess;
+    block_select_kernel<CAP><<<(unsigned)b.first[b.n], 256, smem, st>>>(b);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -363,17 +372,32 @@ size_t mask_workspace_bytes(const Geometry &g) {
     return kAlign + align_up((size_t)g.nrt * g.nblk * sizeof(unsigned long long));
 }
 
+cudaError_t launch_clear_scores(const ScoreLayer *layers, int n, cudaStream_t st) {
+    return for_batches(layers, n, [](const Geometry &) { return (int64_t)1; }, [&](const Batch<ScoreLayer, kBatchLayers> &b) {
+        clear_scores_kernel<kBatchLayers><<<(unsigned)b.n, 256, 0, st>>>(b);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t launch_block_scores(const ScoreLayer *layers, int n, cudaStream_t st) {
+    return for_batches(layers, n, [](const Geometry &g) { return (g.mp() / kM1Rows) * (int64_t)saliency_chunks(g); },
+                       [&](const Batch<ScoreLayer, kBatchLayers> &b) {
+                           const int grid = resident_grid((const void *)block_score_kernel<kBatchLayers>, b.first[b.n]);
+                           block_score_kernel<kBatchLayers><<<grid, kM1Threads, 0, st>>>(b);
+                           return cudaGetLastError();
+                       });
+}
+
+cudaError_t launch_block_selects(const ScoreLayer *layers, int n, cudaStream_t st) {
+    return for_batches(layers, n, select_ctas, [&](const Batch<ScoreLayer, kBatchLayers> &b) { return run_block_select(b, st); });
+}
+
 cudaError_t launch_block_select(const Geometry &g, const void *d_workspace, int32_t *d_blk_col, uint32_t *d_nm_bits,
                                 cudaStream_t st) {
-    const unsigned long long *score =
-        reinterpret_cast<const unsigned long long *>(reinterpret_cast<const uint8_t *>(d_workspace) + kAlign);
-    const size_t smem = (size_t)g.nblk * (sizeof(unsigned long long) + sizeof(int));
-    if (smem + 64 > 48 * 1024) {     // the longest rows (nblk near 4096) need the opt-in shared-memory size
-        cudaError_t e = cudaFuncSetAttribute(block_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    block_select_kernel<<<dim3((unsigned)g.nrt, (unsigned)(g.bm / 32)), 256, smem, st>>>(g, score, d_blk_col, d_nm_bits);
-    return cudaGetLastError();
+    ScoreLayer L = {};
+    L.g = g; L.nm_bits = d_nm_bits; L.blk_col = d_blk_col;
+    L.score = reinterpret_cast<unsigned long long *>(const_cast<uint8_t *>(reinterpret_cast<const uint8_t *>(d_workspace)) + kAlign);
+    return run_block_select(batch_of_one(L, select_ctas(g)), st);
 }
 
 cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, int32_t *d_blk_col,
@@ -387,33 +411,23 @@ cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, i
     cudaError_t e = max_known ? cudaMemsetAsync(score, 0, workspace_bytes - kAlign, st)
                               : cudaMemsetAsync(d_workspace, 0, workspace_bytes, st);
     if (e != cudaSuccess) return e;
-    const bool vec_ok = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(d_s) & 15u) == 0);
+    const bool vec_ok = saliency_vec_ok(d_s, ld);
 
-    // work items of 32 rows x 256 k-elements, dealt out to at most eight resident CTAs per SM
-    const int chunks = (int)((g.kp() + kM1ChunkK - 1) / kM1ChunkK);
+    // work items of 32 rows x 256 k-elements, dealt out to resident CTAs
+    const int chunks = saliency_chunks(g);
     const int64_t items = (g.mp() / kM1Rows) * chunks;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-        sms = 148;
-    // grids of resident CTAs: every CTA is on an SM from the start and takes its share of the items
-    auto resident_grid = [&](const void *kern) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kM1Threads, 0) != cudaSuccess || per_sm <= 0) per_sm = 4;
-        const int64_t cap = (int64_t)sms * per_sm;
-        return (int)(items < cap ? items : cap);
-    };
     if (g.m == 4)
-        group_bits_kernel<4><<<resident_grid((const void *)group_bits_kernel<4>), kM1Threads, 0, st>>>(
+        group_bits_kernel<4><<<resident_grid((const void *)group_bits_kernel<4>, items), kM1Threads, 0, st>>>(
             d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
     else
-        group_bits_kernel<8><<<resident_grid((const void *)group_bits_kernel<8>), kM1Threads, 0, st>>>(
+        group_bits_kernel<8><<<resident_grid((const void *)group_bits_kernel<8>, items), kM1Threads, 0, st>>>(
             d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
-    block_score_kernel<<<resident_grid((const void *)block_score_kernel), kM1Threads, 0, st>>>(
-        d_s, ld, g, vec_ok, items, chunks, max_key, d_nm_bits, score);
+    ScoreLayer L = {};
+    L.g = g; L.s = d_s; L.ld = ld; L.max_key = max_key; L.nm_bits = d_nm_bits; L.score = score; L.blk_col = d_blk_col;
+    block_score_kernel<1><<<resident_grid((const void *)block_score_kernel<1>, items), kM1Threads, 0, st>>>(batch_of_one(L, items));
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_block_select(g, d_workspace, d_blk_col, d_nm_bits, st);
+    return run_block_select(batch_of_one(L, select_ctas(g)), st);
 }
 
 }  // namespace crisp

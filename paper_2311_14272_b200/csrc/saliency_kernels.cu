@@ -3,11 +3,16 @@
 // The gradients come from the caller's training step, one tensor per sample or mini-batch:
 //   crisp_saliency_accumulate  acc += g           (fp32 running sum, once per gradient tensor)
 //   crisp_saliency_finish      S = |acc / H * W|   (fp32, the input of crisp_build_mask)
+// and, for all layers and samples of a network in one launch, saliency_bits_kernel below.
 // Both are element-wise streams and HBM-bound: 16-byte accesses where the rows allow it, one grid-stride
 // pass with a grid of a whole number of waves.
 #include <cuda_bf16.h>
 
+#include <memory>
+#include <new>
+
 #include "crisp_internal.h"
+#include "mask_common.cuh"
 
 namespace crisp {
 namespace {
@@ -87,6 +92,137 @@ saliency_finish_kernel(const float *__restrict__ acc, int64_t ld_a, const uint16
     }
 }
 
+// The gradients of all samples to the saliency and on to the group bits and the layer maximum, for all layers of a network
+// in one launch:
+//     S = |(g_0 + g_1 + ...) * (1 / H) * W|  (fp32, each step rounded, the order of the calls above)
+// The sum stays in registers: a sample costs its own bytes once (2 or 4 an element), where one launch per sample adds a
+// read and a write of the fp32 accumulator to them; the bits and the maximum come from the values the thread already
+// holds instead of from another pass over S.  Work items of 32 rows x 256 elements as in the mask kernels; a lane owns eight
+// consecutive elements of four rows.  Bound by HBM; what a small network waits for is latency, so items are CTAs of
+// their own and all layers share the launch.  Measured (13 layers of VGG-16, 14.7 M weights, four bf16 samples, 206 MB):
+// 44 us, against 390 us for the launches it replaces (52 accumulations, 13 finishing passes, 13 bit passes).
+struct SaliencyLayer {
+    Geometry g;
+    const uint16_t *w;
+    float *s;
+    int64_t ld_w, ld_s;
+    uint32_t *max_key, *nm_bits;
+    float inv;
+    int grad0, samples, chunks, vec_ok;
+};
+struct GradRef {
+    const void *p;
+    int64_t ld;                          // in elements; negative: fp32 with pitch -ld
+};
+constexpr int kBatchGrads = 640;
+struct SaliencyBatch {
+    Batch<SaliencyLayer, kBatchLayers> b;
+    GradRef grad[kBatchGrads];
+};
+static_assert(sizeof(SaliencyBatch) < 32000, "kernel parameters");
+
+template <int M>
+__global__ void __launch_bounds__(kM1Threads)
+saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
+    __shared__ uint8_t s_keep[64];
+    __shared__ uint32_t s_best[kM1Threads / 32];
+    const int l = batch.b.find(blockIdx.x);
+    const SaliencyLayer &L = batch.b.layer[l];
+    const Geometry &g = L.g;
+    if (M == 4 && threadIdx.x < 64) s_keep[threadIdx.x] = (uint8_t)keep_mask_of_outcomes(threadIdx.x, g.n);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const M1Item x = m1_item(blockIdx.x - batch.b.first[l], L.chunks);
+    const int64_t k0 = (int64_t)x.chunk * kM1ChunkK + lane * 8;
+    const int64_t row0 = x.row0 + warp * kM1RowsPerWarp;
+    float v[kM1RowsPerWarp][8];
+    if (L.vec_ok && row0 + kM1RowsPerWarp <= g.rows && k0 + 8 <= g.k) {
+        uint4 wr[kM1RowsPerWarp];
+#pragma unroll
+        for (int i = 0; i < kM1RowsPerWarp; ++i) wr[i] = __ldg(reinterpret_cast<const uint4 *>(L.w + (row0 + i) * L.ld_w + k0));
+        for (int h = 0; h < L.samples; ++h) {
+            const GradRef G = batch.grad[L.grad0 + h];
+            if (G.ld > 0) {
+                uint4 t[kM1RowsPerWarp];
+#pragma unroll
+                for (int i = 0; i < kM1RowsPerWarp; ++i)
+                    t[i] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(G.p) + (row0 + i) * G.ld + k0));
+#pragma unroll
+                for (int i = 0; i < kM1RowsPerWarp; ++i) {
+                    const uint32_t q[4] = {t[i].x, t[i].y, t[i].z, t[i].w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float a = __uint_as_float(q[j] << 16), b = __uint_as_float(q[j] & 0xFFFF0000u);
+                        v[i][2 * j] = h ? __fadd_rn(v[i][2 * j], a) : a;
+                        v[i][2 * j + 1] = h ? __fadd_rn(v[i][2 * j + 1], b) : b;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < kM1RowsPerWarp; ++i) {
+                    // (no read-only loads: the running sum of more samples than the table holds is the layer's own S)
+                    const float4 *p = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(G.p) + (row0 + i) * -G.ld + k0);
+                    const float4 a = p[0], b = p[1];
+                    const float q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[i][j] = h ? __fadd_rn(v[i][j], q[j]) : q[j];
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kM1RowsPerWarp; ++i) {
+            const uint32_t q[4] = {wr[i].x, wr[i].y, wr[i].z, wr[i].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[i][2 * j] = fabsf(__fmul_rn(__fmul_rn(v[i][2 * j], L.inv), __uint_as_float(q[j] << 16)));
+                v[i][2 * j + 1] = fabsf(__fmul_rn(__fmul_rn(v[i][2 * j + 1], L.inv), __uint_as_float(q[j] & 0xFFFF0000u)));
+            }
+            float4 *dst = reinterpret_cast<float4 *>(L.s + (row0 + i) * L.ld_s + k0);
+            dst[0] = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            dst[1] = make_float4(v[i][4], v[i][5], v[i][6], v[i][7]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kM1RowsPerWarp; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int64_t row = row0 + i, k = k0 + j;
+                float a = 0.f;
+                if (row < g.rows && k < g.k) {
+                    for (int h = 0; h < L.samples; ++h) {
+                        const GradRef G = batch.grad[L.grad0 + h];
+                        const float q = G.ld > 0 ? bf16_bits_to_float(reinterpret_cast<const uint16_t *>(G.p)[row * G.ld + k])
+                                                 : reinterpret_cast<const float *>(G.p)[row * -G.ld + k];
+                        a = h ? __fadd_rn(a, q) : q;
+                    }
+                    a = fabsf(__fmul_rn(__fmul_rn(a, L.inv), bf16_bits_to_float(L.w[row * L.ld_w + k])));
+                    L.s[row * L.ld_s + k] = a;
+                }
+                v[i][j] = a;
+            }
+    }
+    if (M == 4) __syncthreads();
+    uint32_t best = 0u;
+    const bool in_kp = k0 < g.kp();
+#pragma unroll
+    for (int i = 0; i < kM1RowsPerWarp; ++i) {
+        uint32_t key[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { key[j] = canonical_bits(__float_as_uint(v[i][j])); best = max(best, key[j]); }
+        uint32_t bits;
+        if constexpr (M == 4) bits = (uint32_t)s_keep[outcomes4(key)] | ((uint32_t)s_keep[outcomes4(key + 4)] << 4);
+        else bits = top_n_bits<M>(key, g.n);
+        if (in_kp) reinterpret_cast<uint8_t *>(L.nm_bits + (row0 + i) * g.wpr)[k0 >> 3] = (uint8_t)bits;
+    }
+    best = __reduce_max_sync(0xFFFFFFFFu, best);
+    if (lane == 0) s_best[warp] = best;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < kM1Threads / 32; ++w) best = max(best, s_best[w]);
+        if (best) atomicMax(L.max_key, best);
+    }
+}
+
 int wave_grid(int64_t work_items) {
     int dev = 0, sm_count = 0;                               // asked for at every call: the current device may change
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -102,6 +238,62 @@ bool vec_ok(const void *p, int64_t ld, int elem_bytes, int k) {
 }
 
 }  // namespace
+
+cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreLayer *scores, int n, cudaStream_t st) {
+    std::unique_ptr<SaliencyBatch> batch(new (std::nothrow) SaliencyBatch);
+    if (!batch) return cudaErrorMemoryAllocation;
+    Batch<SaliencyLayer, kBatchLayers> &b = batch->b;
+    b.n = 0; b.first[0] = 0;
+    int grads = 0;
+    auto flush = [&]() -> cudaError_t {
+        if (b.n == 0) return cudaSuccess;
+        if (b.first[b.n] > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+        if (b.layer[0].g.m == 4) saliency_bits_kernel<4><<<(unsigned)b.first[b.n], kM1Threads, 0, st>>>(*batch);
+        else saliency_bits_kernel<8><<<(unsigned)b.first[b.n], kM1Threads, 0, st>>>(*batch);
+        b.n = 0; grads = 0;
+        return cudaGetLastError();
+    };
+    for (int l = 0; l < n; ++l) {
+        const crisp_prune_layer_t &P = layers[l];
+        const ScoreLayer &S = scores[l];
+        // more samples than the table holds: their running sum is formed in S first, and S takes the place of the samples
+        const bool presum = P.samples > kBatchGrads;
+        if (presum)
+            for (int h = 0; h < P.samples; ++h)
+                if (crisp_saliency_accumulate(P.d_grads[h], P.grad_dtypes[h], P.ld_grads[h], S.g.rows, S.g.k, P.d_saliency, P.ld_s,
+                                              h == 0, st) != CRISP_OK)
+                    return cudaErrorUnknown;
+        const int samples = presum ? 1 : P.samples;
+        if (b.n == kBatchLayers || grads + samples > kBatchGrads) {
+            cudaError_t e = flush();
+            if (e != cudaSuccess) return e;
+        }
+        SaliencyLayer &L = b.layer[b.n];
+        L.g = S.g;
+        L.w = P.d_w_bf16; L.ld_w = P.ld_w;
+        L.s = P.d_saliency; L.ld_s = P.ld_s;
+        L.max_key = const_cast<uint32_t *>(S.max_key); L.nm_bits = S.nm_bits;
+        L.inv = 1.0f / (float)P.samples;
+        L.grad0 = grads; L.samples = samples;
+        L.chunks = (int)((S.g.kp() + kM1ChunkK - 1) / kM1ChunkK);
+        auto vec = [](const void *p, int64_t ld, int bytes) { return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld * bytes % 16 == 0; };
+        bool ok = vec(L.w, L.ld_w, 2) && vec(L.s, L.ld_s, 4);
+        for (int h = 0; h < samples; ++h) {
+            GradRef &G = batch->grad[grads + h];
+            G.p = presum ? P.d_saliency : P.d_grads[h];
+            const bool f32 = presum || P.grad_dtypes[h] == 1;
+            const int64_t ld = presum ? P.ld_s : P.ld_grads[h];
+            G.ld = f32 ? -ld : ld;
+            ok = ok && vec(G.p, ld, f32 ? 4 : 2);
+        }
+        L.vec_ok = ok;
+        grads += samples;
+        b.first[b.n + 1] = b.first[b.n] + (S.g.mp() / kM1Rows) * (int64_t)L.chunks;
+        ++b.n;
+    }
+    return flush();
+}
+
 }  // namespace crisp
 
 extern "C" {

@@ -11,7 +11,7 @@
 // A CTA is persistent over (128-row tile, column tile) pairs; all row tiles of a layer have the same
 // number of kept blocks (uniform block pruning, Sec. III-A), so tiles are load-balanced by construction.
 //
-// The execution image is built by the kernels at the bottom of this file from the canonical format.
+// The execution image is written by the encode kernel (encode_kernels.cu).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -20,7 +20,6 @@
 
 #include "crisp_internal.h"
 #include "tc_common.cuh"
-#include "walks.cuh"
 
 namespace crisp {
 
@@ -769,152 +768,6 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     }
 }
 
-// --------------------------------------------------------------------- execution image kernels
-
-// Walk lists as a kernel of their own (the body, and what it builds, are described in walks.cuh).
-__global__ void __launch_bounds__(256)
-build_walks_kernel(Geometry g, WalkArgs a) {
-    __shared__ WalkShared sh;
-    build_walks_body(g, a, blockIdx.x, sh);
-}
-
-// One CTA per walk entry: assemble the entry's weight tile (and 2:4 metadata) in shared memory from
-// the canonical values and offsets of the row tiles that keep this block column, zeros for row tiles
-// that do not, then write it out with coalesced 16-byte stores.
-// Dense image: element (row, k) of the tile at [k/8][row][k%8].
-// Sparse image: per aligned 4-group two slots (ascending position, zero-padded); slot pair of group
-// q stored at compressed columns 2q, 2q+1 in the same [c/8][row][c%8] layout.  Metadata (2048 bytes):
-// 16-byte row L = row%8 + 8*((k/16)%2) + 16*(row/16), 32-bit word k/32, nibble of the 4-group at bit
-// (k%16) + 16*((row/8)%2), value idx0 | idx1 << 2.
-template <bool kSparse>
-__global__ void __launch_bounds__(256)
-build_image_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *__restrict__ vals,
-                   const uint32_t *__restrict__ idx, int r, int nst, int wcap, int stack,
-                   const int32_t *__restrict__ walk_col, const int32_t *__restrict__ walk_len, uint32_t a_bytes,
-                   uint32_t entry_bytes, int addends, uint8_t *__restrict__ image) {
-    extern __shared__ uint4 s_tile4[];
-    uint8_t *tile = reinterpret_cast<uint8_t *>(s_tile4);
-    __shared__ int s_blk[4];
-    // image entries are ordered [copy][CTA tile][walk entry]; copy q of a stacked layer (one CTA tile of at most
-    // 128 / stack rows) holds the same weights shifted down by q * 128 / stack rows
-    const int per_copy = nst * wcap;
-    const int copy = blockIdx.x / per_copy, in_copy = blockIdx.x - copy * per_copy;
-    const int st = in_copy / wcap, e = in_copy - st * wcap;
-    const int shift = copy * (kTileM / stack);
-    if (e >= walk_len[st]) return;
-    const int jb = walk_col[(int64_t)st * wcap + e];
-    for (uint32_t i = threadIdx.x; i < entry_bytes / 16; i += blockDim.x) s_tile4[i] = make_uint4(0, 0, 0, 0);
-    if (threadIdx.x < r) {
-        // does row tile st*r + threadIdx.x keep block column jb, and in which slot?
-        const int rt = st * r + threadIdx.x;
-        int found = -1;
-        if (rt < g.nrt) {
-            const int32_t *bc = blk_col + (int64_t)rt * g.kkeep;
-            int lo = 0, hi = g.kkeep - 1;
-            while (lo <= hi) {
-                const int mid = (lo + hi) >> 1;
-                const int v = bc[mid];
-                if (v == jb) { found = rt * g.kkeep + mid; break; }
-                if (v < jb) lo = mid + 1; else hi = mid - 1;
-            }
-        }
-        s_blk[threadIdx.x] = found;
-    }
-    __syncthreads();
-    const int groups = g.groups();
-    const int vpb = (int)g.vals_per_block();
-    const int idx_words = vpb * g.idx_bits / 32;
-    const uint32_t field = (1u << g.idx_bits) - 1u;
-    // canonical values and offsets of one kept block, staged with coalesced 16-byte loads
-    uint16_t *vb = reinterpret_cast<uint16_t *>(tile + entry_bytes);
-    uint32_t *ib = reinterpret_cast<uint32_t *>(tile + entry_bytes + (size_t)vpb * 2);
-    for (int sub = 0; sub < r; ++sub) {
-        const int blk = s_blk[sub];
-        if (blk < 0) continue;
-        const int row0 = shift + sub * g.bm;
-        __syncthreads();
-        {
-            const uint4 *vsrc = reinterpret_cast<const uint4 *>(vals + (int64_t)blk * vpb);      // vpb*2 is a multiple of 64
-            for (int i = threadIdx.x; i < vpb / 8; i += blockDim.x) reinterpret_cast<uint4 *>(vb)[i] = __ldg(vsrc + i);
-            const uint32_t *isrc = idx + (int64_t)blk * idx_words;
-            for (int i = threadIdx.x; i < idx_words; i += blockDim.x) ib[i] = __ldg(isrc + i);
-        }
-        __syncthreads();
-        if constexpr (!kSparse) {
-            for (int o = threadIdx.x; o < vpb; o += blockDim.x) {
-                const int item = o / g.n;
-                const int lr = item / groups, gi = item - lr * groups;
-                const int bit = o * g.idx_bits;
-                uint32_t t = ib[bit >> 5] >> (bit & 31);
-                if ((bit & 31) + g.idx_bits > 32) t |= ib[(bit >> 5) + 1] << (32 - (bit & 31));
-                t &= field;
-                const int k = gi * g.m + (int)t, row = row0 + lr;
-                *reinterpret_cast<uint16_t *>(tile + (k >> 3) * 2048 + row * 16 + (k & 7) * 2) = vb[o];
-            }
-        } else {
-            // one thread per (local row, 4-group): at most two kept values per addend.  With one addend the pattern
-            // guarantees that; with two, the first two values (ascending position) go to the first addend and the
-            // rest to the second, each a 2:4-compliant tile with its own metadata, sub bytes apart.
-            const int quads = g.bk / 4;
-            const uint32_t sub = a_bytes + kMetaBytes;
-            for (int item = threadIdx.x; item < g.bm * quads; item += blockDim.x) {
-                const int lr = item / quads, qd = item - lr * quads;
-                const int row = row0 + lr;
-                const int gi = (qd * 4) / g.m;
-                uint16_t v4[4] = {0, 0, 0, 0};
-                int pos4[4] = {0, 0, 0, 0}, cnt4 = 0;
-                for (int vv = 0; vv < g.n; ++vv) {
-                    const int o = (lr * groups + gi) * g.n + vv;
-                    const int bit = o * g.idx_bits;
-                    uint32_t t = ib[bit >> 5] >> (bit & 31);
-                    if ((bit & 31) + g.idx_bits > 32) t |= ib[(bit >> 5) + 1] << (32 - (bit & 31));
-                    t &= field;
-                    const int k = gi * g.m + (int)t;
-                    if ((k >> 2) == qd && cnt4 < 2 * addends) { v4[cnt4] = vb[o]; pos4[cnt4] = k & 3; ++cnt4; }
-                }
-                for (int a = 0; a < addends; ++a) {
-                    uint16_t v[2] = {v4[2 * a], v4[2 * a + 1]};
-                    int pos[2] = {pos4[2 * a], pos4[2 * a + 1]};
-                    const int cnt = cnt4 - 2 * a < 0 ? 0 : (cnt4 - 2 * a > 2 ? 2 : cnt4 - 2 * a);
-                    if (cnt == 0) { v[0] = v[1] = 0; pos[0] = 0; pos[1] = 1; }
-                    else if (cnt == 1) {
-                        v[1] = 0;
-                        if (pos[0] == 3) { v[1] = v[0]; v[0] = 0; pos[1] = 3; pos[0] = 0; }
-                        else pos[1] = 3;
-                    }
-                    uint8_t *ta = tile + a * sub;
-                    uint32_t *meta = reinterpret_cast<uint32_t *>(ta + a_bytes);
-                    const int c0 = 2 * qd;                   // even: both slots share one 16-byte chunk
-                    *reinterpret_cast<uint32_t *>(ta + (c0 >> 3) * 2048 + row * 16 + (c0 & 7) * 2) =
-                        (uint32_t)v[0] | ((uint32_t)v[1] << 16);
-                    const uint32_t nib = (uint32_t)pos[0] | ((uint32_t)pos[1] << 2);
-                    const int k0 = qd * 4;
-                    const int lrow = (row & 7) + 8 * ((k0 >> 4) & 1) + 16 * (row >> 4);
-                    atomicOr(&meta[lrow * 4 + (k0 >> 5)], nib << ((k0 & 15) + 16 * ((row >> 3) & 1)));
-                }
-            }
-        }
-    }
-    if constexpr (kSparse) {
-        // rows that carry no kept block here (row tiles that do not keep it, rows outside a stacked copy's
-        // window) still need valid (distinct, ascending) index pairs
-        for (int a = 0; a < addends; ++a) {
-            uint32_t *meta = reinterpret_cast<uint32_t *>(tile + a * (a_bytes + kMetaBytes) + a_bytes);
-            for (int item = threadIdx.x; item < kTileM * (g.bk / 4); item += blockDim.x) {
-                const int row = item / (g.bk / 4), qd = item - row * (g.bk / 4);
-                const int sub_rt = row >= shift ? (row - shift) / g.bm : r;
-                if (sub_rt < r && s_blk[sub_rt] >= 0) continue;
-                const int k0 = qd * 4;
-                const int lrow = (row & 7) + 8 * ((k0 >> 4) & 1) + 16 * (row >> 4);
-                atomicOr(&meta[lrow * 4 + (k0 >> 5)], 0x4u << ((k0 & 15) + 16 * ((row >> 3) & 1)));
-            }
-        }
-    }
-    __syncthreads();
-    uint4 *out = reinterpret_cast<uint4 *>(image + (int64_t)blockIdx.x * entry_bytes);      // [copy][st][e]
-    for (uint32_t i = threadIdx.x; i < entry_bytes / 16; i += blockDim.x) out[i] = s_tile4[i];
-}
-
 typedef void (*TcKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, TcParams);
 
 constexpr int kMaxDevices = 64;
@@ -1062,44 +915,6 @@ TcImageLayout tc_image_layout(const Geometry &g, int kind) {
     L.image_off = L.walk_len_off + align_up((size_t)L.nst * sizeof(int32_t) + 4);
     L.total_bytes = L.image_off + align_up((size_t)L.stack * L.nst * L.wcap * L.entry_bytes + 16);
     return L;
-}
-
-WalkArgs tc_walk_args(const Geometry &g, int kind, const int32_t *d_blk_col, uint8_t *d_exec) {
-    const TcImageLayout L = tc_image_layout(g, kind);
-    WalkArgs a;
-    a.blk_col = d_blk_col;
-    a.r = L.r; a.nst = L.nst; a.wcap = L.wcap;
-    a.nctas = g.nrt * g.kkeep == 0 ? 0 : L.nst;
-    a.walk_col = reinterpret_cast<int32_t *>(d_exec + L.walk_col_off);
-    a.walk_len = reinterpret_cast<int32_t *>(d_exec + L.walk_len_off);
-    return a;
-}
-
-cudaError_t launch_build_image(const Geometry &g, int kind, const int32_t *d_blk_col, const uint16_t *d_vals,
-                               const uint32_t *d_idx, uint8_t *d_exec, bool tiles_done, bool walks_done,
-                               cudaStream_t st) {
-    const bool sparse = kind != CRISP_PATH_DENSE;
-    const TcImageLayout L = tc_image_layout(g, kind);
-    if (g.nrt * g.kkeep == 0) return cudaSuccess;
-    int32_t *walk_col = reinterpret_cast<int32_t *>(d_exec + L.walk_col_off);
-    int32_t *walk_len = reinterpret_cast<int32_t *>(d_exec + L.walk_len_off);
-    uint8_t *image = d_exec + L.image_off;
-    if (!walks_done) build_walks_kernel<<<L.nst, 256, 0, st>>>(g, tc_walk_args(g, kind, d_blk_col, d_exec));
-    if (tiles_done) return cudaGetLastError();       // the encode kernel already wrote the weight tiles
-    const int grid = L.stack * L.nst * L.wcap;
-    const size_t smem_img = (size_t)L.entry_bytes + (size_t)g.vals_per_block() * 2 + (size_t)(g.vals_per_block() * g.idx_bits / 32) * 4 + 16;
-    if (smem_img > 48 * 1024) {      // large blocks with many kept values need the opt-in shared memory size
-        cudaError_t e = sparse ? cudaFuncSetAttribute(build_image_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_img)
-                               : cudaFuncSetAttribute(build_image_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_img);
-        if (e != cudaSuccess) return e;
-    }
-    if (sparse)
-        build_image_kernel<true><<<grid, 256, smem_img, st>>>(g, d_blk_col, d_vals, d_idx, L.r, L.nst, L.wcap, L.stack, walk_col,
-                                                                    walk_len, L.a_bytes, L.entry_bytes, L.addends, image);
-    else
-        build_image_kernel<false><<<grid, 256, smem_img, st>>>(g, d_blk_col, d_vals, d_idx, L.r, L.nst, L.wcap, L.stack, walk_col,
-                                                                     walk_len, L.a_bytes, L.entry_bytes, L.addends, image);
-    return cudaGetLastError();
 }
 
 // Whether the tensor-core kernel can address these operands (TMA: 16-byte aligned base and pitch).
