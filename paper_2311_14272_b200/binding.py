@@ -155,10 +155,27 @@ def _ptr(t) -> int:
     return t.ctypes.data
 
 
+def _bind_current_stream():
+    """The address of torch's current stream on the current device.  torch.cuda.current_stream() builds a Stream object on
+    every call, 3.2 us of the 9.6 us that a small product used to spend on the host; the two C functions it asks in the
+    end take 0.2 us.  They are not public: without them the public call stays."""
+    global _current_stream
+    import torch
+    torch.cuda.current_stream()                  # initialises CUDA, or says why it cannot
+    device, raw = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device is not None and raw is not None:
+        _current_stream = lambda: raw(device())
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return _current_stream()
+
+
+_current_stream = _bind_current_stream
+
+
 def _stream(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -409,6 +426,7 @@ class HybridLayer:
         mask_bytes, ws_bytes = crisp_mask_sizes(self.desc)
         self.mask_buf = torch.empty(mask_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=self.device)
+        self._bf16 = torch.empty(0, dtype=torch.bfloat16, device=self.device)
         self.mask = 0
         self.handle = 0
         self.canonical_buf = None
@@ -473,10 +491,12 @@ class HybridLayer:
 
     def _adopt(self, kkeep, mask, handle):
         """Take over a mask and a handle that a batched call made in this layer's buffers."""
-        crisp_mask_destroy(self.mask)
-        crisp_destroy(self.handle)
+        if self.mask:
+            _lib.crisp_mask_destroy(self.mask)
+        if self.handle:
+            _lib.crisp_destroy(self.handle)
         self.mask, self.handle = mask, handle
-        self.desc.keep_ratio = crisp_keep_ratio_for_count(self.desc, kkeep)
+        self.desc.keep_ratio = kkeep / self.nblk             # floor(ratio * nblk + 0.5) gives kkeep back
         self.kkeep = kkeep
 
     def export(self, stream=None):
@@ -488,36 +508,39 @@ class HybridLayer:
         crisp_export(self.handle, blk_col, vals, idx, stream)
         return blk_col.reshape(self.nrt, self.kkeep), vals, idx
 
+    # The three calls below are made once per layer and pass; for small layers their host time is the time of the pass, so
+    # they hand their arguments to the library without the wrappers above.
     def decode(self, stream=None):
-        torch = self.torch
-        w = torch.empty((self.desc.rows, self.desc.k), dtype=torch.bfloat16, device=self.device)
-        crisp_decode(self.handle, w, w.stride(0), stream)
+        w = self._bf16.new_empty((self.desc.rows, self.desc.k))
+        code = _lib.crisp_decode(self.handle, w.data_ptr(), w.stride(0), _stream(stream))
+        if code:
+            raise CrispError(code, "crisp_decode")
         return w
 
     def spmm(self, x, y=None, y_dtype=0, stream=None):
-        torch = self.torch
         assert x.is_cuda and x.element_size() == 2 and x.stride(1) == 1 and x.shape[0] == self.desc.k
         ncols = x.shape[1]
         if y is None:
-            y = torch.empty((self.desc.rows, ncols), dtype=torch.float32 if y_dtype else torch.bfloat16,
-                            device=self.device)
-        crisp_spmm(self.handle, x, x.stride(0), ncols, y, y.stride(0), y_dtype, stream)
+            y = self._bf16.new_empty((self.desc.rows, ncols), dtype=self.torch.float32 if y_dtype else self.torch.bfloat16)
+        code = _lib.crisp_spmm(self.handle, x.data_ptr(), x.stride(0), ncols, y.data_ptr(), y.stride(0), y_dtype, _stream(stream))
+        if code:
+            raise CrispError(code, "crisp_spmm")
         return y
 
     def spmm_conv(self, act_nhwc, kernel_h, kernel_w, pad, y=None, y_dtype=0, stream=None, nhwc_out=False):
         """Convolution (stride 1) of an NHWC bf16 activation with this layer's weights, without an X matrix.
         nhwc_out: Y is [batch, ho, wo, rows] (the next convolution's activation) instead of [rows, batch*ho*wo]."""
-        torch = self.torch
         assert act_nhwc.is_cuda and act_nhwc.element_size() == 2 and act_nhwc.is_contiguous() and act_nhwc.dim() == 4
         b, h, w, c = act_nhwc.shape
-        ho, wo = h + 2 * pad - kernel_h + 1, w + 2 * pad - kernel_w + 1
-        dt = torch.float32 if y_dtype else torch.bfloat16
         if y is None:
-            y = torch.empty((b, ho, wo, self.desc.rows) if nhwc_out else (self.desc.rows, b * ho * wo), dtype=dt,
-                            device=self.device)
+            ho, wo = h + 2 * pad - kernel_h + 1, w + 2 * pad - kernel_w + 1
+            dt = self.torch.float32 if y_dtype else self.torch.bfloat16
+            y = self._bf16.new_empty((b, ho, wo, self.desc.rows) if nhwc_out else (self.desc.rows, b * ho * wo), dtype=dt)
         ldy = y.stride(2) if nhwc_out else y.stride(0)
-        crisp_spmm_conv(self.handle, act_nhwc, ConvDesc(b, h, w, c, kernel_h, kernel_w, pad, 1 if nhwc_out else 0), y, ldy,
-                        y_dtype, stream)
+        desc = ConvDesc(b, h, w, c, kernel_h, kernel_w, pad, 1 if nhwc_out else 0)
+        code = _lib.crisp_spmm_conv(self.handle, act_nhwc.data_ptr(), desc, y.data_ptr(), ldy, y_dtype, _stream(stream))
+        if code:
+            raise CrispError(code, "crisp_spmm_conv")
         return y
 
     def set_epilogue(self, bias=None, relu=False):
@@ -593,21 +616,21 @@ class PruningNetwork:
         masks and handles (self.layers[l]) hold the result."""
         torch = self.torch
         bf16 = torch.bfloat16
-        arr = (PruneLayer * len(self.layers))()
-        host = []                                            # the arrays that the table points into
+        count = min(len(self.layers), len(weights), len(grads))
+        weights, grads = weights[:count], grads[:count]
+        assert all(w.is_cuda and w.element_size() == 2 and w.stride(1) == 1 for w in weights)
+        arr = (PruneLayer * count)()
+        flat = [g for gs in grads for g in gs]               # one host array each for the whole network
+        ptrs = (C.c_void_p * len(flat))(*[g.data_ptr() for g in flat])
+        lds = (C.c_int64 * len(flat))(*[g.stride(0) for g in flat])
+        dts = (C.c_int32 * len(flat))(*[0 if g.dtype is bf16 else 1 for g in flat])
+        p0, l0, d0, at = C.addressof(ptrs), C.addressof(lds), C.addressof(dts), 0
         for P, L, w, gs, s in zip(arr, self.layers, weights, grads, self.sal):
-            assert w.is_cuda and w.element_size() == 2 and w.stride(1) == 1
-            h = len(gs)
-            ptrs = (C.c_void_p * h)(*[g.data_ptr() for g in gs])
-            lds = (C.c_int64 * h)(*[g.stride(0) for g in gs])
-            dts = (C.c_int32 * h)(*[0 if g.dtype == bf16 else 1 for g in gs])
-            host.append((ptrs, lds, dts))
-            P.desc = L.desc
-            P.d_w_bf16, P.ld_w = w.data_ptr(), w.stride(0)
-            P.d_grads, P.ld_grads, P.grad_dtypes = C.addressof(ptrs), C.addressof(lds), C.addressof(dts)
-            P.samples = h
-            P.d_saliency, P.ld_s = s.data_ptr(), L.desc.k
+            P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride(0)
+            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, len(gs)
+            P.d_saliency, P.ld_s = s.data_ptr(), s.stride(0)
             P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
+            at += len(gs)
         crisp_prune_score(arr, stream)
         crisp_global_rank(self.rank_arr, crisp_prune_fraction(kappa, self.n, self.m), self.rank_ws, self.d_kkeep, stream)
         if stream is None:
