@@ -52,6 +52,15 @@ struct Batch {
 #endif
 };
 
+#ifdef __CUDACC__
+// Programmatic dependent launch.  A kernel launched with the programmatic-serialization attribute may start before the
+// kernel in front of it in the stream has finished; wait_for_prerequisites() returns when that one has finished and its
+// writes are visible, and every thread that touches global memory another kernel may write or read calls it first.
+// launch_dependents() lets the next kernel of the stream start its own set-up (it waits in the same way).
+__device__ __forceinline__ void wait_for_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 

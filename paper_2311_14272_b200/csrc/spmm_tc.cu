@@ -421,9 +421,6 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         tmem_relinquish();
     }
     const int walk_words = p.walk_cache ? p.nst * (p.wcap + 1) : 0;     // [nst] lengths, then [nst][wcap] columns
-    int32_t walk_w0 = 0;
-    if ((int)threadIdx.x < walk_words)
-        walk_w0 = (int)threadIdx.x < p.nst ? p.walk_len[threadIdx.x] : p.walk_col[(int)threadIdx.x - p.nst];
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_x);
@@ -433,8 +430,11 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if ((int)threadIdx.x < walk_words) s_walk[threadIdx.x] = walk_w0;
-    for (int i = threadIdx.x + blockDim.x; i < walk_words; i += blockDim.x)
+    // Everything above touches this CTA's own memory only, so it may run while the kernel in front of this one in the
+    // stream still does; from here on its results are needed (X, and the image and walk lists after an encode).
+    launch_dependents();
+    wait_for_prerequisites();
+    for (int i = threadIdx.x; i < walk_words; i += blockDim.x)
         s_walk[i] = i < p.nst ? p.walk_len[i] : p.walk_col[i - p.nst];
     const int32_t *walk_len = p.walk_cache ? s_walk : p.walk_len;
     const int32_t *walk_col = p.walk_cache ? s_walk + p.nst : p.walk_col;
@@ -1189,9 +1189,19 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
         plan->has_conv = conv != nullptr;
         if (conv) plan->conv = *conv;
     }
-    plan->variant.kern<<<plan->grid, plan->variant.threads, plan->smem, st>>>(plan->mx, plan->my, plan->ma, plan->p);
-    h->last = plan->info;
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;        // see wait_for_prerequisites
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan->grid);
+    cfg.blockDim = dim3((unsigned)plan->variant.threads);
+    cfg.dynamicSmemBytes = plan->smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, plan->variant.kern, plan->mx, plan->my, plan->ma, plan->p);
+    if (e == cudaSuccess) h->last = plan->info;
+    return e;
 }
 
 }  // namespace crisp
