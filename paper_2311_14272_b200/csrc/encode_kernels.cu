@@ -78,7 +78,7 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
     const Geometry &g = L.g;
     const int cta = (int)(blockIdx.x - batch.first[l]);
     const int r = kTileRows / g.bm;
-    const int per_tile = r == 1 ? g.kkeep : min(r * g.kkeep, g.nblk);     // most entries of a walk list
+    const int per_tile = min(min(r, g.nrt) * g.kkeep, g.nblk);            // most entries of a walk list
     const int st = cta / per_tile, entry = cta - st * per_tile;
     const int first_rt = st * r, n_rt = min(r, g.nrt - first_rt);
     if (cta == 0 && L.header != nullptr && threadIdx.x < 64) L.header[threadIdx.x] = 0u;     // the handle's status block
@@ -439,7 +439,8 @@ cudaError_t encode_batch(const EncodeLayer *layers, int n, cudaStream_t st) {
         // the 16-byte loads of eight elements need every row to start 16-byte aligned (block columns are multiples of 32)
         L.vec_ok = reinterpret_cast<uintptr_t>(L.w) % 16 == 0 && L.ld % 8 == 0;
         const int64_t tiles = (g.mp() + kTileRows - 1) / kTileRows;
-        const int64_t entries = (int64_t)(kTileRows / g.bm) * g.kkeep;
+        const int r = kTileRows / g.bm;
+        const int64_t entries = (int64_t)(r < g.nrt ? r : g.nrt) * g.kkeep;
         b.first[b.n + 1] = b.first[b.n] + tiles * (entries < g.nblk ? entries : g.nblk);
         ++b.n;
     }

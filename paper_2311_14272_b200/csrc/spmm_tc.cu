@@ -69,6 +69,7 @@ struct TcParams {
                                 // fill, so that the wait for it runs into wait_limit
     int a_map;                  // map_a views the image as rows of 256 bytes: weight tiles come in as tiled loads
     int x_map_3d;               // map_x views X as [ncols/64][k][64]: one load fetches all NT boxes
+    uint32_t resident_bytes;    // kResident: the weight tiles of the one walk there is, kept in front of the ring
 };
 
 constexpr uint32_t kWideStageBytes = 2048;                      // epilogue staging tile: 16 rows x 128 bytes
@@ -210,16 +211,44 @@ __device__ __forceinline__ void store_chunk(const TcParams &p, const CUtensorMap
 // as one 4-D bulk tensor store of {32 channels, tw, pixels / tw, 1} (it clips channels beyond `rows` and pixels
 // outside the images), or, where the pixel pitch is not a multiple of 16 bytes, pixel by pixel with the 32
 // lanes on consecutive channels.  `out` is packed as in store_chunk (bf16: pixels 2i, 2i+1 in word i).
+// With 2048-byte staging tiles (bf16) it goes in two passes of 32 pixels.
 template <typename OutT>
 __device__ __forceinline__ void store_chunk_nhwc(const TcParams &p, const CUtensorMap *map_y, uint32_t stg, uint8_t *stg_gen,
                                                  int lane, const uint32_t (&out)[32], const TileOrigin &org, int col0, int y0) {
     constexpr int kOutCols = 128 / (int)sizeof(OutT);
     constexpr int kRowBytes = 32 * (int)sizeof(OutT);           // one pixel: 32 channels
-    const int per_image = p.cv_tw * p.cv_th;
-    const int img = col0 / per_image;
-    const int cx = org.x, cy = org.y + (col0 - img * per_image) / p.cv_tw, cb = org.b + img;
     if (y0 >= p.rows) return;
-    if (lane == 0 && !p.cv_plain) bulk_wait_read<0>();          // the previous store has finished reading the tile
+    if (!p.cv_plain) {
+        const bool halves = sizeof(OutT) == 2 && p.stg_tile_bytes == 2048;
+        const int per_image = p.cv_tw * p.cv_th;
+#pragma unroll
+        for (int h = 0; h < (sizeof(OutT) == 2 ? 2 : 1); ++h) {
+            if (h == 0 || halves) {
+                if (lane == 0) bulk_wait_read<0>();             // the previous store has finished reading the tile
+                __syncwarp();
+            }
+            uint8_t *half = stg_gen + (halves ? 0 : h * 32 * kRowBytes);
+#pragma unroll
+            for (int i = 0; i < (sizeof(OutT) == 2 ? 16 : 32); ++i) {
+                if constexpr (sizeof(OutT) == 2) {
+                    *reinterpret_cast<uint16_t *>(half + (2 * i) * kRowBytes + lane * 2) = (uint16_t)(out[16 * h + i] & 0xFFFFu);
+                    *reinterpret_cast<uint16_t *>(half + (2 * i + 1) * kRowBytes + lane * 2) = (uint16_t)(out[16 * h + i] >> 16);
+                } else {
+                    *reinterpret_cast<uint32_t *>(half + i * kRowBytes + lane * 4) = out[i];
+                }
+            }
+            if (h == 0 && sizeof(OutT) == 2 && !halves) continue;
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                const int first = col0 + (halves ? 32 * h : 0), img = first / per_image;
+                const int cx = org.x, cy = org.y + (first - img * per_image) / p.cv_tw, cb = org.b + img;
+                if (cx < p.cv_wo && cy < p.cv_ho && cb < p.cv_batch) tma_store_4d(map_y, stg, y0, cx, cy, cb);
+                bulk_commit();
+            }
+        }
+        return;
+    }
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
@@ -229,15 +258,6 @@ __device__ __forceinline__ void store_chunk_nhwc(const TcParams &p, const CUtens
         } else {
             *reinterpret_cast<uint32_t *>(stg_gen + i * kRowBytes + lane * 4) = out[i];
         }
-    }
-    if (!p.cv_plain) {
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-            if (cx < p.cv_wo && cy < p.cv_ho && cb < p.cv_batch) tma_store_4d(map_y, stg, y0, cx, cy, cb);
-            bulk_commit();
-        }
-        return;
     }
     __syncwarp();
     const bool row_ok = y0 + lane < p.rows;
@@ -260,10 +280,11 @@ __device__ __forceinline__ void store_chunk_nhwc(const TcParams &p, const CUtens
 // the weight tile advances by 4096 bytes, X by 32 rows (sparse image, 4096 bytes) or 16 rows (2048).
 struct MmaRoleArgs {
     uint32_t ring, bar_full, bar_empty, bar_tfull, bar_tempty, tmem_base;
+    uint32_t weights, bar_weights;      // resident weight tiles and the barrier of their arrival
     const int32_t *walk_len;
     volatile int *abort_flag;
 };
-template <int kTileN, bool kSparse, int kAccStages, int NM, bool kConv>
+template <int kTileN, bool kSparse, int kAccStages, int NM, bool kConv, bool kResident>
 __device__ __forceinline__ void mma_role(const TcParams &p, const MmaRoleArgs &a) {
     // matrix mode: X rows are columns-contiguous (MN-major operand, 64-column boxes box_bytes apart, a K
     // step is 32 or 16 rows); convolution mode: the activation tile is [pixel][bk channels] with the channels
@@ -278,6 +299,45 @@ __device__ __forceinline__ void mma_role(const TcParams &p, const MmaRoleArgs &a
     const uint32_t a_step = p.entry_bytes >> 4, x_step = ((uint32_t)(kTileN / kBoxN) * p.box_bytes) >> 4;   // per block of a stage
     const int group = (int)p.group;
     uint32_t off = 0, full = a.bar_full, empty = a.bar_empty, ph = 0, acc = 0, acc_ph = 0, meta_buf = 0;
+    if constexpr (kResident) {                              // weight tiles stay, a stage is one X tile (one addend, no stack)
+        const uint64_t w_desc = make_smem_desc(a.weights, 2048, 128, kLayoutNone);
+        const uint64_t wm_desc = make_smem_desc(a.weights + p.a_bytes, 128, 128, kLayoutNone);
+        const uint64_t x_desc = kConv ? make_smem_desc(a.ring, 16, 1024, kLayoutSw128) : make_smem_desc(a.ring, p.box_bytes, 1024, kLayoutSw128);
+        const int len = min(a.walk_len[0], p.wcap);
+        if (!mbar_wait(a.bar_weights, 0, a.abort_flag, p.wait_limit)) return;
+        for (int t = blockIdx.x; t < p.num_tiles && !*a.abort_flag; t += gridDim.x) {
+            if (!mbar_wait(a.bar_tempty + 8 * acc, acc_ph ^ 1u, a.abort_flag, p.wait_limit)) break;
+            tc_fence_after();
+            const uint32_t d_tmem = a.tmem_base + acc * kTileN;
+            uint32_t accum = 0, w_off = 0;
+            bool ok = true;
+            for (int e = 0; e < len; ++e, w_off += a_step) {
+                if (!mbar_wait(full, ph, a.abort_flag, p.wait_limit)) { ok = false; break; }
+                tc_fence_after();
+                const uint64_t ad = w_desc + w_off, bd = x_desc + off;
+                if constexpr (kSparse) {
+                    const uint32_t meta_tmem = a.tmem_base + kAccStages * kTileN + 4 * meta_buf;
+                    tmem_copy_128x128b(meta_tmem, wm_desc + w_off);
+#pragma unroll
+                    for (int j = 0; j < NM; ++j)
+                        mma_sparse(d_tmem, ad + j * 256, bd + j * b_step, idesc | (uint32_t)(j & 1), accum | (uint32_t)j,
+                                   meta_tmem + (j & ~1));
+                    meta_buf ^= 1u;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < NM; ++j) mma_dense(d_tmem, ad + j * 256, bd + j * b_step, idesc, accum | (uint32_t)j);
+                }
+                accum = 1u;
+                mma_commit(empty);
+                off += stage_step; full += 8; empty += 8;
+                if (off == ring_span) { off = 0; full = a.bar_full; empty = a.bar_empty; ph ^= 1u; }
+            }
+            if (!ok) break;
+            mma_commit(a.bar_tfull + 8 * acc);
+            if (++acc == kAccStages) { acc = 0; acc_ph ^= 1u; }
+        }
+        return;
+    }
     if (group == 1) {
         // one kept block per stage: the plain loop (large tiles; every extra instruction here costs the headline cells)
         for (int t = blockIdx.x; t < p.num_tiles && !*a.abort_flag; t += gridDim.x) {
@@ -383,7 +443,11 @@ __device__ __forceinline__ void mma_role(const TcParams &p, const MmaRoleArgs &a
 // contiguous, 128 bytes between 8-row groups, 2048 bytes between 16-byte K chunks.
 // X box layout: TMA SWIZZLE_128B, 64 columns (128 bytes) x bk rows; MN-major operand with 1024 bytes
 // between 8-row K groups and box_bytes between 64-column groups.
-template <int NT, bool kSparse, int kAccStages, typename OutT, int kEpi, bool kConv>
+//
+// kResident: with one CTA tile of rows all tiles multiply the same weight tiles; short walks then load them once and keep
+// them, and a stage holds X only.  What bounds a short walk is the number of bytes in flight: a stage's cycle (MMA, release,
+// issue of the copy, L2, arrival) takes 1.4 to 1.6 us whatever it carries.
+template <int NT, bool kSparse, int kAccStages, typename OutT, int kEpi, bool kConv, bool kResident>
 __global__ void __launch_bounds__(96 + 32 * kEpi, 1)
 spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
                const __grid_constant__ CUtensorMap map_a, TcParams p) {
@@ -400,7 +464,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         if (threadIdx.x == 0) atomicCAS(p.status, 0, (int)CRISP_CUDA_ERROR);
         return;
     }
-    const uint32_t ring = smem_base;
+    const uint32_t ring = smem_base + (kResident ? p.resident_bytes : 0u);
     const uint32_t staging = ring + p.num_stages * p.stage_bytes;
     const uint32_t ctrl = staging + kEpi * p.stg_bufs * p.stg_tile_bytes;
     uint8_t *ctrl_gen = smem_gen + (ctrl - smem_base);
@@ -408,6 +472,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const uint32_t bar_full = ctrl, bar_empty = ctrl + 64, bar_tfull = ctrl + 128, bar_tempty = ctrl + 144;
     volatile uint32_t *tmem_base_slot = reinterpret_cast<volatile uint32_t *>(ctrl_gen + 160);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl_gen + 164);
+    const uint32_t bar_weights = ctrl + 168;
     // Optional copy of the walk lists ([nst] lengths, then [nst][wcap] block columns): a tile with a short
     // walk would otherwise spend two dependent global loads per tile in the producer's serial loop.
     int32_t *s_walk = reinterpret_cast<int32_t *>(ctrl_gen + 256);
@@ -427,6 +492,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         if (!(kConv && p.cv_plain)) prefetch_tensormap(&map_y);
         for (uint32_t s = 0; s < p.num_stages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
         for (int a = 0; a < kAccStages; ++a) { mbar_init(bar_tfull + 8 * a, 1); mbar_init(bar_tempty + 8 * a, kEpi); }
+        if constexpr (kResident) mbar_init(bar_weights, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -463,7 +529,12 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             uint32_t dst = ring, full = bar_full, empty = bar_empty, ph = 0;
             int fill_no = 0;     // test hook: fill number p.skip_fill gets no copies, so its `full` barrier never
                                  // completes and the bounded wait of the MMA issuer ends the kernel with CRISP_TIMEOUT
-            if (warp == 0) {
+            if (kResident && warp == 0) {
+                const int len = min(walk_len[0], p.wcap);
+                mbar_expect_tx(bar_weights, (uint32_t)len * p.entry_bytes);
+                for (int e = 0; e < len; ++e)
+                    tma_load_2d(smem_base + (uint32_t)e * p.entry_bytes, &map_a, 0, e * (int)entry_rows, bar_weights);
+            } else if (warp == 0) {
                 if (p.group == 1) {       // one kept block per stage: the plain loop
                     for (int t = blockIdx.x; t < p.num_tiles && !*abort_flag; t += gridDim.x) {
                         const int st = t % p.nst;
@@ -515,9 +586,10 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     }
                 }
             } else {
-                if (p.group == 1) {       // one kept block per stage: the plain loop
+                if (kResident || p.group == 1) {       // one kept block per stage: the plain loop
                     constexpr int kAhead = 8;            // block columns held in registers ahead of their use
-                    dst += p.entry_bytes;
+                    const uint32_t x_at = kResident ? 0u : p.entry_bytes;            // of the X tile in a stage
+                    dst += x_at;
                     for (int t = blockIdx.x; t < p.num_tiles && !*abort_flag; t += gridDim.x) {
                         const int st = t % p.nst, ct = t / p.nst;
                         const int len = min(walk_len[st], p.wcap);
@@ -540,6 +612,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                                     const int krow = jb * p.bk;
                                     if (e + kAhead < len) col_q[u] = cols[e + kAhead];
                                     if (!mbar_wait(empty, ph ^ 1u, abort_flag, p.wait_limit)) { ok = false; break; }
+                                    if constexpr (kResident) mbar_expect_tx(full, x_blk_bytes);
                                     if (fill_no++ != p.skip_fill) {
                                         if constexpr (kConv) {
                                             // block jb = filter tap (i, j), channels [c0, c0 + bk): the tile's pixel box
@@ -556,7 +629,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                                         }
                                     }
                                     dst += p.stage_bytes; full += 8; empty += 8;
-                                    if (dst == ring_end + p.entry_bytes) { dst = ring + p.entry_bytes; full = bar_full; empty = bar_empty; ph ^= 1u; }
+                                    if (dst == ring_end + x_at) { dst = ring + x_at; full = bar_full; empty = bar_empty; ph ^= 1u; }
                                 }
                             }
                         }
@@ -626,21 +699,21 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer: steps 2 + 3
         if (lane == 0) {
-            const MmaRoleArgs a{ring, bar_full, bar_empty, bar_tfull, bar_tempty, tmem_base, walk_len, abort_flag};
+            const MmaRoleArgs a{ring, bar_full, bar_empty, bar_tfull, bar_tempty, tmem_base, smem_base, bar_weights, walk_len, abort_flag};
             const int nmma = kSparse ? p.bk / 32 : p.bk / 16;        // K = 32 (sparse) or K = 16 steps per block
             if constexpr (kSparse) {
                 switch (nmma) {
-                    case 1: mma_role<kTileN, true, kAccStages, 1, kConv>(p, a); break;
-                    case 2: mma_role<kTileN, true, kAccStages, 2, kConv>(p, a); break;
-                    case 3: mma_role<kTileN, true, kAccStages, 3, kConv>(p, a); break;
-                    default: mma_role<kTileN, true, kAccStages, 4, kConv>(p, a); break;
+                    case 1: mma_role<kTileN, true, kAccStages, 1, kConv, kResident>(p, a); break;
+                    case 2: mma_role<kTileN, true, kAccStages, 2, kConv, kResident>(p, a); break;
+                    case 3: mma_role<kTileN, true, kAccStages, 3, kConv, kResident>(p, a); break;
+                    default: mma_role<kTileN, true, kAccStages, 4, kConv, kResident>(p, a); break;
                 }
             } else {
                 switch (nmma) {
-                    case 2: mma_role<kTileN, false, kAccStages, 2, kConv>(p, a); break;
-                    case 4: mma_role<kTileN, false, kAccStages, 4, kConv>(p, a); break;
-                    case 6: mma_role<kTileN, false, kAccStages, 6, kConv>(p, a); break;
-                    default: mma_role<kTileN, false, kAccStages, 8, kConv>(p, a); break;
+                    case 2: mma_role<kTileN, false, kAccStages, 2, kConv, kResident>(p, a); break;
+                    case 4: mma_role<kTileN, false, kAccStages, 4, kConv, kResident>(p, a); break;
+                    case 6: mma_role<kTileN, false, kAccStages, 6, kConv, kResident>(p, a); break;
+                    default: mma_role<kTileN, false, kAccStages, 8, kConv, kResident>(p, a); break;
                 }
             }
         }
@@ -658,7 +731,9 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         uint8_t *stg_gen = smem_gen + (stg - smem_base);
         uint32_t acc = 0, acc_ph = 0, slot = 0;
         for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
+            // (where the tile lies is worked out before the wait: its divisions would sit between accumulator and drain)
             const int st = t % p.nst, ct = t / p.nst;
+            TileOrigin org = tile_origin<kConv>(p, ct, kTileN);
             int go = 0;                                      // lane 0 waits, the warp follows it
             if (lane == 0) go = !*abort_flag && mbar_wait(bar_tfull + 8 * acc, acc_ph, abort_flag, p.wait_limit);
             go = __shfl_sync(0xFFFFFFFFu, go, 0);
@@ -670,7 +745,6 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             // (stack is 1, 2 or 4: 32q / (128 / stack) = q * stack / 4)
             const int grp = (q * p.stack) >> 2;
             const int y0 = st * kTileM + 32 * q - grp * (kTileM >> (p.stack >> 1));
-            TileOrigin org = tile_origin<kConv>(p, ct, kTileN);
             if constexpr (!kConv) org.x = (ct * p.stack + grp) * kTileN;
             // layer epilogue on the fp32 accumulator: this lane's row gets its bias, then the activation
             const bool fuse = p.bias != nullptr || p.relu != 0;
@@ -780,10 +854,10 @@ struct TcVariant {
     std::atomic<size_t> *configured;     // [kMaxDevices]
 };
 
-template <int NT, bool kSparse, int kAccStages, typename OutT, int kEpi, bool kConv>
+template <int NT, bool kSparse, int kAccStages, typename OutT, int kEpi, bool kConv, bool kResident = false>
 TcVariant make_variant() {
     static std::atomic<size_t> configured[kMaxDevices];
-    return TcVariant{spmm_tc_kernel<NT, kSparse, kAccStages, OutT, kEpi, kConv>, 96 + 32 * kEpi, configured};
+    return TcVariant{spmm_tc_kernel<NT, kSparse, kAccStages, OutT, kEpi, kConv, kResident>, 96 + 32 * kEpi, configured};
 }
 
 cudaError_t prepare_variant(const TcVariant &v, int device, size_t smem) {
@@ -902,7 +976,7 @@ TcImageLayout tc_image_layout(const Geometry &g, int kind) {
     L.addends = kind == CRISP_PATH_SPARSE2 ? 2 : 1;
     L.r = kTileM / g.bm;
     L.nst = (g.nrt + L.r - 1) / L.r;
-    const int64_t cap = (int64_t)L.r * g.kkeep;
+    const int64_t cap = (int64_t)(L.r < g.nrt ? L.r : g.nrt) * g.kkeep;      // a tile of fewer row tiles has a shorter union
     L.wcap = (int)(cap < g.nblk ? cap : g.nblk);
     // thin layers (a single CTA tile with at most 64 or 32 rows): 2 or 4 copies of every walk entry, shifted to
     // the other lane quarters, let one accumulator cover 2 or 4 column tiles (see launch_spmm_tc)
@@ -1022,23 +1096,35 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     p.num_tiles = (int)tiles;
     p.a_bytes = L.a_bytes; p.entry_bytes = L.entry_bytes; p.addends = (uint32_t)L.addends;
     p.box_bytes = (uint32_t)(kBoxN * g.bk * 2);
-    const uint32_t block_bytes = p.entry_bytes + nt * p.box_bytes;     // one kept block: weight tile (+ metadata) and X tile
     // Shared memory (the whole 227 KB; the base is 1024-aligned): the ring gets as many stages as fit next
     // to one staging tile per epilogue warp; what is left goes to the walk-list copy and to more staging
     // tiles.  Short walks are store-heavy and need no deep ring: they give stages up for staging tiles.
-    const uint32_t avail = kSmemBudget + 1024;
+    uint32_t avail = kSmemBudget + 1024;
+    // Convolutions of one CTA tile of rows and 2 to 8 blocks keep their weight tiles (kResident): 64 x 576 x 802816 62 us with
+    // them, 66 without (2:4); 60 and 68 (3:4).  A walk of one block gains nothing (10.8 and 10.1 us).
+    const bool resident = conv && short_walk && nt == 4 && L.nst == 1 && L.wcap >= 2 && p.addends == 1 &&
+                          (uint32_t)L.wcap * p.entry_bytes <= 80 * 1024;
+    if (resident) {
+        p.resident_bytes = (uint32_t)L.wcap * p.entry_bytes;     // (a multiple of 1024: so are the tiles and their metadata)
+        avail -= p.resident_bytes;
+    }
     const uint32_t epi = short_walk && nt >= 3 ? 4u * (uint32_t)nt : 8u;
-    const bool nhwc = conv && conv->nhwc_out;                // transposed chunks need whole 4096-byte staging tiles
-    const uint32_t fixed = epi * (nhwc ? 2 * kWideStageBytes : kWideStageBytes) + 256;
+    // transposed chunks of NHWC output: 64 pixels x 32 channels of bf16 in one 4096-byte staging tile, or, where the ring
+    // needs the room (resident weights), 32 pixels at a time; a chunk stored pixel by pixel goes through a whole tile
+    const bool nhwc = conv && conv->nhwc_out;
+    const uint32_t nhwc_tile = resident && y_dtype == 0 && (ldy * 2) % 16 == 0 && reinterpret_cast<uintptr_t>(d_y) % 16 == 0
+                                   ? kWideStageBytes : 2 * kWideStageBytes;
+    const uint32_t fixed = epi * (nhwc ? nhwc_tile : kWideStageBytes) + 256;
     // Blocks per pipeline stage.  A stage costs each single-thread role (weight producer, X producer, MMA issuer)
     // a fixed 300 to 400 cycles of waits, barrier arrivals and loop overhead on top of its copies and MMAs, which
     // for short or narrow blocks is more than the tensor core needs for the block.  Where the ring still holds at
     // least three of them, a stage therefore takes two or four consecutive walk entries: one weight-tile copy, one
     // wait and one commit for all of them.  (Needs the tiled weight map; 256-column tiles of 64-deep blocks stay
     // at one block per stage, two would leave room for two stages only.)
+    const uint32_t block_bytes = (resident ? 0u : p.entry_bytes) + nt * p.box_bytes;   // one kept block: weight tile (+ metadata) and X tile
     uint32_t group = 1;
     const bool bounded = h->group_override > 0;        // a caller's bound: the largest feasible size below it
-    for (uint32_t g = 4; g >= 2; g >>= 1) {
+    for (uint32_t g = 4; g >= 2 && !resident; g >>= 1) {
         if (bounded ? (int)g > h->group_override : L.wcap < 16) continue;   // walks below 16 blocks gain nothing (measured)
         if ((g * p.entry_bytes) % 256 != 0 || (g * p.entry_bytes) / 256 > 256) continue;   // one box of the weight map
         if ((avail - fixed) / (g * block_bytes) >= 3) { group = g; break; }
@@ -1046,7 +1132,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     p.group = group;
     p.stage_bytes = group * block_bytes;
     uint32_t stages = (avail - fixed) / p.stage_bytes;
-    const uint32_t max_stages = block_bytes <= 24 * 1024 ? (wlen <= 8 ? 6u : 7u) : (wlen <= 8 ? 4u : 8u);
+    const uint32_t max_stages = block_bytes <= 24 * 1024 ? (wlen <= 8 ? 6u : 7u) : (wlen <= 8 && !resident ? 4u : 8u);
     if (stages > max_stages) stages = max_stages;
     if (stages < 2) return cudaErrorInvalidValue;
     p.num_stages = stages;
@@ -1056,11 +1142,11 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     if (p.walk_cache) left -= cache_bytes;
     // staging per warp beyond the one 16-row tile already counted: two 32-row tiles, two 16-row tiles, or none
     const uint32_t unit = epi * kWideStageBytes;
-    if (nhwc) { p.stg_bufs = 1; p.stg_tile_bytes = 2 * kWideStageBytes; }
+    if (nhwc) { p.stg_bufs = 1; p.stg_tile_bytes = nhwc_tile; }
     else if (left >= 3 * unit) { p.stg_bufs = 2; p.stg_tile_bytes = 2 * kWideStageBytes; }
     else if (left >= unit) { p.stg_bufs = 2; p.stg_tile_bytes = kWideStageBytes; }
     else { p.stg_bufs = 1; p.stg_tile_bytes = kWideStageBytes; }
-    plan->smem = (size_t)stages * p.stage_bytes + (size_t)epi * p.stg_bufs * p.stg_tile_bytes + 256 +
+    plan->smem = (size_t)p.resident_bytes + (size_t)stages * p.stage_bytes + (size_t)epi * p.stg_bufs * p.stg_tile_bytes + 256 +
                  (p.walk_cache ? cache_bytes : 0);
 
     CUtensorMap &mx = plan->mx, &my = plan->my, &ma = plan->ma;
@@ -1093,7 +1179,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
             // Y [batch][ho][wo][ldy]: a chunk is {32 channels, tw, pixels / tw, 1}, laid out densely in the staging tile
             const uint64_t nd[4] = {(uint64_t)g.rows, wo, ho, (uint64_t)conv->batch};
             const uint64_t ns[3] = {(uint64_t)ldy * es, wo * (uint64_t)ldy * es, ho * wo * (uint64_t)ldy * es};
-            const uint32_t nb[4] = {32u, (uint32_t)p.cv_tw, (uint32_t)((f32 ? 32 : 64) / p.cv_tw), 1u};
+            const uint32_t nb[4] = {32u, (uint32_t)p.cv_tw, p.stg_tile_bytes / (uint32_t)(32 * es) / (uint32_t)p.cv_tw, 1u};
             if (!make_map_4d(&my, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (int)es, d_y, nd, ns, nb,
                              /*swizzle=*/false))
                 return cudaErrorInvalidValue;
@@ -1117,7 +1203,10 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     (acc = ACC, f32 ? make_variant<NTV, SP, ACC, float, EPI, CONV>() : make_variant<NTV, SP, ACC, uint16_t, EPI, CONV>())
 #define CRISP_TC_VARIANT_E(NTV, SP, ACC, EPI) CRISP_TC_VARIANT_C(NTV, SP, ACC, EPI, false)
 #define CRISP_TC_VARIANT(NTV, SP, ACC) CRISP_TC_VARIANT_E(NTV, SP, ACC, 8)
-    if (conv) {                              // the gather uses 128- or 256-pixel tiles only
+#define CRISP_TC_RESIDENT(SP, ACC) (acc = ACC, f32 ? make_variant<4, SP, ACC, float, 16, true, true>() : make_variant<4, SP, ACC, uint16_t, 16, true, true>())
+    if (resident) {
+        plan->variant = sparse ? CRISP_TC_RESIDENT(true, 1) : CRISP_TC_RESIDENT(false, 2);
+    } else if (conv) {                       // the gather uses 128- or 256-pixel tiles only
         if (sparse) {
             if (nt == 2) plan->variant = CRISP_TC_VARIANT_C(2, true, 2, 8, true);
             else plan->variant = epi == 16 ? CRISP_TC_VARIANT_C(4, true, 1, 16, true) : CRISP_TC_VARIANT_C(4, true, 1, 8, true);
@@ -1140,6 +1229,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
             default: plan->variant = epi == 16 ? CRISP_TC_VARIANT_E(4, false, 2, 16) : CRISP_TC_VARIANT(4, false, 2); break;
         }
     }
+#undef CRISP_TC_RESIDENT
 #undef CRISP_TC_VARIANT
 #undef CRISP_TC_VARIANT_E
 #undef CRISP_TC_VARIANT_C
