@@ -59,6 +59,23 @@ struct Batch {
 // launch_dependents() lets the next kernel of the stream start its own set-up (it waits in the same way).
 __device__ __forceinline__ void wait_for_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The kernels of the mask / encode / decode chain begin with this: the next kernel's launch overlaps this one.
+__device__ __forceinline__ void chain_kernels() { launch_dependents(); wait_for_prerequisites(); }
+
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, const Args &...args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
 #endif
 
 constexpr size_t kAlign = 256;

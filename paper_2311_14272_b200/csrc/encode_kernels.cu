@@ -73,6 +73,7 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
     __shared__ uint4 s_lut[16];
     __shared__ uint32_t s_map[kMaxBlockWords];               // kept columns of the tile (the union)
     __shared__ int s_slot[4];                                // where row tile i keeps this column, or -1
+    chain_kernels();
     const int l = batch.find(blockIdx.x);
     const EncodeLayer &L = batch.layer[l];
     const Geometry &g = L.g;
@@ -293,6 +294,7 @@ decode_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *_
               const uint32_t *__restrict__ idx, uint16_t *__restrict__ w, int64_t ld, bool vec_ok, int chunks) {
     constexpr int V = 8 / M * N, kBits = M == 4 ? 2 : 3, kRows = kDecodeRows / 8;
     __shared__ int s_slot[kDecodeCols / 32];
+    chain_kernels();
     const int rg = blockIdx.x / chunks, chunk = blockIdx.x - rg * chunks;
     const int row0 = rg * kDecodeRows, rt = row0 / g.bm;
     const int jb0 = chunk * kDecodeCols / g.bk;
@@ -390,8 +392,7 @@ cudaError_t run_encode_image(const Batch<EncodeLayer, CAP> &b, cudaStream_t st) 
     }
     if (b.first[b.n] == 0) return cudaSuccess;
     if (b.first[b.n] > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-    encode_kernel<M, N, IMAGE, CAP><<<(unsigned)b.first[b.n], 256, smem, st>>>(b);
-    return cudaGetLastError();
+    return launch_chained(encode_kernel<M, N, IMAGE, CAP>, (unsigned)b.first[b.n], 256, smem, st, b);
 }
 template <int M, int N, int CAP>
 cudaError_t run_encode(const Batch<EncodeLayer, CAP> &b, cudaStream_t st) {
@@ -465,7 +466,7 @@ cudaError_t launch_decode(const Geometry &g, const int32_t *d_blk_col, const uin
     if (ctas > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     const bool vec_ok = reinterpret_cast<uintptr_t>(d_w) % 16 == 0 && ld % 8 == 0;
 #define CRISP_DECODE(MV, NV)                                                                                        \
-    case NV: decode_kernel<MV, NV><<<(unsigned)ctas, 256, 0, st>>>(g, d_blk_col, d_vals, d_idx, d_w, ld, vec_ok, chunks); break
+    case NV: return launch_chained(decode_kernel<MV, NV>, (unsigned)ctas, 256, 0, st, g, d_blk_col, d_vals, d_idx, d_w, ld, vec_ok, chunks)
     if (g.m == 4) {
         switch (g.n) { CRISP_DECODE(4, 1); CRISP_DECODE(4, 2); CRISP_DECODE(4, 3); CRISP_DECODE(4, 4); default: return cudaErrorInvalidValue; }
     } else {
@@ -476,7 +477,6 @@ cudaError_t launch_decode(const Geometry &g, const int32_t *d_blk_col, const uin
         }
     }
 #undef CRISP_DECODE
-    return cudaGetLastError();
 }
 
 }  // namespace crisp

@@ -92,6 +92,7 @@ group_bits_kernel(const float *__restrict__ s, int64_t ld, Geometry g, bool vec_
                   bool find_max, uint32_t *__restrict__ max_key, uint32_t *__restrict__ nm_bits) {
     __shared__ uint8_t s_keep[64];
     __shared__ uint32_t s_best[kM1Threads / 32];
+    chain_kernels();
     if (M == 4 && threadIdx.x < 64) s_keep[threadIdx.x] = (uint8_t)keep_mask_of_outcomes(threadIdx.x, g.n);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -168,6 +169,7 @@ __device__ __forceinline__ void floor_parts2(uint64_t v, uint64_t &r, uint64_t &
 template <int CAP>
 __global__ void __launch_bounds__(kM1Threads)
 block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
+    chain_kernels();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t unit = blockIdx.x; unit < batch.first[batch.n]; unit += gridDim.x) {
     const int l = batch.find(unit);
@@ -242,6 +244,7 @@ template <int CAP>
 __global__ void __launch_bounds__(256)
 block_select_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     extern __shared__ unsigned long long sm[];
+    chain_kernels();
     const int l = batch.find(blockIdx.x);
     const ScoreLayer &L = batch.layer[l];
     const Geometry &g = L.g;
@@ -301,6 +304,7 @@ block_select_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
 template <int CAP>
 __global__ void __launch_bounds__(256)
 clear_scores_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
+    chain_kernels();
     const ScoreLayer &L = batch.layer[blockIdx.x];
     if (threadIdx.x == 0) *const_cast<uint32_t *>(L.max_key) = 0u;
     const int64_t n = (int64_t)L.g.nrt * L.g.nblk;
@@ -361,8 +365,7 @@ cudaError_t run_block_select(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
         if (e != cudaSuccess) return e;
     }
     if (b.first[b.n] == 0) return cudaSuccess;
-    block_select_kernel<CAP><<<(unsigned)b.first[b.n], 256, smem, st>>>(b);
-    return cudaGetLastError();
+    return launch_chained(block_select_kernel<CAP>, (unsigned)b.first[b.n], 256, smem, st, b);
 }
 
 }  // namespace
@@ -374,8 +377,7 @@ size_t mask_workspace_bytes(const Geometry &g) {
 
 cudaError_t launch_clear_scores(const ScoreLayer *layers, int n, cudaStream_t st) {
     return for_batches(layers, n, [](const Geometry &) { return (int64_t)1; }, [&](const Batch<ScoreLayer, kBatchLayers> &b) {
-        clear_scores_kernel<kBatchLayers><<<(unsigned)b.n, 256, 0, st>>>(b);
-        return cudaGetLastError();
+        return launch_chained(clear_scores_kernel<kBatchLayers>, (unsigned)b.n, 256, 0, st, b);
     });
 }
 
@@ -383,8 +385,7 @@ cudaError_t launch_block_scores(const ScoreLayer *layers, int n, cudaStream_t st
     return for_batches(layers, n, [](const Geometry &g) { return (g.mp() / kM1Rows) * (int64_t)saliency_chunks(g); },
                        [&](const Batch<ScoreLayer, kBatchLayers> &b) {
                            const int grid = resident_grid((const void *)block_score_kernel<kBatchLayers>, b.first[b.n]);
-                           block_score_kernel<kBatchLayers><<<grid, kM1Threads, 0, st>>>(b);
-                           return cudaGetLastError();
+                           return launch_chained(block_score_kernel<kBatchLayers>, (unsigned)grid, kM1Threads, 0, st, b);
                        });
 }
 
@@ -424,8 +425,10 @@ cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, i
             d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
     ScoreLayer L = {};
     L.g = g; L.s = d_s; L.ld = ld; L.max_key = max_key; L.nm_bits = d_nm_bits; L.score = score; L.blk_col = d_blk_col;
-    block_score_kernel<1><<<resident_grid((const void *)block_score_kernel<1>, items), kM1Threads, 0, st>>>(batch_of_one(L, items));
     e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_chained(block_score_kernel<1>, (unsigned)resident_grid((const void *)block_score_kernel<1>, items), kM1Threads, 0, st,
+                           batch_of_one(L, items));
     if (e != cudaSuccess) return e;
     return run_block_select(batch_of_one(L, select_ctas(g)), st);
 }

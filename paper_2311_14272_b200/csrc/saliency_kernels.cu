@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kM1Threads)
 saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
     __shared__ uint8_t s_keep[64];
     __shared__ uint32_t s_best[kM1Threads / 32];
+    chain_kernels();
     const int l = batch.b.find(blockIdx.x);
     const SaliencyLayer &L = batch.b.layer[l];
     const Geometry &g = L.g;
@@ -248,10 +249,10 @@ cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreL
     auto flush = [&]() -> cudaError_t {
         if (b.n == 0) return cudaSuccess;
         if (b.first[b.n] > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-        if (b.layer[0].g.m == 4) saliency_bits_kernel<4><<<(unsigned)b.first[b.n], kM1Threads, 0, st>>>(*batch);
-        else saliency_bits_kernel<8><<<(unsigned)b.first[b.n], kM1Threads, 0, st>>>(*batch);
+        const cudaError_t e = launch_chained(b.layer[0].g.m == 4 ? saliency_bits_kernel<4> : saliency_bits_kernel<8>,
+                                             (unsigned)b.first[b.n], kM1Threads, 0, st, *batch);
         b.n = 0; grads = 0;
-        return cudaGetLastError();
+        return e;
     };
     for (int l = 0; l < n; ++l) {
         const crisp_prune_layer_t &P = layers[l];
