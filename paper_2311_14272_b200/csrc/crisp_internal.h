@@ -74,7 +74,9 @@ cudaError_t launch_chained(void (*kern)(Params...), unsigned grid, unsigned thre
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();          // reported here, not to the caller's next check
+    return e;
 }
 #endif
 
