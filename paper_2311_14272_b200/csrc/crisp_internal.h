@@ -57,6 +57,10 @@ struct Batch {
 // kernel in front of it in the stream has finished; wait_for_prerequisites() returns when that one has finished and its
 // writes are visible, and every thread that touches global memory another kernel may write or read calls it first.
 // launch_dependents() lets the next kernel of the stream start its own set-up (it waits in the same way).
+// Such a kernel is alive while its predecessors still write, so it reads whatever another kernel may have written (which
+// is every buffer of the caller too: the weights may come from crisp_decode) with plain loads, behind the wait.  The
+// read-only path (__ldg, const __restrict__) is for data that stays as it is for the kernel's whole life: its loads may be
+// moved above the wait and need not see what the wait makes visible.  (Plain loads take the same time.)
 __device__ __forceinline__ void wait_for_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // The kernels of the mask / encode / decode chain begin with this: the next kernel's launch overlaps this one.

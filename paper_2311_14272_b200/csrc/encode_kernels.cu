@@ -86,21 +86,21 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
     const bool lists = L.walk_col != nullptr;
     int jb;
     if (r == 1) {                                            // the walk list is the row tile's kept list
-        jb = __ldg(L.mask_blk_col + (int64_t)st * g.kkeep + entry);
+        jb = L.mask_blk_col[(int64_t)st * g.kkeep + entry];
         if (threadIdx.x < 4) s_slot[threadIdx.x] = threadIdx.x == 0 ? entry : -1;
         if (threadIdx.x >= 32 && threadIdx.x < 48) s_lut[threadIdx.x - 32] = nibble_entry(threadIdx.x - 32);
         if (lists && entry == 0 && threadIdx.x == 0) L.walk_len[st] = g.kkeep;
         __syncthreads();
     } else {
         const int map_words = (g.nblk + 31) / 32, listed = n_rt * g.kkeep;
-        const int c = threadIdx.x < listed ? __ldg(L.mask_blk_col + (int64_t)first_rt * g.kkeep + threadIdx.x) : 0;
+        const int c = threadIdx.x < listed ? L.mask_blk_col[(int64_t)first_rt * g.kkeep + threadIdx.x] : 0;
         for (int i = threadIdx.x; i < map_words; i += blockDim.x) s_map[i] = 0u;
         if (threadIdx.x < 4) s_slot[threadIdx.x] = -1;
         if (threadIdx.x >= 32 && threadIdx.x < 48) s_lut[threadIdx.x - 32] = nibble_entry(threadIdx.x - 32);
         __syncthreads();
         if (threadIdx.x < listed) atomicOr(&s_map[c >> 5], 1u << (c & 31));
         for (int i = threadIdx.x + blockDim.x; i < listed; i += blockDim.x) {
-            const int d = __ldg(L.mask_blk_col + (int64_t)first_rt * g.kkeep + i);
+            const int d = L.mask_blk_col[(int64_t)first_rt * g.kkeep + i];
             atomicOr(&s_map[d >> 5], 1u << (d & 31));
         }
         __syncthreads();
@@ -121,7 +121,7 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
         jb = word * 32 + __ffs(left) - 1;
         if (threadIdx.x < listed && c == jb) { const int q = threadIdx.x / g.kkeep; s_slot[q] = threadIdx.x - q * g.kkeep; }
         for (int i = threadIdx.x + blockDim.x; i < listed; i += blockDim.x)
-            if (__ldg(L.mask_blk_col + (int64_t)first_rt * g.kkeep + i) == jb) { const int q = i / g.kkeep; s_slot[q] = i - q * g.kkeep; }
+            if (L.mask_blk_col[(int64_t)first_rt * g.kkeep + i] == jb) { const int q = i / g.kkeep; s_slot[q] = i - q * g.kkeep; }
         __syncthreads();
     }
     if (lists && threadIdx.x == 0) L.walk_col[(int64_t)st * L.wcap + entry] = jb;
@@ -167,11 +167,11 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
                 if (grow + row < g.rows) {
                     const uint16_t *p = w_col + row * L.ld;
                     if (wide) {
-                        wv[u] = __ldg(reinterpret_cast<const uint4 *>(p));
+                        wv[u] = *reinterpret_cast<const uint4 *>(p);
                     } else {
                         uint32_t e[8];
 #pragma unroll
-                        for (int t = 0; t < 8; ++t) e[t] = col + t < g.k ? (uint32_t)__ldg(p + t) : 0u;
+                        for (int t = 0; t < 8; ++t) e[t] = col + t < g.k ? (uint32_t)p[t] : 0u;
                         wv[u] = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
                     }
                 }
@@ -290,8 +290,8 @@ constexpr int kDecodeRows = 32, kDecodeCols = 256;
 
 template <int M, int N>
 __global__ void __launch_bounds__(256)
-decode_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *__restrict__ vals,
-              const uint32_t *__restrict__ idx, uint16_t *__restrict__ w, int64_t ld, bool vec_ok, int chunks) {
+decode_kernel(Geometry g, const int32_t *blk_col, const uint16_t *vals, const uint32_t *idx, uint16_t *w, int64_t ld,
+              bool vec_ok, int chunks) {
     constexpr int V = 8 / M * N, kBits = M == 4 ? 2 : 3, kRows = kDecodeRows / 8;
     __shared__ int s_slot[kDecodeCols / 32];
     chain_kernels();
@@ -301,7 +301,7 @@ decode_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *_
     if (threadIdx.x < kDecodeCols / 32) s_slot[threadIdx.x] = -1;
     __syncthreads();
     for (int i = threadIdx.x; i < g.kkeep; i += blockDim.x) {
-        const int d = __ldg(blk_col + (int64_t)rt * g.kkeep + i) - jb0;
+        const int d = blk_col[(int64_t)rt * g.kkeep + i] - jb0;
         if (d >= 0 && d < kDecodeCols / 32) s_slot[d] = i;          // (block columns beyond the chunk do no harm)
     }
     __syncthreads();
@@ -321,25 +321,25 @@ decode_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *_
         for (int i = 0; i < kRows; ++i) {
             const int o = ((first + i - rt * g.bm) * groups + (k0 - jb * g.bk) / M) * N;     // (rows of padding are stored too)
             if constexpr (V == 8) {
-                const uint4 t = __ldg(reinterpret_cast<const uint4 *>(vin + o));
+                const uint4 t = *reinterpret_cast<const uint4 *>(vin + o);
                 v[i][0] = (uint16_t)t.x; v[i][1] = (uint16_t)(t.x >> 16); v[i][2] = (uint16_t)t.y; v[i][3] = (uint16_t)(t.y >> 16);
                 v[i][4] = (uint16_t)t.z; v[i][5] = (uint16_t)(t.z >> 16); v[i][6] = (uint16_t)t.w; v[i][7] = (uint16_t)(t.w >> 16);
             } else if constexpr (V == 4) {
-                const uint2 t = __ldg(reinterpret_cast<const uint2 *>(vin + o));
+                const uint2 t = *reinterpret_cast<const uint2 *>(vin + o);
                 v[i][0] = (uint16_t)t.x; v[i][1] = (uint16_t)(t.x >> 16); v[i][2] = (uint16_t)t.y; v[i][3] = (uint16_t)(t.y >> 16);
             } else if constexpr (V % 2 == 0) {
 #pragma unroll
                 for (int j = 0; j < V; j += 2) {
-                    const uint32_t t = __ldg(reinterpret_cast<const uint32_t *>(vin + o + j));
+                    const uint32_t t = *reinterpret_cast<const uint32_t *>(vin + o + j);
                     v[i][j] = (uint16_t)t; v[i][j + 1] = (uint16_t)(t >> 16);
                 }
             } else {
 #pragma unroll
-                for (int j = 0; j < V; ++j) v[i][j] = __ldg(vin + o + j);
+                for (int j = 0; j < V; ++j) v[i][j] = vin[o + j];
             }
             const int bit = o * kBits;
-            uint32_t t = __ldg(iin + (bit >> 5)) >> (bit & 31);
-            if (32 % (V * kBits) != 0 && (bit & 31) + V * kBits > 32) t |= __ldg(iin + (bit >> 5) + 1) << (32 - (bit & 31));
+            uint32_t t = iin[bit >> 5] >> (bit & 31);
+            if (32 % (V * kBits) != 0 && (bit & 31) + V * kBits > 32) t |= iin[(bit >> 5) + 1] << (32 - (bit & 31));
             f[i] = t;
         }
     }

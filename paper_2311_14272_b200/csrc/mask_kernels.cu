@@ -19,16 +19,15 @@ constexpr int kScoreFractionBits = 40;
 
 // Raw bits of eight consecutive saliency values; the caller guarantees row < rows, k0 + 8 <= k and
 // 16-byte alignment.  Kept free of branches so that several of these can be in flight per lane.
-__device__ __forceinline__ void load8_raw(const float *__restrict__ s, int64_t ld, int64_t row, int64_t k0,
-                                          uint32_t key[8]) {
+__device__ __forceinline__ void load8_raw(const float *s, int64_t ld, int64_t row, int64_t k0, uint32_t key[8]) {
     const uint4 *p = reinterpret_cast<const uint4 *>(s + row * ld + k0);
-    const uint4 a = __ldg(p), b = __ldg(p + 1);
+    const uint4 a = p[0], b = p[1];
     key[0] = a.x; key[1] = a.y; key[2] = a.z; key[3] = a.w;
     key[4] = b.x; key[5] = b.y; key[6] = b.z; key[7] = b.w;
 }
 // Eight consecutive saliency values of one row, zero beyond the matrix.
-__device__ __forceinline__ void load8(const float *__restrict__ s, int64_t ld, int rows, int k,
-                                      int64_t row, int64_t k0, bool vec_ok, uint32_t key[8]) {
+__device__ __forceinline__ void load8(const float *s, int64_t ld, int rows, int k, int64_t row, int64_t k0, bool vec_ok,
+                                      uint32_t key[8]) {
     if (row >= rows || k0 >= k) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) key[i] = 0u;
@@ -36,15 +35,15 @@ __device__ __forceinline__ void load8(const float *__restrict__ s, int64_t ld, i
     }
     const float *p = s + row * ld + k0;
     if (vec_ok && k0 + 8 <= k) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        const float4 b = reinterpret_cast<const float4 *>(p)[1];
         key[0] = canonical_key(a.x); key[1] = canonical_key(a.y);
         key[2] = canonical_key(a.z); key[3] = canonical_key(a.w);
         key[4] = canonical_key(b.x); key[5] = canonical_key(b.y);
         key[6] = canonical_key(b.z); key[7] = canonical_key(b.w);
     } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) key[i] = (k0 + i < k) ? canonical_key(__ldg(p + i)) : 0u;
+        for (int i = 0; i < 8; ++i) key[i] = (k0 + i < k) ? canonical_key(p[i]) : 0u;
     }
 }
 
@@ -67,7 +66,7 @@ __device__ __forceinline__ unsigned long long fixed_point_score(uint32_t key, in
 
 // The 8 canonical keys of the lane's elements of row `row` (zero beyond the matrix).  kCap = false leaves infinities in.
 template <bool kCap = true>
-__device__ __forceinline__ void m1_load_rows(const float *__restrict__ s, int64_t ld, const Geometry &g, bool vec_ok,
+__device__ __forceinline__ void m1_load_rows(const float *s, int64_t ld, const Geometry &g, bool vec_ok,
                                              const M1Item &x, int warp, int64_t k0, uint32_t key[kM1RowsPerWarp][8]) {
     if (vec_ok && x.row0 + kM1Rows <= g.rows && (int64_t)(x.chunk + 1) * kM1ChunkK <= g.k) {   // interior item
 #pragma unroll
@@ -90,8 +89,8 @@ __device__ __forceinline__ void m1_load_rows(const float *__restrict__ s, int64_
 // find_max = false when the caller already knows the maximum.
 template <int M>
 __global__ void __launch_bounds__(kM1Threads)
-group_bits_kernel(const float *__restrict__ s, int64_t ld, Geometry g, bool vec_ok, int64_t items, int chunks,
-                  bool find_max, uint32_t *__restrict__ max_key, uint32_t *__restrict__ nm_bits) {
+group_bits_kernel(const float *s, int64_t ld, Geometry g, bool vec_ok, int64_t items, int chunks, bool find_max,
+                  uint32_t *max_key, uint32_t *nm_bits) {
     __shared__ uint8_t s_keep[64];
     __shared__ uint32_t s_best[kM1Threads / 32];
     chain_kernels();
@@ -188,9 +187,9 @@ block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     const int l = batch.find(unit);
     const ScoreLayer &L = batch.layer[l];
     const Geometry &g = L.g;
-    const float *__restrict__ s = L.s;
+    const float *s = L.s;
     const int64_t ld = L.ld;
-    const uint32_t *__restrict__ nm_bits = L.nm_bits;
+    const uint32_t *nm_bits = L.nm_bits;
     const uint32_t mk = *L.max_key;
     if (!mk) continue;                                       // an all-zero layer: every score stays 0
     const int e_max = key_exponent(mk);
@@ -295,9 +294,9 @@ block_select_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     const int l = batch.find(blockIdx.x);
     const ScoreLayer &L = batch.layer[l];
     const Geometry &g = L.g;
-    const unsigned long long *__restrict__ score = L.score;
-    int32_t *__restrict__ blk_col = L.blk_col;
-    uint32_t *__restrict__ nm_bits = L.nm_bits;
+    const unsigned long long *score = L.score;
+    int32_t *blk_col = L.blk_col;
+    uint32_t *nm_bits = L.nm_bits;
     unsigned long long *sc = sm;                                   // [nblk]
     int *kept = reinterpret_cast<int *>(sm + g.nblk);              // [nblk]
     __shared__ int s_warp_tot[8];

@@ -139,14 +139,14 @@ saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
     if (L.vec_ok && row0 + kM1RowsPerWarp <= g.rows && k0 + 8 <= g.k) {
         uint4 wr[kM1RowsPerWarp];
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i) wr[i] = __ldg(reinterpret_cast<const uint4 *>(L.w + (row0 + i) * L.ld_w + k0));
+        for (int i = 0; i < kM1RowsPerWarp; ++i) wr[i] = *reinterpret_cast<const uint4 *>(L.w + (row0 + i) * L.ld_w + k0);
         for (int h = 0; h < L.samples; ++h) {
             const GradRef G = batch.grad[L.grad0 + h];
             if (G.ld > 0) {
                 uint4 t[kM1RowsPerWarp];
 #pragma unroll
                 for (int i = 0; i < kM1RowsPerWarp; ++i)
-                    t[i] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(G.p) + (row0 + i) * G.ld + k0));
+                    t[i] = *reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(G.p) + (row0 + i) * G.ld + k0);
 #pragma unroll
                 for (int i = 0; i < kM1RowsPerWarp; ++i) {
                     const uint32_t q[4] = {t[i].x, t[i].y, t[i].z, t[i].w};
@@ -160,7 +160,6 @@ saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
             } else {
 #pragma unroll
                 for (int i = 0; i < kM1RowsPerWarp; ++i) {
-                    // (no read-only loads: the running sum of more samples than the table holds is the layer's own S)
                     const float4 *p = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(G.p) + (row0 + i) * -G.ld + k0);
                     const float4 a = p[0], b = p[1];
                     const float q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};

@@ -1,0 +1,90 @@
+"""Kernels launched with programmatic dependent launch are alive while the kernels in front of them still write: checks on
+the sources that such a kernel reads no data through the read-only path, which is defined only for data that nobody writes
+during the kernel's life, and, on the GPU, that chains of them hand over what was written last."""
+import glob
+import os
+import re
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2311_14272_b200", "csrc")
+WAIT = re.compile(r"\b(?:chain_kernels|wait_for_prerequisites)\(\)")
+
+
+def functions(text):
+    """(header, name, body) of every function with a body at namespace level."""
+    text = re.sub(r"//[^\n]*|/\*.*?\*/|__launch_bounds__\([^()]*\)", "", text, flags=re.S)
+    for m in re.finditer(r"((?:__global__|__device__)[^;{}]*?(\w+)\s*\([^;{}]*\))\s*\{", text):
+        depth, at = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[at], 0)
+            at += 1
+        yield m.group(1), m.group(2), text[m.end():at - 1]
+
+
+def chained_kernels():
+    out = {}
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = open(path).read() + "".join(open(p).read() for p in sorted(glob.glob(os.path.join(CSRC, "*.cuh"))))
+        fns = list(functions(text))
+        for header, name, body in fns:
+            if "__global__" not in header or not WAIT.search(body):
+                continue
+            # with the device functions it calls, and theirs
+            reached, todo = {}, [body]
+            while todo:
+                b = todo.pop()
+                for h, n, inner in fns:
+                    if n not in reached and "__global__" not in h and re.search(r"\b%s\b\s*[<(]" % n, b):
+                        reached[n] = h + "{" + inner + "}"
+                        todo.append(inner)
+            out[name] = (header, body, reached)
+    return out
+
+
+def test_the_chained_kernels_are_found():
+    assert {"encode_kernel", "decode_kernel", "block_score_kernel", "block_select_kernel", "clear_scores_kernel",
+            "saliency_bits_kernel", "spmm_tc_kernel"} <= set(chained_kernels())
+
+
+@pytest.mark.parametrize("name", sorted(chained_kernels()))
+def test_chained_kernel_has_no_read_only_loads(name):
+    header, body, reached = chained_kernels()[name]
+    for where, text in [(name, header + body)] + sorted(reached.items()):
+        assert "__ldg" not in text and "ld.global.nc" not in text, where
+        assert not re.search(r"\bconst\b[^,;()=]*__restrict__", text), where
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,m,bm,bk", [(2, 4, 128, 64), (4, 8, 32, 32), (3, 4, 64, 96)])
+def test_chain_of_encode_and_decode_hands_over_the_newest_data(n, m, bm, bk):
+    """mask, encode and decode of one layer's buffers over and over, with new weights each time and no wait between."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    rows, k, rounds = 640, 1152, 24
+    g = torch.Generator(device="cuda").manual_seed(n * 100 + bm)
+    ws = [torch.randn(rows, k, generator=g, device="cuda").bfloat16() for _ in range(rounds)]
+    L = B.HybridLayer(rows, k, n, m, bm, bk, 0.5)
+    outs, again = [], []
+    for w in ws:
+        L.build_mask(w.float().abs()).encode(w)
+        outs.append(L.decode())
+        L.encode(outs[-1])                        # the weights of this encode are what decode just wrote
+        again.append(L.decode())
+    # the same, each call finished before the next
+    for w, out, out2 in zip(ws, outs, again):
+        sal = w.float().abs()
+        torch.cuda.synchronize()
+        L.build_mask(sal)
+        torch.cuda.synchronize()
+        L.encode(w)
+        torch.cuda.synchronize()
+        ref = L.decode()
+        torch.cuda.synchronize()
+        assert int((ref != 0).sum()) > 0
+        assert torch.equal(ref.view(torch.int16), out.view(torch.int16))
+        assert torch.equal(ref.view(torch.int16), out2.view(torch.int16))
+    L.close()
