@@ -461,6 +461,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const uint32_t smem_base = smem_u32(smem_raw);
     uint8_t *smem_gen = smem_raw;
     if (smem_base & 1023u) {                 // swizzled operand tiles need it; checked, not assumed
+        wait_for_prerequisites();            // (the kernel behind this one waits for this one only)
         if (threadIdx.x == 0) atomicCAS(p.status, 0, (int)CRISP_CUDA_ERROR);
         return;
     }

@@ -57,6 +57,16 @@ def test_chained_kernel_has_no_read_only_loads(name):
         assert not re.search(r"\bconst\b[^,;()=]*__restrict__", text), where
 
 
+@pytest.mark.parametrize("name", sorted(chained_kernels()))
+def test_no_exit_of_a_chained_kernel_before_its_wait(name):
+    """The kernel behind it waits for this one alone: that it also comes after the one in front of this one holds only if
+    every thread of this one waited."""
+    _, body, _ = chained_kernels()[name]
+    last = [w.start() for w in WAIT.finditer(body)][-1]
+    for r in re.finditer(r"\breturn\b", body[:last]):
+        assert WAIT.search(body, body.rfind("{", 0, r.start()), r.start()), body[:r.end()][-200:]
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,m,bm,bk", [(2, 4, 128, 64), (4, 8, 32, 32), (3, 4, 64, 96)])
 def test_chain_of_encode_and_decode_hands_over_the_newest_data(n, m, bm, bk):
