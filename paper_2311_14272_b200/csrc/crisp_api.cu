@@ -11,10 +11,10 @@
 using crisp::align_up;
 using crisp::Geometry;
 using crisp::kAlign;
+using crisp::kMaxBlocksPerRowTile;
 
 namespace {
 
-constexpr int kMaxBlocksPerRowTile = 4096;   // block_select_kernel keeps a row tile's scores in shared memory
 constexpr int kMaxRowTiles = 65535;
 
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }

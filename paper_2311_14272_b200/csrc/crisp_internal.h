@@ -84,6 +84,7 @@ cudaError_t launch_chained(void (*kern)(Params...), unsigned grid, unsigned thre
 }
 #endif
 
+constexpr int kMaxBlocksPerRowTile = 4096;
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 
@@ -155,7 +156,7 @@ size_t mask_workspace_bytes(const Geometry &g);
 cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreLayer *scores, int n, cudaStream_t st);
 
 // encode_kernels.cu
-constexpr int kMaxBlockWords = 128;      // nblk <= 4096
+constexpr int kMaxBlockWords = kMaxBlocksPerRowTile / 32;
 // One layer of an encode launch: canonical blocks, and the execution image of `kind` with its walk lists (kind DIRECT:
 // canonical blocks only, walk_col = nullptr).  The layers of one launch share n and m.
 struct EncodeLayer {

@@ -75,6 +75,10 @@ struct DirectTile {
     static constexpr int kStageRows = CPL == 4 ? 64 : 128;
     static constexpr int kStages = CPL == 4 ? 3 : 4;
     static constexpr int kPitch = kTileN * 2 + 16;           // a row of X: the aligned 16-byte words that hold kTileN elements
+    // Dynamic shared memory at most: a stage holds kStageRows rows of X and, for each of the kRows rows, up to kStageRows weights
+    // of 2 bytes with offsets of 3 bits (n = m = 8); the weight words and the block list come after the stages.
+    static constexpr int kMostSmem = kStages * kStageRows * (kPitch + kRows * 2 + kRows * 3 / 8) + kRows * kStageRows * 4 + 4 * kMaxBlocksPerRowTile;
+    static_assert(kMostSmem <= 227 * 1024, "shared memory of a CTA");
 };
 
 // ALIGN: bytes every row of X is aligned to (2, 4 or 8), which fixes the columns a lane owns: consecutive ones as far as
@@ -299,10 +303,10 @@ cudaError_t launch_form(const Geometry &g, const int32_t *bc, const uint16_t *va
     if (ctas > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     const uintptr_t al = reinterpret_cast<uintptr_t>(x) | (uintptr_t)(ldx * 2);
     auto launch = [&](auto kern) {
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        // The limit belongs to the function, so it is the same at every call: set to a call's own size, it would refuse the
+        // larger launch of another host thread that set it a moment before.
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kMostSmem);
+        if (e != cudaSuccess) return e;
         kern<<<(unsigned)ctas, T::kThreads, smem, st>>>(g, bc, vals, idx, x, ldx, ncols, y, ldy, epi, sp);
         return cudaGetLastError();
     };
