@@ -416,15 +416,16 @@ cudaError_t run_block_scores_any(const Batch<ScoreLayer, CAP> &b, cudaStream_t s
     return run_block_scores<CAP, 4, 0>(b, st);
 }
 
-size_t select_smem(const Geometry &g) { return (size_t)g.nblk * (sizeof(unsigned long long) + sizeof(int)); }
+size_t select_smem(int nblk) { return (size_t)nblk * (sizeof(unsigned long long) + sizeof(int)); }
 int64_t select_ctas(const Geometry &g) { return (int64_t)g.nrt * (g.bm / 32); }
 
 template <int CAP>
 cudaError_t run_block_select(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
     size_t smem = 0;
-    for (int i = 0; i < b.n; ++i) smem = select_smem(b.layer[i].g) > smem ? select_smem(b.layer[i].g) : smem;
+    for (int i = 0; i < b.n; ++i) smem = select_smem(b.layer[i].g.nblk) > smem ? select_smem(b.layer[i].g.nblk) : smem;
     if (smem + 64 > 48 * 1024) {     // the longest rows (nblk near 4096) need the opt-in shared-memory size
-        cudaError_t e = cudaFuncSetAttribute(block_select_kernel<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // (the same limit at every call: it belongs to the function, which several host threads may be launching)
+        cudaError_t e = cudaFuncSetAttribute(block_select_kernel<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)select_smem(kMaxBlocksPerRowTile));
         if (e != cudaSuccess) return e;
     }
     if (b.first[b.n] == 0) return cudaSuccess;

@@ -854,21 +854,23 @@ constexpr int kMaxDevices = 64;
 struct TcVariant {
     TcKernel kern;
     int threads;
-    std::atomic<size_t> *configured;     // [kMaxDevices]
+    std::atomic<bool> *configured;       // [kMaxDevices]
 };
 
 template <int NT, bool kSparse, int kAccStages, typename OutT, int kEpi, bool kConv, bool kResident = false>
 TcVariant make_variant() {
-    static std::atomic<size_t> configured[kMaxDevices];
+    static std::atomic<bool> configured[kMaxDevices];
     return TcVariant{spmm_tc_kernel<NT, kSparse, kAccStages, OutT, kEpi, kConv, kResident>, 96 + 32 * kEpi, configured};
 }
 
-cudaError_t prepare_variant(const TcVariant &v, int device, size_t smem) {
+// Opts a kernel in to all the shared memory there is (it has none of its own), once per device.  The limit belongs to the
+// function: were it a plan's own size, the smaller plan of another host thread could lower it behind a larger one's back.
+cudaError_t prepare_variant(const TcVariant &v, int device) {
     if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (smem <= v.configured[device].load(std::memory_order_relaxed)) return cudaSuccess;
+    if (v.configured[device].load(std::memory_order_relaxed)) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(v.kern),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) v.configured[device].store(smem, std::memory_order_relaxed);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 1024);
+    if (e == cudaSuccess) v.configured[device].store(true, std::memory_order_relaxed);
     return e;
 }
 
@@ -1246,7 +1248,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     info.ctas = plan->grid;
     info.conv = conv ? 1 : 0;
     info.stage_blocks = (int)p.group;
-    return prepare_variant(plan->variant, device, plan->smem);
+    return prepare_variant(plan->variant, device);
 }
 
 }  // namespace

@@ -57,3 +57,21 @@ def test_direct_products_of_two_threads(ncols):
         assert torch.equal(y, ref)
     for L in layers:
         L.close()
+
+
+def test_block_selections_of_two_threads():
+    """Rows of more than 4090 blocks need more shared memory than a kernel has without asking."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    layers, refs = [], []
+    for nblk, seed in ((4096, 1), (4091, 2)):
+        L = make_layer(B, torch, 32, 32 * nblk, 2, 4, 32, 32, 1.0, seed)
+        layers.append(L.reselect(nblk // 2))
+        refs.append(L.export_mask())
+    jobs = [lambda L=L: L.reselect(L.kkeep) for L in layers]
+    assert run_together(torch, jobs, 3000) == []
+    for L, (blk_col, nm_bits) in zip(layers, refs):
+        got = L.export_mask()
+        assert (got[0] == blk_col).all() and (got[1] == nm_bits).all()
+        L.close()
