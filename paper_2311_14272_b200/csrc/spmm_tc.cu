@@ -907,6 +907,22 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
+// Tensor maps are encoded by the driver, which wants a current context.  The runtime makes one current in a host thread
+// with the first call that needs it; in a thread whose first call is a product, no such call has come yet.
+cudaError_t ensure_context(int device) {
+    typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
+    static CtxGetCurrentFn current = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuCtxGetCurrent", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<CtxGetCurrentFn>(p);
+    }();
+    CUcontext ctx = nullptr;
+    if (current && current(&ctx) == CUDA_SUCCESS && ctx) return cudaSuccess;
+    return cudaSetDevice(device);
+}
+
 bool make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_bytes, const void *base, uint64_t inner,
                  uint64_t outer, uint64_t ld_elems, uint32_t box_inner, uint32_t box_outer) {
     EncodeTiledFn fn = encode_tiled_fn();
@@ -1274,6 +1290,8 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
             h->plan = plan;
         }
         plan->x = nullptr;                                  // not valid until the plan below is complete
+        e = ensure_context(device);
+        if (e != cudaSuccess) return e;
         e = make_plan(h, kind, d_x, ldx, ncols, d_y, ldy, y_dtype, conv, device, plan);
         if (e != cudaSuccess) return e;
         plan->x = d_x; plan->y = d_y; plan->bias = h->epilogue.bias;

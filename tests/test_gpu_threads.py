@@ -75,3 +75,62 @@ def test_block_selections_of_two_threads():
         got = L.export_mask()
         assert (got[0] == blk_col).all() and (got[1] == nm_bits).all()
         L.close()
+
+
+def test_tensor_core_products_of_two_threads():
+    """Two layers of the same kernel, planned anew at every call (the buffers alternate), one with a copy of its walk lists in
+    shared memory beside the ring and one whose ring ends sooner."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    jobs, outs, refs, layers = [], [], [], []
+    for (rows, k, keep, seed) in ((512, 1024, 0.5, 1), (640, 2048, 0.9, 2)):
+        L = make_layer(B, torch, rows, k, 2, 4, 128, 64, keep, seed)
+        x = torch.randn(k, 19200, device="cuda").bfloat16()
+        refs.append(L.spmm(x))
+        assert L.last_launch()["path"] == 2
+        ys = [torch.zeros_like(refs[-1]), torch.zeros_like(refs[-1])]
+        turn = [0]
+
+        def job(L=L, x=x, ys=ys, turn=turn):
+            turn[0] ^= 1
+            L.spmm(x, y=ys[turn[0]])
+        jobs.append(job)
+        outs.append(ys)
+        layers.append(L)
+    torch.cuda.synchronize()
+    assert run_together(torch, jobs, 500) == []
+    for ys, ref, L in zip(outs, refs, layers):
+        assert L.device_status() == 0
+        assert torch.equal(ys[0], ref) and torch.equal(ys[1], ref)
+        L.close()
+
+
+def test_first_call_of_a_host_thread():
+    """A product, or a convolution, as the first CUDA call of a thread, on buffers the layer has not seen: its tensor maps need
+    a context that nothing has made current in that thread yet."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    L = make_layer(B, torch, 128, 64 * 9, 2, 4, 64, 64, 0.5, 5)
+    x = torch.randn(64 * 9, 1024, device="cuda").bfloat16()
+    act = torch.randn(2, 16, 16, 64, device="cuda").bfloat16()
+    stream = torch.cuda.current_stream().cuda_stream
+    want = [L.spmm(x), L.spmm_conv(act, 3, 3, 1)]
+    got = [torch.zeros_like(w) for w in want]
+    torch.cuda.synchronize()
+    for call in (lambda: L.spmm(x, y=got[0], stream=stream), lambda: L.spmm_conv(act, 3, 3, 1, y=got[1], stream=stream)):
+        errors = []
+
+        def work():
+            try:
+                call()
+            except Exception as e:                       # noqa: BLE001 (reported by the test)
+                errors.append(e)
+        t = threading.Thread(target=work)
+        t.start()
+        t.join()
+        torch.cuda.synchronize()
+        assert errors == []
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    L.close()
