@@ -606,32 +606,66 @@ class PruningNetwork:
         self.min_keep = min_keep
         self.layers = [HybridLayer(r, k, n, m, block_rows, block_k, 1.0, device=device) for (r, k) in shapes]
         self.sal = [torch.empty((r, k), dtype=torch.float32, device=self.device) for (r, k) in shapes]
+        self._acc = None
         self.rank_arr = make_rank_layers([L.rank_layer(min_keep) for L in self.layers])
         self.rank_ws = torch.empty(crisp_global_rank_sizes(self.rank_arr), dtype=torch.uint8, device=self.device)
         self.d_kkeep = torch.zeros(len(shapes), dtype=torch.int32, device=self.device)
 
+    @property
+    def acc(self):
+        """The running gradient sums of layers whose gradients come in turn (allocated when first used)."""
+        if self._acc is None:
+            self._acc = [self.torch.empty_like(s) for s in self.sal]
+        return self._acc
+
+    def _score_in_turn(self, weights, grads, stream):
+        """crisp_prune_score in the calls it replaces, one gradient tensor at a time; the number of layers."""
+        count = 0
+        for L, w, gs, acc, s in zip(self.layers, weights, grads, self.acc, self.sal):
+            rows, k = L.desc.rows, L.desc.k
+            for i, g in enumerate(gs):
+                crisp_saliency_accumulate(g, 0 if g.dtype == self.torch.bfloat16 else 1, g.stride(0), rows, k, acc, k, i == 0,
+                                          stream)
+            crisp_saliency_finish_max(acc, k, w, w.stride(0), rows, k, len(gs), s, k, L.workspace, stream)
+            L.desc.keep_ratio = 1.0
+            L.nblk, L.kkeep = crisp_keep_count(L.desc)
+            L.build_mask_max_known(s, stream)
+            count += 1
+        return count
+
     def step(self, weights, grads, kappa, stream=None):
         """weights[l]: bf16 CUDA tensor [rows, k]; grads[l]: list of H gradient tensors (bf16 or fp32) of that shape;
         kappa: overall sparsity target of this iteration.  Returns the kept-block count of every layer; the layers'
-        masks and handles (self.layers[l]) hold the result."""
+        masks and handles (self.layers[l]) hold the result.
+
+        Lists and tuples (or stacked tensors) of gradients are taken for all layers at once.  Anything else that can be iterated over (a generator
+        that makes one layer's gradients after the other, say) is read layer by layer and gradient by gradient, and each
+        gradient's kernel is on the stream before the next one is asked for."""
         torch = self.torch
-        bf16 = torch.bfloat16
-        count = min(len(self.layers), len(weights), len(grads))
-        weights, grads = weights[:count], grads[:count]
+        weights = list(weights)
+        held = (list, tuple, torch.Tensor)                   # every gradient exists, and none is changed by asking for the next
+        at_once = isinstance(grads, held) and all(isinstance(gs, held) for gs in grads)
+        count = min(len(self.layers), len(weights), len(grads) if at_once else len(weights))
+        weights = weights[:count]
         assert all(w.is_cuda and w.element_size() == 2 and w.stride(1) == 1 for w in weights)
+        if not at_once:
+            count = self._score_in_turn(weights, grads, stream)
         arr = (PruneLayer * count)()
-        flat = [g for gs in grads for g in gs]               # one host array each for the whole network
-        ptrs = (C.c_void_p * len(flat))(*[g.data_ptr() for g in flat])
-        lds = (C.c_int64 * len(flat))(*[g.stride(0) for g in flat])
-        dts = (C.c_int32 * len(flat))(*[0 if g.dtype is bf16 else 1 for g in flat])
-        p0, l0, d0, at = C.addressof(ptrs), C.addressof(lds), C.addressof(dts), 0
-        for P, L, w, gs, s in zip(arr, self.layers, weights, grads, self.sal):
+        for P, L, w, s in zip(arr, self.layers, weights, self.sal):
             P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride(0)
-            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, len(gs)
             P.d_saliency, P.ld_s = s.data_ptr(), s.stride(0)
             P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
-            at += len(gs)
-        crisp_prune_score(arr, stream)
+        if at_once:
+            bf16 = torch.bfloat16
+            flat = [g for gs in grads[:count] for g in gs]   # one host array each for the whole network
+            ptrs = (C.c_void_p * len(flat))(*[g.data_ptr() for g in flat])
+            lds = (C.c_int64 * len(flat))(*[g.stride(0) for g in flat])
+            dts = (C.c_int32 * len(flat))(*[0 if g.dtype is bf16 else 1 for g in flat])
+            p0, l0, d0, at = C.addressof(ptrs), C.addressof(lds), C.addressof(dts), 0
+            for P, gs in zip(arr, grads):
+                P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, len(gs)
+                at += len(gs)
+            crisp_prune_score(arr, stream)
         crisp_global_rank(self.rank_arr, crisp_prune_fraction(kappa, self.n, self.m), self.rank_ws, self.d_kkeep, stream)
         if stream is None:
             kk = self.d_kkeep.cpu().tolist()

@@ -123,3 +123,50 @@ def test_finish_max_feeds_the_mask_without_a_second_pass():
     mk = oracle.build_mask(s.cpu().numpy(), 2, 4, 32, 64, 0.5)
     assert np.array_equal(got[0], mk.blk_col) and np.array_equal(got[1], mk.nm_bits)
     L.close()
+
+
+@pytest.mark.parametrize("form", ["tuples", "stacked", "dict_values", "generator", "one_buffer"])
+def test_gradients_in_other_forms_than_lists(form):
+    """What step() does with weights and gradients does not depend on what holds them; a generator may make every gradient
+    in the same buffer, since it is asked for the next one when the last one's kernel is on the stream."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    shapes, samples = [(96, 256), (64, 130), (160, 512)], 3
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    weights = [torch.randn(sh, generator=gen, device="cuda").bfloat16() for sh in shapes]
+    grads = [torch.randn((samples,) + sh, generator=gen, device="cuda") for sh in shapes]
+
+    def results(ws, gs):
+        net = B.PruningNetwork(shapes, 2, 4, 32, 32)
+        kk = net.step(ws, gs, 0.7)
+        out = [kk] + [a for L in net.layers for a in L.export_mask() + L.export()]
+        net.close()
+        return out
+
+    class InOneBuffer:
+        """The samples of a layer, each copied to the same place when it is asked for."""
+        place = torch.empty(max(r * k for r, k in shapes), device="cuda")
+
+        def __init__(self, g):
+            self.g = g
+
+        def __len__(self):
+            return len(self.g)
+
+        def __iter__(self):
+            for one in self.g:
+                yield self.place[:one.numel()].view(one.shape).copy_(one)
+
+    lists = [list(g) for g in grads]
+    want = results(weights, lists)
+    assert sum(want[0]) > 0
+    ws, gs = {
+        "tuples": lambda: (tuple(weights), tuple(tuple(g) for g in lists)),
+        "stacked": lambda: (weights, grads),
+        "dict_values": lambda: (dict(enumerate(weights)).values(), dict(enumerate(lists)).values()),
+        "generator": lambda: (weights, (list(g) for g in grads)),
+        "one_buffer": lambda: ((w for w in weights), (InOneBuffer(g) for g in grads)),
+    }[form]()
+    for a, b in zip(want, results(ws, gs)):
+        assert np.array_equal(a, b)
