@@ -426,6 +426,10 @@ CRISP_API crisp_status_t crisp_set_path(crisp_handle_t h, int32_t path);
 /* Kernel family and tile configuration of the last product launched through this handle. */
 CRISP_API crisp_status_t crisp_last_launch(crisp_handle_t h, crisp_launch_info_t *out);
 
+/* Bytes of weight tiles that every CTA of the handle's last launch kept in shared memory for all of its tiles (0: a
+ * pipeline stage carries them anew).  The paper has no counterpart.  Error: INVALID_ARG. */
+CRISP_API crisp_status_t crisp_last_resident_bytes(crisp_handle_t h, int64_t *bytes);
+
 /* Tuning and failure-detection controls of the tensor-core kernels of this handle (all optional).
  *   tile_boxes        64-column boxes per CTA tile, 1..4; 0 = chosen by the library
  *   wait_limit_cycles every wait inside the kernel (on a pipeline stage, on an accumulator) gives

@@ -107,6 +107,7 @@ def load(path: Optional[str] = None):
         "crisp_set_epilogue": [vp, vp, i32],
         "crisp_device_status": [vp, vp, P(i32)],
         "crisp_last_launch": [vp, P(LaunchInfo)],
+        "crisp_last_resident_bytes": [vp, P(i64)],
         "crisp_set_tuning": [vp, i32, C.c_uint64, i32],
         "crisp_set_stage_blocks": [vp, i32],
         "crisp_reset_status": [vp, vp],
@@ -378,6 +379,13 @@ def crisp_last_launch(handle: int) -> dict:
     return info.as_dict()
 
 
+def crisp_last_resident_bytes(handle: int) -> int:
+    """Bytes of weight tiles that the last product's CTAs kept in shared memory for all of their tiles."""
+    out = C.c_int64()
+    _check(load().crisp_last_resident_bytes(handle, C.byref(out)), "crisp_last_resident_bytes")
+    return out.value
+
+
 def crisp_set_tuning(handle: int, tile_boxes: int = 0, wait_limit_cycles: int = 0, skip_fill: int = -1):
     _check(load().crisp_set_tuning(handle, tile_boxes, wait_limit_cycles, skip_fill), "crisp_set_tuning")
 
@@ -559,6 +567,9 @@ class HybridLayer:
 
     def last_launch(self) -> dict:
         return crisp_last_launch(self.handle)
+
+    def last_resident_bytes(self) -> int:
+        return crisp_last_resident_bytes(self.handle)
 
     def set_tuning(self, tile_boxes=0, wait_limit_cycles=0, skip_fill=-1):
         crisp_set_tuning(self.handle, tile_boxes, wait_limit_cycles, skip_fill)

@@ -99,6 +99,7 @@ crisp_handle_s *new_handle(const uint16_t *d_w_bf16, int64_t ld_w, const crisp_m
     h->debug_skip_stage = -1;
     h->plan = nullptr;
     h->last = crisp_launch_info_t{-1, 0, 0, 1, 0, 0, 0, 0, 1};
+    h->last_resident = 0;
     *L = crisp::EncodeLayer{};
     L->g = g;
     L->w = d_w_bf16; L->ld = ld_w;
@@ -424,7 +425,7 @@ crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ld
     if (path == CRISP_PATH_DIRECT) {
         e = crisp::launch_spmm_direct(h->g, h->d_blk_col, h->d_vals, h->d_idx, d_x_bf16, ldx, ncols,
                                       d_y, ldy, y_dtype, h->epilogue, (cudaStream_t)stream);
-        if (e == cudaSuccess) h->last = crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0};
+        if (e == cudaSuccess) { h->last = crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0}; h->last_resident = 0; }
     } else {
         e = crisp::launch_spmm_tc(h, path, d_x_bf16, ldx, ncols, d_y, ldy, y_dtype, nullptr,
                                   (cudaStream_t)stream);
@@ -463,6 +464,12 @@ crisp_status_t crisp_spmm_conv(crisp_handle_t h, const uint16_t *d_act_nhwc, con
 crisp_status_t crisp_last_launch(crisp_handle_t h, crisp_launch_info_t *out) {
     if (!h || !out) return CRISP_INVALID_ARG;
     *out = h->last;
+    return CRISP_OK;
+}
+
+crisp_status_t crisp_last_resident_bytes(crisp_handle_t h, int64_t *bytes) {
+    if (!h || !bytes) return CRISP_INVALID_ARG;
+    *bytes = h->last_resident;
     return CRISP_OK;
 }
 

@@ -124,6 +124,7 @@ struct crisp_handle_s {
     int debug_skip_stage;   // test hook: the producer leaves out the loads of this pipeline fill (-1 = none)
     crisp::TcPlan *plan;    // cached launch plan of the last tensor-core product (or nullptr)
     crisp_launch_info_t last;               // what the last product on this handle launched
+    int64_t last_resident;                  // and the bytes of weight tiles it kept in shared memory
 };
 
 namespace crisp {

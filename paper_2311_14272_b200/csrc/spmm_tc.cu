@@ -1304,7 +1304,7 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
     }
     e = launch_chained(plan->variant.kern, (unsigned)plan->grid, (unsigned)plan->variant.threads, plan->smem, st, plan->mx, plan->my,
                        plan->ma, plan->p);
-    if (e == cudaSuccess) h->last = plan->info;
+    if (e == cudaSuccess) { h->last = plan->info; h->last_resident = plan->p.resident_bytes; }
     return e;
 }
 

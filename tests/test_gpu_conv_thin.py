@@ -38,6 +38,49 @@ def test_thin_convolution(s_out, ks, pad, c, b, h, w, n, m, bm, keep, nhwc, y_dt
     torch.cuda.synchronize()
     assert L.device_status() == 0
     assert L.last_launch()["tile_cols"] == 256 and L.last_launch()["epilogue_warps"] == 16     # the short-walk form
+    assert L.last_resident_bytes() > 0                                                          # with its weight tiles kept
     got = y_to_f64(y, torch)
     check_tolerance(got.reshape(-1, s_out).T if nhwc else got, ref)
+    L.close()
+
+
+@pytest.mark.parametrize("s_out,ks,c,b,h,w,n,m,bm,keep,why", [
+    (64, 1, 64, 8, 84, 84, 2, 4, 64, 1.0, "a walk of one block"),
+    (64, 3, 64, 8, 84, 84, 2, 4, 64, 1.0, "a walk of nine blocks"),
+    (160, 3, 64, 8, 84, 84, 2, 4, 64, 0.3, "two CTA tiles of rows"),
+    (64, 3, 64, 1, 16, 16, 2, 4, 64, 0.4, "128-pixel tiles"),
+])
+def test_other_convolutions_load_their_weights_with_every_tile(s_out, ks, c, b, h, w, n, m, bm, keep, why):
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    wt, sal, act = conv_inputs(s_out, ks, ks, c, b, h, w, seed=s_out + h)
+    L = gpu_layer(B, torch, wt, sal, n, m, bm, 64, keep)
+    L.spmm_conv(bf16_dev(act, torch), ks, ks, ks // 2)
+    torch.cuda.synchronize()
+    assert L.device_status() == 0 and L.last_resident_bytes() == 0
+    L.close()
+
+
+def test_bounded_wait_with_resident_weights():
+    """The loads of every CTA's second fill are left out under a wait limit of about a millisecond: the kernel returns, the
+    status says why, and the next product is right."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    s_out, ks, c, b, h, w, n, m, bm, keep = 64, 3, 64, 11, 83, 84, 2, 4, 64, 0.4
+    wt, sal, act = conv_inputs(s_out, ks, ks, c, b, h, w, seed=3)
+    _, _, _, wd, _ = oracle_layer(wt, sal, n, m, bm, 64, keep)
+    L = gpu_layer(B, torch, wt, sal, n, m, bm, 64, keep)
+    d_act = bf16_dev(act, torch)
+    L.set_tuning(wait_limit_cycles=2_000_000, skip_fill=1)
+    L.spmm_conv(d_act, ks, ks, 1)
+    torch.cuda.synchronize()
+    assert L.last_resident_bytes() > 0 and L.device_status() == B.TIMEOUT
+    L.set_tuning()
+    L.reset_status()
+    y = L.spmm_conv(d_act, ks, ks, 1)
+    torch.cuda.synchronize()
+    assert L.last_resident_bytes() > 0 and L.device_status() == 0
+    check_tolerance(y_to_f64(y, torch), oracle.conv_fp64(wd, ks, ks, act, 1))
     L.close()
