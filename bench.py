@@ -9,7 +9,8 @@ speedup over a dense bf16 cuBLAS GEMM of the same shape are reported beside it.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints exactly one JSON line on rank 0.
+Prints exactly one JSON line on rank 0: the result, the headline kernel and what else explains it.  Everything measured
+(the cells, the convolutions, the pruning iterations, ...) goes to the file --details names.
 """
 from __future__ import annotations
 
@@ -974,9 +975,52 @@ def run_ours(args, layer, rank, world):
                                "sample": f"mask+encode+decode of the full layer, fp64 product on the first {cols} "
                                          f"of {layer.ncols} columns"}
     if rank == 0:
-        print(json.dumps(out))
+        stored = store_details(out, args.details)
+        print(json.dumps(contract_line(out, stored)))
     if world > 1:
         dist.destroy_process_group()
+
+
+# What the printed line carries of the measured sections; all of it is in the file of store_details().
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+             "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "phases", "device_status", "cpu_baseline")
+LINE_ROOFLINE = ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_kind", "kernel", "t_tensor_us", "t_hbm_us",
+                 "t_kernel_us", "t_kernel_back_to_back_us", "dense_cublas_us", "speedup_vs_dense_cublas")
+LINE_PHASES = ("mask_us", "encode_us", "spmm_us")
+LINE_BYTES = 2500       # readers keep the last few thousand characters of the output
+
+
+def _short(x):
+    """Floats with six significant digits, in nested values too."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_short(v) for v in x]
+    return x
+
+
+def contract_line(out, details=None):
+    """The one line that a run prints: the result and what explains it, short enough to be read from the end of a log.  The
+    cells and the other sections, tens of kilobytes, are in the file `details`."""
+    line = {k: out[k] if k in ("value", "ms_per_step") else _short(out[k]) for k in LINE_KEYS if k in out}
+    line["roofline"] = {k: v for k, v in line["roofline"].items() if k in LINE_ROOFLINE}
+    line["phases"] = {k: v for k, v in line["phases"].items() if k in LINE_PHASES}
+    if details:
+        line["details"] = details
+    return line
+
+
+def store_details(out, path):
+    """Everything measured, as one JSON line in `path` (what --render takes); the path, or None where it cannot be written."""
+    try:
+        with open(path, "w") as f:
+            f.write(json.dumps(out) + "\n")
+    except OSError as e:
+        print(f"details not stored: {e}", file=sys.stderr)
+        return None
+    return path
 
 
 def render_markdown(d):
@@ -1063,7 +1107,9 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-cells", action="store_true", help="skip the per-layer / per-cell SpMM timings")
     ap.add_argument("--cell-iters", type=int, default=50, help="timed launches per cell and protocol")
-    ap.add_argument("--render", metavar="JSON_FILE", help="print the markdown tables of a stored JSON line and exit")
+    ap.add_argument("--details", metavar="JSON_FILE", default=os.path.join(ROOT, "bench_details.json"),
+                    help="where everything measured is stored (the printed line carries the result and the headline kernel)")
+    ap.add_argument("--render", metavar="JSON_FILE", help="print the markdown tables of a stored details file and exit")
     args = ap.parse_args()
     if args.render:
         print(render_markdown(json.loads([l for l in open(args.render) if l.startswith("{")][-1])))
