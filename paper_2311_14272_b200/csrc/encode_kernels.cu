@@ -17,8 +17,8 @@ namespace {
 // values to the front, offset fields, the slot pair of the 2:4 image and its metadata nibble.  Values go straight to
 // global memory (consecutive lanes write consecutive bytes), the tile and the offset fields through shared memory;
 // every metadata byte belongs to one thread, so there are no atomics on it.  What bounds the kernel is the chain of
-// dependent round trips of a CTA (block list, weights, stores), hidden by the five CTAs an SM holds (48 registers; 40 spill
-// and take 20 us where this takes 14).  A thread keeps its chunk column and goes down the rows: with the row and column of
+// dependent round trips of a CTA (block list, weights, stores), hidden by the five CTAs an SM holds (48 registers, for which
+// most forms spill 8 to 48 bytes a thread; with 40 registers they spill more and take 20 us where this takes 14).  A thread keeps its chunk column and goes down the rows: with the row and column of
 // every chunk computed anew, and the image chosen at run time, the same work took 22 us.
 // Measured: 4096 x 4096, 2:4, keep 0.5, 128 x 64 blocks 14.0 us (36 MB moved); the 13 layers of VGG-16 with 64 x 64 blocks in
 // one launch 15.9 us, where a canonical pass and an image pass over it per layer took 62 + 165 us.

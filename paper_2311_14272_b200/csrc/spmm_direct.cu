@@ -15,7 +15,7 @@
 // depend on the tile chosen.
 // Measured (the kernel before staged scalar 2-byte loads and decoded an offset at every use): 256 x 2304 x 6076, 1:4,
 // keep 0.25: 508 -> 51 us (38 M warp instructions, 76 % of the issue slots of busy SMs); 160 x 960 x 49, 2:8, keep 0.5:
-// 147 -> 14.7 us, a chain of four stages on 20 CTAs.  One warp per row that gathers its activations from L2 without
+// 147 -> 16.4 us, a chain of four stages on 20 CTAs.  One warp per row that gathers its activations from L2 without
 // staging took 13-22 us on the second and 65 us on the first; staging through registers with two buffers 70 us.
 #include <cuda_bf16.h>
 

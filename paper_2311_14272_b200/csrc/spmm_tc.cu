@@ -445,8 +445,8 @@ __device__ __forceinline__ void mma_role(const TcParams &p, const MmaRoleArgs &a
 // between 8-row K groups and box_bytes between 64-column groups.
 //
 // kResident: with one CTA tile of rows all tiles multiply the same weight tiles; short walks then load them once and keep
-// them, and a stage holds X only.  What bounds a short walk is the number of bytes in flight: a stage's cycle (MMA, release,
-// issue of the copy, L2, arrival) takes 1.4 to 1.6 us whatever it carries.
+// them, and a stage holds X only.  What bounds a short walk is the rate at which an SM gets X from L2 (four stages of 32 KB and
+// six of 24 KB bring the same bytes per cycle), so the weight tiles' bytes are worth leaving out.
 template <int NT, bool kSparse, int kAccStages, typename OutT, int kEpi, bool kConv, bool kResident>
 __global__ void __launch_bounds__(96 + 32 * kEpi, 1)
 spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
@@ -478,9 +478,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     // walk would otherwise spend two dependent global loads per tile in the producer's serial loop.
     int32_t *s_walk = reinterpret_cast<int32_t *>(ctrl_gen + 256);
 
-    // Set-up, ordered so that its round trips run side by side: warp 1 asks for tensor memory at once, every
-    // thread asks for its first word of the walk lists before thread 0 builds the barriers, and the words are
-    // stored to shared memory afterwards.
+    // Set-up of what is this CTA's own: warp 1 asks for tensor memory while thread 0 builds the barriers.
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 1) {
         tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_base_slot)), kTmemCols);
