@@ -654,28 +654,29 @@ class PruningNetwork:
         gradient's kernel is on the stream before the next one is asked for."""
         torch = self.torch
         weights = list(weights)
-        held = (list, tuple, torch.Tensor)                   # every gradient exists, and none is changed by asking for the next
-        at_once = isinstance(grads, held) and all(isinstance(gs, held) for gs in grads)
+        # every gradient exists, and none is changed by asking for the next
+        held = (list, tuple, torch.Tensor)
+        at_once = isinstance(grads, held) and (set(map(type, grads)) <= {list, tuple} or all(isinstance(gs, held) for gs in grads))
         count = min(len(self.layers), len(weights), len(grads) if at_once else len(weights))
         weights = weights[:count]
         assert all(w.is_cuda and w.element_size() == 2 and w.stride(1) == 1 for w in weights)
         if not at_once:
             count = self._score_in_turn(weights, grads, stream)
+        grads = grads[:count] if at_once else [()] * count
+        bf16 = torch.bfloat16
         arr = (PruneLayer * count)()
-        for P, L, w, s in zip(arr, self.layers, weights, self.sal):
+        flat = [g for gs in grads for g in gs]               # one host array each for the whole network
+        ptrs = (C.c_void_p * len(flat))(*[g.data_ptr() for g in flat])
+        lds = (C.c_int64 * len(flat))(*[g.stride(0) for g in flat])
+        dts = (C.c_int32 * len(flat))(*[0 if g.dtype is bf16 else 1 for g in flat])
+        p0, l0, d0, at = C.addressof(ptrs), C.addressof(lds), C.addressof(dts), 0
+        for P, L, w, gs, s in zip(arr, self.layers, weights, grads, self.sal):
             P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride(0)
+            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, len(gs)
             P.d_saliency, P.ld_s = s.data_ptr(), s.stride(0)
             P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
+            at += len(gs)
         if at_once:
-            bf16 = torch.bfloat16
-            flat = [g for gs in grads[:count] for g in gs]   # one host array each for the whole network
-            ptrs = (C.c_void_p * len(flat))(*[g.data_ptr() for g in flat])
-            lds = (C.c_int64 * len(flat))(*[g.stride(0) for g in flat])
-            dts = (C.c_int32 * len(flat))(*[0 if g.dtype is bf16 else 1 for g in flat])
-            p0, l0, d0, at = C.addressof(ptrs), C.addressof(lds), C.addressof(dts), 0
-            for P, gs in zip(arr, grads):
-                P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, len(gs)
-                at += len(gs)
             crisp_prune_score(arr, stream)
         crisp_global_rank(self.rank_arr, crisp_prune_fraction(kappa, self.n, self.m), self.rank_ws, self.d_kkeep, stream)
         if stream is None:
