@@ -56,3 +56,30 @@ def test_unaligned_product(rows, k, ncols, n, m, bm, bk, keep, off, y_dtype):
     assert np.all(np.abs(y_to_f64(y, torch) - ref) <= bound + 1e-30)
     assert torch.all(ybuf[:off] == 5.0) and torch.all(ybuf[off + rows * ncols:] == 5.0)
     L.close()
+
+
+def test_products_of_falling_size_in_one_graph():
+    """Two layers of one tile form, the one with more shared memory first, captured in one graph and replayed on new data."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    rng = np.random.default_rng(12)
+    layers, xs, ys, refs = [], [], [], []
+    for rows, k, n, m, bk, keep in ((128, 1024, 8, 8, 64, 1.0), (128, 512, 1, 8, 32, 0.25)):
+        w = wl.f32_to_bf16_bits((rng.standard_normal((rows, k)) / 32).astype(np.float32))
+        layers.append(gpu_layer(B, torch, w, np.abs(wl.bf16_bits_to_f32(w)) + 1e-3, n, m, 64, bk, keep))
+        xs.append(torch.zeros(k, 49, dtype=torch.bfloat16, device="cuda"))
+        ys.append(layers[-1].spmm(xs[-1]))
+        assert layers[-1].last_launch()["path"] == 0
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for L, x, y in zip(layers, xs, ys):
+            L.spmm(x, y=y)
+    for L, x in zip(layers, xs):
+        x.copy_(torch.randn(x.shape, device="cuda"))
+        refs.append(L.spmm(x))
+    graph.replay()
+    torch.cuda.synchronize()
+    for L, y, ref in zip(layers, ys, refs):
+        assert int((ref != 0).sum()) > 0 and torch.equal(y, ref)
+        L.close()
