@@ -21,7 +21,7 @@ namespace {
 // most forms spill 8 to 48 bytes a thread; with 40 registers they spill more and take 20 us where this takes 14).  A thread keeps its chunk column and goes down the rows: with the row and column of
 // every chunk computed anew, and the image chosen at run time, the same work took 22 us.
 // Measured: 4096 x 4096, 2:4, keep 0.5, 128 x 64 blocks 14.0 us (36 MB moved); the 13 layers of VGG-16 with 64 x 64 blocks in
-// one launch 15.9 us, where a canonical pass and an image pass over it per layer took 62 + 165 us.
+// one launch 15.9 us (18 under ncu with a cold L2), where a canonical pass and an image pass over it per layer took 62 + 165 us.
 // Shared-memory planes of the tile are padded (2064 or 2080 instead of 2048 bytes), which spreads the eight lanes of a row
 // over the banks.
 // Image layouts: see the tensor-core SpMM.  Stacked thin layers: copy q of the image holds the rows shifted by
