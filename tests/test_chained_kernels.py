@@ -98,3 +98,52 @@ def test_chain_of_encode_and_decode_hands_over_the_newest_data(n, m, bm, bk):
         assert torch.equal(ref.view(torch.int16), out.view(torch.int16))
         assert torch.equal(ref.view(torch.int16), out2.view(torch.int16))
     L.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("rows,k,n,m,bm,bk", [(64, 256, 2, 4, 32, 32), (512, 1024, 3, 8, 64, 64), (2048, 2048, 2, 4, 128, 64)])
+def test_encode_and_decode_of_one_mask_with_new_weights_each_time(rows, k, n, m, bm, bk, graph):
+    """One buffer is written by every encode and read by the decode behind it, which is still there when the next encode's
+    launch begins: queued behind other work, or captured in one graph, every decode gives its own encode's weights."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    g = torch.Generator(device="cuda").manual_seed(rows + n)
+    ws = [torch.randn(rows, k, generator=g, device="cuda").bfloat16() for _ in range(16)]
+    L = B.HybridLayer(rows, k, n, m, bm, bk, 0.5)
+    L.build_mask(torch.rand(rows, k, generator=g, device="cuda") + 0.1)
+    refs = []
+    for w in ws:
+        L.encode(w)
+        torch.cuda.synchronize()
+        refs.append(L.decode())
+        torch.cuda.synchronize()
+    kept = refs[0] != 0
+    assert 0 < int(kept.sum()) < kept.numel()
+    for w, ref in zip(ws, refs):
+        assert torch.equal(ref, torch.where(kept, w, torch.zeros_like(w)))
+    outs = []
+
+    def chain():
+        for w in ws:
+            L.encode(w)
+            outs.append(L.decode())
+
+    if graph:
+        captured = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(captured):
+            chain()
+        for _ in range(3):
+            captured.replay()
+    else:
+        busy = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+        for _ in range(3):
+            outs.clear()
+            for _ in range(20):                       # the chain is queued before the first of it runs
+                busy.zero_()
+            chain()
+    torch.cuda.synchronize()
+    for out, ref in zip(outs, refs):
+        assert torch.equal(out, ref)
+    L.close()
