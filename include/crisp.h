@@ -92,7 +92,9 @@ typedef struct {
     int32_t path;             /* which SpMM kernel the handle runs, see CRISP_PATH_*         */
 } crisp_bytes_t;
 
-#define CRISP_PATH_DIRECT 0   /* CUDA-core kernel on the canonical format (any shape)        */
+#define CRISP_PATH_DIRECT 0   /* any layout: X and Y at any even address and pitch.  CUDA cores on the
+                                 canonical format, or, unless this path was set by crisp_set_path,
+                                 the tensor cores on the handle's image for larger bf16 products */
 #define CRISP_PATH_DENSE  1   /* tcgen05 dense MMA over zero-expanded kept blocks            */
 #define CRISP_PATH_SPARSE 2   /* tcgen05 sparse (2:4) MMA over compressed kept blocks        */
 #define CRISP_PATH_SPARSE2 3  /* the same for patterns with up to four values per aligned 4-group
@@ -106,7 +108,7 @@ typedef struct {
  * steps on every path). */
 typedef struct {
     int32_t path;             /* CRISP_PATH_* of the kernel that was launched, -1 before any    */
-    int32_t tile_cols;        /* columns of X / Y per CTA tile (0 on the direct path)           */
+    int32_t tile_cols;        /* columns of X / Y per CTA tile (0: CUDA cores)                  */
     int32_t accumulators;     /* tensor-memory accumulators per CTA                              */
     int32_t stack;            /* column tiles stacked in one accumulator (thin layers), else 1   */
     int32_t epilogue_warps;
@@ -366,7 +368,7 @@ CRISP_API crisp_status_t crisp_decode(crisp_handle_t h, uint16_t *d_w_dense_bf16
  *            nearest even from the fp32 accumulator) or fp32 (y_dtype 1)
  * Rows of X under blocks that no row tile kept are never read.  A layer with kkeep = 0
  * yields Y = 0.  The tensor-core kernels need X and Y 16-byte aligned with ldx*2 and
- * ldy*sizeof(element) multiples of 16; other layouts run on the direct kernel.
+ * ldy*sizeof(element) multiples of 16; other layouts run on CRISP_PATH_DIRECT.
  */
 CRISP_API crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ldx,
                                     int64_t ncols, void *d_y, int64_t ldy, int32_t y_dtype, void *stream);

@@ -98,6 +98,7 @@ crisp_handle_s *new_handle(const uint16_t *d_w_bf16, int64_t ld_w, const crisp_m
     h->wait_limit_cycles = 0;
     h->debug_skip_stage = -1;
     h->plan = nullptr;
+    h->gather = nullptr;
     h->last = crisp_launch_info_t{-1, 0, 0, 1, 0, 0, 0, 0, 1};
     h->last_resident = 0;
     *L = crisp::EncodeLayer{};
@@ -421,8 +422,12 @@ crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ld
     if ((ncols + 63) / 64 > 0x7FFFFFFFll) return CRISP_UNSUPPORTED;
     int path = h->forced_path >= 0 ? h->forced_path : h->exec_kind;
     if (h->g.kkeep == 0 || !crisp::tc_operands_ok(d_x_bf16, ldx, d_y, ldy, y_dtype, ncols)) path = CRISP_PATH_DIRECT;
-    cudaError_t e;
-    if (path == CRISP_PATH_DIRECT) {
+    cudaError_t e = cudaErrorNotSupported;
+    if (path == CRISP_PATH_DIRECT && h->forced_path != CRISP_PATH_DIRECT && crisp::gather_supported(h, ncols, y_dtype))
+        e = crisp::launch_spmm_gather(h, d_x_bf16, ldx, ncols, d_y, ldy, (cudaStream_t)stream);
+    if (e != cudaErrorNotSupported) {
+        // (done, or failed for another reason than its layout)
+    } else if (path == CRISP_PATH_DIRECT) {
         e = crisp::launch_spmm_direct(h->g, h->d_blk_col, h->d_vals, h->d_idx, d_x_bf16, ldx, ncols,
                                       d_y, ldy, y_dtype, h->epilogue, (cudaStream_t)stream);
         if (e == cudaSuccess) { h->last = crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0}; h->last_resident = 0; }
@@ -534,7 +539,7 @@ crisp_status_t crisp_bytes_model(crisp_handle_t h, int64_t ncols, int32_t y_dtyp
 
 void crisp_mask_destroy(crisp_mask_t mask) { delete mask; }
 void crisp_destroy(crisp_handle_t h) {
-    if (h) crisp::tc_plan_destroy(h->plan);
+    if (h) { crisp::tc_plan_destroy(h->plan); crisp::gather_plan_destroy(h->gather); }
     delete h;
 }
 

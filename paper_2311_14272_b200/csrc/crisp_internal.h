@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "crisp.h"
 
 namespace crisp {
@@ -66,21 +68,29 @@ __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontr
 // The kernels of the mask / encode / decode chain begin with this: the next kernel's launch overlaps this one.
 __device__ __forceinline__ void chain_kernels() { launch_dependents(); wait_for_prerequisites(); }
 
+// (`cluster` CTAs form a thread-block cluster; 1: none)
 template <typename... Params, typename... Args>
-cudaError_t launch_chained(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, const Args &...args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_clusters(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, unsigned cluster,
+                            const Args &...args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
     if (e != cudaSuccess) (void)cudaGetLastError();          // reported here, not to the caller's next check
     return e;
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, const Args &...args) {
+    return launch_clusters(kern, grid, threads, smem, st, 1u, args...);
 }
 #endif
 
@@ -103,6 +113,8 @@ namespace crisp {
 // repeated products on the same buffers skip the tensor-map encoding.
 struct TcPlan;
 void tc_plan_destroy(TcPlan *plan);
+struct GatherPlan;          // tensor map of the execution image for the products of spmm_gather.cu
+void gather_plan_destroy(GatherPlan *plan);
 }  // namespace crisp
 
 struct crisp_handle_s {
@@ -123,6 +135,8 @@ struct crisp_handle_s {
     unsigned long long wait_limit_cycles;   // bound of every in-kernel wait (0 = default)
     int debug_skip_stage;   // test hook: the producer leaves out the loads of this pipeline fill (-1 = none)
     crisp::TcPlan *plan;    // cached launch plan of the last tensor-core product (or nullptr)
+    crisp::GatherPlan *gather;              // made by the first product on a layout TMA cannot address (or nullptr)
+    std::mutex gather_lock;                 // such products may come from several threads at a time
     crisp_launch_info_t last;               // what the last product on this handle launched
     int64_t last_resident;                  // and the bytes of weight tiles it kept in shared memory
 };
@@ -200,6 +214,10 @@ struct ConvGeom { int batch, height, width, channels, kh, kw, pad, ho, wo, nhwc_
 // `h->plan` is reused when the operands, shape and epilogue are those of the previous call; `h->last` is filled in.
 cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols,
                            void *d_y, int64_t ldy, int y_dtype, const ConvGeom *conv, cudaStream_t st);
+// spmm_gather.cu: bf16 products on layouts TMA cannot address, on the same weight tiles
+bool gather_supported(const crisp_handle_s *h, int64_t ncols, int y_dtype);
+cudaError_t launch_spmm_gather(crisp_handle_s *h, const uint16_t *d_x, int64_t ldx, int64_t ncols, void *d_y, int64_t ldy,
+                               cudaStream_t st);
 // spmm_direct.cu
 cudaError_t launch_spmm_direct(const Geometry &g, const int32_t *d_blk_col, const uint16_t *d_vals,
                                const uint32_t *d_idx, const uint16_t *d_x, int64_t ldx, int64_t ncols,

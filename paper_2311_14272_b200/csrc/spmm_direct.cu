@@ -1,8 +1,8 @@
 // Direct SpMM on the canonical format (CUDA cores).  It follows the three steps of Sec. III-E
 // literally: stage the activation rows of kept blocks (step 1), pick for each stored weight the
 // activation its offset names (step 2), multiply-accumulate in fp32 (step 3).  It accepts every
-// shape and alignment and serves the layouts the tensor-core kernels cannot take (row pitches that are
-// not multiples of 16 bytes).
+// shape and alignment and serves the layouts TMA cannot address (row pitches that are not multiples of 16 bytes) where
+// spmm_gather.cu does not: small products, fp32 results, and calls that ask for this path.
 //
 // Large products are bound by instruction issue: a stored weight costs a warp one look-up of its activation row
 // and the multiply-adds of the columns its lanes own, so everything else is taken out of that loop.  A weight and the

@@ -872,6 +872,8 @@ cudaError_t prepare_variant(const TcVariant &v, int device) {
     return e;
 }
 
+}  // namespace
+
 // Multiprocessor count of a device, looked up once per device.
 int sm_count_of(int device) {
     static std::atomic<int> cache[kMaxDevices];
@@ -882,8 +884,6 @@ int sm_count_of(int device) {
     cache[device].store(n, std::memory_order_relaxed);
     return n;
 }
-
-}  // namespace
 
 // ------------------------------------------------------------------------ tensor maps (host)
 
@@ -932,6 +932,17 @@ bool make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_bytes, const
     return fn(map, dt, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_map_rows(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t pitch_bytes, uint32_t box_cols, uint32_t box_rows) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    cuuint64_t dims[2] = {cols, rows};
+    cuuint64_t strides[1] = {pitch_bytes};
+    cuuint32_t box[2] = {box_cols, box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // X viewed as [ncols/64][k][64] (needs ncols % 64 == 0): box = 64 columns x bk rows x nt column groups,

@@ -156,11 +156,17 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // Tensor-map builders (host; defined in spmm_tc.cu).
 bool make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_bytes, const void *base, uint64_t inner,
                  uint64_t outer, uint64_t ld_elems, uint32_t box_inner, uint32_t box_outer);
+// bf16 rows `pitch_bytes` apart, box of box_cols x box_rows, not swizzled
+bool make_map_rows(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t pitch_bytes, uint32_t box_cols, uint32_t box_rows);
 bool make_map_x3d(CUtensorMap *map, const void *base, uint64_t ncols, uint64_t k, uint64_t ldx, uint32_t bk, uint32_t nt);
 bool make_map_image(CUtensorMap *map, const void *image, uint64_t total_bytes, uint32_t entry_bytes);
 bool make_map_4d(CUtensorMap *map, CUtensorMapDataType dt, int elem_bytes, const void *base, const uint64_t (&dims)[4],
                  const uint64_t (&strides_bytes)[3], const uint32_t (&box)[4], bool swizzle = true);
 bool tensor_maps_available();
+cudaError_t ensure_context(int device);
 
 }  // namespace tc
+
+int sm_count_of(int device);                // multiprocessors of a device (spmm_tc.cu)
+
 }  // namespace crisp

@@ -1,0 +1,130 @@
+"""Products on layouts TMA cannot address, on the tensor cores (spmm_gather.cu): edges of its tiles, parts of 32 and 64 rows,
+every alignment of a row, walks split over 2, 4 and 8 CTAs, several tiles a CTA, against the oracle's product in 64 bits.
+
+Tolerance: an fp32 accumulation of t products with one rounding (or truncation) per step is off by at most t * 2^-23 * sum |w x|;
+the bf16 result (8 significant bits) adds at most 2^-8 of the value."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import bf16_dev, gpu_layer, oracle_layer, to_dev, y_to_f64
+from paper_2311_14272_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # rows, k, ncols, pitch, n, m, bm, bk, keep, offset of X's first element
+    (160, 960, 49, 49, 2, 8, 32, 32, 0.5, 0),         # one column tile, walk split over 8
+    (16, 420, 1, 1, 2, 4, 32, 32, 1.0, 1),            # one column, thirteen blocks and a bit
+    (70, 600, 127, 127, 1, 8, 64, 96, 0.6, 3),        # 96-deep blocks, ragged rows, columns and k
+    (130, 1000, 129, 140, 3, 4, 64, 64, 0.9, 4),      # one column beyond a tile, split; pitch a multiple of 8 bytes
+    (256, 512, 3001, 3001, 1, 4, 64, 64, 0.5, 7),     # split over 2, odd pitch
+    (300, 640, 2570, 2574, 4, 4, 128, 128, 0.4, 2),   # 128-deep blocks, as many weights as there can be
+    (384, 256, 9004, 9004, 3, 8, 128, 32, 0.5, 4),    # more tiles than CTAs, 8-byte rows
+    (64, 256, 20001, 20001, 8, 8, 32, 64, 0.5, 5),    # a thin layer (its image has two copies), odd rows
+    (300, 700, 6076, 6076, 1, 4, 64, 64, 0.3, 0),
+    (96, 160, 4100, 4100, 2, 4, 32, 128, 0.7, 6),
+]
+
+
+def make(rows, k, ncols, pitch, n, m, bm, bk, keep, off):
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    rng = np.random.default_rng(rows + ncols)
+    w = wl.f32_to_bf16_bits(rng.standard_normal((rows, k)).astype(np.float32))
+    s = rng.uniform(0.1, 2.0, (rows, k)).astype(np.float32)
+    x = wl.f32_to_bf16_bits(rng.standard_normal((k, ncols)).astype(np.float32))
+    L = gpu_layer(B, torch, w, s, n, m, bm, bk, keep)
+    # what lies between the rows and around the matrix is not finite: it must not be used
+    xbuf = torch.full((off + k * pitch,), float("nan"), dtype=torch.bfloat16, device="cuda")
+    xv = torch.as_strided(xbuf, (k, ncols), (pitch, 1), off)
+    xv.copy_(bf16_dev(x, torch))
+    return torch, L, rng, w, s, x, xv
+
+
+@pytest.mark.parametrize("rows,k,ncols,pitch,n,m,bm,bk,keep,off", CASES)
+def test_product(rows, k, ncols, pitch, n, m, bm, bk, keep, off):
+    torch, L, rng, w, s, x, xv = make(rows, k, ncols, pitch, n, m, bm, bk, keep, off)
+    mk, vals, idx, wd, wb = oracle_layer(w, s, n, m, bm, bk, keep)
+    bias = rng.standard_normal(rows).astype(np.float32)
+    L.set_epilogue(to_dev(bias, torch), relu=True)
+    ybuf = torch.full((rows * pitch + off + 1,), 5.0, dtype=torch.bfloat16, device="cuda")
+    y = torch.as_strided(ybuf, (rows, ncols), (pitch, 1), off)
+    L.spmm(xv, y=y)
+    torch.cuda.synchronize()
+    info = L.last_launch()
+    assert info["path"] == 0 and info["tile_cols"] == 128 and L.device_status() == 0
+    ref = oracle.bias_relu(oracle.spmm_fp64(wd, x), bias, True)
+    x64 = np.abs(wl.bf16_bits_to_f32(x).astype(np.float64))
+    terms = mk.kkeep * bk * n // m + 1
+    bound = terms * 2.0 ** -23 * (np.abs(wd.astype(np.float64)) @ x64 + np.abs(bias)[:, None])
+    bound = bound * (1 + 2.0 ** -8) + 2.0 ** -8 * np.abs(ref)
+    assert np.all(np.abs(y_to_f64(y, torch) - ref) <= bound + 1e-30)
+    outside = torch.ones_like(ybuf, dtype=torch.bool)
+    torch.as_strided(outside, (rows, ncols), (pitch, 1), off).fill_(False)
+    assert torch.all(ybuf[outside] == 5.0)
+    L.close()
+
+
+@pytest.mark.parametrize("rows,k,ncols,bm,bk", [(160, 960, 49, 32, 32), (256, 512, 9003, 64, 64)])
+def test_values_that_are_not_finite_reach_only_the_rows_that_use_them(rows, k, ncols, bm, bk):
+    """An infinity or a NaN under a pruned weight is not part of the sum, as in the kernel on the CUDA cores."""
+    torch, L, rng, w, s, x, xv = make(rows, k, ncols, ncols, 2, 4, bm, bk, 0.5, 1)
+    xv[3, ncols // 2] = float("inf")
+    xv[k // 2, 0] = float("nan")
+    xv[k - 1, ncols - 1] = -float("inf")
+    y = L.spmm(xv)
+    assert L.last_launch()["tile_cols"] == 128
+    L.set_path(0)
+    ref = L.spmm(xv)
+    torch.cuda.synchronize()
+    assert L.last_launch()["tile_cols"] == 0
+    bad = ~torch.isfinite(ref)
+    assert 0 < int(bad.sum()) < 3 * rows and torch.equal(bad, ~torch.isfinite(y))
+    assert torch.equal(torch.isnan(ref), torch.isnan(y)) and torch.equal(ref[torch.isinf(ref)], y[torch.isinf(ref)])
+    a, b = y[~bad].double(), ref[~bad].double()
+    assert float((a - b).norm()) <= 2.0 ** -8 * float(b.norm())
+    L.close()
+
+
+@pytest.mark.parametrize("ncols", [49, 9003])
+def test_a_wait_that_runs_out_is_reported(ncols):
+    torch, L, rng, w, s, x, xv = make(256, 640, ncols, ncols, 2, 4, 64, 64, 0.5, 0)
+    want = L.spmm(xv)
+    L.set_tuning(0, 2_000_000, 1)                      # the second fill gets no weight tile
+    L.spmm(xv)
+    assert L.device_status() == 6
+    L.reset_status()
+    L.set_tuning()
+    y = L.spmm(xv)
+    assert L.device_status() == 0 and torch.equal(y, want)
+    L.close()
+
+
+def test_products_of_two_threads_on_one_layer():
+    """One layer, two host threads with a stream, an input and a row pitch each."""
+    import threading
+    torch, L, rng, w, s, x, xv = make(256, 640, 2049, 2049, 2, 4, 64, 64, 0.5, 0)
+    xs = [xv, torch.randn(640, 1027, device="cuda").bfloat16()]
+    wants = [L.spmm(v) for v in xs]
+    gots = [torch.zeros_like(v) for v in wants]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(i):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            try:
+                for _ in range(500):
+                    L.spmm(xs[i], y=gots[i])
+            except Exception as e:                       # noqa: BLE001 (reported by the test)
+                errors.append(e)
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert errors == [] and L.device_status() == 0
+    assert torch.equal(gots[0], wants[0]) and torch.equal(gots[1], wants[1])
+    L.close()
