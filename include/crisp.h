@@ -464,6 +464,9 @@ CRISP_API crisp_status_t crisp_bytes_model(crisp_handle_t h, int64_t ncols, int3
 
 CRISP_API void crisp_mask_destroy(crisp_mask_t mask);
 CRISP_API void crisp_destroy(crisp_handle_t h);
+/* The same for the masks and handles of n layers (NULL entries are skipped): one call where a
+ * pruning iteration replaces those of a whole network.  Error: INVALID_ARG. */
+CRISP_API crisp_status_t crisp_destroy_layers(int32_t n, const crisp_mask_t *masks, const crisp_handle_t *handles);
 CRISP_API const char *crisp_status_string(crisp_status_t s);
 
 #ifdef __cplusplus

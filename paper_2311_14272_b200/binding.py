@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 from typing import Optional
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -67,11 +68,12 @@ class CrispError(RuntimeError):
 
 
 _lib = None
+_native = None                                            # the same calls on plain integers (csrc/calls.cpp)
 
 
 def load(path: Optional[str] = None):
     """Load libcrisp.so (built in-tree by ``paper_2311_14272_b200.build``)."""
-    global _lib
+    global _lib, _native
     if _lib is not None and path is None:
         return _lib
     p = path or LIB_PATH
@@ -117,6 +119,7 @@ def load(path: Optional[str] = None):
         "crisp_prune_score": [i32, P(PruneLayer), vp],
         "crisp_prune_encode_sizes": [i32, P(PruneLayer), P(sz), P(sz)],
         "crisp_prune_encode": [i32, P(PruneLayer), vp, P(vp), P(vp)],
+        "crisp_destroy_layers": [i32, P(vp), P(vp)],
         "crisp_global_rank": [i32, P(RankLayer), C.c_double, vp, vp, vp],
     }
     for name, args in sig.items():
@@ -129,7 +132,13 @@ def load(path: Optional[str] = None):
     lib.crisp_destroy.restype = None
     lib.crisp_status_string.argtypes = [C.c_int]
     lib.crisp_status_string.restype = C.c_char_p
-    _lib = lib
+    try:
+        from . import _calls
+    except ImportError as e:
+        raise ImportError(f"{e}: build it with `python -m paper_2311_14272_b200.build`") from e
+    _calls.bind(*[C.cast(getattr(lib, "crisp_" + name), vp).value for name in
+                  ("spmm", "spmm_conv", "decode", "build_mask", "encode_sizes", "encode", "mask_destroy", "destroy")])
+    _lib, _native = lib, _calls
     return lib
 
 
@@ -405,6 +414,11 @@ def crisp_bytes_model(handle: int, ncols: int, y_dtype: int = 0) -> dict:
     return b.as_dict()
 
 
+def crisp_destroy_layers(masks, handles):
+    """masks, handles: ctypes arrays of c_void_p of one length (nulls are skipped)."""
+    _check(load().crisp_destroy_layers(len(masks), masks, handles), "crisp_destroy_layers")
+
+
 def crisp_mask_destroy(mask: int):
     if mask:
         load().crisp_mask_destroy(mask)
@@ -434,16 +448,22 @@ class HybridLayer:
         mask_bytes, ws_bytes = crisp_mask_sizes(self.desc)
         self.mask_buf = torch.empty(mask_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=self.device)
-        self._bf16 = torch.empty(0, dtype=torch.bfloat16, device=self.device)
         self.mask = 0
         self.handle = 0
         self.canonical_buf = None
         self.exec_buf = None
 
+    # build_mask, encode, decode, spmm and spmm_conv are made once per layer and pass; for small layers their host time is the
+    # time of the pass, so they hand plain integers to the library (and ask a tensor for all its strides at once, which is cheaper
+    # than for one).
     def build_mask(self, saliency, stream=None):
-        assert saliency.is_cuda and saliency.dtype == self.torch.float32 and saliency.stride(1) == 1
-        crisp_mask_destroy(self.mask)
-        self.mask = crisp_build_mask(saliency, saliency.stride(0), self.desc, self.mask_buf, self.workspace, stream)
+        strides = saliency.stride()
+        assert saliency.is_cuda and saliency.dtype == self.torch.float32 and strides[1] == 1
+        old, self.mask = self.mask, 0
+        code, self.mask = _native.build_mask(saliency.data_ptr(), strides[0], C.addressof(self.desc), self.mask_buf.data_ptr(),
+                                             self.workspace.data_ptr(), _stream(stream), old)
+        if code:
+            raise CrispError(code, "crisp_build_mask")
         return self
 
     def rank_layer(self, min_keep=0):
@@ -485,10 +505,17 @@ class HybridLayer:
         return blk_col, nm_bits
 
     def encode(self, w, stream=None):
-        assert w.is_cuda and w.element_size() == 2 and w.stride(1) == 1
-        self._reserve(*crisp_encode_sizes(self.mask))
-        crisp_destroy(self.handle)
-        self.handle = crisp_encode(w, w.stride(0), self.mask, self.canonical_buf, self.exec_buf, stream)
+        strides = w.stride()
+        assert w.is_cuda and w.element_size() == 2 and strides[1] == 1
+        code, canonical_bytes, exec_bytes = _native.encode_sizes(self.mask)
+        if code:
+            raise CrispError(code, "crisp_encode_sizes")
+        self._reserve(canonical_bytes, exec_bytes)
+        old, self.handle = self.handle, 0
+        code, self.handle = _native.encode(w.data_ptr(), strides[0], self.mask, self.canonical_buf.data_ptr(), self.exec_buf.data_ptr(),
+                                           _stream(stream), old)
+        if code:
+            raise CrispError(code, "crisp_encode")
         return self
 
     def _reserve(self, canonical_bytes, exec_bytes):
@@ -496,16 +523,6 @@ class HybridLayer:
             self.canonical_buf = self.torch.empty(canonical_bytes, dtype=self.torch.uint8, device=self.device)
         if self.exec_buf is None or self.exec_buf.numel() < exec_bytes:
             self.exec_buf = self.torch.empty(exec_bytes, dtype=self.torch.uint8, device=self.device)
-
-    def _adopt(self, kkeep, mask, handle):
-        """Take over a mask and a handle that a batched call made in this layer's buffers."""
-        if self.mask:
-            _lib.crisp_mask_destroy(self.mask)
-        if self.handle:
-            _lib.crisp_destroy(self.handle)
-        self.mask, self.handle = mask, handle
-        self.desc.keep_ratio = kkeep / self.nblk             # floor(ratio * nblk + 0.5) gives kkeep back
-        self.kkeep = kkeep
 
     def export(self, stream=None):
         import numpy as np
@@ -516,21 +533,24 @@ class HybridLayer:
         crisp_export(self.handle, blk_col, vals, idx, stream)
         return blk_col.reshape(self.nrt, self.kkeep), vals, idx
 
-    # The three calls below are made once per layer and pass; for small layers their host time is the time of the pass, so
-    # they hand their arguments to the library without the wrappers above.
+    # (empty_strided is the cheapest of torch's allocating calls: 1.1 us against 3.2 for new_empty and 4.2 for empty)
     def decode(self, stream=None):
-        w = self._bf16.new_empty((self.desc.rows, self.desc.k))
-        code = _lib.crisp_decode(self.handle, w.data_ptr(), w.stride(0), _stream(stream))
+        desc, torch = self.desc, self.torch
+        k = desc.k
+        w = torch.empty_strided((desc.rows, k), (k, 1), dtype=torch.bfloat16, device=self.device)
+        code = _native.decode(self.handle, w.data_ptr(), k, _stream(stream))
         if code:
             raise CrispError(code, "crisp_decode")
         return w
 
     def spmm(self, x, y=None, y_dtype=0, stream=None):
-        assert x.is_cuda and x.element_size() == 2 and x.stride(1) == 1 and x.shape[0] == self.desc.k
-        ncols = x.shape[1]
+        shape, strides = x.shape, x.stride()
+        assert x.is_cuda and x.element_size() == 2 and strides[1] == 1 and shape[0] == self.desc.k
+        ncols = shape[1]
         if y is None:
-            y = self._bf16.new_empty((self.desc.rows, ncols), dtype=self.torch.float32 if y_dtype else self.torch.bfloat16)
-        code = _lib.crisp_spmm(self.handle, x.data_ptr(), x.stride(0), ncols, y.data_ptr(), y.stride(0), y_dtype, _stream(stream))
+            y = self.torch.empty_strided((self.desc.rows, ncols), (ncols, 1), device=self.device,
+                                         dtype=self.torch.float32 if y_dtype else self.torch.bfloat16)
+        code = _native.spmm(self.handle, x.data_ptr(), strides[0], ncols, y.data_ptr(), y.stride()[0], y_dtype, _stream(stream))
         if code:
             raise CrispError(code, "crisp_spmm")
         return y
@@ -543,10 +563,10 @@ class HybridLayer:
         if y is None:
             ho, wo = h + 2 * pad - kernel_h + 1, w + 2 * pad - kernel_w + 1
             dt = self.torch.float32 if y_dtype else self.torch.bfloat16
-            y = self._bf16.new_empty((b, ho, wo, self.desc.rows) if nhwc_out else (self.desc.rows, b * ho * wo), dtype=dt)
-        ldy = y.stride(2) if nhwc_out else y.stride(0)
-        desc = ConvDesc(b, h, w, c, kernel_h, kernel_w, pad, 1 if nhwc_out else 0)
-        code = _lib.crisp_spmm_conv(self.handle, act_nhwc.data_ptr(), desc, y.data_ptr(), ldy, y_dtype, _stream(stream))
+            y = self.torch.empty((b, ho, wo, self.desc.rows) if nhwc_out else (self.desc.rows, b * ho * wo), dtype=dt, device=self.device)
+        ldy = y.stride()[2 if nhwc_out else 0]
+        code = _native.spmm_conv(self.handle, act_nhwc.data_ptr(), b, h, w, c, kernel_h, kernel_w, pad, 1 if nhwc_out else 0,
+                                 y.data_ptr(), ldy, y_dtype, _stream(stream))
         if code:
             raise CrispError(code, "crisp_spmm_conv")
         return y
@@ -659,26 +679,37 @@ class PruningNetwork:
         at_once = isinstance(grads, held) and (set(map(type, grads)) <= {list, tuple} or all(isinstance(gs, held) for gs in grads))
         count = min(len(self.layers), len(weights), len(grads) if at_once else len(weights))
         weights = weights[:count]
-        assert all(w.is_cuda and w.element_size() == 2 and w.stride(1) == 1 for w in weights)
+        assert all(w.is_cuda and w.element_size() == 2 and w.stride()[1] == 1 for w in weights)
         if not at_once:
             count = self._score_in_turn(weights, grads, stream)
         grads = grads[:count] if at_once else [()] * count
-        bf16 = torch.bfloat16
+        bf16, layers = torch.bfloat16, self.layers[:count]
+        # The table of the layers: one host array each for what there is per gradient, and one struct per layer.
+        flat = [g for gs in grads for g in gs]
+        ptrs = array("Q", [g.data_ptr() for g in flat])
+        lds = array("q", [g.stride()[0] for g in flat])
+        dts = array("i", [0 if g.dtype is bf16 else 1 for g in flat])
+        p0, l0, d0, at = ptrs.buffer_info()[0], lds.buffer_info()[0], dts.buffer_info()[0], 0
         arr = (PruneLayer * count)()
-        flat = [g for gs in grads for g in gs]               # one host array each for the whole network
-        ptrs = (C.c_void_p * len(flat))(*[g.data_ptr() for g in flat])
-        lds = (C.c_int64 * len(flat))(*[g.stride(0) for g in flat])
-        dts = (C.c_int32 * len(flat))(*[0 if g.dtype is bf16 else 1 for g in flat])
-        p0, l0, d0, at = C.addressof(ptrs), C.addressof(lds), C.addressof(dts), 0
-        for P, L, w, gs, s in zip(arr, self.layers, weights, grads, self.sal):
-            P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride(0)
-            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, len(gs)
-            P.d_saliency, P.ld_s = s.data_ptr(), s.stride(0)
+        for P, L, w, gs, s in zip(arr, layers, weights, grads, self.sal):
+            P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride()[0]
+            n = len(gs)
+            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, n
+            P.d_saliency, P.ld_s = s.data_ptr(), s.stride()[0]
             P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
-            at += len(gs)
+            at += n
         if at_once:
             crisp_prune_score(arr, stream)
         crisp_global_rank(self.rank_arr, crisp_prune_fraction(kappa, self.n, self.m), self.rank_ws, self.d_kkeep, stream)
+        # While the device scores and ranks: what the encodings need whatever the counts are, and the masks and handles that
+        # they will take the place of.
+        for P, L in zip(arr, layers):
+            if L.canonical_buf is not None:
+                P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
+        have = [(0, 0) if L.canonical_buf is None else (L.canonical_buf.numel(), L.exec_buf.numel()) for L in layers]
+        old_masks, old_handles = (C.c_void_p * count)(*[L.mask for L in layers]), (C.c_void_p * count)(*[L.handle for L in layers])
+        masks, handles = (C.c_void_p * count)(), (C.c_void_p * count)()
+        canonical_bytes, exec_bytes = (C.c_size_t * count)(), (C.c_size_t * count)()
         if stream is None:
             kk = self.d_kkeep.cpu().tolist()
         else:
@@ -686,12 +717,16 @@ class PruningNetwork:
                 kk = self.d_kkeep.cpu().tolist()
         for P, c in zip(arr, kk):
             P.kkeep = c
-        for P, L, cb, eb in zip(arr, self.layers, *crisp_prune_encode_sizes(arr)):
-            L._reserve(cb, eb)
-            P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
-        masks, handles = crisp_prune_encode(arr, stream)
-        for L, c, mask, handle in zip(self.layers, kk, masks, handles):
-            L._adopt(c, mask, handle)
+        _check(_lib.crisp_prune_encode_sizes(count, arr, canonical_bytes, exec_bytes), "crisp_prune_encode_sizes")
+        for P, L, cb, eb, (have_c, have_e) in zip(arr, layers, canonical_bytes, exec_bytes, have):
+            if cb > have_c or eb > have_e:
+                L._reserve(cb, eb)
+                P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
+        _check(_lib.crisp_prune_encode(count, arr, _stream(stream), masks, handles), "crisp_prune_encode")
+        for L, c, mask, handle in zip(layers, kk, masks, handles):
+            L.mask, L.handle, L.kkeep = mask, handle, c
+            L.desc.keep_ratio = c / L.nblk                   # floor(ratio * nblk + 0.5) gives the count back
+        crisp_destroy_layers(old_masks, old_handles)
         return kk
 
     def close(self):

@@ -5,11 +5,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcrisp.so")
+CALLS = os.path.join(HERE, "_calls.so")                      # Python entry points of the hot calls (plain C++)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -22,10 +24,10 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.inl")) \
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.cpp")) \
         + glob.glob(os.path.join(ROOT, "include", "*.h")) + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -39,6 +41,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", tmp] + sources()
     subprocess.check_call(cmd)
     os.replace(tmp, LIB)
+    tmp = CALLS + f".{os.getpid()}.tmp"
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), "-o", tmp,
+                           os.path.join(CSRC, "calls.cpp")])
+    os.replace(tmp, CALLS)
     return LIB
 
 

@@ -542,5 +542,10 @@ void crisp_destroy(crisp_handle_t h) {
     if (h) { crisp::tc_plan_destroy(h->plan); crisp::gather_plan_destroy(h->gather); }
     delete h;
 }
+crisp_status_t crisp_destroy_layers(int32_t n, const crisp_mask_t *masks, const crisp_handle_t *handles) {
+    if (n < 0 || (n > 0 && (!masks || !handles))) return CRISP_INVALID_ARG;
+    for (int32_t l = 0; l < n; ++l) { crisp_mask_destroy(masks[l]); crisp_destroy(handles[l]); }
+    return CRISP_OK;
+}
 
 }  // extern "C"

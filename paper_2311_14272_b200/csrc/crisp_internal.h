@@ -94,6 +94,8 @@ cudaError_t launch_chained(void (*kern)(Params...), unsigned grid, unsigned thre
 }
 #endif
 
+int sm_count_of(int device);                // multiprocessors of a device, looked up once (spmm_tc.cu)
+
 constexpr int kMaxBlocksPerRowTile = 4096;
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }

@@ -8,6 +8,8 @@
 //   K-M2  per row of the block grid: keep the kkeep highest-scored blocks and clear the
 //         bits of the pruned ones (blocks keep their positions)
 // Coalesced 32-byte-per-lane accesses; K-M1a is bound by HBM bandwidth.
+#include <atomic>
+
 #include "crisp_internal.h"
 #include "mask_common.cuh"
 
@@ -16,6 +18,7 @@ namespace crisp {
 namespace {
 
 constexpr int kScoreFractionBits = 40;
+constexpr int kMaxDevices = 64;
 
 // Raw bits of eight consecutive saliency values; the caller guarantees row < rows, k0 + 8 <= k and
 // 16-byte alignment.  Kept free of branches so that several of these can be in flight per lane.
@@ -357,15 +360,24 @@ clear_scores_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) L.score[i] = 0ull;
 }
 
-// Grids of resident CTAs: every CTA is on an SM from the start and takes its share of the items.
-int resident_grid(const void *kern, int64_t items) {
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-        sms = 148;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kM1Threads, 0) != cudaSuccess || per_sm <= 0) per_sm = 4;
-    const int64_t cap = (int64_t)sms * per_sm;
+// Grids of resident CTAs: every CTA is on an SM from the start and takes its share of the items.  What a device holds of a
+// kernel does not change, so it is asked for once (the queries take a microsecond or two of every call).
+template <typename... Params>
+int resident_grid(void (*kern)(Params...), std::atomic<int> *capacity, int64_t items) {
+    int dev = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+    int cap = dev >= 0 && dev < kMaxDevices ? capacity[dev].load(std::memory_order_relaxed) : 0;
+    if (cap <= 0) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kM1Threads, 0) != cudaSuccess || per_sm <= 0) per_sm = 4;
+        cap = sm_count_of(dev) * per_sm;
+        if (dev >= 0 && dev < kMaxDevices) capacity[dev].store(cap, std::memory_order_relaxed);
+    }
     return (int)(items < cap ? items : cap);
+}
+template <int M>
+int group_bits_grid(int64_t items) {
+    static std::atomic<int> capacity[kMaxDevices];
+    return resident_grid(group_bits_kernel<M>, capacity, items);
 }
 
 bool saliency_vec_ok(const float *s, int64_t ld) { return (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(s) & 15u) == 0); }
@@ -401,7 +413,8 @@ Batch<ScoreLayer, 1> batch_of_one(const ScoreLayer &L, int64_t units) {
 
 template <int CAP, int M, int TOP>
 cudaError_t run_block_scores(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
-    const int grid = resident_grid((const void *)block_score_kernel<CAP, M, TOP>, b.first[b.n]);
+    static std::atomic<int> capacity[kMaxDevices];
+    const int grid = resident_grid(block_score_kernel<CAP, M, TOP>, capacity, b.first[b.n]);
     return launch_chained(block_score_kernel<CAP, M, TOP>, (unsigned)grid, kM1Threads, 0, st, b);
 }
 // The selecting forms where n is 1 or 2 and only survivors count (all layers of a launch share n and m); from n = 3 on the
@@ -479,10 +492,10 @@ cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, i
     const int chunks = saliency_chunks(g);
     const int64_t items = (g.mp() / kM1Rows) * chunks;
     if (g.m == 4)
-        group_bits_kernel<4><<<resident_grid((const void *)group_bits_kernel<4>, items), kM1Threads, 0, st>>>(
+        group_bits_kernel<4><<<group_bits_grid<4>(items), kM1Threads, 0, st>>>(
             d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
     else
-        group_bits_kernel<8><<<resident_grid((const void *)group_bits_kernel<8>, items), kM1Threads, 0, st>>>(
+        group_bits_kernel<8><<<group_bits_grid<8>(items), kM1Threads, 0, st>>>(
             d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
     ScoreLayer L = {};
     L.g = g; L.s = d_s; L.ld = ld; L.max_key = max_key; L.nm_bits = d_nm_bits; L.score = score; L.blk_col = d_blk_col;

@@ -167,6 +167,4 @@ cudaError_t ensure_context(int device);
 
 }  // namespace tc
 
-int sm_count_of(int device);                // multiprocessors of a device (spmm_tc.cu)
-
 }  // namespace crisp
