@@ -99,6 +99,7 @@ crisp_handle_s *new_handle(const uint16_t *d_w_bf16, int64_t ld_w, const crisp_m
     h->debug_skip_stage = -1;
     h->plan = nullptr;
     h->gather = nullptr;
+    h->halo = nullptr;
     h->last = crisp_launch_info_t{-1, 0, 0, 1, 0, 0, 0, 0, 1};
     h->last_resident = 0;
     *L = crisp::EncodeLayer{};
@@ -539,7 +540,7 @@ crisp_status_t crisp_bytes_model(crisp_handle_t h, int64_t ncols, int32_t y_dtyp
 
 void crisp_mask_destroy(crisp_mask_t mask) { delete mask; }
 void crisp_destroy(crisp_handle_t h) {
-    if (h) { crisp::tc_plan_destroy(h->plan); crisp::gather_plan_destroy(h->gather); }
+    if (h) { crisp::tc_plan_destroy(h->plan); crisp::gather_plan_destroy(h->gather); crisp::halo_plan_destroy(h->halo); }
     delete h;
 }
 crisp_status_t crisp_destroy_layers(int32_t n, const crisp_mask_t *masks, const crisp_handle_t *handles) {

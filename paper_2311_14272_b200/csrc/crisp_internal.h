@@ -117,6 +117,8 @@ struct TcPlan;
 void tc_plan_destroy(TcPlan *plan);
 struct GatherPlan;          // tensor map of the execution image for the products of spmm_gather.cu
 void gather_plan_destroy(GatherPlan *plan);
+struct HaloPlan;            // launch plan of the last convolution of spmm_halo.cu
+void halo_plan_destroy(HaloPlan *plan);
 }  // namespace crisp
 
 struct crisp_handle_s {
@@ -137,6 +139,7 @@ struct crisp_handle_s {
     unsigned long long wait_limit_cycles;   // bound of every in-kernel wait (0 = default)
     int debug_skip_stage;   // test hook: the producer leaves out the loads of this pipeline fill (-1 = none)
     crisp::TcPlan *plan;    // cached launch plan of the last tensor-core product (or nullptr)
+    crisp::HaloPlan *halo;                  // cached launch plan of the last convolution that shares loads among taps (or nullptr)
     crisp::GatherPlan *gather;              // made by the first product on a layout TMA cannot address (or nullptr)
     std::mutex gather_lock;                 // such products may come from several threads at a time
     crisp_launch_info_t last;               // what the last product on this handle launched
@@ -212,6 +215,16 @@ TcImageLayout tc_image_layout(const Geometry &g, int kind);      // kind: CRISP_
 bool tc_operands_ok(const void *x, int64_t ldx, const void *y, int64_t ldy, int y_dtype, int64_t ncols);
 // Convolution geometry for the implicit-GEMM mode (stride 1): NHWC activation, ho x wo output pixels.
 struct ConvGeom { int batch, height, width, channels, kh, kw, pad, ho, wo, nhwc_out; };
+inline bool same_conv(const ConvGeom &a, const ConvGeom &b) {
+    return a.batch == b.batch && a.height == b.height && a.width == b.width && a.channels == b.channels &&
+           a.kh == b.kh && a.kw == b.kw && a.pad == b.pad && a.nhwc_out == b.nhwc_out;
+}
+// The pixel box tw x th x tb (n pixels) of a column tile of spmm_tc.cu's gather that covers the fewest pixels outside the images, then the
+// widest, then the tallest; `row` pixels of Y fill a 128-byte staging row.  -> pixels covered, -1: none fits
+int64_t conv_box(int n, int row, const ConvGeom &cv, int *tw, int *th, int *tb);
+// spmm_halo.cu: convolutions whose taps share one load of the activation
+cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
+                             cudaStream_t st, bool *done);
 // conv == nullptr: d_x is the [k, ncols] matrix.  Otherwise d_x is the activation and ncols = batch*ho*wo.
 // `h->plan` is reused when the operands, shape and epilogue are those of the previous call; `h->last` is filled in.
 cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols,

@@ -1049,12 +1049,19 @@ struct TcPlan {
 
 void tc_plan_destroy(TcPlan *plan) { delete plan; }
 
-namespace {
-
-bool same_conv(const ConvGeom &a, const ConvGeom &b) {
-    return a.batch == b.batch && a.height == b.height && a.width == b.width && a.channels == b.channels &&
-           a.kh == b.kh && a.kw == b.kw && a.pad == b.pad && a.nhwc_out == b.nhwc_out;
+int64_t conv_box(int n, int row, const ConvGeom &cv, int *tw, int *th, int *tb) {
+    int64_t best = -1;
+    for (int w = 32; w >= 8; w >>= 1)
+        for (int h = 32; h >= 1; h >>= 1) {
+            if (n % (w * h) != 0 || row % w != 0 || (w * h) % row != 0) continue;
+            const int b = n / (w * h);
+            const int64_t covered = (int64_t)((cv.wo + w - 1) / w) * w * ((cv.ho + h - 1) / h) * h * ((cv.batch + b - 1) / b) * b;
+            if (best < 0 || covered < best) { best = covered; *tw = w; *th = h; *tb = b; }
+        }
+    return best;
 }
+
+namespace {
 
 // Tile shape, shared-memory split, tensor maps and kernel variant for one product.
 cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols, void *d_y,
@@ -1087,22 +1094,10 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     TcParams p = {};
     if (conv) {
         // Pixel box of a column tile: tw * th * tb = 256 (or 128) output pixels, tw a power of two that divides
-        // a 128-byte staging row, whole staging rows per image.  Among the shapes that fit, the one that
-        // covers the fewest pixels outside the images wins (then the widest, then the tallest).
+        // a 128-byte staging row, whole staging rows per image.
         if (nt == 3) nt = 4;
         if (nt < 2) nt = 2;
-        const int f32c = y_dtype != 0 ? 32 : 64;
-        int64_t best = -1;
-        for (int tw = 32; tw >= 8; tw >>= 1)
-            for (int th = 32; th >= 1; th >>= 1) {
-                const int n_tile = nt * kBoxN;
-                if (n_tile % (tw * th) != 0 || f32c % tw != 0 || (tw * th) % f32c != 0) continue;
-                const int tb = n_tile / (tw * th);
-                const int64_t covered = (int64_t)((conv->wo + tw - 1) / tw) * tw * ((conv->ho + th - 1) / th) * th *
-                                        ((conv->batch + tb - 1) / tb) * tb;
-                if (best < 0 || covered < best) { best = covered; p.cv_tw = tw; p.cv_th = th; p.cv_tb = tb; }
-            }
-        if (best < 0) return cudaErrorInvalidValue;
+        if (conv_box(nt * kBoxN, y_dtype != 0 ? 32 : 64, *conv, &p.cv_tw, &p.cv_th, &p.cv_tb) < 0) return cudaErrorInvalidValue;
         p.conv = 1;
         p.cv_tiles_x = (conv->wo + p.cv_tw - 1) / p.cv_tw;
         p.cv_tiles_y = (conv->ho + p.cv_th - 1) / p.cv_th;
@@ -1283,6 +1278,12 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
     int device = 0;
     cudaError_t e = cudaGetDevice(&device);
     if (e != cudaSuccess) return e;
+    if (conv) {
+        e = ensure_context(device);                          // (a plan encodes tensor maps)
+        bool done = false;
+        if (e == cudaSuccess) e = launch_spmm_halo(h, d_x, d_y, ldy, y_dtype, *conv, device, st, &done);
+        if (done || e != cudaSuccess) return e;
+    }
     TcPlan *plan = h->plan;
     const bool hit = plan && plan->x == d_x && plan->y == d_y && plan->ldx == ldx && plan->ldy == ldy &&
                      plan->ncols == ncols && plan->y_dtype == y_dtype && plan->bias == h->epilogue.bias &&

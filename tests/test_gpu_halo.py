@@ -1,0 +1,82 @@
+"""Convolutions whose taps share one load of the activation (spmm_halo.cu), at the edges of its tiles: one, two and four
+images a tile, 224 and 256 pixels, ragged in x, y, images and output channels, several slabs of channels and CTA tiles of rows,
+weight tiles that stay and that do not.
+
+Reference: the same layer's product with [channels, pixels] results, which the taps' own loads compute (and the oracle checks
+elsewhere), and the oracle's convolution of one image's top strip.  Both round one fp32 sum of at most t products to bf16; two orders of
+such a sum differ by at most 2 t * 2^-23 * sum |w x|, their bf16 roundings by at most 2^-7 of the value."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import bf16_dev, gpu_layer, oracle_layer, to_dev, y_to_f64
+from test_gpu_conv import conv_inputs
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile
+    (64, 3, 3, 1, 64, 20, 84, 80, 2, 4, 64, 0.4, 224),        # one CTA tile of rows, weight tiles stay
+    (64, 3, 3, 1, 64, 26, 64, 96, 3, 4, 64, 0.9, 256),        # 64-pixel columns: 256 pixels cover less; nine blocks, dense tiles
+    (200, 3, 3, 1, 128, 27, 28, 28, 1, 4, 64, 0.5, 224),      # ragged in x and in the channels, two slabs, two CTA tiles of rows
+    (256, 3, 3, 1, 192, 75, 14, 14, 2, 4, 32, 0.3, 224),      # two images a tile, an odd number of them, three slabs
+    (264, 3, 3, 1, 64, 203, 7, 7, 4, 8, 128, 0.6, 224),       # four images a tile, dense tiles, three CTA tiles of rows
+    (96, 5, 3, 2, 64, 40, 33, 57, 2, 4, 32, 0.8, 224),        # odd sizes, border of four rows and two columns, images of four
+    (160, 3, 3, 0, 64, 17, 34, 66, 2, 8, 32, 0.4, 256),       # no padding, 32-pixel columns
+    (256, 3, 3, 1, 64, 12, 56, 56, 2, 4, 64, 0.9, 256),       # 256 pixels of four images, one accumulator
+]
+
+
+def layer_and_input(s_out, kh, kw, c, b, h, w, n, m, bm, keep, seed):
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    wt, sal, act = conv_inputs(s_out, kh, kw, c, b, h, w, seed=seed)
+    L = gpu_layer(B, torch, wt, sal, n, m, bm, 64, keep)
+    bias = np.random.default_rng(seed).standard_normal(s_out).astype(np.float32)
+    L.set_epilogue(to_dev(bias, torch), relu=True)
+    return torch, B, L, wt, sal, act, bias
+
+
+@pytest.mark.parametrize("s_out,kh,kw,pad,c,b,h,w,n,m,bm,keep,tile", CASES)
+def test_convolution(s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile):
+    torch, B, L, wt, sal, act, bias = layer_and_input(s_out, kh, kw, c, b, h, w, n, m, bm, keep, s_out + h)
+    mk, vals, idx, wd, _ = oracle_layer(wt, sal, n, m, bm, 64, keep)
+    x = bf16_dev(act, torch)
+    ho, wo = h + 2 * pad - kh + 1, w + 2 * pad - kw + 1
+    buf = torch.full((b * ho * wo * s_out + 64,), 7.0, dtype=torch.bfloat16, device="cuda")
+    y = buf[:b * ho * wo * s_out].view(b, ho, wo, s_out)
+    L.spmm_conv(x, kh, kw, pad, y=y, nhwc_out=True)
+    torch.cuda.synchronize()
+    info = L.last_launch()
+    assert L.device_status() == 0 and info["tile_cols"] == tile and info["epilogue_warps"] == 16
+    assert (L.last_resident_bytes() > 0) == (s_out <= 128 and mk.kkeep <= 4)
+    other = L.spmm_conv(x, kh, kw, pad)                         # [channels, pixels]: every tap loads its own pixels
+    assert L.last_launch()["tile_cols"] in (128, 256) and L.last_launch()["stages"] >= 2
+    terms = mk.kkeep * 64 * n // m + 1
+    mag = float(np.abs(wd).max()) * float(x.abs().max()) * terms
+    a, r = y.reshape(-1, s_out).t().double(), other.double()
+    assert bool(((a - r).abs() <= 2.0 ** -7 * r.abs() + 2 * terms * 2.0 ** -23 * mag).all())
+    rows = min(h, 8)
+    ref = oracle.bias_relu(oracle.conv_fp64(wd, kh, kw, np.ascontiguousarray(act[-1:, :rows]), pad), bias, True).reshape(s_out, -1, wo)
+    inner = rows - kh + pad + 1                                 # output rows whose window lies in the strip
+    got = y_to_f64(y[-1, :inner].reshape(-1, s_out), torch).T.reshape(s_out, inner, wo)
+    assert np.all(np.abs(got - ref[:, :inner]) <= 2.0 ** -8 * np.abs(ref[:, :inner]) + terms * 2.0 ** -23 * mag)
+    assert torch.all(buf[b * ho * wo * s_out:] == 7.0)
+    L.close()
+
+
+def test_a_wait_that_runs_out_is_reported():
+    torch, B, L, wt, sal, act, bias = layer_and_input(64, 3, 3, 64, 20, 84, 80, 2, 4, 64, 0.4, 3)
+    x = bf16_dev(act, torch)
+    want = L.spmm_conv(x, 3, 3, 1, nhwc_out=True)
+    L.set_tuning(wait_limit_cycles=2_000_000, skip_fill=1)      # every CTA's second load of the activation is left out
+    L.spmm_conv(x, 3, 3, 1, nhwc_out=True)
+    torch.cuda.synchronize()
+    assert L.last_launch()["tile_cols"] == 224 and L.device_status() == B.TIMEOUT
+    L.set_tuning()
+    L.reset_status()
+    y = L.spmm_conv(x, 3, 3, 1, nhwc_out=True)
+    torch.cuda.synchronize()
+    assert L.device_status() == 0 and torch.equal(y, want)
+    L.close()
