@@ -13,7 +13,7 @@
 // sparse MMAs of an entry (144 each, measured) and some 150 to take in its weight tile and its share of the activation, of 440 in all.
 // A tile is 224 pixels (28 rows of 8, or 14 rows of two images, 7 of four): the image sizes that are multiples of 7 come out even, and two
 // accumulators fit beside the metadata of the sparse image, so that a tile's results leave under the next one's MMAs; 256 pixels
-// where that covers less.
+// where that makes fewer waves of tiles, 128 or 64 where few tiles would leave SMs without one.
 // The walk is taken slab by slab (the list is put in that order when a CTA starts); the weight tiles come through a ring of
 // their own, or stay when there is one CTA tile of rows and the ring holds its whole walk.
 // Results: a warp takes 32 channels x 32 pixels from tensor memory in the layout of the transposing matrix store (stmatrix),
@@ -386,27 +386,32 @@ bool make_map_nhwc(CUtensorMap *map, const void *base, uint64_t c, uint64_t pitc
 bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
                HaloPlan *plan) {
     const Geometry &g = h->g;
-    if (y_dtype != 0 || !cv.nhwc_out || cv.kh * cv.kw < 2 || h->nt_override > 0 || h->group_override > 0) return false;
+    if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return false;
     if (h->exec_kind != CRISP_PATH_SPARSE && h->exec_kind != CRISP_PATH_DENSE) return false;
     if (ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0) return false;
     const bool sparse = h->exec_kind == CRISP_PATH_SPARSE;
     const TcImageLayout L = tc_image_layout(g, h->exec_kind);
     const int sms = sm_count_of(device);
     HaloParams p = {};
-    // Cycles of a launch in its longest CTA, by what was measured: an entry of the walk takes as long as shared memory takes the MMAs'
-    // operands, the weight tile and its share of the activation (1.3 cycles a pixel and 144, or 256 for dense tiles), a tile 300 more, and 1500
-    // where its results leave before the next one begins; an entry of the gather in spmm_tc.cu, 256 pixels, takes 700.
-    // (us, 56 x 56 x 16 images, 256 -> 256 channels, 19 entries: 224 pixels in 4 waves of tiles 25.9, 256 in 3 waves 24.3, the gather in
-    // 3 waves 26.9; 56 x 56 x 4, 384 -> 384, 11 entries: 12.1 in 2 waves, 9.4 in one, 10.0; the second with 3:4 dense tiles 30.4, 28.2, 29.7.)
+    // Cycles of a launch in its longest CTA, by what was measured.  An entry of the walk takes as long as shared memory needs to feed its
+    // MMAs and take in its weight tile, at least the 330 that issuing it takes; a box of the activation a cycle for each pixel of 128
+    // bytes; a tile 300 more, and 1500 where its results leave before the next one begins; the gather in spmm_tc.cu
+    // 700 for an entry of 256 pixels, 500 for one of 128.
+    // Both sides of the lines it draws (us, 3x3, replayed from a graph): 56 x 56 x 16 images, 256 -> 256 channels, 19 entries: 224 pixels in 4
+    // waves of tiles 25.9, 256 in 3 waves 24.1, the gather in 3 waves 26.7; 3:4 dense tiles 30.4, 28.0, 29.7; 56 x 56 x 4, 384 -> 384,
+    // 11 entries: 224 in 2 waves 12.1, 256 in one 9.2, gather 9.9; 14 x 14 x 32, 256 -> 256: 128 pixels 8.8, gather 10.2; 7 x 7 x 8, 512 -> 512:
+    // 64 pixels 15.0, gather 17.1; 1x1, 64 -> 64, 112 x 112 x 16: 11.8 and 14.1; 512 -> 512, 7 x 7 x 3: 6.4 and 6.3.
+    const int cpt = cv.channels / g.bk, boxes = L.wcap < cpt ? L.wcap : cpt;
     auto waves = [&](int64_t tiles) { return (tiles * L.nst + sms - 1) / sms; };
     int n = 0;
     int64_t best = 0, tiles = 0;
-    for (int cand : {224, 256})
+    for (int cand : {224, 256, 128, 64})
         for (int tb = 1; tb <= 4; tb <<= 1) {
             const int th = cand / 8 / tb, pw = 8 + cv.kw - 1, ph = th + cv.kh - 1;
             if (pw > 256 || ph > 256 || (int64_t)pw * ph * tb * 128 > 56 * 1024 || (ph * tb * pw) * 8 > 0xFFFF) continue;
             const int64_t count = (int64_t)((cv.wo + 7) / 8) * ((cv.ho + th - 1) / th) * ((cv.batch + tb - 1) / tb);
-            const int64_t cost = waves(count) * (L.wcap * (13 * cand / 10 + (sparse ? 144 : 256)) + (cand == 256 && sparse ? 1800 : 300)) + 2500;
+            const int fill = cand + (sparse ? 144 : 256), entry = fill > 330 ? fill : 330;
+            const int64_t cost = waves(count) * (L.wcap * entry + boxes * pw * ph * tb + (cand == 256 && sparse ? 1800 : 300)) + 2500;
             if (n && cost >= best) continue;
             best = cost; n = cand; tiles = count * L.nst;
             p.th = th; p.tb = tb; p.pw = pw;
@@ -414,12 +419,12 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     if (!n) return false;
     int bw, bh, bb;
     const int64_t gather = conv_box(256, 64, cv, &bw, &bh, &bb) / 256;
-    const bool narrow = 2 * gather * L.nst < sms;            // (the gather's tiles are half as wide then, 500 cycles an entry)
-    if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 1000) return false;
-    // One CTA tile of rows and a walk of up to eight blocks: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images
+    const bool narrow = 2 * gather * L.nst < sms;            // (the gather's tiles are half as wide then)
+    if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 2500) return false;
+    // One CTA tile of rows and a walk of up to eight blocks, where the gather has its wide tiles: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images
     // of 112 x 112 10.5 and 8.8, 3.4 tiles a CTA; 6 images 9.2 and 8.5; 3 images 6.8 each.  Below the line stays the gather with
     // resident weight tiles, whose form its tests and crisp_last_resident_bytes' callers look for.)
-    if (L.nst == 1 && L.wcap <= 8 && tiles < 3 * (int64_t)sms) return false;
+    if (L.nst == 1 && L.wcap <= 8 && !narrow && tiles < 3 * (int64_t)sms) return false;
     if (tiles > 0x7FFFFFFF) return false;
     if ((int64_t)L.nst * L.wcap * 8 > kListBytes || L.nst > kMaxRowTiles) return false;
     p.tb_log2 = p.tb == 4 ? 2 : p.tb - 1;
@@ -435,10 +440,11 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     const int ph = p.th + cv.kh - 1;
     p.x_bytes = (uint32_t)(p.pw * ph * p.tb * 128);
     p.x_stage = (uint32_t)align_up(p.x_bytes, 1024);
-    // two boxes in flight beside the one in use where the weight tiles leave the room, else one
+    // up to three boxes in flight beside the one in use where the weight tiles leave the room
     const uint32_t fixed = kEpiWarps * kStgTile + 512 + kListBytes, budget = kSmemBudget + 1024, w_stage = kGroup * p.entry_bytes;
     const uint32_t want_w = 3 * w_stage;
-    p.x_stages = fixed + 3 * p.x_stage + want_w <= budget ? 3 : 2;
+    p.x_stages = fixed + want_w + 2 * p.x_stage > budget ? 2u : (budget - fixed - want_w) / p.x_stage;
+    if (p.x_stages > 4) p.x_stages = 4;
     p.w_stages = (budget - fixed - p.x_stages * p.x_stage) / w_stage;
     if (p.w_stages > kMaxStages) p.w_stages = kMaxStages;
     if (p.w_stages < 2) return false;
@@ -450,9 +456,10 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
         !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb))
         return false;
     plan->p = p;
-    plan->which = (n == 256 ? 2 : 0) + (sparse ? 1 : 0);
-    plan->kern = n == 224 ? (sparse ? spmm_halo_kernel<224, true> : spmm_halo_kernel<224, false>)
-                          : (sparse ? spmm_halo_kernel<256, true> : spmm_halo_kernel<256, false>);
+    plan->which = (n == 256 ? 6 : n == 224 ? 4 : n == 128 ? 2 : 0) + (sparse ? 1 : 0);
+    static const HaloKernel kernels[8] = {spmm_halo_kernel<64, false>, spmm_halo_kernel<64, true>, spmm_halo_kernel<128, false>, spmm_halo_kernel<128, true>,
+                                          spmm_halo_kernel<224, false>, spmm_halo_kernel<224, true>, spmm_halo_kernel<256, false>, spmm_halo_kernel<256, true>};
+    plan->kern = kernels[plan->which];
     plan->resident_bytes = p.resident ? (int64_t)L.wcap * p.entry_bytes : 0;
     plan->info = crisp_launch_info_t{h->exec_kind, n, n == 256 && sparse ? 1 : 2, 1, kEpiWarps, (int)p.x_stages, plan->grid, 1, 1};
     return true;
@@ -480,7 +487,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
         *plan = fresh;
     }
     *done = true;
-    static std::atomic<bool> configured[4][64];
+    static std::atomic<bool> configured[8][64];
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     if (!configured[plan->which][device].load(std::memory_order_relaxed)) {
         // the most there is, once: the limit belongs to the function, not to a call

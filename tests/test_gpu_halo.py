@@ -15,15 +15,20 @@ from test_gpu_conv import conv_inputs
 pytestmark = pytest.mark.gpu
 
 CASES = [
-    # s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile
-    (64, 3, 3, 1, 64, 20, 84, 80, 2, 4, 64, 0.4, 224),        # one CTA tile of rows, weight tiles stay
-    (64, 3, 3, 1, 64, 26, 64, 96, 3, 4, 64, 0.9, 256),        # 64-pixel columns: 256 pixels cover less; nine blocks, dense tiles
-    (200, 3, 3, 1, 128, 27, 28, 28, 1, 4, 64, 0.5, 224),      # ragged in x and in the channels, two slabs, two CTA tiles of rows
-    (256, 3, 3, 1, 192, 75, 14, 14, 2, 4, 32, 0.3, 224),      # two images a tile, an odd number of them, three slabs
-    (264, 3, 3, 1, 64, 203, 7, 7, 4, 8, 128, 0.6, 224),       # four images a tile, dense tiles, three CTA tiles of rows
-    (96, 5, 3, 2, 64, 40, 33, 57, 2, 4, 32, 0.8, 224),        # odd sizes, border of four rows and two columns, images of four
-    (160, 3, 3, 0, 64, 17, 34, 66, 2, 8, 32, 0.4, 256),       # no padding, 32-pixel columns
-    (256, 3, 3, 1, 64, 12, 56, 56, 2, 4, 64, 0.9, 256),       # 256 pixels of four images, one accumulator
+    # s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile, whether the weight tiles stay
+    (64, 3, 3, 1, 64, 20, 84, 80, 2, 4, 64, 0.4, 224, True),        # one CTA tile of rows, weight tiles stay
+    (64, 3, 3, 1, 64, 26, 64, 96, 3, 4, 64, 0.9, 256, False),        # 64-pixel columns: 256 pixels cover less; nine blocks, dense tiles
+    (200, 3, 3, 1, 128, 27, 28, 28, 1, 4, 64, 0.5, 224, False),      # ragged in x and in the channels, two slabs, two CTA tiles of rows
+    (256, 3, 3, 1, 192, 75, 14, 14, 2, 4, 32, 0.3, 224, False),      # two images a tile, an odd number of them, three slabs
+    (264, 3, 3, 1, 64, 203, 7, 7, 4, 8, 128, 0.6, 224, False),       # four images a tile, dense tiles, three CTA tiles of rows
+    (96, 5, 3, 2, 64, 40, 33, 57, 2, 4, 32, 0.8, 224, False),        # odd sizes, border of four rows and two columns, images of four
+    (160, 3, 3, 0, 64, 17, 34, 66, 2, 8, 32, 0.4, 256, False),       # no padding, 32-pixel columns
+    (256, 3, 3, 1, 64, 12, 56, 56, 2, 4, 64, 0.9, 256, False),       # 256 pixels of four images, one accumulator
+    (200, 3, 3, 1, 64, 5, 9, 8, 1, 4, 128, 0.34, 64, False),  # few tiles: 64 pixels, ragged in y and in the channels
+    (64, 3, 3, 1, 64, 3, 19, 22, 3, 4, 64, 0.5, 64, True),    # the same with weight tiles that stay, dense
+    (256, 3, 3, 1, 128, 31, 14, 14, 4, 8, 64, 0.2, 128, False),   # 128 pixels, dense tiles, an odd number of images
+    (256, 1, 1, 0, 64, 16, 56, 50, 2, 4, 64, 1.0, 224, False),    # 1x1: no border, ragged in x
+    (72, 1, 1, 0, 192, 50, 45, 41, 1, 8, 32, 0.7, 224, True),
 ]
 
 
@@ -38,8 +43,8 @@ def layer_and_input(s_out, kh, kw, c, b, h, w, n, m, bm, keep, seed):
     return torch, B, L, wt, sal, act, bias
 
 
-@pytest.mark.parametrize("s_out,kh,kw,pad,c,b,h,w,n,m,bm,keep,tile", CASES)
-def test_convolution(s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile):
+@pytest.mark.parametrize("s_out,kh,kw,pad,c,b,h,w,n,m,bm,keep,tile,stay", CASES)
+def test_convolution(s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile, stay):
     torch, B, L, wt, sal, act, bias = layer_and_input(s_out, kh, kw, c, b, h, w, n, m, bm, keep, s_out + h)
     mk, vals, idx, wd, _ = oracle_layer(wt, sal, n, m, bm, 64, keep)
     x = bf16_dev(act, torch)
@@ -50,7 +55,7 @@ def test_convolution(s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile):
     torch.cuda.synchronize()
     info = L.last_launch()
     assert L.device_status() == 0 and info["tile_cols"] == tile and info["epilogue_warps"] == 16
-    assert (L.last_resident_bytes() > 0) == (s_out <= 128 and mk.kkeep <= 4)
+    assert (L.last_resident_bytes() > 0) == stay
     other = L.spmm_conv(x, kh, kw, pad)                         # [channels, pixels]: every tap loads its own pixels
     assert L.last_launch()["tile_cols"] in (128, 256) and L.last_launch()["stages"] >= 2
     terms = mk.kkeep * 64 * n // m + 1
