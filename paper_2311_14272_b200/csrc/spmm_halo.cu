@@ -421,10 +421,10 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     const int64_t gather = conv_box(256, 64, cv, &bw, &bh, &bb) / 256;
     const bool narrow = 2 * gather * L.nst < sms;            // (the gather's tiles are half as wide then)
     if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 2500) return false;
-    // One CTA tile of rows and a walk of up to eight blocks, where the gather has its wide tiles: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images
-    // of 112 x 112 10.5 and 8.8, 3.4 tiles a CTA; 6 images 9.2 and 8.5; 3 images 6.8 each.  Below the line stays the gather with
+    // One CTA tile of rows and a walk of up to eight blocks: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images
+    // of 112 x 112 10.5 and 8.8, 3.4 tiles a CTA; 6 images 9.2 and 8.5; 3 images 6.8 each; one image of 56 x 56 5.5 and 5.9.  Below the line stays the gather with
     // resident weight tiles, whose form its tests and crisp_last_resident_bytes' callers look for.)
-    if (L.nst == 1 && L.wcap <= 8 && !narrow && tiles < 3 * (int64_t)sms) return false;
+    if (L.nst == 1 && L.wcap <= 8 && tiles < 3 * (int64_t)sms) return false;
     if (tiles > 0x7FFFFFFF) return false;
     if ((int64_t)L.nst * L.wcap * 8 > kListBytes || L.nst > kMaxRowTiles) return false;
     p.tb_log2 = p.tb == 4 ? 2 : p.tb - 1;
