@@ -1083,14 +1083,30 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     int stack = conv ? 1 : L.stack;
     if (stack > 1 && (L.wcap * stack > 8 || (ncols + stack * nt * kBoxN - 1) / (stack * nt * kBoxN) < sm_count)) stack = 1;
     const int wlen = L.wcap * stack;                       // blocks per tile
-    // small layers are latency-bound: narrower tiles (down to 2 boxes) until at least half of the SMs have one
-    if (nt_override <= 0)
-        while (nt > 2 && (int64_t)L.nst * ((ncols + stack * nt * kBoxN - 1) / (stack * nt * kBoxN)) < sm_count / 2) --nt;
     // Short walks: the epilogue and the accumulator hand-over are the longest chain.  One warp per 64-column
     // box and lane quarter; under the sparse image three boxes, so that two accumulators fit beside the
     // metadata columns and the next tile's MMAs do not wait for the drain.
     const bool short_walk = wlen <= 8 && nt_override <= 0;
     if (short_walk && wlen <= 2 && sparse && nt == 4 && !conv) nt = 3;
+    if (nt_override > 0) {
+    } else if (conv || stack > 1) {
+        // small layers are latency-bound: narrower tiles (down to 2 boxes) until at least half of the SMs have one
+        while (nt > 2 && (int64_t)L.nst * ((ncols + stack * nt * kBoxN - 1) / (stack * nt * kBoxN)) < sm_count / 2) --nt;
+    } else {
+        // The width whose waves of tiles take the least time.  A tile of 128 or 192 columns takes some 0.66 and 0.80 of the time of one of 256
+        // (long walks on the sparse image, where only the narrowest has a second accumulator and a wave that is not full runs faster, 0.72
+        // and no less).  Measured, us with 256, 192, 128 columns: 256 x 2048, 2:4, 62 tiles of 256: 11.4, 11.6, 9.9; 90: 12.0, 11.6, 15.1;
+        // 160: 21.2, 21.0, 21.5; 240: 28.1, 33.3, 31.3; 512 x 2048, 3:4, 64: 13.3, 13.1, 10.7; 160: 22.7, 20.5, 23.9; 312: 36.0, 32.8, 40.4;
+        // 400: 40.1, 41.9, 50.5; 256 x 768, 2:4, six blocks, 74: 6.6, 6.1, 5.9; 200: 9.9, 8.3, 10.2.
+        const bool long_sparse = sparse && wlen > 8;
+        int64_t best = 0;
+        const int widest = nt;
+        for (int c = widest; c >= 2; --c) {
+            const int64_t waves = (L.nst * ((ncols + c * kBoxN - 1) / (c * kBoxN)) + sm_count - 1) / sm_count;
+            const int64_t cost = waves * (c == 4 ? 100 : c == 3 ? (long_sparse ? 100 : 80) : (long_sparse ? 72 : 66));
+            if (c == widest || cost < best) { best = cost; nt = c; }
+        }
+    }
     TcParams p = {};
     if (conv) {
         // Pixel box of a column tile: tw * th * tb = 256 (or 128) output pixels, tw a power of two that divides
