@@ -593,16 +593,18 @@ struct GatherPlan {
 };
 void gather_plan_destroy(GatherPlan *plan) { delete plan; }
 
-// Which products come here.  A CTA of the kernel in spmm_direct.cu takes some 3 us for every 128 kept activation rows, and again for
-// every wave of its CTAs; a launch of this one 7 to 8 us and little for each further block.  Measured on both sides of the
-// line (us, other kernel and this one): 160 kept rows 7.7 and 7.6 (1280 x 320 x 49), 6.9 and 8.0 (163 x 199 x 98); 256 kept rows 7.8
-// and 8.8 (33 x 1114 x 980); 480 kept rows 14.8 and 8.0 (160 x 960 x 49); 704 kept rows 32.3 and 9.1 (512 x 4608 x 49).  Of few kept rows
-// and many results: 6.6 and 8.0 (105 x 1372 results), 7.0 and 7.9 (39 x 6076), 11.6 and 9.1 (810 x 343), 19.5 and 7.3 (93 x 12348).
-constexpr int64_t kMinKept = 320, kMinResults = 1 << 18;
+// Which products come here.  A CTA of the kernel in spmm_direct.cu takes some 3 us for every 128 kept activation rows or 64 weights of a row, and
+// again for every wave of its CTAs; a launch of this one 7 to 8 us and little for each further block.  Measured on both sides of the
+// lines (us, that kernel and this one).  Kept rows: 256 7.8 and 8.8 (33 x 1114 x 980), 480 14.8 and 8.0 (160 x 960 x 49), 704 32.3 and 9.1.
+// Weights of a row: 96 6.2 and 7.4 (128 x 256 x 98), 7.0 and 7.8 (600 x 128 x 147); 128 9.6 and 8.2 (300 x 200 x 245), 18.1 and 8.3
+// (423 x 281 x 539).  Results, and multiply-adds: 6.9 and 7.9 (200 x 588, 64 weights a row), 7.0 and 7.9 (39 x 6076, 32); 12.6 and 7.7
+// (400 x 490, 96), 11.6 and 9.1 (810 x 343, 32), 19.5 and 7.3 (93 x 12348).
+constexpr int64_t kMinKept = 320, kMinWeights = 128, kMinResults = 1 << 18, kMinMacs = 10000000;
 bool gather_supported(const crisp_handle_s *h, int64_t ncols, int y_dtype) {
     if (y_dtype != 0 || (h->exec_kind != CRISP_PATH_DENSE && h->exec_kind != CRISP_PATH_SPARSE) || h->g.kkeep == 0) return false;
     if (!tensor_maps_available() || ncols >= (1ll << 31)) return false;
-    if ((int64_t)h->g.kkeep * h->g.bk < kMinKept && (int64_t)h->g.rows * ncols < kMinResults) return false;
+    const int64_t kept = (int64_t)h->g.kkeep * h->g.bk, weights = kept * h->g.n / h->g.m, results = (int64_t)h->g.rows * ncols;
+    if (kept < kMinKept && weights < kMinWeights && results < kMinResults && results * weights < kMinMacs) return false;
     const TcImageLayout L = tc_image_layout(h->g, h->exec_kind);
     const int64_t tiles = (int64_t)L.nst * ((ncols + kCols - 1) / kCols);
     return tiles <= 0x7FFFFFFF && (uint64_t)L.stack * L.nst * L.wcap * L.entry_bytes / 256 < (1ull << 31);
