@@ -54,6 +54,8 @@ struct HaloParams {
     int wo, ho, batch;
     uint32_t a_bytes, entry_bytes, x_bytes, x_stage, x_stages, w_stages;       // (a stage of weights: kGroup entries)
     int resident;
+    uint16_t *y;                         // results whose pixels TMA cannot address (pitch or base not a multiple of 16 bytes), else nullptr
+    int64_t ldy;
     unsigned long long wait_limit;
     int skip_fill;                       // test hook: this load of the activation is left out (-1 = none)
 };
@@ -113,7 +115,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_x);
-        prefetch_tensormap(&map_y);
+        if (!p.y) prefetch_tensormap(&map_y);
         for (uint32_t s = 0; s < p.x_stages; ++s) { mbar_init(x_full + 8 * s, 1); mbar_init(x_empty + 8 * s, 1); }
         for (uint32_t s = 0; s < p.w_stages; ++s) { mbar_init(w_full + 8 * s, 1); mbar_init(w_empty + 8 * s, 1); }
         for (int a = 0; a < kAcc; ++a) { mbar_init(t_full + 8 * a, 1); mbar_init(t_empty + 8 * a, kEpiWarps); }
@@ -321,12 +323,24 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         store_matrices(tile + (uint32_t)(512 * g) + my_row, pack(lo[4 * g], lo[4 * g + 1]), pack(lo[4 * g + 2], lo[4 * g + 3]),
                                        pack(hi[4 * g], hi[4 * g + 1]), pack(hi[4 * g + 2], hi[4 * g + 3]));
                     }
-                    fence_async_smem();
-                    __syncwarp();
-                    if (lane == 0) {
-                        const int y = org.y + (4 * c >> p.tb_log2);
-                        if (y < p.ho) tma_store_4d(&map_y, tile, ch0, org.x, org.b, y);
-                        bulk_commit();
+                    if (p.y) {                               // pixel by pixel, the lanes on consecutive channels
+                        __syncwarp();
+                        const bool ch_ok = ch0 + lane < p.rows;
+#pragma unroll 8
+                        for (int px = 0; px < 32; ++px) {
+                            const int g = 4 * c + (px >> 3), y = org.y + (g >> p.tb_log2), b = org.b + (g & (p.tb - 1)), x = org.x + (px & 7);
+                            uint16_t v;
+                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(tile + (uint32_t)(64 * px + (((lane >> 3) ^ (px >> 1 & 3)) << 4) + 2 * (lane & 7))) : "memory");
+                            if (ch_ok && y < p.ho && b < p.batch && x < p.wo) p.y[(((int64_t)b * p.ho + y) * p.wo + x) * p.ldy + ch0 + lane] = v;
+                        }
+                    } else {
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            const int y = org.y + (4 * c >> p.tb_log2);
+                            if (y < p.ho) tma_store_4d(&map_y, tile, ch0, org.x, org.b, y);
+                            bulk_commit();
+                        }
                     }
                 }
             }
@@ -388,7 +402,6 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     const Geometry &g = h->g;
     if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return false;
     if (h->exec_kind != CRISP_PATH_SPARSE && h->exec_kind != CRISP_PATH_DENSE) return false;
-    if (ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0) return false;
     const bool sparse = h->exec_kind == CRISP_PATH_SPARSE;
     const TcImageLayout L = tc_image_layout(g, h->exec_kind);
     const int sms = sm_count_of(device);
@@ -449,11 +462,12 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     if (p.w_stages > kMaxStages) p.w_stages = kMaxStages;
     if (p.w_stages < 2) return false;
     p.resident = L.nst == 1 && (uint32_t)L.wcap <= p.w_stages * kGroup;
+    if (ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0) { p.y = reinterpret_cast<uint16_t *>(d_y); p.ldy = ldy; }
     plan->smem = fixed + (size_t)p.x_stages * p.x_stage + (size_t)p.w_stages * w_stage;
     plan->grid = (int)(tiles < sms ? tiles : sms);
     if (!make_map_image(&plan->ma, h->d_exec + L.image_off, (uint64_t)L.stack * L.nst * L.wcap * L.entry_bytes, L.entry_bytes) ||
         !make_map_nhwc(&plan->mx, d_x, cv.channels, cv.channels, cv.width, cv.height, cv.batch, 64, p.pw, p.tb, ph) ||
-        !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb))
+        (!p.y && !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb)))
         return false;
     plan->p = p;
     plan->which = (n == 256 ? 6 : n == 224 ? 4 : n == 128 ? 2 : 0) + (sparse ? 1 : 0);

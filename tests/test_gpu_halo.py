@@ -27,6 +27,8 @@ CASES = [
     (200, 3, 3, 1, 64, 5, 9, 8, 1, 4, 128, 0.34, 64, False),  # few tiles: 64 pixels, ragged in y and in the channels
     (96, 3, 3, 1, 128, 3, 19, 22, 3, 4, 64, 0.5, 64, False),  # the same with dense tiles, odd sizes
     (256, 3, 3, 1, 128, 31, 14, 14, 4, 8, 64, 0.2, 128, False),   # 128 pixels, dense tiles, an odd number of images
+    (235, 3, 3, 1, 128, 6, 7, 7, 1, 4, 128, 0.3, 64, False),  # 235 channels: stored pixel by pixel
+    (100, 3, 3, 1, 128, 80, 28, 27, 2, 4, 32, 0.5, 224, False),   # 100 channels, several images, ragged in x
     (256, 1, 1, 0, 64, 16, 56, 50, 2, 4, 64, 1.0, 224, False),    # 1x1: no border, ragged in x
     (72, 1, 1, 0, 192, 50, 45, 41, 1, 8, 32, 0.7, 224, True),
 ]
