@@ -68,6 +68,31 @@ __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontr
 // The kernels of the mask / encode / decode chain begin with this: the next kernel's launch overlaps this one.
 __device__ __forceinline__ void chain_kernels() { launch_dependents(); wait_for_prerequisites(); }
 
+// Clusters: rank of this CTA, the place of one of its shared-memory addresses in another rank, loads from there, and the barrier
+// of all threads of a cluster.
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t peer_address(uint32_t smem, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t lds32_peer(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 lds128_peer(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+
 // (`cluster` CTAs form a thread-block cluster; 1: none)
 template <typename... Params, typename... Args>
 cudaError_t launch_clusters(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, unsigned cluster,

@@ -349,6 +349,159 @@ block_select_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     }
 }
 
+// The whole projection of a small layer in one launch: a cluster of up to eight CTAs, each with whole row tiles, so that all that
+// crosses between them is the layer maximum.  Group bits and the maximum in a first pass over S, scores in a second (out of L1 and L2)
+// summed in shared memory, then the selection: what the kernels above compute, from the same definitions.  What bounds it is instructions on
+// one SM (some 250 for eight elements), and for the smallest layers the two passes' round trips.  A memset and three kernels in its place
+// take the device 10 to 15 us and the host about as long.
+constexpr int kSmallThreads = 1024, kSmallMaxBlocks = 512, kSmallCluster = 8;
+template <int M>
+__global__ void __launch_bounds__(kSmallThreads)
+mask_small_kernel(const float *s, int64_t ld, Geometry g, bool vec_ok, bool max_known, uint32_t *max_key, unsigned long long *score,
+                  uint32_t *nm_bits, int32_t *blk_col, int ctas) {
+    __shared__ unsigned long long s_score[kSmallMaxBlocks];
+    __shared__ uint32_t s_part[3][kSmallMaxBlocks];          // a score in pieces of 22 bits: 32-bit shared atomics are native, 64-bit ones a loop
+    __shared__ int s_kept[kSmallMaxBlocks];
+    __shared__ uint32_t s_best[kSmallThreads / 32];
+    __shared__ uint32_t s_max;
+    __shared__ uint8_t s_keep[64];
+    chain_kernels();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x;
+    if (M == 4 && tid < 64) s_keep[tid] = (uint8_t)keep_mask_of_outcomes(tid, g.n);
+    __syncthreads();
+    const int chunks = g.wpr * 4, units = g.bm * chunks;     // chunks of eight elements: of a row, of a row tile
+    // a thread takes every kSmallThreads-th chunk of a row tile: (row, chunk) of the first, and the step
+    const int r_first = tid / chunks, c_first = tid - r_first * chunks, r_step = kSmallThreads / chunks, c_step = kSmallThreads - r_step * chunks;
+    auto load = [&](int64_t row, int c, uint32_t (&key)[8]) {
+        if (vec_ok && row < g.rows && 8 * c + 8 <= g.k) {
+            load8_raw(s, ld, row, 8 * c, key);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) key[j] = canonical_bits(key[j]);
+        } else {
+            load8(s, ld, g.rows, g.k, row, 8 * c, vec_ok, key);
+        }
+    };
+    // group bits and the maximum
+    uint32_t best = 0u;
+    for (int rt = cta; rt < g.nrt; rt += ctas)
+        for (int u = tid, r = r_first, c = c_first; u < units; u += kSmallThreads) {
+            const int64_t row = (int64_t)rt * g.bm + r;
+            uint32_t key[8];
+            load(row, c, key);
+            uint32_t bits;
+            if constexpr (M == 4) bits = (uint32_t)s_keep[outcomes4(key)] | ((uint32_t)s_keep[outcomes4(key + 4)] << 4);
+            else bits = top_n_bits<M>(key, g.n);
+            reinterpret_cast<uint8_t *>(nm_bits + row * g.wpr)[c] = (uint8_t)bits;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) best = max(best, key[j]);
+            r += r_step; c += c_step;
+            if (c >= chunks) { c -= chunks; ++r; }
+        }
+    best = __reduce_max_sync(0xFFFFFFFFu, best);
+    if (lane == 0) s_best[warp] = best;
+    __syncthreads();
+    if (warp == 0) {
+        best = __reduce_max_sync(0xFFFFFFFFu, s_best[lane]);
+        if (lane == 0) s_max = best;
+    }
+    if (ctas > 1) {
+        cluster_arrive();
+        cluster_wait();
+        best = lane < ctas ? lds32_peer(peer_address((uint32_t)__cvta_generic_to_shared(&s_max), (uint32_t)lane)) : 0u;
+    } else {
+        __syncthreads();
+        best = s_max;
+    }
+    best = max_known ? *max_key : __reduce_max_sync(0xFFFFFFFFu, best);
+    if (!max_known && cta == 0 && tid == 0) *max_key = best;
+    const int e_max = best ? key_exponent(best) : 0, scale_exp = kScoreFractionBits - e_max;
+    const bool float_scale = scale_exp >= -126 && scale_exp <= 127;
+    const float scale = float_scale ? __uint_as_float((uint32_t)(127 + scale_exp) << 23) : 0.f;
+    for (int rt = cta; rt < g.nrt; rt += ctas) {
+        // block scores
+        for (int j = tid; j < g.nblk; j += kSmallThreads) s_part[0][j] = s_part[1][j] = s_part[2][j] = 0u;
+        __syncthreads();
+        for (int u0 = 0, r = r_first, c = c_first; u0 < units; u0 += kSmallThreads) {        // (chunks of a row come in fours, so the lanes of a mask word stay together)
+            const int64_t row = (int64_t)rt * g.bm + r;
+            unsigned long long acc = 0ull;
+            if (u0 + tid < units && best) {
+                uint32_t key[8];
+                load(row, c, key);
+                uint32_t counted = 0xFFu;
+                if (g.score_mode == 0) counted = reinterpret_cast<const uint8_t *>(nm_bits + row * g.wpr)[c];       // (this thread's own byte)
+                if (float_scale) {                           // (as in block_score_kernel)
+                    uint64_t r_sum = f32x2(0.f, 0.f), d_sum = r_sum;
+#pragma unroll
+                    for (int j = 0; j < 8; j += 2) {
+                        uint64_t whole, part;
+                        floor_parts2(mul2(f32x2(__uint_as_float(key[j]), __uint_as_float(key[j + 1])),
+                                          f32x2((counted >> j) & 1u ? scale : 0.f, (counted >> (j + 1)) & 1u ? scale : 0.f)), whole, part);
+                        r_sum = add2(r_sum, whole);
+                        d_sum = add2(d_sum, part);
+                    }
+                    acc = ((unsigned long long)__float2uint_rn(f32x2_sum(r_sum) * 9.5367431640625e-07f) << 20) + (unsigned long long)__float2uint_rn(f32x2_sum(d_sum));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if ((counted >> j) & 1u) acc += fixed_point_score(key[j], e_max);
+                }
+            }
+            acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 1);
+            acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 2);
+            if (g.bk % 64 == 0) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 4);
+            if (g.bk % 128 == 0) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 8);
+            // (at most 384 such sums make a block, each below 2^48: no piece overflows)
+            if ((lane & (g.bk % 128 == 0 ? 15 : g.bk % 64 == 0 ? 7 : 3)) == 0 && acc) {
+                const int j = 8 * c / g.bk;
+                atomicAdd(&s_part[0][j], (uint32_t)acc & 0x3FFFFFu);
+                atomicAdd(&s_part[1][j], (uint32_t)(acc >> 22) & 0x3FFFFFu);
+                atomicAdd(&s_part[2][j], (uint32_t)(acc >> 44));
+            }
+            r += r_step; c += c_step;
+            if (c >= chunks) { c -= chunks; ++r; }
+        }
+        __syncthreads();
+        for (int j = tid; j < g.nblk; j += kSmallThreads)
+            s_score[j] = (unsigned long long)s_part[0][j] + ((unsigned long long)s_part[1][j] << 22) + ((unsigned long long)s_part[2][j] << 44);
+        __syncthreads();
+        // selection
+        for (int j = tid; j < g.nblk; j += kSmallThreads) {
+            const unsigned long long mine = s_score[j];
+            int rank = 0;
+            for (int t = 0; t < g.nblk; ++t) rank += s_score[t] > mine || (s_score[t] == mine && t < j);
+            s_kept[j] = rank < g.kkeep;
+            score[(int64_t)rt * g.nblk + j] = mine;
+        }
+        __syncthreads();
+        if (warp == 0) {                                     // kept columns in ascending order
+            int base = 0;
+            for (int j0 = 0; j0 < g.nblk; j0 += 32) {
+                const int f = j0 + lane < g.nblk ? s_kept[j0 + lane] : 0;
+                const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, f);
+                if (f) blk_col[(int64_t)rt * g.kkeep + base + __popc(ballot & ((1u << lane) - 1u))] = j0 + lane;
+                base += __popc(ballot);
+            }
+        }
+        const int wpb = g.bk / 32;
+        for (int i = tid; i < g.bm * g.wpr; i += kSmallThreads)
+            if (!s_kept[i % g.wpr / wpb]) nm_bits[(int64_t)rt * g.bm * g.wpr + i] = 0u;
+        __syncthreads();                                     // (the scores are cleared for the next row tile)
+    }
+    if (ctas > 1) {                                          // no CTA's shared memory goes before all have read it
+        cluster_arrive();
+        cluster_wait();
+    }
+}
+// Layers that it takes: up to 2^14 elements a CTA.  Mask phase replayed from a graph, and mask, encoding and decoding called in a row, us, this kernel and
+// the others: 256 x 256 (2^13 a CTA) 6.3 and 10.4, 14.3 and 19; 128 x 256 (2^14) 8.0 and 10.4, 15.6 and 19; 25 x 489 (2^14, one CTA) 9.2
+// and 13.1, 19.5 and 21; 256 x 512 in four CTAs (2^15) 12.1 and 10.5, 19.9 and 19.
+constexpr int64_t kSmallPerCta = 1 << 14;
+int small_ctas(const Geometry &g) {
+    const int ctas = g.nrt < kSmallCluster ? g.nrt : kSmallCluster;
+    const int64_t most = (int64_t)((g.nrt + ctas - 1) / ctas) * g.bm * g.kp();
+    return g.nblk <= kSmallMaxBlocks && most <= kSmallPerCta ? ctas : 0;
+}
+
 // Scores and maxima of a batch, cleared (one CTA per layer; a memset per layer costs a launch each).
 template <int CAP>
 __global__ void __launch_bounds__(256)
@@ -481,6 +634,13 @@ cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, i
     uint32_t *max_key = reinterpret_cast<uint32_t *>(d_workspace);
     unsigned long long *score =
         reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(d_workspace) + kAlign);
+    if (const int ctas = small_ctas(g)) {
+        auto launch = [&](auto kern) {
+            return launch_clusters(kern, (unsigned)ctas, kSmallThreads, 0, st, (unsigned)ctas, d_s, ld, g, saliency_vec_ok(d_s, ld), max_known, max_key,
+                                   score, d_nm_bits, d_blk_col, ctas);
+        };
+        return g.m == 4 ? launch(mask_small_kernel<4>) : launch(mask_small_kernel<8>);
+    }
     // max_known: the first word already holds the layer's largest canonical |s| (written by the saliency kernel
     // that produced S), so only the scores are cleared and the pass over S that finds the maximum is skipped
     cudaError_t e = max_known ? cudaMemsetAsync(score, 0, workspace_bytes - kAlign, st)
