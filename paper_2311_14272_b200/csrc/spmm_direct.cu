@@ -17,6 +17,8 @@
 // keep 0.25: 508 -> 51 us (38 M warp instructions, 76 % of the issue slots of busy SMs); 160 x 960 x 49, 2:8, keep 0.5:
 // 147 -> 16.4 us, a chain of four stages on 20 CTAs.  One warp per row that gathers its activations from L2 without
 // staging took 13-22 us on the second and 65 us on the first; staging through registers with two buffers 70 us.
+// The next kernel's launch overlaps this one: products in a row, us, 16 x 32 x 49 5.4 -> 4.5, 216 x 106 x 245 7.7 -> 5.8, 64 x 64 x 6076 fp32
+// 12.3 -> 10.0; a product of 93 us keeps its time.
 #include <cuda_bf16.h>
 
 #include "crisp_internal.h"
@@ -85,9 +87,8 @@ struct DirectTile {
 // one shared-memory load can bring them.
 template <int RW, int CPL, int ALIGN, typename OutT>
 __global__ void __launch_bounds__(DirectTile<RW, CPL>::kThreads, 3)
-spmm_direct_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16_t *__restrict__ vals,
-                   const uint32_t *__restrict__ idx, const uint16_t *__restrict__ x, int64_t ldx, int64_t ncols,
-                   OutT *__restrict__ y, int64_t ldy, Epilogue epi, DirectSplit sp) {
+spmm_direct_kernel(Geometry g, const int32_t *blk_col, const uint16_t *vals, const uint32_t *idx, const uint16_t *x, int64_t ldx,
+                   int64_t ncols, OutT *y, int64_t ldy, Epilogue epi, DirectSplit sp) {
     using T = DirectTile<RW, CPL>;
     constexpr int kThreads = T::kThreads, kTileN = T::kTileN, kRows = T::kRows, kStageRows = T::kStageRows, kPitch = T::kPitch;
     constexpr int kRun = ALIGN / 2 < CPL ? ALIGN / 2 : CPL;  // consecutive columns of a lane
@@ -101,6 +102,7 @@ spmm_direct_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16
     const uint32_t s_words = s_x + T::kStages * stage_bytes;                                 // [kRows][group * vpp] weight words
     const int32_t *s_col = reinterpret_cast<const int32_t *>(s_raw + T::kStages * stage_bytes + kRows * group * vpp * 4);   // [kkeep]
 
+    chain_kernels();                                         // (behind it nothing is read through the read-only path)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slabs = g.bm / kRows;                          // CTAs that share a row tile
     const int64_t ct = blockIdx.x / (g.nrt * slabs);         // row slabs fastest: they share X
@@ -114,7 +116,7 @@ spmm_direct_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16
     const int idx_words = vpb * g.idx_bits / 32;
     const uint32_t field = (1u << g.idx_bits) - 1u;
     const int parts = g.kkeep * sp.ppb, stages = (parts + group - 1) / group;
-    for (int i = threadIdx.x; i < g.kkeep; i += kThreads) const_cast<int32_t *>(s_col)[i] = __ldg(blk_col + (int64_t)rt * g.kkeep + i);
+    for (int i = threadIdx.x; i < g.kkeep; i += kThreads) const_cast<int32_t *>(s_col)[i] = blk_col[(int64_t)rt * g.kkeep + i];
     __syncthreads();
 
     // step 1: the activation rows of a stage's parts and the slab's weights and offsets
@@ -134,7 +136,7 @@ spmm_direct_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16
 #pragma unroll
                     for (int t = 0; t < 8; ++t)
                         reinterpret_cast<uint16_t *>(s_raw)[(dst - s_x) / 2 + t] =
-                            p + 2 * t >= x_begin && p + 2 * t < x_end ? __ldg(reinterpret_cast<const uint16_t *>(p) + t) : (uint16_t)0;
+                            p + 2 * t >= x_begin && p + 2 * t < x_end ? reinterpret_cast<const uint16_t *>(p)[t] : (uint16_t)0;
                 } else {                                     // zero beyond the matrix (the address is not used then)
                     const uint32_t bytes = krow >= g.k || p >= x_end ? 0u : (p + 16 <= x_end ? 16u : (uint32_t)(x_end - p));
                     copy16(dst, bytes ? p : reinterpret_cast<uintptr_t>(vals), bytes);
@@ -200,8 +202,8 @@ spmm_direct_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16
                     if ((bit & 31) + g.idx_bits > 32) t |= lds32(a + 4) << (32 - (bit & 31));
                 } else {
                     const int bit = ((slab_row + warp * RW + r) * vpr + sub * vpp + v) * g.idx_bits;
-                    t = __ldg(ib + (bit >> 5)) >> (bit & 31);
-                    if ((bit & 31) + g.idx_bits > 32) t |= __ldg(ib + (bit >> 5) + 1) << (32 - (bit & 31));
+                    t = ib[bit >> 5] >> (bit & 31);
+                    if ((bit & 31) + g.idx_bits > 32) t |= ib[(bit >> 5) + 1] << (32 - (bit & 31));
                 }
                 const uint32_t kin = (uint32_t)(div_small(v, sp.inv_n) * g.m) + (t & field);       // activation row in the part
                 const uint32_t off = ((uint32_t)(b << sp.part_log2) + kin) * (uint32_t)kPitch + ((x_low + (krow0 + kin) * ldx2) & 15u);
@@ -250,7 +252,7 @@ spmm_direct_kernel(Geometry g, const int32_t *__restrict__ blk_col, const uint16
     for (int r = 0; r < RW; ++r) {
         const int64_t row = (int64_t)rt * g.bm + slab_row + warp * RW + r;
         if (row >= g.rows) break;
-        const float bias = epi.bias ? __ldg(epi.bias + row) : 0.f;
+        const float bias = epi.bias ? epi.bias[row] : 0.f;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
             float v = acc[r][c];
@@ -307,8 +309,7 @@ cudaError_t launch_form(const Geometry &g, const int32_t *bc, const uint16_t *va
         // larger launch of another host thread that set it a moment before.
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kMostSmem);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)ctas, T::kThreads, smem, st>>>(g, bc, vals, idx, x, ldx, ncols, y, ldy, epi, sp);
-        return cudaGetLastError();
+        return launch_chained(kern, (unsigned)ctas, T::kThreads, smem, st, g, bc, vals, idx, x, ldx, ncols, y, ldy, epi, sp);
     };
     if (CPL == 4 && al % 8 == 0) return launch(spmm_direct_kernel<RW, CPL, CPL == 4 ? 8 : 4, OutT>);
     if (al % 4 == 0) return launch(spmm_direct_kernel<RW, CPL, 4, OutT>);
