@@ -318,6 +318,8 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         }
     } else if (warp >= kFirstX) {
         // ------------------------------------------------ X: rows res, res + 8, ... of every other block
+        // Every other one of all the blocks this CTA multiplies, whatever tile they belong to: a group that skipped more than num_stages
+        // blocks between two of its own would find the parity of an older release of its stage.
         const int gi = (warp - kFirstX) / kGroupWarps, res = (warp - kFirstX) % kGroupWarps;
         const CUtensorMap *map = &map_x.m[res];
         const int rows = p.g.bk / 8;                         // of a block, for this warp
@@ -331,27 +333,25 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         const uint32_t lane_dst = (uint32_t)res * 128u + p.entry_bytes +
                                   (kWide ? (uint32_t)(lane >> 4) * box_bytes + ((((uint32_t)lane >> 1 & 7u) ^ (uint32_t)res) << 4) + ((uint32_t)lane & 1u) * 8u
                                          : ((((uint32_t)lane >> 2) ^ (uint32_t)res) << 4) + ((uint32_t)lane & 3u) * 4u);
-        uint32_t stage = 0, ph = 0, slot = 0, slot_ph = 0;
-        int tile_no = 0;
+        uint32_t stage = (uint32_t)gi, ph = 0, slot = 0, slot_ph = 0;
+        int tile_no = 0, first = gi;                         // the group's first block of the tile
         bool ok = true;
 #pragma unroll 1
         for (int t = first_tile; t < p.num_tiles && ok; t += tile_step, ++tile_no) {
             const int ct = t / p.nst, st = t - ct * p.nst;
             const int32_t *cols = p.walk_col + (int64_t)st * p.wcap + rank;
             int window = 0, col_of_lane = 0;                 // block columns of entries window .. window + 31 of this rank
-            auto load_window = [&](int first) {
-                window = first;
-                const int e = (first + lane) << p.split_log2;
+            auto load_window = [&](int from) {
+                window = from;
+                const int e = (from + lane) << p.split_log2;
                 col_of_lane = rank + e < p.wcap ? cols[e] : 0;
             };
             load_window(0);
-            const int count = walk_share(p, st, rank), mine = (count - gi + 1) >> 1;      // blocks gi, gi + 2, ...
-            auto next_stage = [&] { if (++stage == p.num_stages) { stage = 0; ph ^= 1u; } };
+            const int count = walk_share(p, st, rank), mine = (count - first + 1) >> 1;   // blocks first, first + 2, ...
             uint32_t probe = 0, to = slot;                   // slot to ask for next; one block is moved, the one `ahead` on asked for
 #pragma unroll 1
             for (int i = 0; i < mine + p.ahead; ++i) {
                 if (i >= p.ahead) {
-                    if (gi == 1) next_stage();               // (the other group's block)
                     if (!mbar_wait(my_bar + 8 * slot, slot_ph, abort_flag, p.wait_limit) ||
                         !mbar_wait(bar_empty + 8 * stage, ph ^ 1u, abort_flag, p.wait_limit)) { ok = false; break; }
                     const uint32_t src = my_raw + slot * slot_step + lane_src, dst = ring + stage * p.stage_bytes + lane_dst;
@@ -391,12 +391,12 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_full + 8 * stage);
-                    next_stage();
-                    if (gi == 0) next_stage();
+                    stage += 2;                              // (past the other group's block)
+                    if (stage >= p.num_stages) { stage -= p.num_stages; ph ^= 1u; }
                     if (++slot == (uint32_t)p.ahead) { slot = 0; slot_ph ^= 1u; }
                 }
                 if (i < mine) {
-                    const int e = gi + 2 * i;
+                    const int e = first + 2 * i;
                     if (e >= window + 32) load_window(e);
                     const int col = __shfl_sync(0xFFFFFFFFu, col_of_lane, e - window);
                     if (lane == 0) {
@@ -407,9 +407,7 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     if (++to == (uint32_t)p.ahead) to = 0;
                 }
             }
-            // blocks of the walk behind this group's last one
-            if (gi == 0 ? (count & 1) : 0) { if (stage == 0) { stage = p.num_stages; ph ^= 1u; } --stage; }
-            if (gi == 1 && (count & 1)) next_stage();
+            first ^= count & 1;
         }
         if (warp == kFirstX) launch_dependents();            // (this CTA has asked for its last tile)
     } else if (p.split == 1) {

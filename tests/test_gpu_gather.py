@@ -27,13 +27,15 @@ CASES = [
 ]
 
 
-def make(rows, k, ncols, pitch, n, m, bm, bk, keep, off):
+def make(rows, k, ncols, pitch, n, m, bm, bk, keep, off, favour=None):
     import torch
     from paper_2311_14272_b200 import binding as B
     B.load()
     rng = np.random.default_rng(rows + ncols)
     w = wl.f32_to_bf16_bits(rng.standard_normal((rows, k)).astype(np.float32))
     s = rng.uniform(0.1, 2.0, (rows, k)).astype(np.float32)
+    if favour is not None:
+        favour(s)
     x = wl.f32_to_bf16_bits(rng.standard_normal((k, ncols)).astype(np.float32))
     L = gpu_layer(B, torch, w, s, n, m, bm, bk, keep)
     # what lies between the rows and around the matrix is not finite: it must not be used
@@ -127,4 +129,40 @@ def test_products_of_two_threads_on_one_layer():
     torch.cuda.synchronize()
     assert errors == [] and L.device_status() == 0
     assert torch.equal(gots[0], wants[0]) and torch.equal(gots[1], wants[1])
+    L.close()
+
+
+def one_long_walk_in_nine(s):
+    """Saliency of row tiles of 64 that all keep block 0, but for one of the 18, which keeps block 1."""
+    s[:, :32] += 4.0
+    s[576:640] = s[576:640, ::-1]
+
+
+@pytest.mark.parametrize("rows,k,ncols,n,m,bm,bk,keep,favour", [
+    (1034, 413, 2206, 3, 4, 64, 128, 0.4, None),        # a ring of two stages, walks of two or three blocks, two tiles a CTA
+    (700, 300, 9001, 2, 4, 32, 128, 0.34, None),        # the same with the 2:4 image, walks of one or two blocks
+    (1300, 800, 4999, 4, 4, 64, 96, 0.4, None),         # 96-deep blocks, walks of four to seven
+    (1152, 64, 38401, 2, 4, 64, 32, 0.5, one_long_walk_in_nine),     # eight stages, walks of one block and every ninth of two
+    (1152, 64, 38401, 4, 4, 64, 32, 0.5, one_long_walk_in_nine),
+])
+def test_several_tiles_with_walks_of_unlike_length(rows, k, ncols, n, m, bm, bk, keep, favour):
+    """The two groups of X warps take every other block of all tiles of a CTA: neither may get ahead of the other by more than the ring.
+
+    Reference: the kernel on the CUDA cores (checked against the oracle elsewhere).  Two orders of an fp32 sum of t products
+    differ by at most 2 t * 2^-23 * sum |w x|, their bf16 roundings by at most 2^-7 of the value."""
+    torch, L, rng, w, s, x, xv = make(rows, k, ncols, ncols, n, m, bm, bk, keep, 0, favour)
+    mk, vals, idx, wd, wb = oracle_layer(w, s, n, m, bm, bk, keep)
+    y = L.spmm(xv)
+    info = L.last_launch()
+    tiles = -(-rows // 128) * -(-ncols // 128)
+    assert info["tile_cols"] == 128 and info["ctas"] < tiles
+    walks = {len(set(mk.blk_col.reshape(-1, mk.kkeep)[i:i + 128 // bm].ravel())) for i in range(0, -(-rows // bm), 128 // bm)}
+    assert len(walks) > 1
+    L.set_path(0)
+    ref = L.spmm(xv).double()
+    torch.cuda.synchronize()
+    assert L.last_launch()["tile_cols"] == 0 and L.device_status() == 0
+    size = to_dev(np.abs(wd.astype(np.float64)), torch) @ xv.double().abs()
+    terms = mk.kkeep * bk * n // m
+    assert bool(((y.double() - ref).abs() <= 2.0 ** -7 * ref.abs() + 2 * terms * 2.0 ** -23 * size).all())
     L.close()
