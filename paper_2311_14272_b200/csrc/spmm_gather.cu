@@ -352,8 +352,11 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 #pragma unroll 1
             for (int i = 0; i < mine + p.ahead; ++i) {
                 if (i >= p.ahead) {
-                    if (!mbar_wait(my_bar + 8 * slot, slot_ph, abort_flag, p.wait_limit) ||
-                        !mbar_wait(bar_empty + 8 * stage, ph ^ 1u, abort_flag, p.wait_limit)) { ok = false; break; }
+                    // (the lanes wait on their own and give up together: those that went on alone would wait in a warp operation
+                    // without a bound for lanes that are in the teardown)
+                    const bool have = mbar_wait(my_bar + 8 * slot, slot_ph, abort_flag, p.wait_limit) &&
+                                      mbar_wait(bar_empty + 8 * stage, ph ^ 1u, abort_flag, p.wait_limit);
+                    if (!__all_sync(0xFFFFFFFFu, have)) { ok = false; break; }
                     const uint32_t src = my_raw + slot * slot_step + lane_src, dst = ring + stage * p.stage_bytes + lane_dst;
 #pragma unroll 1
                     for (int r = 0; r < rows; r += 4) {

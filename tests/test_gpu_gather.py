@@ -104,6 +104,23 @@ def test_a_wait_that_runs_out_is_reported(ncols):
     L.close()
 
 
+@pytest.mark.parametrize("ncols,limit", [(49, 1), (49, 20_000), (9003, 1), (9003, 20_000)])
+def test_warps_that_give_up_at_different_times_leave_together(ncols, limit):
+    """Short limits and a missing weight tile: the lanes of a warp find out one by one that there is nothing to wait for."""
+    torch, L, rng, w, s, x, xv = make(256, 2048, ncols, ncols, 2, 4, 64, 64, 0.5, 0)
+    want = L.spmm(xv)
+    for fill in (0, 1, 2):                              # (a rank of the split walk has three)
+        for _ in range(5):
+            L.set_tuning(0, limit, fill)
+            L.spmm(xv)
+            assert L.device_status() == 6
+            L.reset_status()
+    L.set_tuning()
+    y = L.spmm(xv)
+    assert L.device_status() == 0 and torch.equal(y, want)
+    L.close()
+
+
 def test_products_of_two_threads_on_one_layer():
     """One layer, two host threads with a stream, an input and a row pitch each."""
     import threading
