@@ -54,8 +54,12 @@ struct HaloParams {
     int wo, ho, batch;
     uint32_t a_bytes, entry_bytes, x_bytes, x_stage, x_stages, w_stages;       // (a stage of weights: kGroup entries)
     int resident;
-    uint16_t *y;                         // results whose pixels TMA cannot address (pitch or base not a multiple of 16 bytes), else nullptr
+    uint16_t *y;
     int64_t ldy;
+    // From this channel on (a multiple of 32) results are stored pixel by pixel: all where TMA cannot address the pixels (pitch or base not a
+    // multiple of 16 bytes), the last 32 or fewer where their number is not a multiple of 8: TMA clips at 16 bytes, and what lies
+    // behind the last channel is the caller's.
+    int plain_from;
     unsigned long long wait_limit;
     int skip_fill;                       // test hook: this load of the activation is left out (-1 = none)
 };
@@ -115,7 +119,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_x);
-        if (!p.y) prefetch_tensormap(&map_y);
+        if (p.plain_from > 0) prefetch_tensormap(&map_y);
         for (uint32_t s = 0; s < p.x_stages; ++s) { mbar_init(x_full + 8 * s, 1); mbar_init(x_empty + 8 * s, 1); }
         for (uint32_t s = 0; s < p.w_stages; ++s) { mbar_init(w_full + 8 * s, 1); mbar_init(w_empty + 8 * s, 1); }
         for (int a = 0; a < kAcc; ++a) { mbar_init(t_full + 8 * a, 1); mbar_init(t_empty + 8 * a, kEpiWarps); }
@@ -323,7 +327,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         store_matrices(tile + (uint32_t)(512 * g) + my_row, pack(lo[4 * g], lo[4 * g + 1]), pack(lo[4 * g + 2], lo[4 * g + 3]),
                                        pack(hi[4 * g], hi[4 * g + 1]), pack(hi[4 * g + 2], hi[4 * g + 3]));
                     }
-                    if (p.y) {                               // pixel by pixel, the lanes on consecutive channels
+                    if (ch0 >= p.plain_from) {               // pixel by pixel, the lanes on consecutive channels
                         __syncwarp();
                         const bool ch_ok = ch0 + lane < p.rows;
 #pragma unroll 8
@@ -462,12 +466,13 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     if (p.w_stages > kMaxStages) p.w_stages = kMaxStages;
     if (p.w_stages < 2) return false;
     p.resident = L.nst == 1 && (uint32_t)L.wcap <= p.w_stages * kGroup;
-    if (ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0) { p.y = reinterpret_cast<uint16_t *>(d_y); p.ldy = ldy; }
+    p.y = reinterpret_cast<uint16_t *>(d_y); p.ldy = ldy;
+    p.plain_from = ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0 ? 0 : g.rows % 8 != 0 ? g.rows / 32 * 32 : g.rows;
     plan->smem = fixed + (size_t)p.x_stages * p.x_stage + (size_t)p.w_stages * w_stage;
     plan->grid = (int)(tiles < sms ? tiles : sms);
     if (!make_map_image(&plan->ma, h->d_exec + L.image_off, (uint64_t)L.stack * L.nst * L.wcap * L.entry_bytes, L.entry_bytes) ||
         !make_map_nhwc(&plan->mx, d_x, cv.channels, cv.channels, cv.width, cv.height, cv.batch, 64, p.pw, p.tb, ph) ||
-        (!p.y && !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb)))
+        (p.plain_from > 0 && !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb)))
         return false;
     plan->p = p;
     plan->which = (n == 256 ? 6 : n == 224 ? 4 : n == 128 ? 2 : 0) + (sparse ? 1 : 0);

@@ -56,6 +56,8 @@ struct TcParams {
     int cv_wo, cv_ho, cv_batch; // output width, height, images
     int cv_plain;               // Y rows are not TMA-addressable (wo * element size not a multiple of 16 bytes):
                                 // the epilogue stores element by element
+    int cv_plain_from;          // the same for NHWC results from this channel on (a multiple of 32): the last ones where their
+                                // bytes are not a multiple of 16, all where the pixels are not TMA-addressable
     int cv_tw_log2, cv_img_log2;   // log2(tw), log2(tw * th)
     int cv_nhwc;                // Y is [batch, ho, wo, ldy] (output channel fastest): the next convolution's activation
     // Thin layers (one CTA tile, at most 128 / stack rows; matrix mode): a tile covers `stack` column tiles, one per
@@ -208,9 +210,9 @@ __device__ __forceinline__ void store_chunk(const TcParams &p, const CUtensorMap
 // One epilogue chunk of a convolution whose output is NHWC: the lane holds one output channel (row y0 + lane) of
 // kOutCols pixels, memory wants the 32 channels of a pixel side by side.  The chunk is transposed through the
 // warp's staging tile, [pixel][32 channels] (64 or 128 bytes per pixel, 4096 bytes per chunk), and goes out
-// as one 4-D bulk tensor store of {32 channels, tw, pixels / tw, 1} (it clips channels beyond `rows` and pixels
-// outside the images), or, where the pixel pitch is not a multiple of 16 bytes, pixel by pixel with the 32
-// lanes on consecutive channels.  `out` is packed as in store_chunk (bf16: pixels 2i, 2i+1 in word i).
+// as one 4-D bulk tensor store of {32 channels, tw, pixels / tw, 1} (it clips pixels outside the images, and channels
+// beyond `rows` at 16 bytes), or, where the pixel pitch or the end of the channels is not a multiple of 16 bytes, pixel by
+// pixel with the 32 lanes on consecutive channels.  `out` is packed as in store_chunk (bf16: pixels 2i, 2i+1 in word i).
 // With 2048-byte staging tiles (bf16) it goes in two passes of 32 pixels.
 template <typename OutT>
 __device__ __forceinline__ void store_chunk_nhwc(const TcParams &p, const CUtensorMap *map_y, uint32_t stg, uint8_t *stg_gen,
@@ -218,7 +220,7 @@ __device__ __forceinline__ void store_chunk_nhwc(const TcParams &p, const CUtens
     constexpr int kOutCols = 128 / (int)sizeof(OutT);
     constexpr int kRowBytes = 32 * (int)sizeof(OutT);           // one pixel: 32 channels
     if (y0 >= p.rows) return;
-    if (!p.cv_plain) {
+    if (y0 < p.cv_plain_from) {
         const bool halves = sizeof(OutT) == 2 && p.stg_tile_bytes == 2048;
         const int per_image = p.cv_tw * p.cv_th;
 #pragma unroll
@@ -249,6 +251,7 @@ __device__ __forceinline__ void store_chunk_nhwc(const TcParams &p, const CUtens
         }
         return;
     }
+    if (lane == 0) bulk_wait_read<0>();                         // (the warp may have stored whole channels of another tile in bulk)
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
@@ -1153,7 +1156,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     // transposed chunks of NHWC output: 64 pixels x 32 channels of bf16 in one 4096-byte staging tile, or, where the ring
     // needs the room (resident weights), 32 pixels at a time; a chunk stored pixel by pixel goes through a whole tile
     const bool nhwc = conv && conv->nhwc_out;
-    const uint32_t nhwc_tile = resident && y_dtype == 0 && (ldy * 2) % 16 == 0 && reinterpret_cast<uintptr_t>(d_y) % 16 == 0
+    const uint32_t nhwc_tile = resident && y_dtype == 0 && (ldy * 2) % 16 == 0 && g.rows % 8 == 0 && reinterpret_cast<uintptr_t>(d_y) % 16 == 0
                                    ? kWideStageBytes : 2 * kWideStageBytes;
     const uint32_t fixed = epi * (nhwc ? nhwc_tile : kWideStageBytes) + 256;
     // Blocks per pipeline stage.  A stage costs each single-thread role (weight producer, X producer, MMA issuer)
@@ -1203,6 +1206,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
         p.cv_nhwc = conv->nhwc_out;
         p.cv_plain = (!p.cv_nhwc && ((int64_t)conv->wo * (f32 ? 4 : 2)) % 16 != 0) || (ldy * (f32 ? 4 : 2)) % 16 != 0 ||
                      reinterpret_cast<uintptr_t>(d_y) % 16 != 0;
+        p.cv_plain_from = p.cv_plain ? 0 : g.rows * (f32 ? 4 : 2) % 16 != 0 ? g.rows / 32 * 32 : g.rows;
         for (p.cv_tw_log2 = 0; (1 << p.cv_tw_log2) < p.cv_tw; ++p.cv_tw_log2) {}
         for (p.cv_img_log2 = 0; (1 << p.cv_img_log2) < p.cv_tw * p.cv_th; ++p.cv_img_log2) {}
         // activation [batch][height][width][channels] and Y [rows][batch][ho][wo] as 4-D tensors

@@ -73,6 +73,30 @@ def test_convolution(s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile, stay)
     L.close()
 
 
+@pytest.mark.parametrize("y_dtype", [0, 1])
+@pytest.mark.parametrize("s_out,ldy,b,h,w", [
+    (100, 104, 20, 28, 28), (100, 128, 1, 28, 28), (235, 240, 6, 7, 7), (45, 48, 4, 56, 56), (45, 48, 1, 14, 14), (45, 48, 40, 112, 112),
+    (30, 32, 3, 56, 56), (130, 144, 9, 28, 28), (67, 68, 2, 19, 21), (96, 104, 5, 28, 28),
+])
+def test_what_lies_behind_the_channels_of_a_pixel_stays(s_out, ldy, b, h, w, y_dtype):
+    """Pixels further apart than their channels, in both convolution kernels (fp32 results leave by the older one)."""
+    torch, B, L, wt, sal, act, bias = layer_and_input(s_out, 3, 3, 64, b, h, w, 2, 4, 32, 0.6, s_out + h)
+    x = bf16_dev(act, torch)
+    buf = torch.full((b, h, w, ldy), 7.0, dtype=torch.float32 if y_dtype else torch.bfloat16, device="cuda")
+    terms = 5 * 64 * 2 // 4 + 1                                 # five of nine blocks, and the bias
+    mag = terms * max(1.0, float(x.abs().max())) * float(bf16_dev(wt, torch).abs().max()) + float(np.abs(bias).max())
+    for stage_blocks in (0, 1):                                 # (a bound on the blocks of a stage: the older kernel)
+        buf.fill_(7.0)
+        L.set_stage_blocks(stage_blocks)
+        L.spmm_conv(x, 3, 3, 1, y=buf[..., :s_out], y_dtype=y_dtype, nhwc_out=True)
+        torch.cuda.synchronize()
+        assert L.device_status() == 0 and bool((buf[..., s_out:] == 7.0).all())
+        other = L.spmm_conv(x, 3, 3, 1, y_dtype=1).t().reshape(b, h, w, s_out)
+        order = 2 * terms * 2.0 ** -23 * mag                    # two orders of an fp32 sum
+        assert bool(((buf[..., :s_out].float() - other).abs() <= (0.0 if y_dtype else 2.0 ** -8) * other.abs() + order).all())
+    L.close()
+
+
 def test_a_wait_that_runs_out_is_reported():
     torch, B, L, wt, sal, act, bias = layer_and_input(64, 3, 3, 64, 20, 84, 80, 2, 4, 64, 0.4, 3)
     x = bf16_dev(act, torch)
