@@ -288,12 +288,13 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         // lane l writes pixel l % 8 of a group, channels 8 (l / 8) ..: 16-byte chunk c of pixel row r lies at c ^ (r / 2 % 4)
         const uint32_t my_row = (uint32_t)((lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4));
         uint32_t acc = 0, acc_ph = 0;
-        const float floor_v = p.relu ? 0.f : -__int_as_float(0x7f800000);
+        const float floor_v = p.relu ? 0.f : __int_as_float(0x7FFFFFFF);     // max(v, NaN) is v, whatever v is: a NaN stays
         const bool fuse = p.bias != nullptr || p.relu != 0;
         for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
             const int ct = t / p.nst, st = t - ct * p.nst;
             const Tile org = tile_at(p, ct);
             const int ch0 = st * kTileM + 32 * q;
+            const bool plain = ch0 >= p.plain_from;
             float bias[4];                                   // of channels l / 4, + 8, + 16, + 24
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -327,7 +328,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         store_matrices(tile + (uint32_t)(512 * g) + my_row, pack(lo[4 * g], lo[4 * g + 1]), pack(lo[4 * g + 2], lo[4 * g + 3]),
                                        pack(hi[4 * g], hi[4 * g + 1]), pack(hi[4 * g + 2], hi[4 * g + 3]));
                     }
-                    if (ch0 >= p.plain_from) {               // pixel by pixel, the lanes on consecutive channels
+                    if (plain) {                             // pixel by pixel, the lanes on consecutive channels
                         __syncwarp();
                         const bool ch_ok = ch0 + lane < p.rows;
 #pragma unroll 8

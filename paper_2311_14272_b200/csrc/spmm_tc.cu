@@ -750,7 +750,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             // layer epilogue on the fp32 accumulator: this lane's row gets its bias, then the activation
             const bool fuse = p.bias != nullptr || p.relu != 0;
             const float bias_v = (p.bias != nullptr && y0 + lane < p.rows) ? p.bias[y0 + lane] : 0.f;
-            const float floor_v = p.relu ? 0.f : -__int_as_float(0x7f800000);
+            const float floor_v = p.relu ? 0.f : __int_as_float(0x7FFFFFFF);     // max(v, NaN) is v, whatever v is: a NaN stays
             if (y0 >= p.rows) {
                 // this lane quarter lies below the last row of W: nothing to drain
                 tc_fence_before();

@@ -121,3 +121,37 @@ def test_two_pointwise_layers_chain_through_bf16(env):
     y1_bits = y1.contiguous().view(torch.int16).cpu().numpy().view(np.uint16)      # what layer 2 actually read
     check_tolerance(y_to_f64(y2, torch), oracle.bias_relu(oracle.spmm_fp64(wd2, y1_bits), b2, False))
     L1.close(); L2.close()
+
+
+@pytest.mark.parametrize("use_bias,relu", [(True, False), (False, False), (True, True)])
+@pytest.mark.parametrize("kind", ["aligned", "aligned fp32", "dense tiles", "short walk", "thin", "odd pitch", "odd pitch fp32", "CUDA cores",
+                                  "shared taps", "conv", "conv fp32", "conv of one tap a load"])
+def test_a_sum_that_is_not_a_number_stays_one(env, kind, use_bias, relu):
+    """A column of NaN under every kernel: with a bias alone the result is NaN (not the lowest value), under ReLU it is 0."""
+    B, torch = env
+    f32 = "fp32" in kind
+    conv = kind.startswith("conv") or kind == "shared taps"
+    rows, k = (32, 64) if kind == "thin" else (128, 576) if conv else (256, 96 if kind == "short walk" else 512)
+    rng = np.random.default_rng(rows + k)
+    w = wl.f32_to_bf16_bits(rng.standard_normal((rows, k)).astype(np.float32))
+    L = gpu_layer(B, torch, w, np.abs(wl.bf16_bits_to_f32(w)) + 1e-3, 4 if kind == "dense tiles" else 2, 4, 32, 32 if kind == "short walk" else 64, 1.0)
+    L.set_epilogue(torch.ones(rows, device="cuda") if use_bias else None, relu)
+    if conv:
+        x = torch.ones(20, 28, 28, 64, dtype=torch.bfloat16, device="cuda")
+        x[0, 4:7, 4:7] = float("nan")                        # all that pixel (5, 5) sees
+        if kind == "conv of one tap a load":
+            L.set_stage_blocks(1)
+        y = L.spmm_conv(x, 3, 3, 1, nhwc_out=kind != "conv", y_dtype=int(f32))
+        got, clean = (y[:, 5 * 28 + 5], y[:, 15 * 28 + 15]) if kind == "conv" else (y[0, 5, 5], y[0, 15, 15])
+    else:
+        if kind == "CUDA cores":
+            L.set_path(B.PATH_DIRECT)
+        n = 400000 if kind == "thin" else 1023 if "odd" in kind else 1024
+        x = torch.ones(k, n, dtype=torch.bfloat16, device="cuda")
+        x[:, 5] = float("nan")
+        y = L.spmm(x, y_dtype=int(f32))
+        got, clean = y[:, 5], y[:, 6]
+    torch.cuda.synchronize()
+    assert L.device_status() == 0 and bool(torch.isfinite(clean).all())
+    assert bool((got == 0).all()) if relu else bool(torch.isnan(got).all())
+    L.close()
