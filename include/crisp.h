@@ -369,6 +369,8 @@ CRISP_API crisp_status_t crisp_decode(crisp_handle_t h, uint16_t *d_w_dense_bf16
  * Rows of X under blocks that no row tile kept are never read.  A layer with kkeep = 0
  * yields Y = 0.  The tensor-core kernels need X and Y 16-byte aligned with ldx*2 and
  * ldy*sizeof(element) multiples of 16; other layouts run on CRISP_PATH_DIRECT.
+ * Products and convolutions of one handle may be issued by several host threads; a handle's settings (crisp_set_*) are
+ * changed, and it is destroyed, only while none of them is in such a call.
  */
 CRISP_API crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ldx,
                                     int64_t ncols, void *d_y, int64_t ldy, int32_t y_dtype, void *stream);

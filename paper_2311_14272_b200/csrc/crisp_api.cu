@@ -431,7 +431,7 @@ crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ld
     } else if (path == CRISP_PATH_DIRECT) {
         e = crisp::launch_spmm_direct(h->g, h->d_blk_col, h->d_vals, h->d_idx, d_x_bf16, ldx, ncols,
                                       d_y, ldy, y_dtype, h->epilogue, (cudaStream_t)stream);
-        if (e == cudaSuccess) { h->last = crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0}; h->last_resident = 0; }
+        if (e == cudaSuccess) crisp::note_launch(h, crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0}, 0);
     } else {
         e = crisp::launch_spmm_tc(h, path, d_x_bf16, ldx, ncols, d_y, ldy, y_dtype, nullptr,
                                   (cudaStream_t)stream);
@@ -469,12 +469,14 @@ crisp_status_t crisp_spmm_conv(crisp_handle_t h, const uint16_t *d_act_nhwc, con
 
 crisp_status_t crisp_last_launch(crisp_handle_t h, crisp_launch_info_t *out) {
     if (!h || !out) return CRISP_INVALID_ARG;
+    std::lock_guard<std::mutex> hold(h->plan_lock);
     *out = h->last;
     return CRISP_OK;
 }
 
 crisp_status_t crisp_last_resident_bytes(crisp_handle_t h, int64_t *bytes) {
     if (!h || !bytes) return CRISP_INVALID_ARG;
+    std::lock_guard<std::mutex> hold(h->plan_lock);
     *bytes = h->last_resident;
     return CRISP_OK;
 }

@@ -166,7 +166,9 @@ struct crisp_handle_s {
     crisp::TcPlan *plan;    // cached launch plan of the last tensor-core product (or nullptr)
     crisp::HaloPlan *halo;                  // cached launch plan of the last convolution that shares loads among taps (or nullptr)
     crisp::GatherPlan *gather;              // made by the first product on a layout TMA cannot address (or nullptr)
-    std::mutex gather_lock;                 // such products may come from several threads at a time
+    // Products and convolutions of one handle may come from several host threads: the three plans above and what follows are read and
+    // written under this lock, and a launch is made from copies.
+    std::mutex plan_lock;
     crisp_launch_info_t last;               // what the last product on this handle launched
     int64_t last_resident;                  // and the bytes of weight tiles it kept in shared memory
 };
@@ -250,6 +252,7 @@ int64_t conv_box(int n, int row, const ConvGeom &cv, int *tw, int *th, int *tb);
 // spmm_halo.cu: convolutions whose taps share one load of the activation
 cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
                              cudaStream_t st, bool *done);
+void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes);          // for crisp_last_launch
 // conv == nullptr: d_x is the [k, ncols] matrix.  Otherwise d_x is the activation and ncols = batch*ho*wo.
 // `h->plan` is reused when the operands, shape and epilogue are those of the previous call; `h->last` is filled in.
 cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols,

@@ -599,7 +599,7 @@ cudaError_t launch_spmm_gather(crisp_handle_s *h, const uint16_t *d_x, int64_t l
     CUtensorMap image;
     RowMaps rows;
     {
-        std::lock_guard<std::mutex> hold(h->gather_lock);
+        std::lock_guard<std::mutex> hold(h->plan_lock);
         if (!h->gather) {
             e = ensure_context(device);
             if (e != cudaSuccess) return e;
@@ -669,10 +669,7 @@ cudaError_t launch_spmm_gather(crisp_handle_s *h, const uint16_t *d_x, int64_t l
     }
     const int grid = p.split > 1 ? p.num_tiles * p.split : (p.num_tiles < sms ? p.num_tiles : sms);
     e = launch_clusters(kern, (unsigned)grid, (unsigned)kThreads, smem, st, (unsigned)p.split, image, rows, p);
-    if (e == cudaSuccess) {
-        h->last = crisp_launch_info_t{CRISP_PATH_DIRECT, kCols, 2, 1, kEpiWarps, (int)stages, grid, 0, 1};
-        h->last_resident = 0;
-    }
+    if (e == cudaSuccess) note_launch(h, crisp_launch_info_t{CRISP_PATH_DIRECT, kCols, 2, 1, kEpiWarps, (int)stages, grid, 0, 1}, 0);
     return e;
 }
 

@@ -375,12 +375,8 @@ typedef void (*HaloKernel)(const CUtensorMap, const CUtensorMap, const CUtensorM
 
 }  // namespace
 
-// Launch plan: tensor maps and tile shape for one set of operands.
-struct HaloPlan {
-    const void *x, *y;
-    int64_t ldy;
-    ConvGeom conv;
-    int device;
+// What a launch takes.
+struct HaloLaunch {
     CUtensorMap mx, my, ma;
     HaloParams p;
     HaloKernel kern;
@@ -388,6 +384,14 @@ struct HaloPlan {
     size_t smem;
     crisp_launch_info_t info;
     int64_t resident_bytes;
+};
+// Launch plan: tensor maps and tile shape for one set of operands.
+struct HaloPlan {
+    const void *x, *y;
+    int64_t ldy;
+    ConvGeom conv;
+    int device;
+    HaloLaunch launch;
 };
 void halo_plan_destroy(HaloPlan *plan) { delete plan; }
 
@@ -403,7 +407,7 @@ bool make_map_nhwc(CUtensorMap *map, const void *base, uint64_t c, uint64_t pitc
 
 // Whether this convolution goes through the kernel above, and its plan if so.
 bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
-               HaloPlan *plan) {
+               HaloLaunch *plan) {
     const Geometry &g = h->g;
     if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return false;
     if (h->exec_kind != CRISP_PATH_SPARSE && h->exec_kind != CRISP_PATH_DENSE) return false;
@@ -492,36 +496,41 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
 cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
                              cudaStream_t st, bool *done) {
     *done = false;
-    HaloPlan *plan = h->halo;
-    const bool hit = plan && plan->x == d_x && plan->y == d_y && plan->ldy == ldy && plan->device == device && same_conv(plan->conv, cv) &&
-                     y_dtype == 0 && h->nt_override <= 0 && h->group_override <= 0;
-    if (!hit) {
-        HaloPlan fresh = {};
-        if (!plan_halo(h, d_x, d_y, ldy, y_dtype, cv, device, &fresh)) return cudaSuccess;
-        fresh.x = d_x; fresh.y = d_y; fresh.ldy = ldy; fresh.conv = cv; fresh.device = device;
-        if (!plan) {
-            plan = new (std::nothrow) HaloPlan;
-            if (!plan) return cudaErrorMemoryAllocation;
-            h->halo = plan;
+    HaloLaunch launch;
+    {
+        std::lock_guard<std::mutex> hold(h->plan_lock);
+        HaloPlan *plan = h->halo;
+        const bool hit = plan && plan->x == d_x && plan->y == d_y && plan->ldy == ldy && plan->device == device && same_conv(plan->conv, cv) &&
+                         y_dtype == 0 && h->nt_override <= 0 && h->group_override <= 0;
+        if (!hit) {
+            HaloPlan fresh = {};
+            if (!plan_halo(h, d_x, d_y, ldy, y_dtype, cv, device, &fresh.launch)) return cudaSuccess;
+            fresh.x = d_x; fresh.y = d_y; fresh.ldy = ldy; fresh.conv = cv; fresh.device = device;
+            if (!plan) {
+                plan = new (std::nothrow) HaloPlan;
+                if (!plan) return cudaErrorMemoryAllocation;
+                h->halo = plan;
+            }
+            *plan = fresh;
         }
-        *plan = fresh;
+        launch = plan->launch;
     }
     *done = true;
     static std::atomic<bool> configured[8][64];
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
-    if (!configured[plan->which][device].load(std::memory_order_relaxed)) {
+    if (!configured[launch.which][device].load(std::memory_order_relaxed)) {
         // the most there is, once: the limit belongs to the function, not to a call
-        const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(plan->kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(launch.kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)kSmemBudget + 1024);
         if (e != cudaSuccess) return e;
-        configured[plan->which][device].store(true, std::memory_order_relaxed);
+        configured[launch.which][device].store(true, std::memory_order_relaxed);
     }
-    HaloParams &p = plan->p;
+    HaloParams &p = launch.p;
     p.bias = h->epilogue.bias; p.relu = h->epilogue.relu;
     p.wait_limit = h->wait_limit_cycles ? h->wait_limit_cycles : kWaitLimitCycles;
     p.skip_fill = h->debug_skip_stage;
-    const cudaError_t e = launch_chained(plan->kern, (unsigned)plan->grid, (unsigned)kThreads, plan->smem, st, plan->mx, plan->my, plan->ma, p);
-    if (e == cudaSuccess) { h->last = plan->info; h->last_resident = plan->resident_bytes; }
+    const cudaError_t e = launch_chained(launch.kern, (unsigned)launch.grid, (unsigned)kThreads, launch.smem, st, launch.mx, launch.my, launch.ma, p);
+    if (e == cudaSuccess) note_launch(h, launch.info, launch.resident_bytes);
     return e;
 }
 

@@ -1031,7 +1031,17 @@ bool tc_operands_ok(const void *x, int64_t ldx, const void *y, int64_t ldy, int 
            (ldx * 2) % 16 == 0 && (ldy * ye) % 16 == 0 && ncols < (1ll << 31) && encode_tiled_fn() != nullptr;
 }
 
-// Everything one launch needs, and the operands it was planned for.  Encoding three tensor maps costs a few
+// Everything one launch needs.
+struct TcLaunch {
+    CUtensorMap mx, my, ma;
+    TcParams p;
+    TcVariant variant;
+    int grid;
+    size_t smem;
+    crisp_launch_info_t info;
+};
+
+// A launch and the operands it was planned for.  Encoding three tensor maps costs a few
 // microseconds of host time per call, which small layers notice; a product on the same buffers reuses the plan.
 struct TcPlan {
     // key
@@ -1041,16 +1051,16 @@ struct TcPlan {
     unsigned long long wait_limit;
     bool has_conv;
     ConvGeom conv;
-    // plan
-    CUtensorMap mx, my, ma;
-    TcParams p;
-    TcVariant variant;
-    int grid;
-    size_t smem;
-    crisp_launch_info_t info;
+    TcLaunch launch;
 };
 
 void tc_plan_destroy(TcPlan *plan) { delete plan; }
+
+void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes) {
+    std::lock_guard<std::mutex> hold(h->plan_lock);
+    h->last = info;
+    h->last_resident = resident_bytes;
+}
 
 int64_t conv_box(int n, int row, const ConvGeom &cv, int *tw, int *th, int *tb) {
     int64_t best = -1;
@@ -1068,7 +1078,7 @@ namespace {
 
 // Tile shape, shared-memory split, tensor maps and kernel variant for one product.
 cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols, void *d_y,
-                      int64_t ldy, int y_dtype, const ConvGeom *conv, int device, TcPlan *plan) {
+                      int64_t ldy, int y_dtype, const ConvGeom *conv, int device, TcLaunch *plan) {
     const Geometry &g = h->g;
     const uint8_t *d_exec = h->d_exec;
     const int nt_override = h->nt_override;
@@ -1304,37 +1314,42 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
         if (e == cudaSuccess) e = launch_spmm_halo(h, d_x, d_y, ldy, y_dtype, *conv, device, st, &done);
         if (done || e != cudaSuccess) return e;
     }
-    TcPlan *plan = h->plan;
-    const bool hit = plan && plan->x == d_x && plan->y == d_y && plan->ldx == ldx && plan->ldy == ldy &&
-                     plan->ncols == ncols && plan->y_dtype == y_dtype && plan->bias == h->epilogue.bias &&
-                     plan->relu == h->epilogue.relu && plan->nt_override == h->nt_override &&
-                     plan->group_override == h->group_override &&
-                     plan->device == device && plan->skip_stage == h->debug_skip_stage &&
-                     plan->wait_limit == h->wait_limit_cycles && plan->has_conv == (conv != nullptr) &&
-                     (!conv || same_conv(plan->conv, *conv)) && plan->p.status == h->d_status &&
-                     plan->info.path == kind;
-    if (!hit) {
-        if (!plan) {
-            plan = new (std::nothrow) TcPlan;
-            if (!plan) return cudaErrorMemoryAllocation;
-            h->plan = plan;
+    TcLaunch launch;
+    {
+        std::lock_guard<std::mutex> hold(h->plan_lock);
+        TcPlan *plan = h->plan;
+        const bool hit = plan && plan->x == d_x && plan->y == d_y && plan->ldx == ldx && plan->ldy == ldy &&
+                         plan->ncols == ncols && plan->y_dtype == y_dtype && plan->bias == h->epilogue.bias &&
+                         plan->relu == h->epilogue.relu && plan->nt_override == h->nt_override &&
+                         plan->group_override == h->group_override &&
+                         plan->device == device && plan->skip_stage == h->debug_skip_stage &&
+                         plan->wait_limit == h->wait_limit_cycles && plan->has_conv == (conv != nullptr) &&
+                         (!conv || same_conv(plan->conv, *conv)) && plan->launch.p.status == h->d_status &&
+                         plan->launch.info.path == kind;
+        if (!hit) {
+            if (!plan) {
+                plan = new (std::nothrow) TcPlan;
+                if (!plan) return cudaErrorMemoryAllocation;
+                h->plan = plan;
+            }
+            plan->x = nullptr;                                  // not valid until the plan below is complete
+            e = ensure_context(device);
+            if (e != cudaSuccess) return e;
+            e = make_plan(h, kind, d_x, ldx, ncols, d_y, ldy, y_dtype, conv, device, &plan->launch);
+            if (e != cudaSuccess) return e;
+            plan->x = d_x; plan->y = d_y; plan->bias = h->epilogue.bias;
+            plan->ldx = ldx; plan->ldy = ldy; plan->ncols = ncols;
+            plan->y_dtype = y_dtype; plan->relu = h->epilogue.relu; plan->nt_override = h->nt_override;
+            plan->group_override = h->group_override;
+            plan->device = device; plan->skip_stage = h->debug_skip_stage; plan->wait_limit = h->wait_limit_cycles;
+            plan->has_conv = conv != nullptr;
+            if (conv) plan->conv = *conv;
         }
-        plan->x = nullptr;                                  // not valid until the plan below is complete
-        e = ensure_context(device);
-        if (e != cudaSuccess) return e;
-        e = make_plan(h, kind, d_x, ldx, ncols, d_y, ldy, y_dtype, conv, device, plan);
-        if (e != cudaSuccess) return e;
-        plan->x = d_x; plan->y = d_y; plan->bias = h->epilogue.bias;
-        plan->ldx = ldx; plan->ldy = ldy; plan->ncols = ncols;
-        plan->y_dtype = y_dtype; plan->relu = h->epilogue.relu; plan->nt_override = h->nt_override;
-        plan->group_override = h->group_override;
-        plan->device = device; plan->skip_stage = h->debug_skip_stage; plan->wait_limit = h->wait_limit_cycles;
-        plan->has_conv = conv != nullptr;
-        if (conv) plan->conv = *conv;
+        launch = plan->launch;
     }
-    e = launch_chained(plan->variant.kern, (unsigned)plan->grid, (unsigned)plan->variant.threads, plan->smem, st, plan->mx, plan->my,
-                       plan->ma, plan->p);
-    if (e == cudaSuccess) { h->last = plan->info; h->last_resident = plan->p.resident_bytes; }
+    e = launch_chained(launch.variant.kern, (unsigned)launch.grid, (unsigned)launch.variant.threads, launch.smem, st, launch.mx, launch.my,
+                       launch.ma, launch.p);
+    if (e == cudaSuccess) note_launch(h, launch.info, launch.p.resident_bytes);
     return e;
 }
 

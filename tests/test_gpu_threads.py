@@ -134,3 +134,36 @@ def test_first_call_of_a_host_thread():
         assert errors == []
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     L.close()
+
+
+@pytest.mark.parametrize("kind", ["shared taps", "one tap a load", "matrix", "matrix fp32", "all in turn"])
+def test_one_layer_from_two_threads(kind):
+    """Two threads with a stream, an input and a result each on one layer, whose plans for the last operands they take from each other."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    L = make_layer(B, torch, 128, 64 * 9, 2, 4, 64, 64, 0.5, 5)
+    acts = [torch.randn(20, 28, 28, 64, device="cuda").bfloat16(), torch.randn(24, 14, 14, 64, device="cuda").bfloat16()]
+    xs = [torch.randn(64 * 9, 4096, device="cuda").bfloat16(), torch.randn(64 * 9, 520, device="cuda").bfloat16()]
+    calls = {
+        "shared taps": lambda i, y: L.spmm_conv(acts[i], 3, 3, 1, y=y, nhwc_out=True),
+        "one tap a load": lambda i, y: L.spmm_conv(acts[i], 3, 3, 1, y=y),
+        "matrix": lambda i, y: L.spmm(xs[i], y=y),
+        "matrix fp32": lambda i, y: L.spmm(xs[i], y=y, y_dtype=1),
+    }
+    names = list(calls)[:3] if kind == "all in turn" else [kind]
+    wants = [[calls[n](i, None) for n in names] for i in range(2)]
+    if kind == "shared taps":
+        assert L.last_launch()["epilogue_warps"] == 16 and L.last_launch()["conv"] == 1
+    gots = [[torch.zeros_like(w) for w in ws] for ws in wants]
+    torch.cuda.synchronize()
+
+    def job(i):
+        for n, y in zip(names, gots[i]):
+            calls[n](i, y)
+    assert run_together(torch, [lambda: job(0), lambda: job(1)], 500) == []
+    assert L.device_status() == 0
+    for ws, gs in zip(wants, gots):
+        for w, g in zip(ws, gs):
+            assert torch.equal(w, g)
+    L.close()
