@@ -443,6 +443,19 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     const int64_t gather = conv_box(256, 64, cv, &bw, &bh, &bb) / 256;
     const bool narrow = 2 * gather * L.nst < sms;            // (the gather's tiles are half as wide then)
     if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 2500) return false;
+    // Where an entry's cost decides, the estimates above are too low: with every SM at work an entry of 128, 224 and 256 pixels takes some
+    // 410, 560 and 520 cycles, and what a tile costs besides is 1500 less than in the gather.  (us, gather and this kernel, 2 waves of
+    // tiles there and 3 here: 512 -> 448 channels, 55 x 57 x 5, 72 entries 51.2 and 59.7; 256 -> 256, 112 x 112 x 3, 24 entries 21.0 and 23.4;
+    // one and two: 128 -> 128, 28 x 28 x 40, 18 entries 11.4 and 13.4.  On the other side: 4 and 5 waves, 256 -> 256, 12 entries and more 1.08 times
+    // faster here in the median; as many waves on both sides 1.2 times.)  Walks of up to four blocks in one wave of 128-pixel tiles gain nothing that
+    // the set-up does not cost: 64 -> 448, 1x1, 28 x 28 x 4 5.0 and 5.4.
+    // (Channels that are no multiple of 8 leave the gather element by element, 1.2 to 1.6 times slower on all of these.)
+    if (g.rows % 8 == 0 && narrow) {
+        if (n == 128 && L.wcap <= 4) return false;
+    } else if (g.rows % 8 == 0) {
+        const int busy = n == 128 || n == 64 ? 410 : n == 224 ? 560 : 520, entry = sparse || busy > n + 256 ? busy : n + 256;
+        if ((tiles + sms - 1) / sms * (L.wcap * entry + 1000) > waves(gather) * (L.wcap * 700 + 2500)) return false;
+    }
     // One CTA tile of rows and a walk of up to eight blocks: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images
     // of 112 x 112 10.5 and 8.8, 3.4 tiles a CTA; 6 images 9.2 and 8.5; 3 images 6.8 each; one image of 56 x 56 5.5 and 5.9.  Below the line stays the gather with
     // resident weight tiles, whose form its tests and crisp_last_resident_bytes' callers look for.)

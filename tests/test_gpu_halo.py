@@ -73,6 +73,26 @@ def test_convolution(s_out, kh, kw, pad, c, b, h, w, n, m, bm, keep, tile, stay)
     L.close()
 
 
+@pytest.mark.parametrize("s_out,kh,c,b,h,w,n,m,bm,keep", [
+    (384, 3, 512, 1, 112, 112, 1, 4, 64, 0.69),      # two waves of tiles here, one in the kernel that loads the pixels of each tap
+    (128, 3, 128, 40, 28, 28, 1, 4, 64, 0.59),
+    (448, 3, 512, 5, 55, 57, 2, 8, 64, 0.9),         # three and two
+    (448, 1, 64, 4, 28, 28, 2, 8, 128, 1.0),         # one wave, one block
+])
+def test_convolutions_that_sharing_loads_would_slow_down(s_out, kh, c, b, h, w, n, m, bm, keep):
+    torch, B, L, wt, sal, act, bias = layer_and_input(s_out, kh, kh, c, b, h, w, n, m, bm, keep, 1)
+    x = bf16_dev(act, torch)
+    y = L.spmm_conv(x, kh, kh, kh // 2, nhwc_out=True)
+    taken = L.last_launch()
+    L.set_stage_blocks(1)                                       # (one tap a load)
+    other = L.spmm_conv(x, kh, kh, kh // 2, nhwc_out=True)
+    torch.cuda.synchronize()
+    forced = L.last_launch()
+    assert all(taken[f] == forced[f] for f in ("tile_cols", "epilogue_warps", "accumulators", "ctas"))
+    assert L.device_status() == 0 and torch.equal(y, other)
+    L.close()
+
+
 @pytest.mark.parametrize("y_dtype", [0, 1])
 @pytest.mark.parametrize("s_out,ldy,b,h,w", [
     (100, 104, 20, 28, 28), (100, 128, 1, 28, 28), (235, 240, 6, 7, 7), (45, 48, 4, 56, 56), (45, 48, 1, 14, 14), (45, 48, 40, 112, 112),
