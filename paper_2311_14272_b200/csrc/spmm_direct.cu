@@ -17,8 +17,8 @@
 // keep 0.25: 508 -> 51 us (38 M warp instructions, 76 % of the issue slots of busy SMs); 160 x 960 x 49, 2:8, keep 0.5:
 // 147 -> 16.4 us, a chain of four stages on 20 CTAs.  One warp per row that gathers its activations from L2 without
 // staging took 13-22 us on the second and 65 us on the first; staging through registers with two buffers 70 us.
-// The next kernel's launch overlaps this one: products in a row, us, 16 x 32 x 49 5.4 -> 4.5, 216 x 106 x 245 7.7 -> 5.8, 64 x 64 x 6076 fp32
-// 12.3 -> 10.0; a product of 93 us keeps its time.
+// The next kernel's launch overlaps the end of this one: products in a row, us, without and with it, 216 x 106 x 245 6.2 and 4.0, 64 x 64 x 6076 fp32
+// 14.4 and 11.4, 3554 x 199 x 3332 fp32 178 and 175.
 #include <cuda_bf16.h>
 
 #include "crisp_internal.h"
@@ -102,7 +102,7 @@ spmm_direct_kernel(Geometry g, const int32_t *blk_col, const uint16_t *vals, con
     const uint32_t s_words = s_x + T::kStages * stage_bytes;                                 // [kRows][group * vpp] weight words
     const int32_t *s_col = reinterpret_cast<const int32_t *>(s_raw + T::kStages * stage_bytes + kRows * group * vpp * 4);   // [kkeep]
 
-    chain_kernels();                                         // (behind it nothing is read through the read-only path)
+    wait_for_prerequisites();                                // (behind it nothing is read through the read-only path)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slabs = g.bm / kRows;                          // CTAs that share a row tile
     const int64_t ct = blockIdx.x / (g.nrt * slabs);         // row slabs fastest: they share X
@@ -247,6 +247,9 @@ spmm_direct_kernel(Geometry g, const int32_t *blk_col, const uint16_t *vals, con
         __syncwarp();                                        // the warp's weight words may be overwritten
     }
     wait_copies<0>();
+    // The next kernel may begin now.  Asked for at the start, its CTAs wait beside this one's on some SMs and leave others empty: 47 x 1048 x 196
+    // fp32 37.5 us in a row instead of 29.7 (32.5 without overlap), 1783 x 107 x 7 14.9 instead of 12.2 (14.4).
+    launch_dependents();
 
 #pragma unroll
     for (int r = 0; r < RW; ++r) {

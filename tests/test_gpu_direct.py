@@ -83,3 +83,36 @@ def test_products_of_falling_size_in_one_graph():
     for L, y, ref in zip(layers, ys, refs):
         assert int((ref != 0).sum()) > 0 and torch.equal(y, ref)
         L.close()
+
+
+def test_products_that_read_each_others_results():
+    """A chain of products in a row, each reading what the one before wrote; the launches overlap."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    rng = np.random.default_rng(5)
+    rows = 96
+    layers = []
+    for n, bk in ((2, 32), (3, 96), (1, 64)):                   # whole blocks, blocks in parts
+        w = wl.f32_to_bf16_bits((rng.standard_normal((rows, rows)) / 4).astype(np.float32))
+        layers.append(gpu_layer(B, torch, w, np.abs(wl.bf16_bits_to_f32(w)) + 1e-3, n, 4, 32, bk, 1.0))
+        layers[-1].set_path(B.PATH_DIRECT)
+    for ncols in (1, 49, 3001):
+        xs = [torch.randn(rows, ncols, device="cuda").bfloat16() for _ in range(20)]
+        wants, gots = [], []
+        for x in xs:                                            # one at a time
+            for L in layers:
+                x = L.spmm(x)
+                torch.cuda.synchronize()
+            wants.append(x)
+        bufs = [torch.zeros(rows, ncols, dtype=torch.bfloat16, device="cuda") for _ in layers]
+        for x in xs:                                            # all in a row, through the same buffers
+            for L, y in zip(layers, bufs):
+                x = L.spmm(x, y=y)
+            gots.append(x.clone())
+        torch.cuda.synchronize()
+        assert layers[0].last_launch()["tile_cols"] == 0
+        for w, g in zip(wants, gots):
+            assert torch.equal(w, g)
+    for L in layers:
+        L.close()
