@@ -1110,13 +1110,16 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
         // (long walks on the sparse image, where only the narrowest has a second accumulator and a wave that is not full runs faster, 0.72
         // and no less).  Measured, us with 256, 192, 128 columns: 256 x 2048, 2:4, 62 tiles of 256: 11.4, 11.6, 9.9; 90: 12.0, 11.6, 15.1;
         // 160: 21.2, 21.0, 21.5; 240: 28.1, 33.3, 31.3; 512 x 2048, 3:4, 64: 13.3, 13.1, 10.7; 160: 22.7, 20.5, 23.9; 312: 36.0, 32.8, 40.4;
-        // 400: 40.1, 41.9, 50.5; 256 x 768, 2:4, six blocks, 74: 6.6, 6.1, 5.9; 200: 9.9, 8.3, 10.2.
-        const bool long_sparse = sparse && wlen > 8;
+        // 400: 40.1, 41.9, 50.5; 256 x 768, 2:4, six blocks, 74: 6.6, 6.1, 5.9; 200: 9.9, 8.3, 10.2.  With dense tiles and short walks the
+        // epilogue is the longest role, for which only the widest tile has 16 warps: from the second wave on the others take all of its time, and
+        // three quarters (256 and 192 columns, one block, 55 x 79 x 39776, 3:4 6.8, 7.9; three, 600 x 400 x 26576 18.3, 20.5; seven, fp32, 4160 columns 11.2, 13.0).
+        const bool long_sparse = sparse && wlen > 8, short_dense = !sparse && wlen <= 8;
         int64_t best = 0;
         const int widest = nt;
         for (int c = widest; c >= 2; --c) {
             const int64_t waves = (L.nst * ((ncols + c * kBoxN - 1) / (c * kBoxN)) + sm_count - 1) / sm_count;
-            const int64_t cost = waves * (c == 4 ? 100 : c == 3 ? (long_sparse ? 100 : 80) : (long_sparse ? 72 : 66));
+            const int64_t cost = waves * (short_dense && waves > 1 ? (c == 2 ? 75 : 100)
+                                                                   : c == 4 ? 100 : c == 3 ? (long_sparse ? 100 : 80) : (long_sparse ? 72 : 66));
             if (c == widest || cost < best) { best = cost; nt = c; }
         }
     }
