@@ -68,7 +68,39 @@ class CrispError(RuntimeError):
 
 
 _lib = None
-_native = None                                            # the same calls on plain integers (csrc/calls.cpp)
+_native = None                                            # the hot ones of the same calls on plain integers (csrc/calls.cpp)
+
+
+class _CtypesCalls:
+    """The calls of csrc/calls.cpp through ctypes: the same arguments and results, 1.5 us slower each.  For a tree where that
+    module could not be built (it needs Python's headers)."""
+
+    def __init__(self, lib):
+        self._lib = lib
+        self.spmm, self.decode = lib.crisp_spmm, lib.crisp_decode
+
+    def spmm_conv(self, handle, activation, *rest):
+        *conv, y, ldy, y_dtype, stream = rest
+        if any(v != C.c_int32(v).value for v in conv):
+            return BAD_SHAPE
+        return self._lib.crisp_spmm_conv(handle, activation, ConvDesc(*conv), y, ldy, y_dtype, stream)
+
+    def build_mask(self, saliency, ld, desc, mask_buf, workspace, stream, replaced):
+        self._lib.crisp_mask_destroy(replaced)
+        mask = C.c_void_p()
+        code = self._lib.crisp_build_mask(saliency, ld, LayerDesc.from_address(desc), mask_buf, workspace, stream, C.byref(mask))
+        return code, mask.value or 0
+
+    def encode_sizes(self, mask):
+        canonical, execution = C.c_size_t(), C.c_size_t()
+        code = self._lib.crisp_encode_sizes(mask, C.byref(canonical), C.byref(execution))
+        return code, canonical.value, execution.value
+
+    def encode(self, w, ld, mask, canonical_buf, exec_buf, stream, replaced):
+        self._lib.crisp_destroy(replaced)
+        handle = C.c_void_p()
+        code = self._lib.crisp_encode(w, ld, mask, canonical_buf, exec_buf, stream, C.byref(handle))
+        return code, handle.value or 0
 
 
 def load(path: Optional[str] = None):
@@ -133,12 +165,12 @@ def load(path: Optional[str] = None):
     lib.crisp_status_string.argtypes = [C.c_int]
     lib.crisp_status_string.restype = C.c_char_p
     try:
-        from . import _calls
-    except ImportError as e:
-        raise ImportError(f"{e}: build it with `python -m paper_2311_14272_b200.build`") from e
-    _calls.bind(*[C.cast(getattr(lib, "crisp_" + name), vp).value for name in
-                  ("spmm", "spmm_conv", "decode", "build_mask", "encode_sizes", "encode", "mask_destroy", "destroy")])
-    _lib, _native = lib, _calls
+        from . import _calls as native
+        native.bind(*[C.cast(getattr(lib, "crisp_" + name), vp).value for name in
+                      ("spmm", "spmm_conv", "decode", "build_mask", "encode_sizes", "encode", "mask_destroy", "destroy")])
+    except ImportError:
+        native = _CtypesCalls(lib)
+    _lib, _native = lib, native
     return lib
 
 

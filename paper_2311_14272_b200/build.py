@@ -12,6 +12,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcrisp.so")
 CALLS = os.path.join(HERE, "_calls.so")                      # Python entry points of the hot calls (plain C++)
+PYTHON_INCLUDE = sysconfig.get_paths()["include"]
+HAVE_PYTHON_H = os.path.exists(os.path.join(PYTHON_INCLUDE, "Python.h"))       # without it the binding makes those calls through ctypes
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -24,9 +26,10 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALLS):
+    built = [LIB] + ([CALLS] if HAVE_PYTHON_H else [])
+    if not all(os.path.exists(f) for f in built):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
+    t = min(os.path.getmtime(f) for f in built)
     deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.cpp")) \
         + glob.glob(os.path.join(ROOT, "include", "*.h")) + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -41,9 +44,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", tmp] + sources()
     subprocess.check_call(cmd)
     os.replace(tmp, LIB)
+    if not HAVE_PYTHON_H:
+        print(f"no Python.h in {PYTHON_INCLUDE}: the hot calls go through ctypes", file=sys.stderr)
+        return LIB
     tmp = CALLS + f".{os.getpid()}.tmp"
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), "-o", tmp,
+                           "-I", PYTHON_INCLUDE, "-I", os.path.join(ROOT, "include"), "-o", tmp,
                            os.path.join(CSRC, "calls.cpp")])
     os.replace(tmp, CALLS)
     return LIB
