@@ -480,6 +480,7 @@ class HybridLayer:
         mask_bytes, ws_bytes = crisp_mask_sizes(self.desc)
         self.mask_buf = torch.empty(mask_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=self.device)
+        self.device = self.mask_buf.device                   # with its index: results lie beside the buffers, whatever device is current by then
         self.mask = 0
         self.handle = 0
         self.canonical_buf = None

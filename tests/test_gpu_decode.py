@@ -29,3 +29,17 @@ def test_decode_is_exact(rows, k, bm, bk, keep, pad, n, m):
     assert np.array_equal(got[:, :k], wb)
     assert torch.all(out[:, k:] == 7.0)                       # nothing written past k
     L.close()
+
+
+def test_a_layer_knows_its_device():
+    """Results of a layer made on "cuda" lie beside its buffers: the device is settled when the layer is made, not at each call."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    here = torch.device("cuda", torch.cuda.current_device())
+    L = B.HybridLayer(64, 64, 2, 4, 32, 32, 1.0, device="cuda")
+    assert L.device == here and L.mask_buf.device == here
+    w = torch.randn(64, 64, device="cuda").bfloat16()
+    L.build_mask(w.float().abs()).encode(w)
+    assert L.decode().device == here and L.spmm(w).device == here
+    L.close()
