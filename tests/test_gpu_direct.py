@@ -69,8 +69,9 @@ def test_products_of_falling_size_in_one_graph():
         w = wl.f32_to_bf16_bits((rng.standard_normal((rows, k)) / 32).astype(np.float32))
         layers.append(gpu_layer(B, torch, w, np.abs(wl.bf16_bits_to_f32(w)) + 1e-3, n, m, 64, bk, keep))
         xs.append(torch.zeros(k, 49, dtype=torch.bfloat16, device="cuda"))
+        layers[-1].set_path(B.PATH_DIRECT)
         ys.append(layers[-1].spmm(xs[-1]))
-        assert layers[-1].last_launch()["path"] == 0
+        assert layers[-1].last_launch()["path"] == 0 and layers[-1].last_launch()["tile_cols"] == 0
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
         for L, x, y in zip(layers, xs, ys):

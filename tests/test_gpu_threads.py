@@ -46,8 +46,9 @@ def test_direct_products_of_two_threads(ncols):
     jobs, outs, refs = [], [], []
     for L in layers:
         x = torch.randn(L.desc.k, ncols, device="cuda").bfloat16()
+        L.set_path(B.PATH_DIRECT)
         refs.append(L.spmm(x))
-        assert L.last_launch()["path"] == 0              # the direct product
+        assert L.last_launch()["path"] == 0 and L.last_launch()["tile_cols"] == 0        # the kernel on the CUDA cores
         y = torch.zeros_like(refs[-1])
         outs.append(y)
         jobs.append(lambda L=L, x=x, y=y: L.spmm(x, y=y))
