@@ -385,12 +385,14 @@ struct HaloLaunch {
     crisp_launch_info_t info;
     int64_t resident_bytes;
 };
-// Launch plan: tensor maps and tile shape for one set of operands.
+// Launch plan: tensor maps and tile shape for one set of operands; or that convolutions of this shape stay with the other kernel,
+// so that this is not worked out at every call.
 struct HaloPlan {
     const void *x, *y;
     int64_t ldy;
     ConvGeom conv;
     int device;
+    bool refused;
     HaloLaunch launch;
 };
 void halo_plan_destroy(HaloPlan *plan) { delete plan; }
@@ -405,12 +407,13 @@ bool make_map_nhwc(CUtensorMap *map, const void *base, uint64_t c, uint64_t pitc
     return make_map_4d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box);
 }
 
-// Whether this convolution goes through the kernel above, and its plan if so.
-bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
+enum class Choice { kTaken, kRefused, kNoMaps };
+
+// Whether convolutions of this shape go through the kernel above, and the plan of this one if so.
+Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, const ConvGeom &cv, int device,
                HaloLaunch *plan) {
     const Geometry &g = h->g;
-    if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return false;
-    if (h->exec_kind != CRISP_PATH_SPARSE && h->exec_kind != CRISP_PATH_DENSE) return false;
+    if (h->exec_kind != CRISP_PATH_SPARSE && h->exec_kind != CRISP_PATH_DENSE) return Choice::kRefused;
     const bool sparse = h->exec_kind == CRISP_PATH_SPARSE;
     const TcImageLayout L = tc_image_layout(g, h->exec_kind);
     const int sms = sm_count_of(device);
@@ -438,11 +441,11 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
             best = cost; n = cand; tiles = count * L.nst;
             p.th = th; p.tb = tb; p.pw = pw;
         }
-    if (!n) return false;
+    if (!n) return Choice::kRefused;
     int bw, bh, bb;
     const int64_t gather = conv_box(256, 64, cv, &bw, &bh, &bb) / 256;
     const bool narrow = 2 * gather * L.nst < sms;            // (the gather's tiles are half as wide then)
-    if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 2500) return false;
+    if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 2500) return Choice::kRefused;
     // Where an entry's cost decides, the estimates above are too low: with every SM at work an entry of 128, 224 and 256 pixels takes some
     // 410, 560 and 520 cycles, and what a tile costs besides is 1500 less than in the gather.  (us, gather and this kernel, 2 waves of
     // tiles there and 3 here: 512 -> 448 channels, 55 x 57 x 5, 72 entries 51.2 and 59.7; 256 -> 256, 112 x 112 x 3, 24 entries 21.0 and 23.4;
@@ -451,17 +454,17 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     // the set-up does not cost: 64 -> 448, 1x1, 28 x 28 x 4 5.0 and 5.4.
     // (Channels that are no multiple of 8 leave the gather element by element, 1.2 to 1.6 times slower on all of these.)
     if (g.rows % 8 == 0 && narrow) {
-        if (n == 128 && L.wcap <= 4) return false;
+        if (n == 128 && L.wcap <= 4) return Choice::kRefused;
     } else if (g.rows % 8 == 0) {
         const int busy = n == 128 || n == 64 ? 410 : n == 224 ? 560 : 520, entry = sparse || busy > n + 256 ? busy : n + 256;
-        if ((tiles + sms - 1) / sms * (L.wcap * entry + 1000) > waves(gather) * (L.wcap * 700 + 2500)) return false;
+        if ((tiles + sms - 1) / sms * (L.wcap * entry + 1000) > waves(gather) * (L.wcap * 700 + 2500)) return Choice::kRefused;
     }
     // One CTA tile of rows and a walk of up to eight blocks: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images
     // of 112 x 112 10.5 and 8.8, 3.4 tiles a CTA; 6 images 9.2 and 8.5; 3 images 6.8 each; one image of 56 x 56 5.5 and 5.9.  Below the line stays the gather with
     // resident weight tiles, whose form its tests and crisp_last_resident_bytes' callers look for.)
-    if (L.nst == 1 && L.wcap <= 8 && tiles < 3 * (int64_t)sms) return false;
-    if (tiles > 0x7FFFFFFF) return false;
-    if ((int64_t)L.nst * L.wcap * 8 > kListBytes || L.nst > kMaxRowTiles) return false;
+    if (L.nst == 1 && L.wcap <= 8 && tiles < 3 * (int64_t)sms) return Choice::kRefused;
+    if (tiles > 0x7FFFFFFF) return Choice::kRefused;
+    if ((int64_t)L.nst * L.wcap * 8 > kListBytes || L.nst > kMaxRowTiles) return Choice::kRefused;
     p.tb_log2 = p.tb == 4 ? 2 : p.tb - 1;
     p.tiles_x = (cv.wo + 7) / 8; p.tiles_y = (cv.ho + p.th - 1) / p.th;
     p.num_tiles = (int)tiles;
@@ -482,7 +485,7 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     if (p.x_stages > 4) p.x_stages = 4;
     p.w_stages = (budget - fixed - p.x_stages * p.x_stage) / w_stage;
     if (p.w_stages > kMaxStages) p.w_stages = kMaxStages;
-    if (p.w_stages < 2) return false;
+    if (p.w_stages < 2) return Choice::kRefused;
     p.resident = L.nst == 1 && (uint32_t)L.wcap <= p.w_stages * kGroup;
     p.y = reinterpret_cast<uint16_t *>(d_y); p.ldy = ldy;
     p.plain_from = ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0 ? 0 : g.rows % 8 != 0 ? g.rows / 32 * 32 : g.rows;
@@ -491,7 +494,7 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     if (!make_map_image(&plan->ma, h->d_exec + L.image_off, (uint64_t)L.stack * L.nst * L.wcap * L.entry_bytes, L.entry_bytes) ||
         !make_map_nhwc(&plan->mx, d_x, cv.channels, cv.channels, cv.width, cv.height, cv.batch, 64, p.pw, p.tb, ph) ||
         (p.plain_from > 0 && !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb)))
-        return false;
+        return Choice::kNoMaps;
     plan->p = p;
     plan->which = (n == 256 ? 6 : n == 224 ? 4 : n == 128 ? 2 : 0) + (sparse ? 1 : 0);
     static const HaloKernel kernels[8] = {spmm_halo_kernel<64, false>, spmm_halo_kernel<64, true>, spmm_halo_kernel<128, false>, spmm_halo_kernel<128, true>,
@@ -499,7 +502,7 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
     plan->kern = kernels[plan->which];
     plan->resident_bytes = p.resident ? (int64_t)L.wcap * p.entry_bytes : 0;
     plan->info = crisp_launch_info_t{h->exec_kind, n, n == 256 && sparse ? 1 : 2, 1, kEpiWarps, (int)p.x_stages, plan->grid, 1, 1};
-    return true;
+    return Choice::kTaken;
 }
 
 }  // namespace
@@ -509,22 +512,28 @@ bool plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t 
 cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
                              cudaStream_t st, bool *done) {
     *done = false;
+    if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return cudaSuccess;
     HaloLaunch launch;
     {
         std::lock_guard<std::mutex> hold(h->plan_lock);
         HaloPlan *plan = h->halo;
-        const bool hit = plan && plan->x == d_x && plan->y == d_y && plan->ldy == ldy && plan->device == device && same_conv(plan->conv, cv) &&
-                         y_dtype == 0 && h->nt_override <= 0 && h->group_override <= 0;
-        if (!hit) {
+        const bool same = plan && plan->device == device && same_conv(plan->conv, cv);
+        if (same && plan->refused) return cudaSuccess;
+        if (!same || plan->x != d_x || plan->y != d_y || plan->ldy != ldy) {
+            const cudaError_t e = ensure_context(device);    // (a plan encodes tensor maps)
+            if (e != cudaSuccess) return e;
             HaloPlan fresh = {};
-            if (!plan_halo(h, d_x, d_y, ldy, y_dtype, cv, device, &fresh.launch)) return cudaSuccess;
+            const Choice choice = plan_halo(h, d_x, d_y, ldy, cv, device, &fresh.launch);
+            if (choice == Choice::kNoMaps) return cudaSuccess;
             fresh.x = d_x; fresh.y = d_y; fresh.ldy = ldy; fresh.conv = cv; fresh.device = device;
+            fresh.refused = choice == Choice::kRefused;
             if (!plan) {
                 plan = new (std::nothrow) HaloPlan;
                 if (!plan) return cudaErrorMemoryAllocation;
                 h->halo = plan;
             }
             *plan = fresh;
+            if (fresh.refused) return cudaSuccess;
         }
         launch = plan->launch;
     }

@@ -1312,9 +1312,8 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
     cudaError_t e = cudaGetDevice(&device);
     if (e != cudaSuccess) return e;
     if (conv) {
-        e = ensure_context(device);                          // (a plan encodes tensor maps)
         bool done = false;
-        if (e == cudaSuccess) e = launch_spmm_halo(h, d_x, d_y, ldy, y_dtype, *conv, device, st, &done);
+        e = launch_spmm_halo(h, d_x, d_y, ldy, y_dtype, *conv, device, st, &done);
         if (done || e != cudaSuccess) return e;
     }
     TcLaunch launch;
