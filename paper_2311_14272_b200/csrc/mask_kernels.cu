@@ -494,12 +494,13 @@ mask_small_kernel(const float *s, int64_t ld, Geometry g, bool vec_ok, bool max_
 }
 // Layers that it takes: up to 2^14 elements a CTA.  Mask phase replayed from a graph, and mask, encoding and decoding called in a row, us, this kernel and
 // the others: 256 x 256 (2^13 a CTA) 6.3 and 10.4, 14.3 and 19; 128 x 256 (2^14) 8.0 and 10.4, 15.6 and 19; 25 x 489 (2^14, one CTA) 9.2
-// and 13.1, 19.5 and 21; 256 x 512 in four CTAs (2^15) 12.1 and 10.5, 19.9 and 19.
+// and 13.1, 19.5 and 21; 256 x 512 in four CTAs (2^15) 12.1 and 10.5, 19.9 and 19.  A CTA takes its row tiles one after the other, so of two at most (mask
+// phase: two, 435 x 35 9.0 and 13.2, 464 x 218 12.2 and 12.6; four, 1949 x 46 15.3 and 13.2; six, 1497 x 58 19.0 and 12.4).
 constexpr int64_t kSmallPerCta = 1 << 14;
 int small_ctas(const Geometry &g) {
     const int ctas = g.nrt < kSmallCluster ? g.nrt : kSmallCluster;
-    const int64_t most = (int64_t)((g.nrt + ctas - 1) / ctas) * g.bm * g.kp();
-    return g.nblk <= kSmallMaxBlocks && most <= kSmallPerCta ? ctas : 0;
+    const int row_tiles = (g.nrt + ctas - 1) / ctas;
+    return g.nblk <= kSmallMaxBlocks && row_tiles <= 2 && (int64_t)row_tiles * g.bm * g.kp() <= kSmallPerCta ? ctas : 0;
 }
 
 // Scores and maxima of a batch, cleared (one CTA per layer; a memset per layer costs a launch each).

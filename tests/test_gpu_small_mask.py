@@ -19,6 +19,8 @@ CASES = [
     (290, 60, 5, 8, 32, 32, 0.7, 0, 64),              # ten row tiles: two CTAs have two
     (128, 128, 4, 8, 128, 32, 0.0, 0, 128),           # no kept block
     (129, 100, 8, 8, 128, 32, 0.3, 0, 100),
+    (512, 60, 2, 4, 32, 64, 1.0, 0, 60),              # two row tiles a CTA: the most
+    (513, 60, 2, 4, 32, 64, 1.0, 0, 60),              # three: the kernels for any size
     (257, 512, 2, 4, 32, 64, 0.5, 0, 512),            # a row more than it takes: the kernels for any size
     (32, 544, 2, 4, 32, 32, 0.25, 0, 544),            # a block more than one CTA takes
 ]
