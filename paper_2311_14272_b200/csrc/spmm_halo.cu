@@ -86,7 +86,8 @@ __device__ __forceinline__ void store_matrices(uint32_t addr, uint32_t a, uint32
 // ----------------------------------------------------------------------------------- kernel
 //
 // Shared memory: x_stages x [pixel box with border] | w_stages x 2 x [weight tile | metadata] | 16 staging tiles | barriers | walks
-template <int kN, bool kSparse>
+// kPlain: some channels are stored pixel by pixel (HaloParams::plain_from)
+template <int kN, bool kSparse, bool kPlain>
 __global__ void __launch_bounds__(kThreads, 1)
 spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y,
                  const __grid_constant__ CUtensorMap map_a, const __grid_constant__ HaloParams p) {
@@ -119,7 +120,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_x);
-        if (p.plain_from > 0) prefetch_tensormap(&map_y);
+        if (!kPlain || p.plain_from > 0) prefetch_tensormap(&map_y);
         for (uint32_t s = 0; s < p.x_stages; ++s) { mbar_init(x_full + 8 * s, 1); mbar_init(x_empty + 8 * s, 1); }
         for (uint32_t s = 0; s < p.w_stages; ++s) { mbar_init(w_full + 8 * s, 1); mbar_init(w_empty + 8 * s, 1); }
         for (int a = 0; a < kAcc; ++a) { mbar_init(t_full + 8 * a, 1); mbar_init(t_empty + 8 * a, kEpiWarps); }
@@ -294,7 +295,6 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             const int ct = t / p.nst, st = t - ct * p.nst;
             const Tile org = tile_at(p, ct);
             const int ch0 = st * kTileM + 32 * q;
-            const bool plain = ch0 >= p.plain_from;
             float bias[4];                                   // of channels l / 4, + 8, + 16, + 24
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -328,7 +328,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         store_matrices(tile + (uint32_t)(512 * g) + my_row, pack(lo[4 * g], lo[4 * g + 1]), pack(lo[4 * g + 2], lo[4 * g + 3]),
                                        pack(hi[4 * g], hi[4 * g + 1]), pack(hi[4 * g + 2], hi[4 * g + 3]));
                     }
-                    if (plain) {                             // pixel by pixel, the lanes on consecutive channels
+                    if (kPlain && ch0 >= p.plain_from) {     // pixel by pixel, the lanes on consecutive channels
                         __syncwarp();
                         const bool ch_ok = ch0 + lane < p.rows;
 #pragma unroll 8
@@ -496,9 +496,11 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
         (p.plain_from > 0 && !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb)))
         return Choice::kNoMaps;
     plan->p = p;
-    plan->which = (n == 256 ? 6 : n == 224 ? 4 : n == 128 ? 2 : 0) + (sparse ? 1 : 0);
-    static const HaloKernel kernels[8] = {spmm_halo_kernel<64, false>, spmm_halo_kernel<64, true>, spmm_halo_kernel<128, false>, spmm_halo_kernel<128, true>,
-                                          spmm_halo_kernel<224, false>, spmm_halo_kernel<224, true>, spmm_halo_kernel<256, false>, spmm_halo_kernel<256, true>};
+    const bool plain = p.plain_from < g.rows;
+    plan->which = (n == 256 ? 12 : n == 224 ? 8 : n == 128 ? 4 : 0) + (sparse ? 2 : 0) + (plain ? 1 : 0);
+#define CRISP_HALO_KERNELS(N) spmm_halo_kernel<N, false, false>, spmm_halo_kernel<N, false, true>, spmm_halo_kernel<N, true, false>, spmm_halo_kernel<N, true, true>
+    static const HaloKernel kernels[16] = {CRISP_HALO_KERNELS(64), CRISP_HALO_KERNELS(128), CRISP_HALO_KERNELS(224), CRISP_HALO_KERNELS(256)};
+#undef CRISP_HALO_KERNELS
     plan->kern = kernels[plan->which];
     plan->resident_bytes = p.resident ? (int64_t)L.wcap * p.entry_bytes : 0;
     plan->info = crisp_launch_info_t{h->exec_kind, n, n == 256 && sparse ? 1 : 2, 1, kEpiWarps, (int)p.x_stages, plan->grid, 1, 1};
@@ -538,7 +540,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
         launch = plan->launch;
     }
     *done = true;
-    static std::atomic<bool> configured[8][64];
+    static std::atomic<bool> configured[16][64];
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     if (!configured[launch.which][device].load(std::memory_order_relaxed)) {
         // the most there is, once: the limit belongs to the function, not to a call
