@@ -10,7 +10,7 @@
 // (Asynchronous 16-byte copies by the same warps instead of TMA: 0.55 us a block, of which the copies' issue alone took half.)
 // Y goes through a staging tile and out in 4-byte stores, row by row.
 // What bounds a long walk is the X warps' chain, 0.37 us a block; what a launch costs besides is set-up, the first load and the rows of
-// Y, a third each.  Measured: 256 x 2304 x 6076, 1:4, keep 0.25: 51.2 us on the CUDA cores, 13.0 here; 512 x 4608 x 588, 2:4: 103 and 11.6.
+// Y, a third each.  Measured: 256 x 2304 x 6076, 1:4, keep 0.25: 51.2 us on the CUDA cores, 13.4 here; 512 x 4608 x 588, 2:4: 103 and 11.6.
 //
 // Few tiles and long walks leave most SMs without work: the walk of a tile is then split over a cluster of 2, 4 or 8 CTAs,
 // each of which owns a slice of the tile's rows in the end.  The partial sums travel through distributed shared memory
@@ -19,7 +19,10 @@
 //
 // Zeros in a weight tile (pruned places, row tiles that do not keep the block) multiply activations that the pattern does
 // not touch: an infinity or a NaN there must not reach the result.  The warps that shift X notice one on the way (one fused
-// multiply-add by zero per two elements), and a tile that had any is computed anew from the canonical format.
+// multiply-add by zero per two elements), put 1 or -1 in its place and leave a note of the tile, the block and the row.  When a
+// CTA has multiplied all its tiles, all its warps go through the noted ones: a result with such a term in the canonical format becomes
+// what its terms that are not finite add up to, the others stay.  (us, clean, one infinity a column tile, all NaN, and the CUDA cores: 256 x 2304 x 6076, 1:4
+// 13.1, 19.6, 31.3, 49.2; 160 x 960 x 49 8.1, 10.3, 11.8, 14.7; 64 x 64 x 50001, where a tile's work is little, 15.7, 31.3, 34.7, 23.0.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -45,7 +48,7 @@ constexpr uint32_t kStagePitch = 144;                    // a row of 64 results 
 constexpr uint32_t kStageTile = 16 * kStagePitch;
 constexpr int kMaxSplit = 8;
 constexpr uint32_t kSumPitch = kCols * 4 + 16;           // a row of partial sums of a split tile (odd number of 16-byte words)
-constexpr int kFlagSlots = 16;                           // tiles the X warps may be ahead of the epilogue: at most the ring's stages
+constexpr uint32_t kTileBits = 2048;                      // notes of the tiles of a CTA that had a value that is not finite, by number modulo this
 
 // Blocks as they lie in memory, of all warps: [group][slot][residue][bk / 8 rows], a residue's rows from a 128-byte boundary; `ahead`
 // slots a group: 1 block of 128 or 96 rows, 2 of 64 or 4 of 32 (these take the most, 4 rows in 1152 bytes).
@@ -151,54 +154,147 @@ __device__ __forceinline__ void mma_loop(const GatherParams &p, const MmaArgs &a
     }
 }
 
-// Y from the canonical format for rows [row0, row0 + nrows) and columns [col0, col0 + width) (width <= 64), one warp; two
-// columns a lane, sums in the order of blocks, groups and values.
-__device__ __noinline__ void canonical_rows(const GatherParams &p, int row0, int nrows, int row_step, int64_t col0, int width) {
+// Blocks and rows of X that had a value that is not finite: block columns modulo 32, rows of a block modulo 32.
+struct Notes { uint32_t blocks, rows; };
+
+// One row of a tile with values that are not finite, 128 columns from col0, four a lane, one warp: what such terms of the row add up to takes
+// the place of the result, which was made with 1 or -1 in their place.  A result that is not finite by itself (from a weight or the bias) is
+// one more term.  ReLU comes last, and for all results of such a tile here (after the rounding to bf16, which changes no sign).
+// The lanes look through 32 kept blocks, then decode 32 weights at a time, and then all take the noted ones among them, two by two, until every
+// sum is a NaN, which nothing changes.  What it costs are a few round trips to L2.
+// (Part of the kernel and at one place of it: as a function that is called it reads the launch's parameters through memory, three times the
+// repair's time, and the calls cost products without such values 0.4 us.)
+__device__ __forceinline__ void repair_row(const GatherParams &p, Notes notes, int row, int64_t col0) {
     const Geometry &g = p.g;
-    const int lane = threadIdx.x & 31, gpb = g.bk / g.m, vpb = (int)g.vals_per_block();
-    const int64_t ca = col0 + lane, cb = ca + 32;
-    const bool a_ok = lane < width && ca < p.ncols, b_ok = lane + 32 < width && cb < p.ncols;
-    for (int i = 0; i < nrows; ++i) {
-        const int row = row0 + i * row_step;
-        if (row >= g.rows) break;
-        const int rt = row / g.bm, local = row - rt * g.bm;
-        float sa = 0.f, sb = 0.f;
-        for (int slot = 0; slot < g.kkeep; ++slot) {
-            const int64_t blk = (int64_t)rt * g.kkeep + slot;
-            const int krow0 = p.blk_col[blk] * g.bk;
+    const int lane = threadIdx.x & 31, vpr = g.bk / g.m * g.n, vpb = (int)g.vals_per_block();
+    const int rt = row / g.bm, local = row - rt * g.bm, valid = (int)min((int64_t)kCols, p.ncols - col0) - lane;      // this lane's columns: 0, 32, 64, 96 below it
+    const uint16_t *x0 = p.x + col0 + lane;
+    auto value = [](const uint16_t *at) { return __uint_as_float((uint32_t)*at << 16); };
+    auto odd = [](float v) { return !(fabsf(v) < __int_as_float(0x7f800000)); };
+    float extra[4] = {0.f, 0.f, 0.f, 0.f};
+    bool settled = false;
+    for (int s0 = 0; s0 < g.kkeep && !settled; s0 += 32) {
+        const int col_of_lane = s0 + lane < g.kkeep ? p.blk_col[(int64_t)rt * g.kkeep + s0 + lane] : 0;
+        uint32_t slots = __ballot_sync(0xFFFFFFFFu, s0 + lane < g.kkeep && (notes.blocks >> (col_of_lane & 31) & 1u));
+        for (; slots && !settled; slots &= slots - 1) {
+            const int in32 = __ffs(slots) - 1;
+            const int64_t blk = (int64_t)rt * g.kkeep + s0 + in32;
+            const int krow0 = __shfl_sync(0xFFFFFFFFu, col_of_lane, in32) * g.bk;
             const uint32_t *iw = p.idx + blk * (vpb * g.idx_bits / 32);
-#pragma unroll 4
-            for (int v = 0; v < gpb * g.n; ++v) {
-                const int at = local * gpb * g.n + v, bit = at * g.idx_bits;
-                uint32_t f = iw[bit >> 5] >> (bit & 31);
-                if ((bit & 31) + g.idx_bits > 32) f |= iw[(bit >> 5) + 1] << (32 - (bit & 31));
-                const int krow = krow0 + v / g.n * g.m + (int)(f & ((1u << g.idx_bits) - 1u));
-                const float w = __uint_as_float((uint32_t)p.vals[blk * vpb + at] << 16);
-                if (krow < g.k) {
-                    const uint16_t *xr = p.x + (int64_t)krow * p.ldx;
-                    if (a_ok) sa = fmaf(w, __uint_as_float((uint32_t)xr[ca] << 16), sa);
-                    if (b_ok) sb = fmaf(w, __uint_as_float((uint32_t)xr[cb] << 16), sb);
+            for (int v0 = 0; v0 < vpr && !settled; v0 += 32) {
+                const int v = v0 + lane;
+                bool hit = v < vpr;
+                uint32_t entry = 0;                          // weight and row of the block
+                if (hit) {
+                    const int at = local * vpr + v, bit = at * g.idx_bits;
+                    uint32_t f = iw[bit >> 5] >> (bit & 31);
+                    if ((bit & 31) + g.idx_bits > 32) f |= iw[(bit >> 5) + 1] << (32 - (bit & 31));
+                    const int kin = v / g.n * g.m + (int)(f & ((1u << g.idx_bits) - 1u));
+                    entry = (uint32_t)p.vals[blk * vpb + at] << 16 | (uint32_t)kin;
+                    hit = (notes.rows >> (kin & 31) & 1u) && krow0 + kin < g.k;
+                }
+                uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
+                while (hits && !settled) {
+                    float w[2], xv[2][4];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const uint32_t e = __shfl_sync(0xFFFFFFFFu, entry, hits ? __ffs(hits) - 1 : 0);
+                        const uint16_t *xr = x0 + (int64_t)(krow0 + (int)(e & 0xFFFFu)) * p.ldx;
+                        w[u] = __uint_as_float(e & 0xFFFF0000u);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) xv[u][c] = hits && 32 * c < valid ? value(xr + 32 * c) : 0.f;
+                        hits &= hits - 1;
+                    }
+                    bool nan = true;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+                            if (odd(xv[u][c])) extra[c] = fmaf(w[u], xv[u][c], extra[c]);
+                        nan = nan && (32 * c >= valid || extra[c] != extra[c]);
+                    }
+                    settled = __all_sync(0xFFFFFFFFu, nan);
                 }
             }
         }
-        if (p.bias) { sa += p.bias[row]; sb += p.bias[row]; }
-        if (p.relu) { sa = fmaxf(sa, 0.f); sb = fmaxf(sb, 0.f); }
-        if (a_ok) p.y[row * p.ldy + ca] = __bfloat16_as_ushort(__float2bfloat16_rn(sa));
-        if (b_ok) p.y[row * p.ldy + cb] = __bfloat16_as_ushort(__float2bfloat16_rn(sb));
+    }
+    uint16_t *y = p.y + (int64_t)row * p.ldy + col0 + lane;
+    float was[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) was[c] = 32 * c < valid && (odd(extra[c]) || p.relu) ? value(y + 32 * c) : 0.f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        float v = !odd(extra[c]) ? was[c] : odd(was[c]) ? was[c] + extra[c] : extra[c];
+        if (p.relu) v = fmaxf(v, 0.f);
+        if (32 * c < valid && (odd(extra[c]) || p.relu)) y[32 * c] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
     }
 }
 
 // Y = act(sum + bias) as the kernel on the CUDA cores rounds it: without a bias nothing is added, and a NaN becomes 0 only under ReLU.
+// (`noted`: the tile goes through repair_row, which applies ReLU)
 template <int N>
-__device__ __forceinline__ void finish(const GatherParams &p, float (&v)[N], float bias) {
+__device__ __forceinline__ void finish(const GatherParams &p, float (&v)[N], float bias, bool noted) {
     if (p.bias) {
 #pragma unroll
         for (int i = 0; i < N; ++i) v[i] += bias;
     }
-    if (p.relu) {
+    if (p.relu && !noted) {
 #pragma unroll
         for (int i = 0; i < N; ++i) v[i] = fmaxf(v[i], 0.f);
     }
+}
+
+// 1 or -1 in the place of a bf16 value that is not finite, two at a time; whether there was one
+__device__ __forceinline__ bool finite_only(uint32_t &w) {
+    const bool lo = (w & 0x7F80u) == 0x7F80u, hi = (w & 0x7F800000u) == 0x7F800000u;
+    if (lo) w = (w & 0xFFFF8000u) | 0x3F80u;
+    if (hi) w = (w & 0x8000FFFFu) | 0x3F800000u;
+    return lo | hi;
+}
+
+// An X warp's rows of a block, from where they arrived to the operand tile.  The result is not 0 if there was a value that is not finite in
+// the lane's columns.  kClean: with such values replaced, and the result says in which of the rows 0, 1, 2 and so on they were (modulo 4).
+template <bool kWide, bool kClean>
+__device__ __forceinline__ uint32_t move_rows(uint32_t src, uint32_t dst, int rows, uint32_t at, uint32_t box_bytes) {
+    uint32_t probe = 0, which = 0;
+#pragma unroll 1
+    for (int r = 0; r < rows; r += 4) {
+        const uint32_t s4 = src + (uint32_t)r * kRawPitch, d4 = dst + (uint32_t)r * 1024u;
+        if constexpr (kWide) {
+            uint2 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = lds64(s4 + u * kRawPitch);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if constexpr (kClean) which |= (uint32_t)(finite_only(v[u].x) | finite_only(v[u].y)) << u;
+                else probe = finite_probe(v[u].y, finite_probe(v[u].x, probe));
+                sts64(d4 + 1024u * u, v[u].x, v[u].y);
+            }
+        } else {
+            uint32_t v[4][2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { v[u][0] = lds32(s4 + u * kRawPitch); v[u][1] = lds32(s4 + u * kRawPitch + 128u); }
+            if (at & 2u) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    v[u][0] = __funnelshift_r(v[u][0], lds32(s4 + u * kRawPitch + 4u), 16);
+                    v[u][1] = __funnelshift_r(v[u][1], lds32(s4 + u * kRawPitch + 132u), 16);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if constexpr (kClean) which |= (uint32_t)(finite_only(v[u][0]) | finite_only(v[u][1])) << u;
+                else probe = finite_probe(v[u][1], finite_probe(v[u][0], probe));
+                sts32(d4 + 1024u * u, v[u][0]);
+                sts32(d4 + 1024u * u + box_bytes, v[u][1]);
+            }
+        }
+    }
+    return kClean ? which : probe & 0x7FFF7FFFu;
+}
+template <bool kWide>
+__device__ __noinline__ uint32_t clean_rows(uint32_t src, uint32_t dst, int rows, uint32_t at, uint32_t box_bytes) {
+    return move_rows<kWide, true>(src, dst, rows, at, box_bytes);
 }
 
 // A row of results, packed two columns a word: word u of the row in `v`, the one after it in `next`; `valid` columns of it
@@ -255,7 +351,8 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     const uint32_t bar_full = ctrl, bar_empty = ctrl + 64, bar_tfull = ctrl + 128, bar_tempty = ctrl + 144;
     volatile uint32_t *tmem_base_slot = reinterpret_cast<volatile uint32_t *>(ctrl_gen + 160);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl_gen + 164);
-    volatile int *tile_flags = reinterpret_cast<volatile int *>(ctrl_gen + 192);       // [kFlagSlots] number of the last tile with a value that is not finite, plus one
+    volatile Notes *notes = reinterpret_cast<volatile Notes *>(ctrl_gen + 192);
+    volatile uint32_t *tile_bits = reinterpret_cast<volatile uint32_t *>(ctrl_gen + 768);          // [kTileBits / 32]
     const uint32_t bar_raw = ctrl + 256;                     // [X warp][4]: its rows of a block have arrived
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -268,8 +365,11 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         for (uint32_t s = 0; s < p.num_stages; ++s) { mbar_init(bar_full + 8 * s, 1 + kGroupWarps); mbar_init(bar_empty + 8 * s, 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(bar_tfull + 8 * a, 1); mbar_init(bar_tempty + 8 * a, kEpiWarps); }
         *abort_flag = 0;
-        for (int i = 0; i < kFlagSlots; ++i) tile_flags[i] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 2) {
+        notes->blocks = notes->rows = 0;
+        tile_bits[lane] = tile_bits[32 + lane] = 0;
     }
     if (warp >= kFirstX && lane == 0) {
         for (int i = 0; i < 4; ++i) mbar_init(bar_raw + 32u * (uint32_t)(warp - kFirstX) + 8u * i, 1);
@@ -348,7 +448,7 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             };
             load_window(0);
             const int count = walk_share(p, st, rank), mine = (count - first + 1) >> 1;   // blocks first, first + 2, ...
-            uint32_t probe = 0, to = slot;                   // slot to ask for next; one block is moved, the one `ahead` on asked for
+            uint32_t to = slot;                              // slot to ask for next; one block is moved, the one `ahead` on asked for
 #pragma unroll 1
             for (int i = 0; i < mine + p.ahead; ++i) {
                 if (i >= p.ahead) {
@@ -358,39 +458,15 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                                       mbar_wait(bar_empty + 8 * stage, ph ^ 1u, abort_flag, p.wait_limit);
                     if (!__all_sync(0xFFFFFFFFu, have)) { ok = false; break; }
                     const uint32_t src = my_raw + slot * slot_step + lane_src, dst = ring + stage * p.stage_bytes + lane_dst;
-#pragma unroll 1
-                    for (int r = 0; r < rows; r += 4) {
-                        const uint32_t s4 = src + (uint32_t)r * kRawPitch, d4 = dst + (uint32_t)r * 1024u;
-                        if constexpr (kWide) {
-                            uint2 v[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) v[u] = lds64(s4 + u * kRawPitch);
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                probe = finite_probe(v[u].y, finite_probe(v[u].x, probe));
-                                sts64(d4 + 1024u * u, v[u].x, v[u].y);
-                            }
-                        } else {
-                            uint32_t v[4][2];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) { v[u][0] = lds32(s4 + u * kRawPitch); v[u][1] = lds32(s4 + u * kRawPitch + 128u); }
-                            if (at & 2u) {
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) {
-                                    v[u][0] = __funnelshift_r(v[u][0], lds32(s4 + u * kRawPitch + 4u), 16);
-                                    v[u][1] = __funnelshift_r(v[u][1], lds32(s4 + u * kRawPitch + 132u), 16);
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                probe = finite_probe(v[u][1], finite_probe(v[u][0], probe));
-                                sts32(d4 + 1024u * u, v[u][0]);
-                                sts32(d4 + 1024u * u + box_bytes, v[u][1]);
-                            }
-                        }
+                    if (__builtin_expect(move_rows<kWide, false>(src, dst, rows, at, box_bytes) != 0u, 0)) {
+                        // (said before the stage is handed over: the epilogue reads it behind the accumulator.  The warp's rows are res,
+                        // res + 8 and so on: bit 8 u + res for the u-th of four)
+                        const uint32_t which = clean_rows<kWide>(src, dst, rows, at, box_bytes);
+                        const int col = cols[(first + 2 * (i - p.ahead)) << p.split_log2];
+                        atomicOr(const_cast<uint32_t *>(&notes->blocks), 1u << (col & 31));
+                        atomicOr(const_cast<uint32_t *>(&notes->rows), ((which & 1u) | (which & 2u) << 7 | (which & 4u) << 14 | (which & 8u) << 21) << res);
+                        atomicOr(const_cast<uint32_t *>(tile_bits) + (tile_no % kTileBits >> 5), 1u << (tile_no & 31));
                     }
-                    // (said before the stage is handed over: the epilogue reads it behind the accumulator)
-                    if (probe & 0x7FFF7FFFu) tile_flags[tile_no % kFlagSlots] = tile_no + 1;
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_full + 8 * stage);
@@ -428,7 +504,7 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             tc_fence_after();
             const int y0 = st * kTileM + 32 * q;
             const int64_t x0 = (int64_t)ct * kCols + 64 * half;
-            const bool again = tile_flags[tile_no % kFlagSlots] == tile_no + 1;
+            const bool noted = tile_bits[tile_no % kTileBits >> 5] >> (tile_no & 31) & 1u;
             uint32_t out[32];                                // 64 columns of the lane's row, packed
             const float bias = p.bias && y0 + lane < p.g.rows ? p.bias[y0 + lane] : 0.f;
 #pragma unroll
@@ -439,7 +515,7 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 tmem_ld_wait();
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(bits[i]);
-                finish(p, v, bias);
+                finish(p, v, bias, noted);
 #pragma unroll
                 for (int i = 0; i < 16; ++i) out[16 * c + i] = pack_bf16(v[2 * i], v[2 * i + 1]);
             }
@@ -447,26 +523,23 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty + 8 * acc);
             if (y0 < p.g.rows && x0 < p.ncols) {
-                if (again) {
-                    canonical_rows(p, y0, 32, 1, x0, 64);
-                } else {
 #pragma unroll 1
-                    for (int h = 0; h < 2; ++h) {            // lanes 0..15, then 16..31
-                        if (y0 + 16 * h >= p.g.rows) break;
-                        __syncwarp();
-                        if ((lane >> 4) == h) {
+                for (int h = 0; h < 2; ++h) {                // lanes 0..15, then 16..31
+                    if (y0 + 16 * h >= p.g.rows) break;
+                    __syncwarp();
+                    if ((lane >> 4) == h) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                sts128(stg + (uint32_t)(lane & 15) * kStagePitch + 16u * i, out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
-                        }
-                        __syncwarp();
-                        store_rows(p, stg, lane, y0 + 16 * h, x0);
+                        for (int i = 0; i < 8; ++i)
+                            sts128(stg + (uint32_t)(lane & 15) * kStagePitch + 16u * i, out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
                     }
+                    __syncwarp();
+                    store_rows(p, stg, lane, y0 + 16 * h, x0);
                 }
             }
             if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
         }
     }
+    Notes all = {0u, 0u};                                    // of a cluster
     if (p.split > 1) {
         // ------------------------------------------------ a split tile: one tile a cluster
         // A rank leaves its sums in its own shared memory ([row][128 columns], where the X warps' rings were: they are done when
@@ -503,35 +576,32 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         cluster_arrive();
         cluster_wait();
         const int per_rank = kTileM >> p.split_log2;
-        const uint32_t flag = smem_u32(const_cast<int *>(tile_flags));
-        const bool again = __any_sync(0xFFFFFFFFu, lane < p.split ? lds32_peer(peer_address(flag, (uint32_t)lane)) : 0u);
+        const uint32_t note = peer_address(smem_u32(const_cast<Notes *>(notes)), (uint32_t)(lane < p.split ? lane : rank));
+        const uint32_t noted_blocks = lds32_peer(note), noted_rows = lds32_peer(note + 4);
+        all = {__reduce_or_sync(0xFFFFFFFFu, noted_blocks), __reduce_or_sync(0xFFFFFFFFu, noted_rows)};
         const int row0 = st * kTileM + rank * per_rank;
         constexpr int kWarps = kThreads / 32;
-        if (again) {
-            for (int h = 0; h < valid; h += 64) canonical_rows(p, row0 + warp, (per_rank - warp + kWarps - 1) / kWarps, kWarps, x0 + h, min(64, valid - h));
-        } else {
-            for (int r = warp; r < per_rank && row0 + r < p.g.rows; r += kWarps) {
-                const int row = row0 + r;
-                const uint32_t at = raw + (uint32_t)(rank * per_rank + r) * kSumPitch + 16u * lane;
-                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int r = warp; r < per_rank && row0 + r < p.g.rows; r += kWarps) {
+            const int row = row0 + r;
+            const uint32_t at = raw + (uint32_t)(rank * per_rank + r) * kSumPitch + 16u * lane;
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-                for (int s0 = 0; s0 < p.split; s0 += 4) {    // four loads from the others at a time
-                    float4 part[4];
+            for (int s0 = 0; s0 < p.split; s0 += 4) {    // four loads from the others at a time
+                float4 part[4];
 #pragma unroll
-                    for (int s = 0; s < 4; ++s)
-                        part[s] = s0 + s < p.split && 4 * lane < valid ? lds128_peer(peer_address(at, (uint32_t)(s0 + s))) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int s = 0; s < 4; ++s)
+                    part[s] = s0 + s < p.split && 4 * lane < valid ? lds128_peer(peer_address(at, (uint32_t)(s0 + s))) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) { sum.x += part[s].x; sum.y += part[s].y; sum.z += part[s].z; sum.w += part[s].w; }
-                }
-                const float bias = p.bias ? p.bias[row] : 0.f;
-                float v[4] = {sum.x, sum.y, sum.z, sum.w};
-                finish(p, v, bias);
-                const uint32_t lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
-                const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, lo, 1);
-                uint16_t *dst = p.y + (int64_t)row * p.ldy + x0;
-                store_words(dst, 2 * lane, valid, lo, hi);
-                store_words(dst, 2 * lane + 1, valid, hi, next);
+                for (int s = 0; s < 4; ++s) { sum.x += part[s].x; sum.y += part[s].y; sum.z += part[s].z; sum.w += part[s].w; }
             }
+            const float bias = p.bias ? p.bias[row] : 0.f;
+            float v[4] = {sum.x, sum.y, sum.z, sum.w};
+            finish(p, v, bias, all.blocks != 0u);
+            const uint32_t lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
+            const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, lo, 1);
+            uint16_t *dst = p.y + (int64_t)row * p.ldy + x0;
+            store_words(dst, 2 * lane, valid, lo, hi);
+            store_words(dst, 2 * lane + 1, valid, hi, next);
         }
         __syncwarp();
         cluster_arrive();                                    // no rank's shared memory goes before all have read it
@@ -540,7 +610,21 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // ------------------------------------------------ teardown (every wait above is bounded)
     tc_fence_before();
     __syncthreads();
-    if (*abort_flag) {
+    // (The unlikely branches here and in the X warps are marked as such: left in line their code costs every product 0.3 us.)
+    if (p.split == 1) { all.blocks = notes->blocks; all.rows = notes->rows; }
+    if (__builtin_expect(all.blocks != 0u && !*abort_flag, 0)) {         // (the same for the whole CTA; a cluster's CTAs have one tile, and their share of its rows)
+        constexpr int kWarps = kThreads / 32;
+        const int nrows = kTileM >> p.split_log2;
+        int no = 0, turn = 0;                                // the warps take turns over the rows of all such tiles; the next one's
+        for (int t = first_tile; t < p.num_tiles; t += tile_step, ++no) {
+            if (p.split == 1 && !(tile_bits[no % kTileBits >> 5] >> (no & 31) & 1u)) continue;
+            const int row0 = t % p.nst * kTileM + rank * nrows, count = max(0, min(nrows, p.g.rows - row0));
+            for (int r = warp >= turn ? warp - turn : warp - turn + kWarps; r < count; r += kWarps)
+                repair_row(p, all, row0 + r, (int64_t)(t / p.nst) * kCols);
+            turn = (turn + count) % kWarps;
+        }
+    }
+    if (__builtin_expect(*abort_flag != 0, 0)) {
         if (threadIdx.x == 0) atomicCAS(p.status, 0, (int)CRISP_TIMEOUT);
         const unsigned long long t0 = clock64();             // let copies that may still be in flight land
         while ((unsigned long long)(clock64() - t0) < 2000000ull) __nanosleep(1000);

@@ -90,6 +90,93 @@ def test_values_that_are_not_finite_reach_only_the_rows_that_use_them(rows, k, n
     L.close()
 
 
+def spoil(xv, where, torch):
+    """Values that are not finite: one, a row and a column, one in a hundred, all."""
+    k, ncols = xv.shape
+    inf, nan = float("inf"), float("nan")
+    if where == "one":
+        xv[k // 2, ncols // 2] = inf
+    elif where == "row and column":
+        xv[k // 3, :] = -inf
+        xv[:, ncols // 3] = nan
+        xv[k - 1, ncols - 1] = inf
+    elif where == "sprinkled":
+        r = torch.rand(k, ncols, device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+        xv[r < 0.004] = inf
+        xv[(r > 0.004) & (r < 0.007)] = -inf
+        xv[(r > 0.007) & (r < 0.008)] = nan
+    else:
+        xv.fill_({"all NaN": nan, "all infinite": inf}[where])
+
+
+SPOILT = [
+    # rows, k, ncols, pitch, n, m, bm, bk, keep
+    (160, 960, 49, 49, 2, 8, 32, 32, 0.5),            # walk split over 8
+    (130, 1000, 131, 140, 3, 4, 64, 64, 0.9),         # split, ragged rows, 8-byte rows
+    (256, 600, 6076, 6076, 1, 4, 64, 64, 0.25),
+    (700, 300, 9001, 9001, 2, 4, 32, 128, 0.34),      # two tiles a CTA, odd rows
+    (42, 70, 70001, 70004, 8, 8, 32, 96, 1.0),        # four tiles a CTA, k in the middle of a block
+]
+
+
+@pytest.mark.parametrize("rows,k,ncols,pitch,n,m,bm,bk,keep", SPOILT)
+@pytest.mark.parametrize("where", ["one", "row and column", "sprinkled", "all NaN", "all infinite"])
+@pytest.mark.parametrize("use_bias,relu,weights", [(False, False, False), (True, True, False), (True, False, True), (False, True, True)])
+def test_values_that_are_not_finite(rows, k, ncols, pitch, n, m, bm, bk, keep, where, use_bias, relu, weights):
+    """NaN and infinities of X, and of the weights and the bias, give what the kernel on the CUDA cores gives, and change no other result."""
+    torch, L, rng, w, s, x, xv = make(rows, k, ncols, pitch, n, m, bm, bk, keep, 0)
+    wd = bf16_dev(w, torch)
+    if weights:
+        wd[1, :] = 0.0                                          # a stored zero times an infinity is a NaN
+        wd[2, ::3] = float("inf")
+        wd[rows - 1, 1::5] = float("nan")
+        L.encode(wd)
+    bias = torch.randn(rows, device="cuda")
+    bias[3] = -float("inf")
+    L.set_epilogue(bias if use_bias else None, relu)
+    spoil(xv, where, torch)
+    y = L.spmm(xv)
+    assert L.last_launch()["tile_cols"] == 128
+    L.set_path(0)
+    ref = L.spmm(xv)
+    torch.cuda.synchronize()
+    assert L.last_launch()["tile_cols"] == 0 and L.device_status() == 0
+    assert torch.equal(torch.isnan(ref), torch.isnan(y))
+    fin = torch.isfinite(ref)
+    odd = ~fin & ~torch.isnan(ref)
+    assert torch.equal(fin, torch.isfinite(y)) and torch.equal(ref[odd], y[odd])
+    a, b = y[fin].double(), ref[fin].double()
+    assert float((a - b).norm()) <= 2.0 ** -8 * float(b.norm())
+    L.close()
+
+
+@pytest.mark.parametrize("rows,k,ncols,n,m,bm,bk,keep", [(160, 960, 49, 2, 8, 32, 32, 0.5), (256, 2304, 6076, 1, 4, 64, 64, 0.25), (512, 4608, 588, 2, 4, 64, 64, 0.5)])
+@pytest.mark.parametrize("where", ["one a column tile", "all NaN", "all infinite"])
+def test_values_that_are_not_finite_cost_no_more_than_on_the_cuda_cores(rows, k, ncols, n, m, bm, bk, keep, where):
+    torch, L, rng, w, s, x, xv = make(rows, k, ncols, ncols, n, m, bm, bk, keep, 0)
+    if where == "one a column tile":
+        xv[k // 2, 5::128] = float("inf")
+    else:
+        spoil(xv, where, torch)
+    y = torch.empty(rows, ncols, dtype=torch.bfloat16, device="cuda")
+
+    def time():
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                L.spmm(xv, y=y)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+    mine = time()
+    L.set_path(0)
+    assert mine <= 1.25 * time()
+    L.close()
+
+
 @pytest.mark.parametrize("ncols", [49, 9003])
 def test_a_wait_that_runs_out_is_reported(ncols):
     torch, L, rng, w, s, x, xv = make(256, 640, ncols, ncols, 2, 4, 64, 64, 0.5, 0)
