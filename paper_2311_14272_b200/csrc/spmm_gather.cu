@@ -660,13 +660,14 @@ void gather_plan_destroy(GatherPlan *plan) { delete plan; }
 // lines (us, that kernel and this one).  Kept rows: 256 7.8 and 8.8 (33 x 1114 x 980), 480 14.8 and 8.0 (160 x 960 x 49), 704 32.3 and 9.1.
 // Weights of a row: 96 6.2 and 7.4 (128 x 256 x 98), 7.0 and 7.8 (600 x 128 x 147); 128 9.6 and 8.2 (300 x 200 x 245), 18.1 and 8.3
 // (423 x 281 x 539).  Results, and multiply-adds: 6.9 and 7.9 (200 x 588, 64 weights a row), 7.0 and 7.9 (39 x 6076, 32); 12.6 and 7.7
-// (400 x 490, 96), 11.6 and 9.1 (810 x 343, 32), 19.5 and 7.3 (93 x 12348).
-constexpr int64_t kMinKept = 320, kMinWeights = 128, kMinResults = 1 << 18, kMinMacs = 10000000;
+// (400 x 490, 96), 11.6 and 9.1 (810 x 343, 32), 19.5 and 7.3 (93 x 12348); many results of fewer than eight weights are stores alone, 4.3 and 6.9 (49 x 7644, 4),
+// 10.4 and 7.4 (191 x 2891, 8).
+constexpr int64_t kMinKept = 320, kMinWeights = 128, kMinResults = 1 << 18, kMinTerms = 8, kMinMacs = 10000000;
 bool gather_supported(const crisp_handle_s *h, int64_t ncols, int y_dtype) {
     if (y_dtype != 0 || (h->exec_kind != CRISP_PATH_DENSE && h->exec_kind != CRISP_PATH_SPARSE) || h->g.kkeep == 0) return false;
     if (!tensor_maps_available() || ncols >= (1ll << 31)) return false;
     const int64_t kept = (int64_t)h->g.kkeep * h->g.bk, weights = kept * h->g.n / h->g.m, results = (int64_t)h->g.rows * ncols;
-    if (kept < kMinKept && weights < kMinWeights && results < kMinResults && results * weights < kMinMacs) return false;
+    if (kept < kMinKept && weights < kMinWeights && (results < kMinResults || weights < kMinTerms) && results * weights < kMinMacs) return false;
     const TcImageLayout L = tc_image_layout(h->g, h->exec_kind);
     const int64_t tiles = (int64_t)L.nst * ((ncols + kCols - 1) / kCols);
     return tiles <= 0x7FFFFFFF && (uint64_t)L.stack * L.nst * L.wcap * L.entry_bytes / 256 < (1ull << 31);

@@ -270,3 +270,17 @@ def test_several_tiles_with_walks_of_unlike_length(rows, k, ncols, n, m, bm, bk,
     terms = mk.kkeep * bk * n // m
     assert bool(((y.double() - ref).abs() <= 2.0 ** -7 * ref.abs() + 2 * terms * 2.0 ** -23 * size).all())
     L.close()
+
+
+@pytest.mark.parametrize("rows,k,ncols,n,m,bm,bk,cuda_cores", [(49, 93, 7644, 1, 8, 128, 32, True), (191, 93, 2891, 2, 8, 32, 32, False)])
+def test_many_results_of_few_weights(rows, k, ncols, n, m, bm, bk, cuda_cores):
+    """One kept block of four or eight weights a row: which kernel takes it."""
+    torch, L, rng, w, s, x, xv = make(rows, k, ncols, ncols, n, m, bm, bk, 0.34, 0)
+    assert L.kkeep == 1
+    y = L.spmm(xv)
+    assert (L.last_launch()["tile_cols"] == 0) == cuda_cores
+    L.set_path(0)
+    ref = L.spmm(xv).double()
+    torch.cuda.synchronize()
+    assert float((y.double() - ref).norm()) <= 2.0 ** -8 * float(ref.norm())
+    L.close()
