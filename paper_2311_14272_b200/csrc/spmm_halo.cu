@@ -9,7 +9,7 @@
 // apart, pw = 8 + kernel width - 1.  Images of one tile are interleaved by rows ([y][image][x]), so the groups of a tile are
 // evenly spaced for any number of images.
 // What bounds it: for one slab and few taps HBM (64 -> 64 channels, 224 x 224 x 16, 4 taps: 241 MB in 36.3 us when replayed from a graph, 56.3 with the
-// gather; 48.7 and 63.7 on buffers that L2 does not hold); for long walks shared memory, which takes 288 cycles to feed the two
+// gather; 46.6 and 63.7 on buffers that L2 does not hold); for long walks shared memory, which takes 288 cycles to feed the two
 // sparse MMAs of an entry (144 each, measured) and some 150 to take in its weight tile and its share of the activation, of 440 in all.
 // A tile is 224 pixels (28 rows of 8, or 14 rows of two images, 7 of four): the image sizes that are multiples of 7 come out even, and two
 // accumulators fit beside the metadata of the sparse image, so that a tile's results leave under the next one's MMAs; 256 pixels
@@ -447,16 +447,18 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
     const bool narrow = 2 * gather * L.nst < sms;            // (the gather's tiles are half as wide then)
     if (best >= (narrow ? waves(2 * gather) * (L.wcap * 500 + 500) : waves(gather) * (L.wcap * 700 + (sparse ? 2000 : 500))) + 2500) return Choice::kRefused;
     // Where an entry's cost decides, the estimates above are too low: with every SM at work an entry of 128, 224 and 256 pixels takes some
-    // 410, 560 and 520 cycles, and what a tile costs besides is 1500 less than in the gather.  (us, gather and this kernel, 2 waves of
-    // tiles there and 3 here: 512 -> 448 channels, 55 x 57 x 5, 72 entries 51.2 and 59.7; 256 -> 256, 112 x 112 x 3, 24 entries 21.0 and 23.4;
-    // one and two: 128 -> 128, 28 x 28 x 40, 18 entries 11.4 and 13.4.  On the other side: 4 and 5 waves, 256 -> 256, 12 entries and more 1.08 times
-    // faster here in the median; as many waves on both sides 1.2 times.)  Walks of up to four blocks in one wave of 128-pixel tiles gain nothing that
-    // the set-up does not cost: 64 -> 448, 1x1, 28 x 28 x 4 5.0 and 5.4.
+    // 410, 560 and 520 cycles (dense tiles what was estimated), and what a tile costs besides is 1500 less than in the gather.  (us, gather
+    // and this kernel, 2 waves of tiles there and 3 here: 512 -> 448 channels, 55 x 57 x 5, 72 entries 51.2 and 59.7; 256 -> 256, 112 x 112 x 3, 24 entries 21.0
+    // and 23.4; one and two: 128 -> 128, 28 x 28 x 40, 18 entries 11.4 and 13.4.  On the other side: 4 and 5 waves, 256 -> 256, 12 entries and more 1.08
+    // times faster here in the median, 3 and 4 waves of dense tiles, 256 -> 448, 28 x 28 x 30, 36 entries 51.2 and 48.5; as many waves on both sides 1.2
+    // times.)  Walks of up to four blocks in one wave of 128-pixel tiles gain nothing that the set-up does not cost, where the gather's tiles are as
+    // narrow: 64 -> 448, 1x1, 28 x 28 x 4 5.0 and 5.4; 128 -> 320, 28 x 28 x 6, 256-pixel tiles there, 6.4 and 5.6.
     // (Channels that are no multiple of 8 leave the gather element by element, 1.2 to 1.6 times slower on all of these.)
     if (g.rows % 8 == 0 && narrow) {
-        if (n == 128 && L.wcap <= 4) return Choice::kRefused;
+        const int64_t pixels = (int64_t)cv.batch * cv.ho * cv.wo;
+        if (n == 128 && L.wcap <= 4 && L.nst * ((pixels + 191) / 192) < sms / 2) return Choice::kRefused;
     } else if (g.rows % 8 == 0) {
-        const int busy = n == 128 || n == 64 ? 410 : n == 224 ? 560 : 520, entry = sparse || busy > n + 256 ? busy : n + 256;
+        const int entry = n <= 128 ? 410 : !sparse ? n + 256 : n == 224 ? 560 : 520;
         if ((tiles + sms - 1) / sms * (L.wcap * entry + 1000) > waves(gather) * (L.wcap * 700 + 2500)) return Choice::kRefused;
     }
     // One CTA tile of rows and a walk of up to eight blocks: from three tiles a CTA on.  (us, gather and this kernel, 64 -> 64 channels: 9 images

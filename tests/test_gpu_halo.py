@@ -31,6 +31,8 @@ CASES = [
     (100, 3, 3, 1, 128, 80, 28, 27, 2, 4, 32, 0.5, 224, False),   # 100 channels, several images, ragged in x
     (256, 1, 1, 0, 64, 16, 56, 50, 2, 4, 64, 1.0, 224, False),    # 1x1: no border, ragged in x
     (72, 1, 1, 0, 192, 50, 45, 41, 1, 8, 32, 0.7, 224, True),
+    (448, 3, 3, 1, 256, 30, 28, 28, 4, 8, 32, 0.59, 224, False),  # dense tiles, four waves where the other kernel has three
+    (320, 1, 1, 0, 128, 6, 28, 28, 1, 8, 64, 1.0, 128, False),    # two blocks, 256-pixel tiles in the other kernel
 ]
 
 
