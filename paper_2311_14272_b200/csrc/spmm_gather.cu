@@ -48,7 +48,7 @@ constexpr uint32_t kStagePitch = 144;                    // a row of 64 results 
 constexpr uint32_t kStageTile = 16 * kStagePitch;
 constexpr int kMaxSplit = 8;
 constexpr uint32_t kSumPitch = kCols * 4 + 16;           // a row of partial sums of a split tile (odd number of 16-byte words)
-constexpr uint32_t kTileBits = 2048;                      // notes of the tiles of a CTA that had a value that is not finite, by number modulo this
+constexpr uint32_t kTileBitsAt = 768, kTileBits = 2048;   // (place among the barriers) notes of the tiles of a CTA that had a value that is not finite, by number modulo this
 
 // Blocks as they lie in memory, of all warps: [group][slot][residue][bk / 8 rows], a residue's rows from a 128-byte boundary; `ahead`
 // slots a group: 1 block of 128 or 96 rows, 2 of 64 or 4 of 32 (these take the most, 4 rows in 1152 bytes).
@@ -352,7 +352,7 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     volatile uint32_t *tmem_base_slot = reinterpret_cast<volatile uint32_t *>(ctrl_gen + 160);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl_gen + 164);
     volatile Notes *notes = reinterpret_cast<volatile Notes *>(ctrl_gen + 192);
-    volatile uint32_t *tile_bits = reinterpret_cast<volatile uint32_t *>(ctrl_gen + 768);          // [kTileBits / 32]
+    volatile uint32_t *tile_bits = reinterpret_cast<volatile uint32_t *>(ctrl_gen + kTileBitsAt);          // [kTileBits / 32]
     const uint32_t bar_raw = ctrl + 256;                     // [X warp][4]: its rows of a block have arrived
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -610,16 +610,21 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // ------------------------------------------------ teardown (every wait above is bounded)
     tc_fence_before();
     __syncthreads();
-    // (The unlikely branches here and in the X warps are marked as such: left in line their code costs every product 0.3 us.)
+    // (The unlikely branches here and in the X warps are marked as such, and what the repair starts from is worked out anew: left in line, or with
+    // its values kept in registers from the start of the kernel, it costs every product 0.3 us.)
     if (p.split == 1) { all.blocks = notes->blocks; all.rows = notes->rows; }
     if (__builtin_expect(all.blocks != 0u && !*abort_flag, 0)) {         // (the same for the whole CTA; a cluster's CTAs have one tile, and their share of its rows)
         constexpr int kWarps = kThreads / 32;
-        const int nrows = kTileM >> p.split_log2;
+        uint32_t cta, tid, stages = p.num_stages;
+        asm volatile("mov.u32 %0, %%ctaid.x;\n\tmov.u32 %1, %%tid.x;" : "=r"(cta), "=r"(tid));
+        asm volatile("" : "+r"(stages));
+        const uint32_t *bits = reinterpret_cast<const uint32_t *>(smem_raw + stages * p.stage_bytes + kRawBytes + kEpiWarps * kStageTile + kTileBitsAt);
+        const int nrows = kTileM >> p.split_log2, my_warp = (int)tid >> 5, row_in_tile = p.split > 1 ? (int)cluster_rank() * nrows : 0;
         int no = 0, turn = 0;                                // the warps take turns over the rows of all such tiles; the next one's
-        for (int t = first_tile; t < p.num_tiles; t += tile_step, ++no) {
-            if (p.split == 1 && !(tile_bits[no % kTileBits >> 5] >> (no & 31) & 1u)) continue;
-            const int row0 = t % p.nst * kTileM + rank * nrows, count = max(0, min(nrows, p.g.rows - row0));
-            for (int r = warp >= turn ? warp - turn : warp - turn + kWarps; r < count; r += kWarps)
+        for (int t = (int)cta >> p.split_log2; t < p.num_tiles; t += (int)gridDim.x >> p.split_log2, ++no) {
+            if (p.split == 1 && !(bits[no % kTileBits >> 5] >> (no & 31) & 1u)) continue;
+            const int row0 = t % p.nst * kTileM + row_in_tile, count = max(0, min(nrows, p.g.rows - row0));
+            for (int r = my_warp >= turn ? my_warp - turn : my_warp - turn + kWarps; r < count; r += kWarps)
                 repair_row(p, all, row0 + r, (int64_t)(t / p.nst) * kCols);
             turn = (turn + count) % kWarps;
         }
@@ -632,7 +637,7 @@ spmm_gather_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     }
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc(*tmem_base_slot, kTmemCols);
     }
 }
 
