@@ -189,7 +189,8 @@ CRISP_API crisp_status_t crisp_keep_ratio_for_count(const crisp_layer_desc_t *de
  * start-up, a process whose pool is fully committed).  The paper has no counterpart of this
  * call; it is a packaging variant of the mask projection.
  *
- * The scratch lives in a fixed array of CRISP_STATIC_SCRATCH_BYTES inside the library image;
+ * The scratch lives in a fixed array inside the library image (4.3 MiB: CRISP_STATIC_SCRATCH_BYTES for
+ * maximum and scores, and sixteen times that for what the scores are made from);
  * every GPU that loads the library holds it until the process exits.  The call allocates and
  * frees no device memory and calls no allocating CUDA routine; the only allocation is the small
  * host object behind the returned crisp_mask_t (a few dozen bytes from the C++ heap, freed by
@@ -197,15 +198,15 @@ CRISP_API crisp_status_t crisp_keep_ratio_for_count(const crisp_layer_desc_t *de
  * (crisp_mask_sizes gives its size) and the returned mask.
  *
  * Limits and rules
- *   - The layer's workspace (256 bytes + 8 bytes per coarse block, i.e. per (row tile,
- *     k-block) pair) must fit: at most 32736 coarse blocks.  Larger layers are refused with
+ *   - The layer's maximum and scores (256 bytes + 8 bytes per coarse block, i.e. per (row tile,
+ *     k-block) pair) must fit into CRISP_STATIC_SCRATCH_BYTES: at most 32736 coarse blocks.  Larger layers are refused with
  *     CRISP_BUFFER_TOO_SMALL before anything is launched; use crisp_build_mask for them.
  *   - Every call looks up the array's device address with the current device current; the first
  *     call on a device also makes the runtime load the library's module there.  Make that first
  *     call during set-up, before any stream capture begins.  The address is never kept across
  *     calls, so cudaDeviceReset or a second context on the device cannot leave a stale one.
  *   - All calls on a device share the one array, and it keeps what the last call wrote.  Each
- *     call clears it on `stream` before use, so calls issued one after another on the same
+ *     call writes what it reads of it on `stream` before use, so calls issued one after another on the same
  *     stream are safe; calls that may run concurrently on the GPU (different streams or host
  *     threads without ordering between them) race on it and give wrong masks.
  */

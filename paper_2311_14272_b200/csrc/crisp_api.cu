@@ -181,7 +181,7 @@ crisp_status_t crisp_build_mask_ex(const float *d_saliency, int64_t ld_s, const 
     mk->d_nm_bits = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(d_mask_buf) + blk_col_bytes(g));
     mk->image_kind = image_kind(g);
     cudaError_t e = crisp::launch_build_mask(d_saliency, ld_s, g, mk->d_blk_col, mk->d_nm_bits, d_workspace,
-                                             crisp::mask_workspace_bytes(g), (flags & CRISP_MASK_MAX_KNOWN) != 0,
+                                             (flags & CRISP_MASK_MAX_KNOWN) != 0,
                                              (cudaStream_t)stream);
     if (e != cudaSuccess) { delete mk; return CRISP_CUDA_ERROR; }
     *out = mk;
@@ -289,8 +289,8 @@ crisp_status_t crisp_prune_score(int32_t n_layers, const crisp_prune_layer_t *la
         crisp::ScoreLayer &S = sc[l];
         S.g = g;
         S.s = P.d_saliency; S.ld = P.ld_s;
-        S.max_key = reinterpret_cast<const uint32_t *>(P.d_workspace);
-        S.score = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(P.d_workspace) + kAlign);
+        S.maxima = nullptr; S.n_maxima = 0;
+        crisp::set_workspace(&S, P.d_workspace);
         S.blk_col = reinterpret_cast<int32_t *>(P.d_mask_buf);
         S.nm_bits = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(P.d_mask_buf) + blk_col_bytes(g));
     }
@@ -352,7 +352,7 @@ crisp_status_t crisp_prune_encode(int32_t n_layers, const crisp_prune_layer_t *l
         crisp::ScoreLayer &S = sc[l];
         S = crisp::ScoreLayer{};
         S.g = g;
-        S.score = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(P.d_workspace) + kAlign);
+        crisp::set_workspace(&S, P.d_workspace);
         S.blk_col = masks[l]->d_blk_col; S.nm_bits = masks[l]->d_nm_bits;
     }
     if (s == CRISP_OK) {

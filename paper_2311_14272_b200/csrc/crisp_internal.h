@@ -179,29 +179,35 @@ namespace crisp {
 
 // mask_kernels.cu
 cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, int32_t *d_blk_col,
-                              uint32_t *d_nm_bits, void *d_workspace, size_t workspace_bytes, bool max_known,
-                              cudaStream_t st);
-// One layer of a batched launch: the saliency that is scored, the group bits and scores (in the mask workspace) and where
-// the selection writes its block list.
+                              uint32_t *d_nm_bits, void *d_workspace, bool max_known, cudaStream_t st);
+// One layer of a batched launch: the saliency that is scored, the group bits, scores and what they are made from (in the mask workspace)
+// and where the selection writes its block list.
 struct ScoreLayer {
     Geometry g;
     const float *s;
     int64_t ld;
-    const uint32_t *max_key;
+    uint32_t *max_key;
+    const uint32_t *maxima;              // partial maxima that max_key is made from, n_maxima of them; nullptr: max_key stands
+    int n_maxima;
     uint32_t *nm_bits;
-    unsigned long long *score;
+    unsigned long long *score, *records;
     int32_t *blk_col;
-    int chunks, vec_ok;                  // (filled in by the launchers)
+    int vec_ok;                          // (filled in by the launchers)
 };
-cudaError_t launch_clear_scores(const ScoreLayer *layers, int n, cudaStream_t st);     // scores and max_key
+constexpr int kMaxMaxima = 2048;         // CTAs of the pass over S
+void set_workspace(ScoreLayer *L, void *d_workspace);        // max_key, score, records of a layer whose geometry is set
+// Whether only a group's n largest values count, so that they are found with minima and maxima (1, 2; 0: no).
+inline int top_counted(int n, bool all_count) { return !all_count && n <= 2 ? n : 0; }
+cudaError_t launch_clear_scores(const ScoreLayer *layers, int n, cudaStream_t st);     // max_key
 cudaError_t launch_block_scores(const ScoreLayer *layers, int n, cudaStream_t st);
 cudaError_t launch_block_selects(const ScoreLayer *layers, int n, cudaStream_t st);
 // per-row-tile selection alone, on the scores and group bits an earlier launch_build_mask left behind
 cudaError_t launch_block_select(const Geometry &g, const void *d_workspace, int32_t *d_blk_col, uint32_t *d_nm_bits,
                                 cudaStream_t st);
 size_t mask_workspace_bytes(const Geometry &g);
+size_t mask_score_bytes(const Geometry &g);                  // its first part: the maximum and the scores
 
-// saliency_kernels.cu: saliency, group bits and layer maxima of a network in one launch (max_key cleared before)
+// saliency_kernels.cu: saliency, group bits, score records and layer maxima of a network in one launch (max_key cleared before)
 cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreLayer *scores, int n, cudaStream_t st);
 
 // encode_kernels.cu

@@ -1,13 +1,11 @@
 // Mask projection kernels: saliency -> hybrid (block + N:M) mask.
 //
 // Algorithm 1 of the paper, restricted to one layer with the block keep count given:
-//   K-M1a per group of M: keep the N largest (fine-grained N:M step), and the layer-wide maximum
-//         of the canonical saliency (it sets the fixed-point scale): one pass over S from HBM
-//   K-M1b block scores s_j = sum |T_w| as exact fixed-point integers: second pass over S, which
-//         for layers up to the size of L2 is served from there
+//   K-M1a per group of M: keep the N largest (fine-grained N:M step), the layer-wide maximum of the canonical saliency (it sets
+//         the fixed-point scale of the scores), and sums of 32 x 32 elements in their own scale: the one pass over S
+//   K-M1b block scores s_j = sum |T_w| as exact fixed-point integers, from those sums
 //   K-M2  per row of the block grid: keep the kkeep highest-scored blocks and clear the
 //         bits of the pruned ones (blocks keep their positions)
-// Coalesced 32-byte-per-lane accesses; K-M1a is bound by HBM bandwidth.
 #include <atomic>
 
 #include "crisp_internal.h"
@@ -67,89 +65,79 @@ __device__ __forceinline__ unsigned long long fixed_point_score(uint32_t key, in
     return ((unsigned long long)__funnelshift_l(down, 0u, up) << 32) | (unsigned long long)(down << up);
 }
 
-// The 8 canonical keys of the lane's elements of row `row` (zero beyond the matrix).  kCap = false leaves infinities in.
-template <bool kCap = true>
-__device__ __forceinline__ void m1_load_rows(const float *s, int64_t ld, const Geometry &g, bool vec_ok,
-                                             const M1Item &x, int warp, int64_t k0, uint32_t key[kM1RowsPerWarp][8]) {
-    if (vec_ok && x.row0 + kM1Rows <= g.rows && (int64_t)(x.chunk + 1) * kM1ChunkK <= g.k) {   // interior item
+// Eight consecutive fp32 values from a 32-byte boundary, one load.
+__device__ __forceinline__ void load8_wide(const float *p, uint32_t key[8]) {
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(key[0]), "=r"(key[1]), "=r"(key[2]), "=r"(key[3]), "=r"(key[4]), "=r"(key[5]), "=r"(key[6]), "=r"(key[7]) : "l"(p) : "memory");
+}
+// Canonical bits of the lane's elements of a patch, zero beyond the matrix; vec_ok: S and its rows lie on 16-byte boundaries.
+__device__ __forceinline__ void load_patch(const float *s, int64_t ld, const Geometry &g, bool vec_ok, int64_t row0, int64_t col0, int lane,
+                                           uint32_t (&key)[kM1LaneRows][8]) {
+    const int64_t row = row0 + (lane >> 2), k0 = col0 + 8 * (lane & 3);
+    if (vec_ok && row0 + kM1Rows <= g.rows && k0 + 8 <= g.k) {
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i) load8_raw(s, ld, x.row0 + warp * kM1RowsPerWarp + i, k0, key[i]);
+        for (int i = 0; i < kM1LaneRows; ++i) load8_raw(s, ld, row + 8 * i, k0, key[i]);
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i)
+        for (int i = 0; i < kM1LaneRows; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                key[i][j] = kCap ? canonical_bits(key[i][j]) : __float_as_uint(fmaxf(fabsf(__uint_as_float(key[i][j])), 0.f));
+            for (int j = 0; j < 8; ++j) key[i][j] = canonical_bits(key[i][j]);
     } else {
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i)
-            load8(s, ld, g.rows, g.k, x.row0 + warp * kM1RowsPerWarp + i, k0, vec_ok, key[i]);
+        for (int i = 0; i < kM1LaneRows; ++i) load8(s, ld, g.rows, g.k, row + 8 * i, k0, vec_ok, key[i]);
     }
 }
 
-// K-M1a: the fine-grained N:M step (which does not depend on the score scale) and the layer maximum (which fixes
-// the scale) in ONE pass over S, the pass that comes from HBM: per group of M the N largest are marked, a lane
-// stores its eight mask bits as one byte, and the largest key goes to max_key (one atomic per CTA).
-// find_max = false when the caller already knows the maximum.
-template <int M>
-__global__ void __launch_bounds__(kM1Threads)
-group_bits_kernel(const float *s, int64_t ld, Geometry g, bool vec_ok, int64_t items, int chunks, bool find_max,
-                  uint32_t *max_key, uint32_t *nm_bits) {
+// K-M1a: the one pass over S.  The fine-grained N:M step does not depend on the score scale, and the sums of bits_and_record wait for it with a
+// shift, so mask bits, layer maximum (one partial maximum a CTA, in `maxima`; nullptr: known) and the records of the scores come from the same load.
+// What bounds it is DRAM: S comes in while the results of the calls in front, dirty in L2, leave for it (67 MB read and some 40 written back in 17 us; 13 instructions an
+// element fill 45 % of the issue slots).  Copies of the next patch into shared memory while this one is worked on (cp.async, two stages) gained nothing, 18.2 to
+// 18.5 us where this took 18.0; nor did 2 or 4 resident CTAs, 20.5 and 18.0.
+// align: of S and its rows, 32 bytes (one load for eight elements), 16 or less.
+template <int M, int TOP>
+__global__ void __launch_bounds__(kM1Threads, 3)
+group_bits_kernel(const float *s, int64_t ld, Geometry g, int align, int64_t items, uint32_t *maxima, uint32_t *nm_bits,
+                  unsigned long long *records) {
     __shared__ uint8_t s_keep[64];
-    __shared__ uint32_t s_best[kM1Threads / 32];
+    __shared__ uint32_t s_best[kM1Warps];
     chain_kernels();
     if (M == 4 && threadIdx.x < 64) s_keep[threadIdx.x] = (uint8_t)keep_mask_of_outcomes(threadIdx.x, g.n);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t best = 0u;
     for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-        const M1Item x = m1_item(it, chunks);
-        const int64_t k0 = (int64_t)x.chunk * kM1ChunkK + lane * 8;
-        uint32_t key[kM1RowsPerWarp][8];
-        m1_load_rows(s, ld, g, vec_ok, x, warp, k0, key);
-        const bool in_kp = k0 < g.kp();
+        const Patch x = patch_of(it, warp, g);
+        if (!x.any) continue;
+        const int64_t row = x.row0 + (lane >> 2), k0 = (int64_t)x.word * 32 + 8 * (lane & 3);
+        auto reload = [&](int i, uint32_t (&q)[8]) { load8(s, ld, g.rows, g.k, row + 8 * i, k0, align >= 16, q); };
+        uint32_t key[kM1LaneRows][8];
+        if (align >= 16 && x.row0 + kM1Rows <= g.rows && k0 + 8 <= g.k) {
+            const float *p = s + row * ld + k0;
+            if (align >= 32) {
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i) {
-            const int64_t row = x.row0 + warp * kM1RowsPerWarp + i;
-            uint32_t bits;
-            if constexpr (M == 4)
-                bits = (uint32_t)s_keep[outcomes4(key[i])] | ((uint32_t)s_keep[outcomes4(key[i] + 4)] << 4);
-            else
-                bits = top_n_bits<M>(key[i], g.n);
-            // the lane's eight bits are byte (k0 / 8) mod 4 of their little-endian mask word: a warp stores 32
-            // consecutive bytes of the row
-            if (in_kp) reinterpret_cast<uint8_t *>(nm_bits + row * g.wpr)[k0 >> 3] = (uint8_t)bits;
+                for (int i = 0; i < kM1LaneRows; ++i) load8_wide(p + 8 * i * ld, key[i]);
+            } else {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) best = max(best, key[i][j]);
+                for (int i = 0; i < kM1LaneRows; ++i) load8_raw(s, ld, row + 8 * i, k0, key[i]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kM1LaneRows; ++i) reload(i, key[i]);
         }
+        unsigned long long record;
+        const uint32_t bits = mask_words(bits_and_record<M, TOP>(key, g.n, g.score_mode != 0, s_keep, reload, best, record), lane);
+        nm_bits[(x.row0 + mask_word_row(lane)) * g.wpr + x.word] = bits;
+        if (lane == 0) records[x.at] = record;
     }
-    if (find_max) {
-        best = __reduce_max_sync(0xFFFFFFFFu, best);
+    if (maxima) {
         if (lane == 0) s_best[warp] = best;
         __syncthreads();
         if (threadIdx.x == 0) {
 #pragma unroll
-            for (int w = 1; w < kM1Threads / 32; ++w) best = max(best, s_best[w]);
-            if (best) atomicMax(max_key, best);
+            for (int w = 1; w < kM1Warps; ++w) best = max(best, s_best[w]);
+            maxima[blockIdx.x] = best;
         }
     }
 }
-
-// Two fp32 values in one 64-bit register and the packed fp32 instructions of sm_100 on them (one instruction
-// per pair; each half is rounded as the scalar instruction would round it).
-__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float f32x2_sum(uint64_t v) {       // lo + hi
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-    return __fadd_rn(lo, hi);
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ uint64_t add2_down(uint64_t a, uint64_t b) { uint64_t r; asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 
 // floor(v) of fp32 values 0 <= v < 2^41, two at a time, without a float-to-integer conversion per element (those
 // run at a fraction of the fp32 rate and were what bound this kernel): v = r + d with r = v rounded DOWN to a
@@ -164,126 +152,68 @@ __device__ __forceinline__ void floor_parts2(uint64_t v, uint64_t &r, uint64_t &
     fd = sub2(add2_down(sub2(v, r), mid), mid);
 }
 
-// The two largest of four values (as a pair; equal values count as often as they occur).
-struct Two { float a, b; };
-__device__ __forceinline__ Two top2_of4(float x0, float x1, float x2, float x3) {
-    const float h0 = fmaxf(x0, x1), l0 = fminf(x0, x1), h1 = fmaxf(x2, x3), l1 = fminf(x2, x3);
-    return Two{fmaxf(h0, h1), fmaxf(fminf(h0, h1), fmaxf(l0, l1))};
-}
-
-// K-M1b: the block scores s_j = sum |T_w| as exact fixed-point integers, once the scale is known.  Second pass
-// over S (for layers that fit, out of L2, where K-M1a left it).  Warps are independent (no shared memory, no
-// barrier): a lane adds floor(|s| * 2^(40 - e_max)) of its counted elements over its warp's four rows, the four lanes of a
-// 32-element word add up (a mask word never straddles a block: block_k is a multiple of 32), and one lane per word adds the
-// partial score to the block's 64-bit total with an atomic (integer addition: any order gives the same sum).
-// Which elements count: TOP = 0, the N:M survivors, read back as the byte K-M1a stored, or all of them.  TOP = 1 or 2
-// (score mode 0 and n = TOP): a group contributes the sum of its n largest values, whichever of equal ones the mask keeps,
-// so the values themselves are selected with minima and maxima and only they are scaled and floored: half of the
-// elements for 2:4, an eighth for 1:8.  Measured (4096 x 4096, 2:4, S of 64 MiB): 18.2 -> 14.4 us under ncu with a cold L2,
-// 4.4 us off the mask phase in a stream; what is left is mostly the wait between an item's loads and the next item's.
-template <int CAP, int M, int TOP>
+// K-M1b: the block scores from the records of K-M1a, once the scale is known: a warp a block, a lane a record.  A record whose sum does
+// not stand (see bits_and_record) has its 32 x 32 elements counted again, the mask bits telling which.
+// Measured (us, 4096 x 4096, 2:4, S of 64 MiB): the pass over S and this kernel 17.0 + 3.8, where a memset, a pass for bits and maximum and a second one
+// for the scores took 1.8 + 16.2 + 11.4; mask, encoding and decoding in a row 59.3 -> 47.2.
+template <int CAP>
 __global__ void __launch_bounds__(kM1Threads)
 block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
+    __shared__ uint32_t s_best[kM1Threads / 32];
     chain_kernels();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t unit = blockIdx.x; unit < batch.first[batch.n]; unit += gridDim.x) {
-    const int l = batch.find(unit);
+    const int l = batch.find(blockIdx.x);
     const ScoreLayer &L = batch.layer[l];
     const Geometry &g = L.g;
-    const float *s = L.s;
-    const int64_t ld = L.ld;
-    const uint32_t *nm_bits = L.nm_bits;
-    const uint32_t mk = *L.max_key;
-    if (!mk) continue;                                       // an all-zero layer: every score stays 0
-    const int e_max = key_exponent(mk);
-    // floor(value * 2^(40 - e_max)): when that power of two is an fp32 number, the product is exact
-    // (value <= layer maximum, so it stays below 2^41)
-    const int scale_exp = kScoreFractionBits - e_max;
-    const bool float_scale = scale_exp >= -126 && scale_exp <= 127;
-    const float scale = float_scale ? __uint_as_float((uint32_t)(127 + scale_exp) << 23) : 0.f;
-        const M1Item x = m1_item(unit - batch.first[l], L.chunks);
-        const int64_t k0 = (int64_t)x.chunk * kM1ChunkK + lane * 8;
-        const int rt = (int)(x.row0 / g.bm);
-        uint32_t key[kM1RowsPerWarp][8];
-        m1_load_rows<TOP == 0>(s, ld, g, L.vec_ok != 0, x, warp, k0, key);
-        const bool in_kp = k0 < g.kp();
-        unsigned long long acc = 0ull;
-        if (TOP != 0 && float_scale) {
-            uint64_t r_sum = f32x2(0.f, 0.f), d_sum = r_sum;                     // exact for eight values: see floor_parts2
-            auto count = [&](float a, float b) {
-                uint64_t r, fd;
-                floor_parts2(mul2(f32x2(fminf(a, 3.402823466e+38f), fminf(b, 3.402823466e+38f)), f32x2(scale, scale)), r, fd);
-                r_sum = add2(r_sum, r);
-                d_sum = add2(d_sum, fd);
-            };
-            auto flush = [&]() {
-                acc += ((unsigned long long)__float2uint_rn(f32x2_sum(r_sum) * 9.5367431640625e-07f) << 20) +
-                       (unsigned long long)__float2uint_rn(f32x2_sum(d_sum));
-                r_sum = d_sum = f32x2(0.f, 0.f);
-            };
-            float best_before = 0.f;
+    const int64_t cta = blockIdx.x - batch.first[l], block = cta * (kM1Threads / 32) + warp;
+    uint32_t mk;
+    if (L.maxima) {
+        mk = 0u;
+        for (int i = threadIdx.x; i < L.n_maxima; i += kM1Threads) mk = max(mk, L.maxima[i]);
+        mk = __reduce_max_sync(0xFFFFFFFFu, mk);
+        if (lane == 0) s_best[warp] = mk;
+        __syncthreads();
 #pragma unroll
-            for (int i = 0; i < kM1RowsPerWarp; ++i) {
-                float v[8];
+        for (int w = 0; w < kM1Threads / 32; ++w) mk = max(mk, s_best[w]);
+        if (cta == 0 && threadIdx.x == 0) *L.max_key = mk;
+    } else {
+        mk = *L.max_key;
+    }
+    if (block >= (int64_t)g.nrt * g.nblk) return;
+    const int rt = (int)(block / g.nblk), jb = (int)(block - (int64_t)rt * g.nblk);
+    const int wpb = g.bk / 32, parts = g.bm / kM1Rows * wpb;                   // at most 16
+    const int64_t rec0 = (int64_t)rt * (g.bm / kM1Rows) * g.wpr + jb * wpb;    // (a record a mask word of every 32nd row)
+    unsigned long long acc = 0ull;
+    bool stands = true;
+    if (lane < parts) {
+        const unsigned long long rec = L.records[rec0 + lane / wpb * g.wpr + lane % wpb];
+        const int d = (int)(mk >> 23) - (int)(rec >> kRecordExpShift), code = (int)(rec >> kRecordCodeShift) & 31;
+        const unsigned long long sum = rec & kRecordSum;
+        // nothing counted; all elements below one unit; or a sum that stands
+        if (code == 18 && sum == 0ull) acc = 0ull;
+        else if (d >= kScoreFractionBits + 1) acc = 0ull;
+        else if (d >= 0 && d < code) acc = sum >> d;
+        else stands = false;
+    }
+    const int e_max = mk ? key_exponent(mk) : 0;
+    for (uint32_t left = __ballot_sync(0xFFFFFFFFu, !stands); left; left &= left - 1u) {
+        const int part = __ffs(left) - 1;
+        const int64_t row0 = (int64_t)rt * g.bm + part / wpb * kM1Rows;
+        const int word = jb * wpb + part % wpb;
+        uint32_t key[kM1LaneRows][8];
+        load_patch(L.s, L.ld, g, L.vec_ok != 0, row0, (int64_t)word * 32, lane, key);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(key[i][j]);
-                const Two p = top2_of4(v[0], v[1], v[2], v[3]), q = top2_of4(v[4], v[5], v[6], v[7]);
-                if constexpr (TOP == 2 && M == 4) {
-                    count(p.a, p.b);
-                    count(q.a, q.b);
-                    if (i & 1) flush();
-                } else if constexpr (TOP == 1 && M == 4) {
-                    count(p.a, q.a);
-                } else if constexpr (TOP == 2) {
-                    count(fmaxf(p.a, q.a), fmaxf(fminf(p.a, q.a), fmaxf(p.b, q.b)));
-                } else {
-                    if (i & 1) count(best_before, fmaxf(p.a, q.a));
-                    best_before = fmaxf(p.a, q.a);
-                }
-            }
-            if (!(TOP == 2 && M == 4)) flush();
-        } else if (float_scale) {
+        for (int i = 0; i < kM1LaneRows; ++i) {
+            uint32_t counted = 0xFFu;
+            if (g.score_mode == 0) counted = L.nm_bits[(row0 + (lane >> 2) + 8 * i) * g.wpr + word] >> (8 * (lane & 3));
 #pragma unroll
-            for (int i = 0; i < kM1RowsPerWarp; ++i) {
-                const int64_t row = x.row0 + warp * kM1RowsPerWarp + i;
-                uint32_t counted = 0xFFu;
-                if (g.score_mode == 0) counted = in_kp ? reinterpret_cast<const uint8_t *>(nm_bits + row * g.wpr)[k0 >> 3] : 0u;
-                // an element that is not counted is multiplied by zero instead of by the scale: its parts are zero
-                uint64_t r_sum = f32x2(0.f, 0.f), d_sum = r_sum;             // exact: see floor_parts2
-#pragma unroll
-                for (int j = 0; j < 8; j += 2) {
-                    const uint64_t sc = f32x2((counted >> j) & 1u ? scale : 0.f, (counted >> (j + 1)) & 1u ? scale : 0.f);
-                    uint64_t r, fd;
-                    floor_parts2(mul2(f32x2(__uint_as_float(key[i][j]), __uint_as_float(key[i][j + 1])), sc), r, fd);
-                    r_sum = add2(r_sum, r);
-                    d_sum = add2(d_sum, fd);
-                }
-                acc += ((unsigned long long)__float2uint_rn(f32x2_sum(r_sum) * 9.5367431640625e-07f) << 20) +
-                       (unsigned long long)__float2uint_rn(f32x2_sum(d_sum));
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < kM1RowsPerWarp; ++i) {
-                const int64_t row = x.row0 + warp * kM1RowsPerWarp + i;
-                uint32_t counted = 0xFFu;
-                if (g.score_mode == 0) counted = in_kp ? reinterpret_cast<const uint8_t *>(nm_bits + row * g.wpr)[k0 >> 3] : 0u;
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if ((counted >> j) & 1u) acc += fixed_point_score(canonical_bits(key[i][j]), e_max);
-            }
-        }
-        acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 1);
-        acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 2);
-        // lanes that share a block column (block_k / 8 of them, 4, 8, 12 or 16): add up as far as the lane groups
-        // of a power of two allow, then one atomic per group
-        if (g.bk % 64 == 0) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 4);
-        if (g.bk % 128 == 0) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 8);
-        const int grp = g.bk % 128 == 0 ? 15 : (g.bk % 64 == 0 ? 7 : 3);
-        if ((lane & grp) == 0 && in_kp && acc) {
-            const int jb = (int)(k0 / g.bk);
-            if (jb < g.nblk) atomicAdd(&L.score[(int64_t)rt * g.nblk + jb], acc);
+            for (int j = 0; j < 8; ++j)
+                if ((counted >> j) & 1u) acc += fixed_point_score(key[i][j], e_max);
         }
     }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    if (lane == 0) L.score[block] = acc;
 }
 
 // K-M2.  One CTA per 32 rows of a row tile.  Every CTA ranks its row tile's block scores (cheap)
@@ -503,15 +433,12 @@ int small_ctas(const Geometry &g) {
     return g.nblk <= kSmallMaxBlocks && row_tiles <= 2 && (int64_t)row_tiles * g.bm * g.kp() <= kSmallPerCta ? ctas : 0;
 }
 
-// Scores and maxima of a batch, cleared (one CTA per layer; a memset per layer costs a launch each).
+// Maxima of a batch, cleared (a memset per layer costs a launch each).
 template <int CAP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kBatchLayers)
 clear_scores_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
     chain_kernels();
-    const ScoreLayer &L = batch.layer[blockIdx.x];
-    if (threadIdx.x == 0) *const_cast<uint32_t *>(L.max_key) = 0u;
-    const int64_t n = (int64_t)L.g.nrt * L.g.nblk;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) L.score[i] = 0ull;
+    if ((int)threadIdx.x < batch.n) *batch.layer[threadIdx.x].max_key = 0u;
 }
 
 // Grids of resident CTAs: every CTA is on an SM from the start and takes its share of the items.  What a device holds of a
@@ -528,14 +455,7 @@ int resident_grid(void (*kern)(Params...), std::atomic<int> *capacity, int64_t i
     }
     return (int)(items < cap ? items : cap);
 }
-template <int M>
-int group_bits_grid(int64_t items) {
-    static std::atomic<int> capacity[kMaxDevices];
-    return resident_grid(group_bits_kernel<M>, capacity, items);
-}
-
 bool saliency_vec_ok(const float *s, int64_t ld) { return (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(s) & 15u) == 0); }
-int saliency_chunks(const Geometry &g) { return (int)((g.kp() + kM1ChunkK - 1) / kM1ChunkK); }
 
 // Layers [0, n) in launches of up to kBatchLayers; units(layer) = work units of a layer, launch(batch, units of the batch).
 template <typename Units, typename Launch>
@@ -546,7 +466,6 @@ cudaError_t for_batches(const ScoreLayer *layers, int n, Units units, Launch lau
         b.first[0] = 0;
         for (int i = 0; i < b.n; ++i) {
             b.layer[i] = layers[at + i];
-            b.layer[i].chunks = saliency_chunks(b.layer[i].g);
             b.layer[i].vec_ok = saliency_vec_ok(b.layer[i].s, b.layer[i].ld);
             b.first[i + 1] = b.first[i] + units(b.layer[i].g);
         }
@@ -560,27 +479,25 @@ Batch<ScoreLayer, 1> batch_of_one(const ScoreLayer &L, int64_t units) {
     Batch<ScoreLayer, 1> b;
     b.n = 1; b.first[0] = 0; b.first[1] = units;
     b.layer[0] = L;
-    b.layer[0].chunks = saliency_chunks(L.g);
     b.layer[0].vec_ok = saliency_vec_ok(L.s, L.ld);
     return b;
 }
 
-template <int CAP, int M, int TOP>
-cudaError_t run_block_scores(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
+template <int M, int TOP>
+cudaError_t run_group_bits(const ScoreLayer &L, int *ctas, cudaStream_t st) {
     static std::atomic<int> capacity[kMaxDevices];
-    const int grid = resident_grid(block_score_kernel<CAP, M, TOP>, capacity, b.first[b.n]);
-    return launch_chained(block_score_kernel<CAP, M, TOP>, (unsigned)grid, kM1Threads, 0, st, b);
+    const int64_t items = patch_ctas(L.g);
+    if (items > 0x0FFFFFFF) return cudaErrorInvalidValue;    // (patches are numbered in 32 bits: 2^31 of them are 2^41 elements)
+    const int align = L.ld % 8 == 0 && reinterpret_cast<uintptr_t>(L.s) % 32 == 0 ? 32 : saliency_vec_ok(L.s, L.ld) ? 16 : 4;
+    *ctas = resident_grid(group_bits_kernel<M, TOP>, capacity, items < kMaxMaxima ? items : kMaxMaxima);
+    return launch_chained(group_bits_kernel<M, TOP>, (unsigned)*ctas, kM1Threads, 0, st, L.s, L.ld, L.g, align, items,
+                          const_cast<uint32_t *>(L.maxima), L.nm_bits, const_cast<unsigned long long *>(L.records));
 }
-// The selecting forms where n is 1 or 2 and only survivors count (all layers of a launch share n and m); from n = 3 on the
-// selection network is longer than the work it saves.
+
+int64_t score_ctas(const Geometry &g) { return ((int64_t)g.nrt * g.nblk + kM1Threads / 32 - 1) / (kM1Threads / 32); }
 template <int CAP>
-cudaError_t run_block_scores_any(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
-    const Geometry &g = b.layer[0].g;
-    bool survivors = true;
-    for (int i = 0; i < b.n; ++i) survivors = survivors && b.layer[i].g.score_mode == 0;
-    if (survivors && g.n == 1) return g.m == 4 ? run_block_scores<CAP, 4, 1>(b, st) : run_block_scores<CAP, 8, 1>(b, st);
-    if (survivors && g.n == 2) return g.m == 4 ? run_block_scores<CAP, 4, 2>(b, st) : run_block_scores<CAP, 8, 2>(b, st);
-    return run_block_scores<CAP, 4, 0>(b, st);
+cudaError_t run_block_scores(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
+    return launch_chained(block_score_kernel<CAP>, (unsigned)b.first[b.n], kM1Threads, 0, st, b);
 }
 
 size_t select_smem(int nblk) { return (size_t)nblk * (sizeof(unsigned long long) + sizeof(int)); }
@@ -601,20 +518,27 @@ cudaError_t run_block_select(const Batch<ScoreLayer, CAP> &b, cudaStream_t st) {
 
 }  // namespace
 
-// workspace: [0] max key (uint32), padded to 256 B; then score[nrt * nblk] uint64.
-size_t mask_workspace_bytes(const Geometry &g) {
-    return kAlign + align_up((size_t)g.nrt * g.nblk * sizeof(unsigned long long));
+// workspace: [0] max key (uint32), padded to 256 B; then score[nrt * nblk] uint64; the records of the pass over S, a uint64 for 32 x 32
+// elements; and that pass's partial maxima.
+static size_t score_bytes(const Geometry &g) { return align_up((size_t)g.nrt * g.nblk * sizeof(unsigned long long)); }
+static size_t record_bytes(const Geometry &g) { return align_up((size_t)(g.mp() / kM1Rows) * g.wpr * sizeof(unsigned long long)); }
+size_t mask_workspace_bytes(const Geometry &g) { return mask_score_bytes(g) + record_bytes(g) + kMaxMaxima * sizeof(uint32_t); }
+size_t mask_score_bytes(const Geometry &g) { return kAlign + score_bytes(g); }
+void set_workspace(ScoreLayer *L, void *d_workspace) {
+    uint8_t *ws = reinterpret_cast<uint8_t *>(d_workspace);
+    L->max_key = reinterpret_cast<uint32_t *>(ws);
+    L->score = reinterpret_cast<unsigned long long *>(ws + kAlign);
+    L->records = reinterpret_cast<unsigned long long *>(ws + mask_score_bytes(L->g));
 }
 
 cudaError_t launch_clear_scores(const ScoreLayer *layers, int n, cudaStream_t st) {
     return for_batches(layers, n, [](const Geometry &) { return (int64_t)1; }, [&](const Batch<ScoreLayer, kBatchLayers> &b) {
-        return launch_chained(clear_scores_kernel<kBatchLayers>, (unsigned)b.n, 256, 0, st, b);
+        return launch_chained(clear_scores_kernel<kBatchLayers>, 1u, kBatchLayers, 0, st, b);
     });
 }
 
 cudaError_t launch_block_scores(const ScoreLayer *layers, int n, cudaStream_t st) {
-    return for_batches(layers, n, [](const Geometry &g) { return (g.mp() / kM1Rows) * (int64_t)saliency_chunks(g); },
-                       [&](const Batch<ScoreLayer, kBatchLayers> &b) { return run_block_scores_any(b, st); });
+    return for_batches(layers, n, score_ctas, [&](const Batch<ScoreLayer, kBatchLayers> &b) { return run_block_scores(b, st); });
 }
 
 cudaError_t launch_block_selects(const ScoreLayer *layers, int n, cudaStream_t st) {
@@ -625,43 +549,31 @@ cudaError_t launch_block_select(const Geometry &g, const void *d_workspace, int3
                                 cudaStream_t st) {
     ScoreLayer L = {};
     L.g = g; L.nm_bits = d_nm_bits; L.blk_col = d_blk_col;
-    L.score = reinterpret_cast<unsigned long long *>(const_cast<uint8_t *>(reinterpret_cast<const uint8_t *>(d_workspace)) + kAlign);
+    set_workspace(&L, const_cast<void *>(d_workspace));
     return run_block_select(batch_of_one(L, select_ctas(g)), st);
 }
 
 cudaError_t launch_build_mask(const float *d_s, int64_t ld, const Geometry &g, int32_t *d_blk_col,
-                              uint32_t *d_nm_bits, void *d_workspace, size_t workspace_bytes, bool max_known,
-                              cudaStream_t st) {
-    uint32_t *max_key = reinterpret_cast<uint32_t *>(d_workspace);
-    unsigned long long *score =
-        reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(d_workspace) + kAlign);
+                              uint32_t *d_nm_bits, void *d_workspace, bool max_known, cudaStream_t st) {
+    ScoreLayer L = {};
+    L.g = g; L.s = d_s; L.ld = ld; L.nm_bits = d_nm_bits; L.blk_col = d_blk_col;
+    set_workspace(&L, d_workspace);
     if (const int ctas = small_ctas(g)) {
         auto launch = [&](auto kern) {
-            return launch_clusters(kern, (unsigned)ctas, kSmallThreads, 0, st, (unsigned)ctas, d_s, ld, g, saliency_vec_ok(d_s, ld), max_known, max_key,
-                                   score, d_nm_bits, d_blk_col, ctas);
+            return launch_clusters(kern, (unsigned)ctas, kSmallThreads, 0, st, (unsigned)ctas, d_s, ld, g, saliency_vec_ok(d_s, ld), max_known, L.max_key,
+                                   L.score, d_nm_bits, d_blk_col, ctas);
         };
         return g.m == 4 ? launch(mask_small_kernel<4>) : launch(mask_small_kernel<8>);
     }
-    // max_known: the first word already holds the layer's largest canonical |s| (written by the saliency kernel
-    // that produced S), so only the scores are cleared and the pass over S that finds the maximum is skipped
-    cudaError_t e = max_known ? cudaMemsetAsync(score, 0, workspace_bytes - kAlign, st)
-                              : cudaMemsetAsync(d_workspace, 0, workspace_bytes, st);
-    if (e != cudaSuccess) return e;
-    const bool vec_ok = saliency_vec_ok(d_s, ld);
-
-    // work items of 32 rows x 256 k-elements, dealt out to resident CTAs
-    const int chunks = saliency_chunks(g);
-    const int64_t items = (g.mp() / kM1Rows) * chunks;
-    if (g.m == 4)
-        group_bits_kernel<4><<<group_bits_grid<4>(items), kM1Threads, 0, st>>>(
-            d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
-    else
-        group_bits_kernel<8><<<group_bits_grid<8>(items), kM1Threads, 0, st>>>(
-            d_s, ld, g, vec_ok, items, chunks, !max_known, max_key, d_nm_bits);
-    ScoreLayer L = {};
-    L.g = g; L.s = d_s; L.ld = ld; L.max_key = max_key; L.nm_bits = d_nm_bits; L.score = score; L.blk_col = d_blk_col;
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = run_block_scores_any(batch_of_one(L, items), st);
+    // max_known: the first word already holds the layer's largest canonical |s| (written by the saliency kernel that produced S)
+    if (!max_known)
+        L.maxima = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(d_workspace) + mask_score_bytes(g) + record_bytes(g));
+    const int top = top_counted(g.n, g.score_mode != 0);
+    cudaError_t e = g.m == 4 ? (top == 0 ? run_group_bits<4, 0>(L, &L.n_maxima, st) : top == 1 ? run_group_bits<4, 1>(L, &L.n_maxima, st)
+                                                                                              : run_group_bits<4, 2>(L, &L.n_maxima, st))
+                             : (top == 0 ? run_group_bits<8, 0>(L, &L.n_maxima, st) : top == 1 ? run_group_bits<8, 1>(L, &L.n_maxima, st)
+                                                                                              : run_group_bits<8, 2>(L, &L.n_maxima, st));
+    if (e == cudaSuccess) e = run_block_scores(batch_of_one(L, score_ctas(g)), st);
     if (e != cudaSuccess) return e;
     return run_block_select(batch_of_one(L, select_ctas(g)), st);
 }

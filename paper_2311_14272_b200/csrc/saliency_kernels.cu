@@ -97,16 +97,21 @@ saliency_finish_kernel(const float *__restrict__ acc, int64_t ld_a, const uint16
 //     S = |(g_0 + g_1 + ...) * (1 / H) * W|  (fp32, each step rounded, the order of the calls above)
 // The sum stays in registers: a sample costs its own bytes once (2 or 4 an element), where one launch per sample adds a
 // read and a write of the fp32 accumulator to them; the bits and the maximum come from the values the thread already
-// holds instead of from another pass over S.  Work items of 32 rows x 256 elements as in the mask kernels; a lane owns eight
-// consecutive elements of four rows.  Bound by HBM; what a small network waits for is latency, so items are CTAs of
-// their own and all layers share the launch.  Measured (13 layers of VGG-16, 14.7 M weights, four bf16 samples, 206 MB):
-// 44 to 48 us, against 390 us for the launches it replaces (52 accumulations, 13 finishing passes, 13 bit passes).
+// holds instead of from another pass over S, and so do the records that the block scores are made of (bits_and_record's, of 32 x 32 elements: the
+// CTA's 16 warps agree on a scale through shared memory).  Work items of 32 rows x 256 elements; a lane owns eight consecutive elements of two
+// rows, and a warp 512 consecutive bytes of each row (32 x 32 elements a warp: 64 us on the first below, twice the requests).  Bound by HBM; what a small network waits
+// for is latency, so items are CTAs of their own, all layers share the launch and a sample is asked for before the last one is added.
+// Measured (us, this kernel and the score kernel; 13 layers of VGG-16, 14.7 M weights, four bf16 samples, 206 MB): 52.2 + 3.4, before the
+// records 51.1 + 14.8; 35 layers of MobileNetV2 13.0 + 3.2, 15.0 + 5.8.  Four rows a lane 56.5 and 17.1, two CTAs an SM 53.6 and 15.9.
+constexpr int kSalChunk = 256, kSalWords = kSalChunk / 32;                     // k-elements of a work item: 32 lanes x 8
+constexpr int kSalLaneRows = 2, kSalItemThreads = kM1Rows / kSalLaneRows * 32;
 struct SaliencyLayer {
     Geometry g;
     const uint16_t *w;
     float *s;
     int64_t ld_w, ld_s;
     uint32_t *max_key, *nm_bits;
+    unsigned long long *records;
     float inv;
     int grad0, samples, chunks, vec_ok;
 };
@@ -121,34 +126,46 @@ struct SaliencyBatch {
 };
 static_assert(sizeof(SaliencyBatch) < 32000, "kernel parameters");
 
-template <int M>
-__global__ void __launch_bounds__(kM1Threads)
+template <int M, int TOP>
+__global__ void __launch_bounds__(kSalItemThreads, 3)
 saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
     __shared__ uint8_t s_keep[64];
-    __shared__ uint32_t s_best[kM1Threads / 32];
+    __shared__ uint32_t s_top[kSalWords], s_low[kSalWords], s_r[kSalWords];        // of the CTA's 32 x 32 elements in a mask word's columns
+    __shared__ int s_d[kSalWords];
     chain_kernels();
     const int l = batch.b.find(blockIdx.x);
     const SaliencyLayer &L = batch.b.layer[l];
     const Geometry &g = L.g;
     if (M == 4 && threadIdx.x < 64) s_keep[threadIdx.x] = (uint8_t)keep_mask_of_outcomes(threadIdx.x, g.n);
+    if (threadIdx.x < kSalWords) { s_top[threadIdx.x] = 0u; s_low[threadIdx.x] = 0xFFFFFFFFu; s_r[threadIdx.x] = 0u; s_d[threadIdx.x] = 0; }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const M1Item x = m1_item(blockIdx.x - batch.b.first[l], L.chunks);
-    const int64_t k0 = (int64_t)x.chunk * kM1ChunkK + lane * 8;
-    const int64_t row0 = x.row0 + warp * kM1RowsPerWarp;
-    float v[kM1RowsPerWarp][8];
-    if (L.vec_ok && row0 + kM1RowsPerWarp <= g.rows && k0 + 8 <= g.k) {
-        uint4 wr[kM1RowsPerWarp];
+    const uint32_t item = blockIdx.x - (uint32_t)batch.b.first[l], rg = item / (uint32_t)L.chunks, chunk = item - rg * (uint32_t)L.chunks;
+    const int64_t k0 = (int64_t)chunk * kSalChunk + lane * 8;
+    const int64_t row0 = (int64_t)rg * kM1Rows + warp * kSalLaneRows;
+    float v[kSalLaneRows][8];
+    if (L.vec_ok && row0 + kSalLaneRows <= g.rows && k0 + 8 <= g.k) {
+        uint4 wr[kSalLaneRows];
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i) wr[i] = *reinterpret_cast<const uint4 *>(L.w + (row0 + i) * L.ld_w + k0);
+        for (int i = 0; i < kSalLaneRows; ++i) wr[i] = *reinterpret_cast<const uint4 *>(L.w + (row0 + i) * L.ld_w + k0);
+        // (a bf16 sample is asked for before the one in front of it is added)
+        uint4 t[kSalLaneRows];
+        auto ask = [&](const GradRef &G, uint4 (&to)[kSalLaneRows]) {
+#pragma unroll
+            for (int i = 0; i < kSalLaneRows; ++i)
+                to[i] = *reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(G.p) + (row0 + i) * G.ld + k0);
+        };
+        GradRef G = batch.grad[L.grad0];
+        if (G.ld > 0) ask(G, t);
         for (int h = 0; h < L.samples; ++h) {
-            const GradRef G = batch.grad[L.grad0 + h];
+            uint4 next[kSalLaneRows];
+            GradRef N = G;
+            if (h + 1 < L.samples) {
+                N = batch.grad[L.grad0 + h + 1];
+                if (N.ld > 0) ask(N, next);
+            }
             if (G.ld > 0) {
-                uint4 t[kM1RowsPerWarp];
 #pragma unroll
-                for (int i = 0; i < kM1RowsPerWarp; ++i)
-                    t[i] = *reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(G.p) + (row0 + i) * G.ld + k0);
-#pragma unroll
-                for (int i = 0; i < kM1RowsPerWarp; ++i) {
+                for (int i = 0; i < kSalLaneRows; ++i) {
                     const uint32_t q[4] = {t[i].x, t[i].y, t[i].z, t[i].w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -159,7 +176,7 @@ saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < kM1RowsPerWarp; ++i) {
+                for (int i = 0; i < kSalLaneRows; ++i) {
                     const float4 *p = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(G.p) + (row0 + i) * -G.ld + k0);
                     const float4 a = p[0], b = p[1];
                     const float q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -167,9 +184,12 @@ saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
                     for (int j = 0; j < 8; ++j) v[i][j] = h ? __fadd_rn(v[i][j], q[j]) : q[j];
                 }
             }
+            G = N;
+#pragma unroll
+            for (int i = 0; i < kSalLaneRows; ++i) t[i] = next[i];
         }
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i) {
+        for (int i = 0; i < kSalLaneRows; ++i) {
             const uint32_t q[4] = {wr[i].x, wr[i].y, wr[i].z, wr[i].w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -182,7 +202,7 @@ saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < kM1RowsPerWarp; ++i)
+        for (int i = 0; i < kSalLaneRows; ++i)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int64_t row = row0 + i, k = k0 + j;
@@ -200,26 +220,46 @@ saliency_bits_kernel(const __grid_constant__ SaliencyBatch batch) {
                 v[i][j] = a;
             }
     }
-    if (M == 4) __syncthreads();
-    uint32_t best = 0u;
+    __syncthreads();                                         // (the tables)
+    uint32_t key[kSalLaneRows][8];
+#pragma unroll
+    for (int i = 0; i < kSalLaneRows; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) key[i][j] = __float_as_uint(v[i][j]) & 0x7FFFFFFFu;
+    auto reload = [&](int i, uint32_t (&q)[8]) {             // (this thread's own stores)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) q[j] = row0 + i < g.rows && k0 + j < g.k ? canonical_bits(__float_as_uint(L.s[(row0 + i) * L.ld_s + k0 + j])) : 0u;
+    };
+    float counted[kSalLaneRows][kCounted<M, TOP>];
+    uint32_t top;
+    const uint32_t bits = select_rows<M, TOP>(key, g.n, g.score_mode != 0, s_keep, reload, counted, top);
     const bool in_kp = k0 < g.kp();
+    // a lane's eight bits are byte (k0 / 8) mod 4 of their little-endian mask word: a warp stores 32 consecutive bytes of a row
+    if (in_kp)
 #pragma unroll
-    for (int i = 0; i < kM1RowsPerWarp; ++i) {
-        uint32_t key[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { key[j] = canonical_bits(__float_as_uint(v[i][j])); best = max(best, key[j]); }
-        uint32_t bits;
-        if constexpr (M == 4) bits = (uint32_t)s_keep[outcomes4(key)] | ((uint32_t)s_keep[outcomes4(key + 4)] << 4);
-        else bits = top_n_bits<M>(key, g.n);
-        if (in_kp) reinterpret_cast<uint8_t *>(L.nm_bits + (row0 + i) * g.wpr)[k0 >> 3] = (uint8_t)bits;
-    }
-    best = __reduce_max_sync(0xFFFFFFFFu, best);
-    if (lane == 0) s_best[warp] = best;
+        for (int i = 0; i < kSalLaneRows; ++i) reinterpret_cast<uint8_t *>(L.nm_bits + (row0 + i) * g.wpr)[k0 >> 3] = (uint8_t)(bits >> (8 * i));
+    // A record is of four lanes of every warp: their largest first, for the unit that all of them add up in.
+    const int q = lane >> 2;
+    top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, 1));
+    top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, 2));
+    if ((lane & 3) == 0) atomicMax(&s_top[q], top);
     __syncthreads();
-    if (threadIdx.x == 0) {
+    top = s_top[q];
+    LaneSums s = sum_rows<M, TOP>(counted, (int)(top >> 23));
 #pragma unroll
-        for (int w = 1; w < kM1Threads / 32; ++w) best = max(best, s_best[w]);
-        if (best) atomicMax(L.max_key, best);
+    for (int o = 1; o <= 2; o <<= 1) {
+        s.low = min(s.low, __shfl_xor_sync(0xFFFFFFFFu, s.low, o));
+        s.r += __shfl_xor_sync(0xFFFFFFFFu, s.r, o);
+        s.d += __shfl_xor_sync(0xFFFFFFFFu, s.d, o);
+    }
+    if ((lane & 3) == 0) { atomicMin(&s_low[q], s.low); atomicAdd(&s_r[q], s.r); atomicAdd(&s_d[q], s.d); }
+    __syncthreads();
+    if (threadIdx.x < kSalWords) {
+        const int word = (int)chunk * kSalWords + (int)threadIdx.x;
+        const uint32_t t = s_top[threadIdx.x];
+        if (word < g.wpr) L.records[(int64_t)rg * g.wpr + word] = make_record((int)(t >> 23), s_low[threadIdx.x], s_r[threadIdx.x], s_d[threadIdx.x]);
+        const uint32_t best = __reduce_max_sync((1u << kSalWords) - 1u, t);
+        if (threadIdx.x == 0 && best) atomicMax(L.max_key, best);
     }
 }
 
@@ -248,8 +288,12 @@ cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreL
     auto flush = [&]() -> cudaError_t {
         if (b.n == 0) return cudaSuccess;
         if (b.first[b.n] > 0x7FFFFFFFll) return cudaErrorInvalidValue;
-        const cudaError_t e = launch_chained(b.layer[0].g.m == 4 ? saliency_bits_kernel<4> : saliency_bits_kernel<8>,
-                                             (unsigned)b.first[b.n], kM1Threads, 0, st, *batch);
+        bool all_count = false;                              // (score modes may differ between the layers of a call, n and m may not)
+        for (int i = 0; i < b.n; ++i) all_count = all_count || b.layer[i].g.score_mode != 0;
+        const int top = top_counted(b.layer[0].g.n, all_count);
+        const auto kern = b.layer[0].g.m == 4 ? (top == 0 ? saliency_bits_kernel<4, 0> : top == 1 ? saliency_bits_kernel<4, 1> : saliency_bits_kernel<4, 2>)
+                                              : (top == 0 ? saliency_bits_kernel<8, 0> : top == 1 ? saliency_bits_kernel<8, 1> : saliency_bits_kernel<8, 2>);
+        const cudaError_t e = launch_chained(kern, (unsigned)b.first[b.n], kSalItemThreads, 0, st, *batch);
         b.n = 0; grads = 0;
         return e;
     };
@@ -272,10 +316,10 @@ cudaError_t launch_saliency_bits(const crisp_prune_layer_t *layers, const ScoreL
         L.g = S.g;
         L.w = P.d_w_bf16; L.ld_w = P.ld_w;
         L.s = P.d_saliency; L.ld_s = P.ld_s;
-        L.max_key = const_cast<uint32_t *>(S.max_key); L.nm_bits = S.nm_bits;
+        L.max_key = S.max_key; L.nm_bits = S.nm_bits; L.records = S.records;
         L.inv = 1.0f / (float)P.samples;
+        L.chunks = (int)((S.g.kp() + kSalChunk - 1) / kSalChunk);
         L.grad0 = grads; L.samples = samples;
-        L.chunks = (int)((S.g.kp() + kM1ChunkK - 1) / kM1ChunkK);
         auto vec = [](const void *p, int64_t ld, int bytes) { return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld * bytes % 16 == 0; };
         bool ok = vec(L.w, L.ld_w, 2) && vec(L.s, L.ld_s, 4);
         for (int h = 0; h < samples; ++h) {
