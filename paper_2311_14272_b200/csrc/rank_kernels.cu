@@ -134,6 +134,51 @@ rank_columns_kernel(const RankLayer *__restrict__ layers, int n_layers, ulonglon
     for (int o = threadIdx.x; o < L.candidates; o += kRankThreads) add(o, s_row[o]);
 }
 
+// K-R1 of layers that a CTA holds in shared memory, with the candidates made from it: a thread a score, whose rank is its place in the row, then
+// a thread a column.  No sums in global memory, so nothing to clear, and the table travels as a kernel parameter: a copy, a memset and two
+// kernels less in front of the selection.  Bound by latency (the longest layer's row, some 10 cycles a score of it, and the launch).
+// Measured (13 layers of VGG-16, us): 4.8 where copy, memset and the two kernels below took 0.9 + 1.5 + 4.1 + 3.0 and the gaps between them, some 8.
+// The line: a score is compared with its row by one thread, so a layer's 2^19 comparisons are some 500 a thread, 5 us; beyond, and for more layers than the
+// parameter holds, rows are CTAs of their own (4096 x 4096 in 32 x 32 blocks is 2^21).
+constexpr int kRankLayers = 64, kRankScores = 2560, kRankLayerThreads = 1024;
+constexpr long long kRankCompares = 1 << 19;         // of a layer: each score with the others of its row
+struct RankTable { RankLayer layer[kRankLayers]; };
+__global__ void __launch_bounds__(kRankLayerThreads)
+rank_layer_kernel(const __grid_constant__ RankTable table, RankEntry *entries, int32_t *kkeep) {
+    __shared__ unsigned long long s_score[kRankScores], s_sorted[kRankScores];
+    wait_for_prerequisites();
+    const RankLayer &L = table.layer[blockIdx.x];
+    const int n = L.nrt * L.nblk;
+    for (int i = threadIdx.x; i < n; i += kRankLayerThreads) s_score[i] = L.scores[i];
+    if (threadIdx.x == 0) kkeep[blockIdx.x] = L.nblk;        // the selection takes the pruned positions off
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kRankLayerThreads) {
+        const int at = i % L.nblk;
+        const unsigned long long *row = s_score + (i - at), mine = s_score[i];
+        int rank = 0;
+#pragma unroll 4
+        for (int j = 0; j < L.nblk; ++j) {
+            const unsigned long long o = row[j];
+            rank += (o < mine) | ((o == mine) & (j < at));
+        }
+        s_sorted[i - at + rank] = mine;
+    }
+    __syncthreads();
+    const int e = float_bits_exponent(*L.max_key);
+    for (int o = threadIdx.x; o < L.candidates; o += kRankLayerThreads) {
+        unsigned long long lo = 0ull, hi = 0ull;
+        for (int r = 0; r < L.nrt; ++r) {
+            const unsigned long long v = s_sorted[r * L.nblk + o];
+            lo += v;
+            hi += lo < v;
+        }
+        entries[L.entry_off + o] = make_entry(lo, hi, e, (int)blockIdx.x, o, (unsigned long long)L.nrt * (unsigned long long)L.block_elems);
+    }
+}
+bool rank_layer_fits(const RankLayer &L) {
+    return (long long)L.nrt * L.nblk <= kRankScores && (long long)L.nrt * L.nblk * L.nblk <= kRankCompares;
+}
+
 // The candidates in the form they are compared in.
 __global__ void __launch_bounds__(kRankThreads)
 rank_entries_kernel(const RankLayer *__restrict__ layers, int n_layers, int n, const ulonglong2 *__restrict__ sums,
@@ -157,9 +202,9 @@ rank_entries_kernel(const RankLayer *__restrict__ layers, int n_layers, int n, c
 // each adds up the weight of those that precede i in the global order, and a shuffle reduction gives the
 // weight pruned before i.
 __global__ void __launch_bounds__(kRankThreads)
-global_select_kernel(const RankEntry *__restrict__ entries, int n, unsigned long long target,
-                     int32_t *__restrict__ kkeep) {
+global_select_kernel(const RankEntry *entries, int n, unsigned long long target, int32_t *kkeep) {
     __shared__ RankEntry s_tile[kRankThreads];
+    wait_for_prerequisites();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * (kRankThreads / 32) + warp;
     RankEntry mine;
@@ -264,19 +309,28 @@ CRISP_API crisp_status_t crisp_global_rank(int32_t n_layers, const crisp_rank_la
     ulonglong2 *d_sums = reinterpret_cast<ulonglong2 *>(ws + lay.sums_off);
     RankEntry *d_entries = reinterpret_cast<RankEntry *>(ws + lay.entries_off);
     const int n = (int)lay.n_entries;
-    // the table is read from pageable host memory: the call returns once it has been staged
-    if (cudaMemcpyAsync(d_table, table.get(), (size_t)n_layers * sizeof(RankLayer), cudaMemcpyHostToDevice, st) != cudaSuccess)
-        return CRISP_CUDA_ERROR;
-    if (n > 0) {
-        if (cudaMemsetAsync(d_sums, 0, (size_t)n * sizeof(ulonglong2), st) != cudaSuccess) return CRISP_CUDA_ERROR;
-        crisp::rank_columns_kernel<<<(unsigned)lay.n_rows, crisp::kRankThreads, 0, st>>>(d_table, n_layers, d_sums);
+    bool fits = n_layers <= crisp::kRankLayers;
+    for (int l = 0; l < n_layers && fits; ++l) fits = crisp::rank_layer_fits(table[l]);
+    if (fits) {
+        crisp::RankTable param;
+        for (int l = 0; l < n_layers; ++l) param.layer[l] = table[l];
+        if (crisp::launch_chained(crisp::rank_layer_kernel, (unsigned)n_layers, crisp::kRankLayerThreads, 0, st, param, d_entries, d_kkeep) != cudaSuccess)
+            return CRISP_CUDA_ERROR;
+    } else {
+        // the table is read from pageable host memory: the call returns once it has been staged
+        if (cudaMemcpyAsync(d_table, table.get(), (size_t)n_layers * sizeof(RankLayer), cudaMemcpyHostToDevice, st) != cudaSuccess)
+            return CRISP_CUDA_ERROR;
+        if (n > 0) {
+            if (cudaMemsetAsync(d_sums, 0, (size_t)n * sizeof(ulonglong2), st) != cudaSuccess) return CRISP_CUDA_ERROR;
+            crisp::rank_columns_kernel<<<(unsigned)lay.n_rows, crisp::kRankThreads, 0, st>>>(d_table, n_layers, d_sums);
+        }
+        const int most = n > n_layers ? n : n_layers;
+        crisp::rank_entries_kernel<<<(most + crisp::kRankThreads - 1) / crisp::kRankThreads, crisp::kRankThreads, 0, st>>>(
+            d_table, n_layers, n, d_sums, d_entries, d_kkeep);
     }
-    const int most = n > n_layers ? n : n_layers;
-    crisp::rank_entries_kernel<<<(most + crisp::kRankThreads - 1) / crisp::kRankThreads, crisp::kRankThreads, 0, st>>>(
-        d_table, n_layers, n, d_sums, d_entries, d_kkeep);
-    if (n > 0)
-        crisp::global_select_kernel<<<(n + crisp::kRankThreads / 32 - 1) / (crisp::kRankThreads / 32), crisp::kRankThreads, 0, st>>>(
-            d_entries, n, target, d_kkeep);
+    if (n > 0 && crisp::launch_chained(crisp::global_select_kernel, (unsigned)((n + crisp::kRankThreads / 32 - 1) / (crisp::kRankThreads / 32)), crisp::kRankThreads,
+                                       0, st, (const RankEntry *)d_entries, n, target, d_kkeep) != cudaSuccess)
+        return CRISP_CUDA_ERROR;
     return cudaGetLastError() == cudaSuccess ? CRISP_OK : CRISP_CUDA_ERROR;
 }
 
