@@ -69,6 +69,22 @@ class CrispError(RuntimeError):
 
 _lib = None
 _native = None                                            # the hot ones of the same calls on plain integers (csrc/calls.cpp)
+_network = None                                           # what goes over all tensors of a network (csrc/network.cpp); False: not built
+
+
+def _bind_network():
+    """csrc/network.cpp for the library that is loaded, or False in a tree where it could not be built (it needs torch's headers)."""
+    global _network
+    lib = load()
+    if _network is not False:
+        import torch                                      # noqa: F401  (the module's libraries)
+        try:
+            from . import _network as module
+            module.bind(C.cast(lib.crisp_decode, C.c_void_p).value)
+            _network = module
+        except ImportError:
+            _network = False
+    return _network
 
 
 class _CtypesCalls:
@@ -171,6 +187,8 @@ def load(path: Optional[str] = None):
     except ImportError:
         native = _CtypesCalls(lib)
     _lib, _native = lib, native
+    if _network:
+        _bind_network()
     return lib
 
 
@@ -485,6 +503,7 @@ class HybridLayer:
         self.handle = 0
         self.canonical_buf = None
         self.exec_buf = None
+        self._gpu = self.device.index if (_network or _bind_network()) else None       # (decode makes its tensors through it)
 
     # build_mask, encode, decode, spmm and spmm_conv are made once per layer and pass; for small layers their host time is the
     # time of the pass, so they hand plain integers to the library (and ask a tensor for all its strides at once, which is cheaper
@@ -566,10 +585,15 @@ class HybridLayer:
         crisp_export(self.handle, blk_col, vals, idx, stream)
         return blk_col.reshape(self.nrt, self.kkeep), vals, idx
 
-    # (empty_strided is the cheapest of torch's allocating calls: 1.1 us against 3.2 for new_empty and 4.2 for empty)
+    # (of the calls in Python empty_strided is the cheapest that allocates: 1.1 us against 3.2 for new_empty and 4.2 for empty)
     def decode(self, stream=None):
         desc, torch = self.desc, self.torch
         k = desc.k
+        if self._gpu is not None:
+            code, w = _network.decode(self.handle, desc.rows, k, self._gpu, _stream(stream))
+            if code:
+                raise CrispError(code, "crisp_decode")
+            return w
         w = torch.empty_strided((desc.rows, k), (k, 1), dtype=torch.bfloat16, device=self.device)
         code = _native.decode(self.handle, w.data_ptr(), k, _stream(stream))
         if code:
@@ -674,6 +698,8 @@ class PruningNetwork:
         self.rank_arr = make_rank_layers([L.rank_layer(min_keep) for L in self.layers])
         self.rank_ws = torch.empty(crisp_global_rank_sizes(self.rank_arr), dtype=torch.uint8, device=self.device)
         self.d_kkeep = torch.zeros(len(shapes), dtype=torch.int32, device=self.device)
+        self._h_kkeep = torch.zeros(len(shapes), dtype=torch.int32, pin_memory=True)
+        self._blocks = (C.c_int32 * len(shapes))(*[L.nblk for L in self.layers])
 
     @property
     def acc(self):
@@ -697,6 +723,23 @@ class PruningNetwork:
             count += 1
         return count
 
+    def _table(self, arr, layers, weights, grads):
+        """Fills in the table of the layers: one host array each for what there is per gradient (returned; the entries point into them),
+        and one struct per layer."""
+        flat = [g for gs in grads for g in gs]
+        ptrs = array("Q", [g.data_ptr() for g in flat])
+        lds = array("q", [g.stride()[0] for g in flat])
+        dts = array("i", [0 if g.dtype is self.torch.bfloat16 else 1 for g in flat])
+        p0, l0, d0, at = ptrs.buffer_info()[0], lds.buffer_info()[0], dts.buffer_info()[0], 0
+        for P, L, w, gs, s in zip(arr, layers, weights, grads, self.sal):
+            P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride()[0]
+            n = len(gs)
+            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, n
+            P.d_saliency, P.ld_s = s.data_ptr(), s.stride()[0]
+            P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
+            at += n
+        return ptrs, lds, dts, flat
+
     def step(self, weights, grads, kappa, stream=None):
         """weights[l]: bf16 CUDA tensor [rows, k]; grads[l]: list of H gradient tensors (bf16 or fp32) of that shape;
         kappa: overall sparsity target of this iteration.  Returns the kept-block count of every layer; the layers'
@@ -711,54 +754,50 @@ class PruningNetwork:
         held = (list, tuple, torch.Tensor)
         at_once = isinstance(grads, held) and (set(map(type, grads)) <= {list, tuple} or all(isinstance(gs, held) for gs in grads))
         count = min(len(self.layers), len(weights), len(grads) if at_once else len(weights))
-        weights = weights[:count]
-        assert all(w.is_cuda and w.element_size() == 2 and w.stride()[1] == 1 for w in weights)
-        if not at_once:
-            count = self._score_in_turn(weights, grads, stream)
-        grads = grads[:count] if at_once else [()] * count
-        bf16, layers = torch.bfloat16, self.layers[:count]
-        # The table of the layers: one host array each for what there is per gradient, and one struct per layer.
-        flat = [g for gs in grads for g in gs]
-        ptrs = array("Q", [g.data_ptr() for g in flat])
-        lds = array("q", [g.stride()[0] for g in flat])
-        dts = array("i", [0 if g.dtype is bf16 else 1 for g in flat])
-        p0, l0, d0, at = ptrs.buffer_info()[0], lds.buffer_info()[0], dts.buffer_info()[0], 0
-        arr = (PruneLayer * count)()
-        for P, L, w, gs, s in zip(arr, layers, weights, grads, self.sal):
-            P.desc, P.d_w_bf16, P.ld_w = L.desc, w.data_ptr(), w.stride()[0]
-            n = len(gs)
-            P.d_grads, P.ld_grads, P.grad_dtypes, P.samples = p0 + 8 * at, l0 + 8 * at, d0 + 4 * at, n
-            P.d_saliency, P.ld_s = s.data_ptr(), s.stride()[0]
-            P.d_mask_buf, P.d_workspace = L.mask_buf.data_ptr(), L.workspace.data_ptr()
-            at += n
+        weights, layers = weights[:count], self.layers[:count]
+        arr, table = (PruneLayer * count)(), None
+        if at_once and _network:
+            gradients = [gs if type(gs) in (list, tuple) else list(gs) for gs in grads[:count]]
+            table = _network.table(layers, weights, gradients, self.sal, C.addressof(arr))
+        if table is None:
+            assert all(w.is_cuda and w.element_size() == 2 and w.stride()[1] == 1 for w in weights)
+            if not at_once:
+                count = self._score_in_turn(weights, grads, stream)
+                arr, layers = (PruneLayer * count)(), layers[:count]
+            table = self._table(arr, layers, weights, grads[:count] if at_once else [()] * count)
         if at_once:
             crisp_prune_score(arr, stream)
         crisp_global_rank(self.rank_arr, crisp_prune_fraction(kappa, self.n, self.m), self.rank_ws, self.d_kkeep, stream)
         # While the device scores and ranks: what the encodings need whatever the counts are, and the masks and handles that
         # they will take the place of.
-        for P, L in zip(arr, layers):
-            if L.canonical_buf is not None:
-                P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
-        have = [(0, 0) if L.canonical_buf is None else (L.canonical_buf.numel(), L.exec_buf.numel()) for L in layers]
-        old_masks, old_handles = (C.c_void_p * count)(*[L.mask for L in layers]), (C.c_void_p * count)(*[L.handle for L in layers])
-        masks, handles = (C.c_void_p * count)(), (C.c_void_p * count)()
-        canonical_bytes, exec_bytes = (C.c_size_t * count)(), (C.c_size_t * count)()
-        if stream is None:
-            kk = self.d_kkeep.cpu().tolist()
-        else:
-            with torch.cuda.stream(stream):
-                kk = self.d_kkeep.cpu().tolist()
+        old_masks, old_handles, masks, handles = [(C.c_void_p * count)() for _ in range(4)]
+        canonical_bytes, exec_bytes, have_c, have_e = [(C.c_size_t * count)() for _ in range(4)]
+        if not (_network and _network.encodings(layers, *map(C.addressof, (arr, have_c, have_e, old_masks, old_handles)))):
+            for i, (P, L) in enumerate(zip(arr, layers)):
+                if L.canonical_buf is not None:
+                    P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
+                    have_c[i], have_e[i] = L.canonical_buf.numel(), L.exec_buf.numel()
+                old_masks[i], old_handles[i] = L.mask, L.handle
+        # (a copy into pinned memory and a wait for the stream: 10 us less than a copy into pageable memory)
+        with torch.cuda.stream(stream):                      # (None: the current one)
+            self._h_kkeep.copy_(self.d_kkeep, non_blocking=True)
+            torch.cuda.current_stream(self.d_kkeep.device).synchronize()
+        kk = self._h_kkeep.tolist()
         for P, c in zip(arr, kk):
             P.kkeep = c
         _check(_lib.crisp_prune_encode_sizes(count, arr, canonical_bytes, exec_bytes), "crisp_prune_encode_sizes")
-        for P, L, cb, eb, (have_c, have_e) in zip(arr, layers, canonical_bytes, exec_bytes, have):
-            if cb > have_c or eb > have_e:
+        for i, (cb, eb) in enumerate(zip(canonical_bytes, exec_bytes)):
+            if cb > have_c[i] or eb > have_e[i]:
+                P, L = arr[i], layers[i]
                 L._reserve(cb, eb)
                 P.d_canonical_buf, P.d_exec_buf = L.canonical_buf.data_ptr(), L.exec_buf.data_ptr()
         _check(_lib.crisp_prune_encode(count, arr, _stream(stream), masks, handles), "crisp_prune_encode")
-        for L, c, mask, handle in zip(layers, kk, masks, handles):
-            L.mask, L.handle, L.kkeep = mask, handle, c
-            L.desc.keep_ratio = c / L.nblk                   # floor(ratio * nblk + 0.5) gives the count back
+        if _network:
+            _network.encoded(layers, kk, *map(C.addressof, (self._blocks, masks, handles)))
+        else:
+            for L, c, mask, handle in zip(layers, kk, masks, handles):
+                L.mask, L.handle, L.kkeep = mask, handle, c
+                L.desc.keep_ratio = c / L.nblk               # floor(ratio * nblk + 0.5) gives the count back
         crisp_destroy_layers(old_masks, old_handles)
         return kk
 

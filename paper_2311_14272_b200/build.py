@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import subprocess
 import sys
@@ -12,8 +13,16 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcrisp.so")
 CALLS = os.path.join(HERE, "_calls.so")                      # Python entry points of the hot calls (plain C++)
+NETWORK = os.path.join(HERE, "_network.so")                  # and of what goes over the tensors of a network (C++ with torch's headers)
 PYTHON_INCLUDE = sysconfig.get_paths()["include"]
 HAVE_PYTHON_H = os.path.exists(os.path.join(PYTHON_INCLUDE, "Python.h"))       # without it the binding makes those calls through ctypes
+
+
+def torch_dir():
+    """Where torch is installed with its headers, or None (found without importing it)."""
+    spec = importlib.util.find_spec("torch")
+    d = os.path.dirname(spec.origin) if spec and spec.origin else None
+    return d if d and os.path.exists(os.path.join(d, "include", "torch", "csrc", "autograd", "python_variable.h")) else None
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -26,7 +35,7 @@ def sources():
 
 
 def _stale() -> bool:
-    built = [LIB] + ([CALLS] if HAVE_PYTHON_H else [])
+    built = [LIB] + ([CALLS] if HAVE_PYTHON_H else []) + ([NETWORK] if HAVE_PYTHON_H and torch_dir() else [])
     if not all(os.path.exists(f) for f in built):
         return True
     t = min(os.path.getmtime(f) for f in built)
@@ -52,6 +61,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
                            "-I", PYTHON_INCLUDE, "-I", os.path.join(ROOT, "include"), "-o", tmp,
                            os.path.join(CSRC, "calls.cpp")])
     os.replace(tmp, CALLS)
+    where = torch_dir()
+    if not where:
+        print("no headers of torch: a pruning iteration's table is made in Python", file=sys.stderr)
+        return LIB
+    tmp = NETWORK + f".{os.getpid()}.tmp"
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                           "-I", PYTHON_INCLUDE, "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(where, "include"),
+                           "-isystem", os.path.join(where, "include", "torch", "csrc", "api", "include"), "-o", tmp,
+                           os.path.join(CSRC, "network.cpp"), "-L", os.path.join(where, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"])
+    os.replace(tmp, NETWORK)
     return LIB
 
 
