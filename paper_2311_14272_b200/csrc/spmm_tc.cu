@@ -1102,6 +1102,12 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
     const bool short_walk = wlen <= 8 && nt_override <= 0;
     if (short_walk && wlen <= 2 && sparse && nt == 4 && !conv) nt = 3;
     if (nt_override > 0) {
+    } else if (!conv && stack == 1 && L.nst * boxes <= sm_count) {
+        // Every SM gets one tile of 64 columns at most: what counts is the chain of a single tile, and the narrowest has the shortest fills and drain.  Of 90
+        // random products with up to 450 such tiles all 72 below the line are faster than with 128 columns, by 12 % in the mean (us, replayed: one tile
+        // 21 x 1903 x 104, 3:4 10.6 -> 8.4, 8 tiles 413 x 661 x 88 5.4 -> 4.8, 143 tiles 1315 x 180 x 832 5.4 -> 4.9), and all 18 beyond it
+        // slower or equal (154 tiles 1341 x 186 x 864 4.5 -> 5.2, 252 1497 x 1220 x 1328 8.8 -> 10.8).
+        nt = 1;
     } else if (conv || stack > 1) {
         // small layers are latency-bound: narrower tiles (down to 2 boxes) until at least half of the SMs have one
         while (nt > 2 && (int64_t)L.nst * ((ncols + stack * nt * kBoxN - 1) / (stack * nt * kBoxN)) < sm_count / 2) --nt;
