@@ -450,7 +450,10 @@ cudaError_t encode_batch(const EncodeLayer *layers, int n, cudaStream_t st) {
 
 }  // namespace
 
+std::atomic<uint64_t> encode_launches{0};
+
 cudaError_t launch_encode(const EncodeLayer *layers, int n, cudaStream_t st) {
+    encode_launches.fetch_add(1, std::memory_order_relaxed);
     if (n == 1) return encode_batch<1>(layers, 1, st);
     for (int at = 0; at < n; at += kBatchLayers) {
         cudaError_t e = encode_batch<kBatchLayers>(layers + at, n - at < kBatchLayers ? n - at : kBatchLayers, st);

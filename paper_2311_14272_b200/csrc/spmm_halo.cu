@@ -54,6 +54,7 @@ struct HaloParams {
     int wo, ho, batch;
     uint32_t a_bytes, entry_bytes, x_bytes, x_stage, x_stages, w_stages;       // (a stage of weights: kGroup entries)
     int resident;
+    int early;                           // weight tiles and walks may be read before the kernel in front has finished (weights_settled)
     uint16_t *y;
     int64_t ldy;
     // From this channel on (a multiple of 32) results are stored pixel by pixel: all where TMA cannot address the pixels (pitch or base not a
@@ -127,7 +128,8 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    wait_for_prerequisites();
+    // (where the weights have not just been encoded, the walks and the first weight tiles come while the kernel in front finishes)
+    if (!p.early) wait_for_prerequisites();
     for (int i = threadIdx.x; i < p.nst * p.wcap; i += kThreads) {
         const int jb = p.walk_col[i], tap = jb / p.cpt, ti = tap / p.kw;
         s_cols[i] = (jb - tap * p.cpt) << 16 | ((ti * p.tb * p.pw + tap - ti * p.kw) * 8);       // slab | start of the tap
@@ -153,6 +155,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if (p.early && warp != 0) wait_for_prerequisites();      // the activation, the bias and the results' place
 
     if (warp == 0) {
         // ------------------------------------------------ weight tiles
@@ -163,7 +166,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             for (int t = blockIdx.x; t < p.num_tiles && ok && !*abort_flag; t += gridDim.x) {
                 const int st = t % p.nst, len = s_len[st];
                 for (int i = 0; i < len; i += kGroup) {
-                    if (!mbar_wait(w_empty + 8 * stage, ph ^ 1u, abort_flag, p.wait_limit)) { ok = false; break; }
+                    if (!mbar_wait_early(w_empty + 8 * stage, ph ^ 1u, abort_flag, p.wait_limit)) { ok = false; break; }
                     const int n = min(kGroup, len - i);
                     mbar_expect_tx(w_full + 8 * stage, (uint32_t)n * p.entry_bytes);
                     for (int g = 0; g < n; ++g)
@@ -174,6 +177,7 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 if (p.resident) break;                       // (the only walk there is: its tiles stay)
             }
         }
+        wait_for_prerequisites();                            // (there may have been nothing to wait for)
     } else if (warp == 2 + kEpiWarps) {
         // ------------------------------------------------ activations: a box with its border per slab
         if (lane == 0) {
@@ -517,6 +521,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
                              cudaStream_t st, bool *done) {
     *done = false;
     if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return cudaSuccess;
+    const uint64_t encodes = encode_launches.load(std::memory_order_relaxed);
     HaloLaunch launch;
     {
         std::lock_guard<std::mutex> hold(h->plan_lock);
@@ -540,6 +545,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
             if (fresh.refused) return cudaSuccess;
         }
         launch = plan->launch;
+        launch.p.early = weights_settled(h, st, encodes);
     }
     *done = true;
     static std::atomic<bool> configured[16][64];
@@ -556,7 +562,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
     p.wait_limit = h->wait_limit_cycles ? h->wait_limit_cycles : kWaitLimitCycles;
     p.skip_fill = h->debug_skip_stage;
     const cudaError_t e = launch_chained(launch.kern, (unsigned)launch.grid, (unsigned)kThreads, launch.smem, st, launch.mx, launch.my, launch.ma, p);
-    if (e == cudaSuccess) note_launch(h, launch.info, launch.resident_bytes);
+    if (e == cudaSuccess) note_launch(h, launch.info, launch.resident_bytes, st, encodes);
     return e;
 }
 

@@ -6,7 +6,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
-#include "crisp.h"
+#include "crisp_internal.h"
 
 namespace crisp {
 namespace tc {
@@ -53,6 +53,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return false; }
         }
     }
+}
+// The same for a role that may run before the kernel in front of this one has finished: the limit counts from then on.
+__device__ __forceinline__ bool mbar_wait_early(uint32_t bar, uint32_t parity, volatile int *abort_flag, unsigned long long limit) {
+    if (mbar_try_wait(bar, parity)) return true;
+    wait_for_prerequisites();
+    return mbar_wait(bar, parity, abort_flag, limit);
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
     asm volatile(
