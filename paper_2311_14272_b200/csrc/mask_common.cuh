@@ -129,15 +129,21 @@ constexpr unsigned long long kRecordSum = (1ull << kRecordCodeShift) - 1;
 // The N:M step on a lane's rows.  `key`: the bits of its elements (signs, infinities and NaN among them).  Returns its mask bits, byte i for row i of R; v: the
 // values that count in the scores, top: the bits of the largest.  TOP = 1 or 2: n is TOP and only survivors count, so a group's largest values are selected with
 // minima and maxima, which serve both the mask (an element is kept if it reaches the smallest of them) and the sums (whichever of equal values is
-// kept).  TOP = 0: any n, and all elements where all_count is set.  Two cases are left to reload(i, key), which reads the canonical bits of the
-// lane's row i again, so that no register holds them: infinities or NaN, and ties, where more than n elements reach the smallest.
+// kept; ties, where more than n elements reach the smallest, go by rank).  TOP = 0: any n, and all elements where all_count is set.  reload(i, key) reads the
+// canonical bits of the lane's row i again, for infinities and NaN, so that no register holds them until then.
 template <int M, int TOP> constexpr int kCounted = TOP ? TOP * (8 / M) : 8;     // values that count, of a row of a lane
 template <int M, int TOP, int R, typename Reload>
 __device__ __forceinline__ uint32_t select_rows(uint32_t (&key)[R][8], int n, bool all_count, const uint8_t *s_keep, const Reload &reload,
                                                 float (&v)[R][kCounted<M, TOP>], uint32_t &top) {
     constexpr int kGroups = 8 / M;
+    // Ties of a row, while its elements are in registers, where those are not what there is too little of (4096 x 4096, 2:4, three of four elements zero: 26.3 us
+    // for the mask, 31.7 with the rows read again; but 15.6 instead of 13.0 for the saliency of 35 small layers, two rows a lane at 40 registers).
+    constexpr bool kTiesByRow = R == kM1LaneRows;
     uint32_t bits = 0u;
-    auto ranked = [&](const uint32_t (&q)[8]) -> uint32_t {
+    auto ranked = [&](const uint32_t (&raw)[8]) -> uint32_t {
+        uint32_t q[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) q[j] = raw[j] & 0x7FFFFFFFu;
         if constexpr (M == 4) return (uint32_t)s_keep[outcomes4(q)] | ((uint32_t)s_keep[outcomes4(q + 4)] << 4);
         else return top_n_bits<M>(q, TOP ? TOP : n);
     };
@@ -167,9 +173,12 @@ __device__ __forceinline__ uint32_t select_rows(uint32_t (&key)[R][8], int n, bo
                 v[i][0] = fmaxf(p.a, q.a);
                 if constexpr (TOP == 2) v[i][1] = fmaxf(fminf(p.a, q.a), fmaxf(p.b, q.b));
             }
+            uint32_t row = 0u;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (x[j] >= v[i][(M == 4 ? j / 4 : 0) * TOP + TOP - 1]) bits |= 1u << (8 * i + j);
+                if (x[j] >= v[i][(M == 4 ? j / 4 : 0) * TOP + TOP - 1]) row |= 1u << j;
+            if (kTiesByRow && __popc(row) != kGroups * TOP) row = ranked(q8);
+            bits |= row << (8 * i);
         };
 #pragma unroll
         for (int i = 0; i < R; ++i) select(i, key[i]);
@@ -182,16 +191,16 @@ __device__ __forceinline__ uint32_t select_rows(uint32_t (&key)[R][8], int n, bo
                 select(i, q);
             }
         }
-        if (top_f == 0.f) {                                  // (zeros: columns beyond the matrix, blocks pruned before)
+        if (kTiesByRow) {
+        } else if (top_f == 0.f) {                           // (zeros: columns beyond the matrix, blocks pruned before)
             bits = (M == 4 ? 0x11111111u : 0x01010101u) * ((1u << TOP) - 1u) >> (32 - 8 * R);
         } else if (__popc(bits) != R * kGroups * TOP) {
+            uint32_t q[R][8];
             bits = 0u;
-#pragma unroll 1
-            for (int i = 0; i < R; ++i) {
-                uint32_t q[8];
-                reload(i, q);
-                bits |= ranked(q) << (8 * i);
-            }
+#pragma unroll
+            for (int i = 0; i < R; ++i) reload(i, q[i]);
+#pragma unroll
+            for (int i = 0; i < R; ++i) bits |= ranked(q[i]) << (8 * i);
         }
         top = __float_as_uint(top_f);
     }

@@ -155,7 +155,8 @@ __device__ __forceinline__ void floor_parts2(uint64_t v, uint64_t &r, uint64_t &
 // K-M1b: the block scores from the records of K-M1a, once the scale is known: a warp a block, a lane a record.  A record whose sum does
 // not stand (see bits_and_record) has its 32 x 32 elements counted again, the mask bits telling which.
 // Measured (us, 4096 x 4096, 2:4, S of 64 MiB): the pass over S and this kernel 17.0 + 3.8, where a memset, a pass for bits and maximum and a second one
-// for the scores took 1.8 + 16.2 + 11.4; mask, encoding and decoding in a row 59.3 -> 47.2.
+// for the scores took 1.8 + 16.2 + 11.4; mask, encoding and decoding in a row 59.3 -> 47.2.  The mask phase alone, in a row: 28.8 -> 18.5, 4:8 in blocks of 32 x 32
+// 41.1 -> 39.8.  Where no record stands (elements spread over 20 binades evenly) this kernel is a second pass over S: 28.8 -> 31.5 and 41.1 -> 52.6.
 template <int CAP>
 __global__ void __launch_bounds__(kM1Threads)
 block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
@@ -195,20 +196,59 @@ block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
         else if (d >= 0 && d < code) acc = sum >> d;
         else stands = false;
     }
-    const int e_max = mk ? key_exponent(mk) : 0;
-    for (uint32_t left = __ballot_sync(0xFFFFFFFFu, !stands); left; left &= left - 1u) {
-        const int part = __ffs(left) - 1;
-        const int64_t row0 = (int64_t)rt * g.bm + part / wpb * kM1Rows;
-        const int word = jb * wpb + part % wpb;
-        uint32_t key[kM1LaneRows][8];
-        load_patch(L.s, L.ld, g, L.vec_ok != 0, row0, (int64_t)word * 32, lane, key);
+    if (const uint32_t again = __ballot_sync(0xFFFFFFFFu, !stands)) {
+        // The elements of these records once more, the next record's on their way while one is counted.  floor(value * 2^(40 - e_max)): when that
+        // power of two is an fp32 number, the product is exact (value <= layer maximum, so it stays below 2^41).
+        const int e_max = mk ? key_exponent(mk) : 0, scale_exp = kScoreFractionBits - e_max;
+        const bool float_scale = scale_exp >= -126 && scale_exp <= 127;
+        const float scale = float_scale ? __uint_as_float((uint32_t)(127 + scale_exp) << 23) : 0.f;
+        auto load = [&](uint32_t left, uint32_t (&key)[kM1LaneRows][8], uint32_t &counted) {
+            const int part = __ffs(left) - 1, word = jb * wpb + part % wpb;
+            const int64_t row0 = (int64_t)rt * g.bm + part / wpb * kM1Rows;
+            load_patch(L.s, L.ld, g, L.vec_ok != 0, row0, (int64_t)word * 32, lane, key);
+            counted = 0xFFFFFFFFu;
+            if (g.score_mode == 0) {
+                const uint8_t *bits = reinterpret_cast<const uint8_t *>(L.nm_bits + (row0 + (lane >> 2)) * g.wpr + word) + (lane & 3);
+                counted = 0u;
 #pragma unroll
-        for (int i = 0; i < kM1LaneRows; ++i) {
-            uint32_t counted = 0xFFu;
-            if (g.score_mode == 0) counted = L.nm_bits[(row0 + (lane >> 2) + 8 * i) * g.wpr + word] >> (8 * (lane & 3));
+                for (int i = 0; i < kM1LaneRows; ++i) counted |= (uint32_t)bits[(int64_t)32 * i * g.wpr] << (8 * i);
+            }
+        };
+        auto count = [&](const uint32_t (&key)[kM1LaneRows][8], uint32_t counted) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if ((counted >> j) & 1u) acc += fixed_point_score(key[i][j], e_max);
+            for (int i = 0; i < kM1LaneRows; ++i) {
+                if (float_scale) {
+                    // an element that does not count is multiplied by zero instead of by the scale: its parts are zero
+                    uint64_t r_sum = f32x2(0.f, 0.f), d_sum = r_sum;             // exact for eight values: see floor_parts2
+#pragma unroll
+                    for (int j = 0; j < 8; j += 2) {
+                        const uint32_t two = counted >> (8 * i + j);
+                        uint64_t r, fd;
+                        floor_parts2(mul2(f32x2(__uint_as_float(key[i][j]), __uint_as_float(key[i][j + 1])),
+                                          f32x2(two & 1u ? scale : 0.f, two & 2u ? scale : 0.f)), r, fd);
+                        r_sum = add2(r_sum, r);
+                        d_sum = add2(d_sum, fd);
+                    }
+                    acc += ((unsigned long long)__float2uint_rn(f32x2_sum(r_sum) * 9.5367431640625e-07f) << 20) +
+                           (unsigned long long)__float2uint_rn(f32x2_sum(d_sum));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if ((counted >> (8 * i + j)) & 1u) acc += fixed_point_score(key[i][j], e_max);
+                }
+            }
+        };
+        uint32_t key[2][kM1LaneRows][8], counted[2], left = again;
+        load(left, key[0], counted[0]);
+        for (;;) {
+            left &= left - 1u;
+            if (left) load(left, key[1], counted[1]);
+            count(key[0], counted[0]);
+            if (!left) break;
+            left &= left - 1u;
+            if (left) load(left, key[0], counted[0]);
+            count(key[1], counted[1]);
+            if (!left) break;
         }
     }
 #pragma unroll
