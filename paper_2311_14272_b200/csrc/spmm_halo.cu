@@ -310,47 +310,74 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             go = __shfl_sync(0xFFFFFFFFu, go, 0);
             if (!go) break;
             tc_fence_after();
+            // a chunk: channels 0..15 and 16..31 of 32 pixels
+            auto load = [&](int c, uint32_t (&lo)[16], uint32_t (&hi)[16]) {
+                const uint32_t taddr = tmem_base + acc * kN + 32 * c + ((uint32_t)(32 * q) << 16);
+                tmem_ld_16x32(taddr, lo);
+                tmem_ld_16x32(taddr + (16u << 16), hi);
+            };
+            auto store = [&](int c, uint32_t (&lo)[16], uint32_t (&hi)[16]) {
+                if (fuse) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        lo[i] = __float_as_uint(fmaxf(__uint_as_float(lo[i]) + bias[i >> 1 & 1], floor_v));
+                        hi[i] = __float_as_uint(fmaxf(__uint_as_float(hi[i]) + bias[2 + (i >> 1 & 1)], floor_v));
+                    }
+                }
+                if (lane == 0) bulk_wait_read<0>();      // the store that last used the staging tile has read it
+                __syncwarp();
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {            // groups of 8 pixels
+                    auto pack = [](uint32_t a, uint32_t b) { return pack_bf16(__uint_as_float(a), __uint_as_float(b)); };
+                    store_matrices(tile + (uint32_t)(512 * g) + my_row, pack(lo[4 * g], lo[4 * g + 1]), pack(lo[4 * g + 2], lo[4 * g + 3]),
+                                   pack(hi[4 * g], hi[4 * g + 1]), pack(hi[4 * g + 2], hi[4 * g + 3]));
+                }
+                if (kPlain && ch0 >= p.plain_from) {     // pixel by pixel, the lanes on consecutive channels
+                    __syncwarp();
+                    const bool ch_ok = ch0 + lane < p.rows;
+#pragma unroll 8
+                    for (int px = 0; px < 32; ++px) {
+                        const int g = 4 * c + (px >> 3), y = org.y + (g >> p.tb_log2), b = org.b + (g & (p.tb - 1)), x = org.x + (px & 7);
+                        uint16_t v;
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(tile + (uint32_t)(64 * px + (((lane >> 3) ^ (px >> 1 & 3)) << 4) + 2 * (lane & 7))) : "memory");
+                        if (ch_ok && y < p.ho && b < p.batch && x < p.wo) p.y[(((int64_t)b * p.ho + y) * p.wo + x) * p.ldy + ch0 + lane] = v;
+                    }
+                } else {
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        const int y = org.y + (4 * c >> p.tb_log2);
+                        if (y < p.ho) tma_store_4d(&map_y, tile, ch0, org.x, org.b, y);
+                        bulk_commit();
+                    }
+                }
+            };
+            if constexpr (kAcc == 1) {
+                // One accumulator: the warp takes all of its share before the next tile's MMAs may begin, and stores it under them (three
+                // convolutions of 56 x 56, 256 pixels a tile: 61.7 -> 58.5 us).
+                constexpr int kMine = kChunks / kParts;
+                uint32_t lo[kMine][16], hi[kMine][16];
+                if (ch0 < p.rows) {
+#pragma unroll
+                    for (int i = 0; i < kMine; ++i) load(part + kParts * i, lo[i], hi[i]);
+                    tmem_ld_wait();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(t_empty);
+                if (ch0 < p.rows) {
+#pragma unroll
+                    for (int i = 0; i < kMine; ++i) store(part + kParts * i, lo[i], hi[i]);
+                }
+                acc_ph ^= 1u;
+                continue;
+            }
             if (ch0 < p.rows) {
                 for (int c = part; c < kChunks; c += kParts) {
-                    uint32_t lo[16], hi[16];                 // channels 0..15 and 16..31 of 32 pixels
-                    const uint32_t taddr = tmem_base + acc * kN + 32 * c + ((uint32_t)(32 * q) << 16);
-                    tmem_ld_16x32(taddr, lo);
-                    tmem_ld_16x32(taddr + (16u << 16), hi);
+                    uint32_t lo[16], hi[16];
+                    load(c, lo, hi);
                     tmem_ld_wait();
-                    if (fuse) {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            lo[i] = __float_as_uint(fmaxf(__uint_as_float(lo[i]) + bias[i >> 1 & 1], floor_v));
-                            hi[i] = __float_as_uint(fmaxf(__uint_as_float(hi[i]) + bias[2 + (i >> 1 & 1)], floor_v));
-                        }
-                    }
-                    if (lane == 0) bulk_wait_read<0>();      // the store that last used the staging tile has read it
-                    __syncwarp();
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {            // groups of 8 pixels
-                        auto pack = [](uint32_t a, uint32_t b) { return pack_bf16(__uint_as_float(a), __uint_as_float(b)); };
-                        store_matrices(tile + (uint32_t)(512 * g) + my_row, pack(lo[4 * g], lo[4 * g + 1]), pack(lo[4 * g + 2], lo[4 * g + 3]),
-                                       pack(hi[4 * g], hi[4 * g + 1]), pack(hi[4 * g + 2], hi[4 * g + 3]));
-                    }
-                    if (kPlain && ch0 >= p.plain_from) {     // pixel by pixel, the lanes on consecutive channels
-                        __syncwarp();
-                        const bool ch_ok = ch0 + lane < p.rows;
-#pragma unroll 8
-                        for (int px = 0; px < 32; ++px) {
-                            const int g = 4 * c + (px >> 3), y = org.y + (g >> p.tb_log2), b = org.b + (g & (p.tb - 1)), x = org.x + (px & 7);
-                            uint16_t v;
-                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(tile + (uint32_t)(64 * px + (((lane >> 3) ^ (px >> 1 & 3)) << 4) + 2 * (lane & 7))) : "memory");
-                            if (ch_ok && y < p.ho && b < p.batch && x < p.wo) p.y[(((int64_t)b * p.ho + y) * p.wo + x) * p.ldy + ch0 + lane] = v;
-                        }
-                    } else {
-                        fence_async_smem();
-                        __syncwarp();
-                        if (lane == 0) {
-                            const int y = org.y + (4 * c >> p.tb_log2);
-                            if (y < p.ho) tma_store_4d(&map_y, tile, ch0, org.x, org.b, y);
-                            bulk_commit();
-                        }
-                    }
+                    store(c, lo, hi);
                 }
             }
             tc_fence_before();
@@ -424,12 +451,13 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
     HaloParams p = {};
     // Cycles of a launch in its longest CTA, by what was measured.  An entry of the walk takes as long as shared memory needs to feed its
     // MMAs and take in its weight tile, at least the 330 that issuing it takes; a box of the activation a cycle for each pixel of 128
-    // bytes; a tile 300 more, and 1500 where its results leave before the next one begins; the gather in spmm_tc.cu
+    // bytes; a tile 300 more, and 800 where its accumulator has to be drained before the next one begins; the gather in spmm_tc.cu
     // 700 for an entry of 256 pixels, 500 for one of 128.
     // Both sides of the lines it draws (us, 3x3, replayed from a graph): 56 x 56 x 16 images, 256 -> 256 channels, 19 entries: 224 pixels in 4
     // waves of tiles 25.9, 256 in 3 waves 24.1, the gather in 3 waves 26.7; 3:4 dense tiles 30.4, 28.0, 29.7; 56 x 56 x 4, 384 -> 384,
     // 11 entries: 224 in 2 waves 12.1, 256 in one 9.2, gather 9.9; 14 x 14 x 32, 256 -> 256: 128 pixels 8.8, gather 10.2; 7 x 7 x 8, 512 -> 512:
-    // 64 pixels 15.0, gather 17.1; 1x1, 64 -> 64, 112 x 112 x 16: 11.8 and 14.1; 512 -> 512, 7 x 7 x 3: 6.4 and 6.3.
+    // 64 pixels 15.0, gather 17.1; 1x1, 64 -> 64, 112 x 112 x 16: 11.8 and 14.1; 512 -> 512, 7 x 7 x 3: 6.4 and 6.3.  (The 800: 224 and 256 pixels, 128 -> 128, 224 x 224 x 3
+    // 30.5 and 26.8, x 4 38.1 and 34.9, which 1800 left with 224; 256 -> 112, 1x1, 224 x 224 x 2 10.2 and 11.7, 64 -> 509, 1x1 50.3 and 56.1, which 300 would take to 256.)
     const int cpt = cv.channels / g.bk, boxes = L.wcap < cpt ? L.wcap : cpt;
     auto waves = [&](int64_t tiles) { return (tiles * L.nst + sms - 1) / sms; };
     int n = 0;
@@ -440,7 +468,7 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
             if (pw > 256 || ph > 256 || (int64_t)pw * ph * tb * 128 > 56 * 1024 || (ph * tb * pw) * 8 > 0xFFFF) continue;
             const int64_t count = (int64_t)((cv.wo + 7) / 8) * ((cv.ho + th - 1) / th) * ((cv.batch + tb - 1) / tb);
             const int fill = cand + (sparse ? 144 : 256), entry = fill > 330 ? fill : 330;
-            const int64_t cost = waves(count) * (L.wcap * entry + boxes * pw * ph * tb + (cand == 256 && sparse ? 1800 : 300)) + 2500;
+            const int64_t cost = waves(count) * (L.wcap * entry + boxes * pw * ph * tb + (cand == 256 && sparse ? 800 : 300)) + 2500;
             if (n && cost >= best) continue;
             best = cost; n = cand; tiles = count * L.nst;
             p.th = th; p.tb = tb; p.pw = pw;
