@@ -64,6 +64,8 @@ struct Batch {
 // is every buffer of the caller too: the weights may come from crisp_decode) with plain loads, behind the wait.  The
 // read-only path (__ldg, const __restrict__) is for data that stays as it is for the kernel's whole life: its loads may be
 // moved above the wait and need not see what the wait makes visible.  (Plain loads take the same time.)
+// What weights_settled() allows ahead of the wait, a handle's walk lists and weight tiles, is read from L2 (__ldcg, and TMA): an SM's L1 may hold a line from
+// before the encode.
 __device__ __forceinline__ void wait_for_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // The kernels of the mask / encode / decode chain begin with this.  The next kernel may begin as this one's last CTAs end; asked for at the

@@ -131,10 +131,10 @@ spmm_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     // (where the weights have not just been encoded, the walks and the first weight tiles come while the kernel in front finishes)
     if (!p.early) wait_for_prerequisites();
     for (int i = threadIdx.x; i < p.nst * p.wcap; i += kThreads) {
-        const int jb = p.walk_col[i], tap = jb / p.cpt, ti = tap / p.kw;
+        const int jb = __ldcg(p.walk_col + i), tap = jb / p.cpt, ti = tap / p.kw;
         s_cols[i] = (jb - tap * p.cpt) << 16 | ((ti * p.tb * p.pw + tap - ti * p.kw) * 8);       // slab | start of the tap
     }
-    if ((int)threadIdx.x < p.nst) s_len[threadIdx.x] = min(p.walk_len[threadIdx.x], p.wcap);
+    if ((int)threadIdx.x < p.nst) s_len[threadIdx.x] = min(__ldcg(p.walk_len + threadIdx.x), p.wcap);
     __syncthreads();
     for (int i = threadIdx.x; i < p.nst * p.wcap; i += kThreads) {
         const int st = i / p.wcap, e = i - st * p.wcap, len = s_len[st];

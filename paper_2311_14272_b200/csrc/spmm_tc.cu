@@ -505,7 +505,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     // walks are also put in order, 34 random ones 0.92, three of 56 x 56 67.0 -> 61.9.  In the kernel for odd pitches it gained nothing, 13.15 -> 13.3 us.)
     if (!p.early) wait_for_prerequisites();
     for (int i = threadIdx.x; i < walk_words; i += blockDim.x)
-        s_walk[i] = i < p.nst ? p.walk_len[i] : p.walk_col[i - p.nst];
+        s_walk[i] = __ldcg(i < p.nst ? p.walk_len + i : p.walk_col + (i - p.nst));
     const int32_t *walk_len = p.walk_cache ? s_walk : p.walk_len;
     const int32_t *walk_col = p.walk_cache ? s_walk + p.nst : p.walk_col;
     tc_fence_before();
@@ -1369,7 +1369,7 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
             if (conv) plan->conv = *conv;
         }
         launch = plan->launch;
-        launch.p.early = weights_settled(h, st, encodes);
+        launch.p.early = launch.p.walk_cache && weights_settled(h, st, encodes);      // (lists that are read in place are read behind the wait)
     }
     e = launch_chained(launch.variant.kern, (unsigned)launch.grid, (unsigned)launch.variant.threads, launch.smem, st, launch.mx, launch.my,
                        launch.ma, launch.p);
