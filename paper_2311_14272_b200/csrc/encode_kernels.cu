@@ -289,7 +289,7 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
 // much takes 10.8); several slabs of 32 rows a CTA, the next one's loads ahead, gained nothing.
 // With one or two values a group a byte permute puts a pair of values into a word of the result, and what it does follows from the group's offset
 // fields: a table of selectors in shared memory, 2 bytes for a word of two elements.  (Placing value by value with 64-bit shifts, as from three values a group on, took 160
-// instructions a lane and row, two thirds of the issue slots, and 11.3 us.)
+// instructions a lane and row, two thirds of the issue slots, and 11.3 us.  That form is kept there as it was.)
 constexpr int kDecodeRows = 32, kDecodeCols = 256;
 // Selectors of the words of a group of M whose fields are `code`: value j (bytes 2 j, 2 j + 1) where field j says, zero (bytes 4..) elsewhere.
 template <int M, int N>
@@ -316,12 +316,12 @@ decode_kernel(Geometry g, const int32_t *blk_col, const uint16_t *vals, const ui
     constexpr int kCodes = 1 << (N * kBits);
     __shared__ int s_slot[kDecodeCols / 32];
     __shared__ uint2 s_place[kTable ? kCodes : 1];
+    if (kTable && threadIdx.x < kCodes) s_place[threadIdx.x] = place_selectors<M, N>(threadIdx.x);
     chain_kernels();
     const int rg = blockIdx.x / chunks, chunk = blockIdx.x - rg * chunks;
     const int row0 = rg * kDecodeRows, rt = row0 / g.bm;
     const int jb0 = chunk * kDecodeCols / g.bk;
     if (threadIdx.x < kDecodeCols / 32) s_slot[threadIdx.x] = -1;
-    if (kTable && threadIdx.x >= 64 && threadIdx.x < 64 + kCodes) s_place[threadIdx.x - 64] = place_selectors<M, N>(threadIdx.x - 64);
     __syncthreads();
     for (int i = threadIdx.x; i < g.kkeep; i += blockDim.x) {
         const int d = blk_col[(int64_t)rt * g.kkeep + i] - jb0;
@@ -333,67 +333,111 @@ decode_kernel(Geometry g, const int32_t *blk_col, const uint16_t *vals, const ui
     if (k0 >= g.k) return;
     const int jb = k0 / g.bk, slot = s_slot[jb - jb0];
     const int first = row0 + warp * kRows;
-    uint32_t v[kRows][(V + 1) / 2], f[kRows];                // values two a word, offset fields
-    if (slot >= 0) {
-        const int vpb = (int)g.vals_per_block(), vpr = g.groups() * N;
-        const int64_t blk = (int64_t)rt * g.kkeep + slot;
-        const int o0 = (first - rt * g.bm) * vpr + (k0 - jb * g.bk) / M * N;             // (rows of padding are stored too)
-        const uint16_t *vin = vals + blk * vpb + o0;
-        const uint32_t *iin = idx + blk * (vpb * kBits / 32);
-#pragma unroll
-        for (int i = 0; i < kRows; ++i, vin += vpr) {
-            if constexpr (V == 8) {
-                const uint4 t = *reinterpret_cast<const uint4 *>(vin);
-                v[i][0] = t.x; v[i][1] = t.y; v[i][2] = t.z; v[i][3] = t.w;
-            } else if constexpr (V == 4) {
-                const uint2 t = *reinterpret_cast<const uint2 *>(vin);
-                v[i][0] = t.x; v[i][1] = t.y;
-            } else if constexpr (V % 2 == 0) {
-#pragma unroll
-                for (int j = 0; j < V / 2; ++j) v[i][j] = *reinterpret_cast<const uint32_t *>(vin + 2 * j);
-            } else {
-#pragma unroll
-                for (int j = 0; j < V; j += 2) v[i][j / 2] = (uint32_t)vin[j] | (j + 1 < V ? (uint32_t)vin[j + 1] << 16 : 0u);
-            }
-            const int bit = (o0 + i * vpr) * kBits;
-            uint32_t t = iin[bit >> 5] >> (bit & 31);
-            if (32 % (V * kBits) != 0 && (bit & 31) + V * kBits > 32) t |= iin[(bit >> 5) + 1] << (32 - (bit & 31));
-            f[i] = t;
-        }
-    }
-    uint16_t *dst = w + (int64_t)first * ld + k0;
-#pragma unroll
-    for (int i = 0; i < kRows; ++i, dst += ld) {
-        if (first + i >= g.rows) break;
-        uint4 out = make_uint4(0u, 0u, 0u, 0u);              // the row's eight elements
+    if constexpr (kTable) {
+        uint32_t v[kRows][(V + 1) / 2], f[kRows];                // values two a word, offset fields
         if (slot >= 0) {
-            if constexpr (kTable && M == 4) {
-                const uint32_t e0 = s_place[f[i] & (kCodes - 1)].x, e1 = s_place[(f[i] >> (N * kBits)) & (kCodes - 1)].x;
-                const uint32_t w0 = v[i][0], w1 = N == 1 ? v[i][0] >> 16 : v[i][N - 1];
-                out = make_uint4(__byte_perm(w0, 0u, e0 & 0xFFFFu), __byte_perm(w0, 0u, e0 >> 16), __byte_perm(w1, 0u, e1 & 0xFFFFu), __byte_perm(w1, 0u, e1 >> 16));
-            } else if constexpr (kTable) {
-                const uint2 e = s_place[f[i] & (kCodes - 1)];
-                const uint32_t w0 = v[i][0];
-                out = make_uint4(__byte_perm(w0, 0u, e.x & 0xFFFFu), __byte_perm(w0, 0u, e.x >> 16), __byte_perm(w0, 0u, e.y & 0xFFFFu), __byte_perm(w0, 0u, e.y >> 16));
+            const int vpb = (int)g.vals_per_block(), vpr = g.groups() * N;
+            const int64_t blk = (int64_t)rt * g.kkeep + slot;
+            const int o0 = (first - rt * g.bm) * vpr + (k0 - jb * g.bk) / M * N;             // (rows of padding are stored too)
+            const uint16_t *vin = vals + blk * vpb + o0;
+            const uint32_t *iin = idx + blk * (vpb * kBits / 32);
+#pragma unroll
+            for (int i = 0; i < kRows; ++i, vin += vpr) {
+                if constexpr (V == 4) {
+                    const uint2 t = *reinterpret_cast<const uint2 *>(vin);
+                    v[i][0] = t.x; v[i][1] = t.y;
+                } else if constexpr (V == 2) {
+                    v[i][0] = *reinterpret_cast<const uint32_t *>(vin);
+                } else {
+                    v[i][0] = *vin;
+                }
+                const int bit = (o0 + i * vpr) * kBits;
+                uint32_t t = iin[bit >> 5] >> (bit & 31);
+                if (32 % (V * kBits) != 0 && (bit & 31) + V * kBits > 32) t |= iin[(bit >> 5) + 1] << (32 - (bit & 31));
+                f[i] = t;
+            }
+        }
+        uint16_t *dst = w + (int64_t)first * ld + k0;
+#pragma unroll
+        for (int i = 0; i < kRows; ++i, dst += ld) {
+            if (first + i >= g.rows) break;
+            uint4 out = make_uint4(0u, 0u, 0u, 0u);              // the row's eight elements
+            if (slot >= 0) {
+                if constexpr (M == 4) {
+                    const uint32_t e0 = s_place[f[i] & (kCodes - 1)].x, e1 = s_place[(f[i] >> (N * kBits)) & (kCodes - 1)].x;
+                    const uint32_t w0 = v[i][0], w1 = N == 1 ? v[i][0] >> 16 : v[i][N - 1];
+                    out = make_uint4(__byte_perm(w0, 0u, e0 & 0xFFFFu), __byte_perm(w0, 0u, e0 >> 16), __byte_perm(w1, 0u, e1 & 0xFFFFu), __byte_perm(w1, 0u, e1 >> 16));
+                } else {
+                    const uint2 e = s_place[f[i] & (kCodes - 1)];
+                    const uint32_t w0 = v[i][0];
+                    out = make_uint4(__byte_perm(w0, 0u, e.x & 0xFFFFu), __byte_perm(w0, 0u, e.x >> 16), __byte_perm(w0, 0u, e.y & 0xFFFFu), __byte_perm(w0, 0u, e.y >> 16));
+                }
+            }
+            if (vec_ok && k0 + 8 <= g.k) {
+                *reinterpret_cast<uint4 *>(dst) = out;
             } else {
-                unsigned long long half[2] = {0ull, 0ull};           // elements 0..3 and 4..7
+                const uint32_t word[4] = {out.x, out.y, out.z, out.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (k0 + j < g.k) dst[j] = (uint16_t)(word[j >> 1] >> (16 * (j & 1)));
+            }
+        }
+    } else {
+        uint16_t v[kRows][V];
+        uint32_t f[kRows];
+        if (slot >= 0) {
+            const int vpb = (int)g.vals_per_block(), groups = g.groups();
+            const int64_t blk = (int64_t)rt * g.kkeep + slot;
+            const uint16_t *vin = vals + blk * vpb;
+            const uint32_t *iin = idx + blk * (vpb * kBits / 32);
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                const int o = ((first + i - rt * g.bm) * groups + (k0 - jb * g.bk) / M) * N;     // (rows of padding are stored too)
+                if constexpr (V == 8) {
+                    const uint4 t = *reinterpret_cast<const uint4 *>(vin + o);
+                    v[i][0] = (uint16_t)t.x; v[i][1] = (uint16_t)(t.x >> 16); v[i][2] = (uint16_t)t.y; v[i][3] = (uint16_t)(t.y >> 16);
+                    v[i][4] = (uint16_t)t.z; v[i][5] = (uint16_t)(t.z >> 16); v[i][6] = (uint16_t)t.w; v[i][7] = (uint16_t)(t.w >> 16);
+                } else if constexpr (V == 4) {
+                    const uint2 t = *reinterpret_cast<const uint2 *>(vin + o);
+                    v[i][0] = (uint16_t)t.x; v[i][1] = (uint16_t)(t.x >> 16); v[i][2] = (uint16_t)t.y; v[i][3] = (uint16_t)(t.y >> 16);
+                } else if constexpr (V % 2 == 0) {
+#pragma unroll
+                    for (int j = 0; j < V; j += 2) {
+                        const uint32_t t = *reinterpret_cast<const uint32_t *>(vin + o + j);
+                        v[i][j] = (uint16_t)t; v[i][j + 1] = (uint16_t)(t >> 16);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < V; ++j) v[i][j] = vin[o + j];
+                }
+                const int bit = o * kBits;
+                uint32_t t = iin[bit >> 5] >> (bit & 31);
+                if (32 % (V * kBits) != 0 && (bit & 31) + V * kBits > 32) t |= iin[(bit >> 5) + 1] << (32 - (bit & 31));
+                f[i] = t;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const int row = first + i;
+            if (row >= g.rows) break;
+            unsigned long long half[2] = {0ull, 0ull};                   // elements 0..3 and 4..7
+            if (slot >= 0) {
 #pragma unroll
                 for (int j = 0; j < V; ++j) {
                     const uint32_t t = (f[i] >> (j * kBits)) & ((1u << kBits) - 1u);
-                    const unsigned long long at = (unsigned long long)(v[i][j / 2] >> (16 * (j & 1)) & 0xFFFFu) << (16 * (t & 3u));
+                    const unsigned long long at = (unsigned long long)v[i][j] << (16 * (t & 3u));
                     if constexpr (M == 4) half[j / N] |= at;
                     else { half[0] |= t < 4u ? at : 0ull; half[1] |= t < 4u ? 0ull : at; }
                 }
-                out = make_uint4((uint32_t)half[0], (uint32_t)(half[0] >> 32), (uint32_t)half[1], (uint32_t)(half[1] >> 32));
             }
-        }
-        if (vec_ok && k0 + 8 <= g.k) {
-            *reinterpret_cast<uint4 *>(dst) = out;
-        } else {
-            const uint32_t word[4] = {out.x, out.y, out.z, out.w};
+            uint16_t *dst = w + (int64_t)row * ld + k0;
+            if (vec_ok && k0 + 8 <= g.k) {
+                *reinterpret_cast<uint4 *>(dst) = make_uint4((uint32_t)half[0], (uint32_t)(half[0] >> 32), (uint32_t)half[1], (uint32_t)(half[1] >> 32));
+            } else {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (k0 + j < g.k) dst[j] = (uint16_t)(word[j >> 1] >> (16 * (j & 1)));
+                for (int j = 0; j < 8; ++j)
+                    if (k0 + j < g.k) dst[j] = (uint16_t)(half[j >> 2] >> (16 * (j & 3)));
+            }
         }
     }
 }
