@@ -701,7 +701,7 @@ spmm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 }
             }
         }
-        wait_for_prerequisites();                            // (the weight producer may have had nothing to wait for)
+        if (warp == 0) wait_for_prerequisites();             // (the weight producer may have had nothing to wait for; the other has waited)
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer: steps 2 + 3
         if (lane == 0) {
