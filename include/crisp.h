@@ -343,7 +343,10 @@ CRISP_API crisp_status_t crisp_encode_sizes(crisp_mask_t mask, size_t *canonical
  *                   [o*b, o*b+b) of the uint32 stream, LSB first; offsets are zero-based
  *                   positions inside the m-vector (Sec. III-E example).  Values in the zero
  *                   padding are stored as 0.
- *   d_exec_buf      out: tensor-core-ready copy used by crisp_spmm (opaque) + status word.
+ *   d_exec_buf      out: tensor-core-ready copy used by crisp_spmm (opaque) + status word.  Only the library writes it while
+ *                   the handle is in use; a caller that puts a saved copy back does so by a copy (cudaMemcpyAsync), or waits
+ *                   for its own kernel before the next product: a product may begin to read it while a kernel in front of
+ *                   it in the stream finishes, unless that is an encode (of any handle, captured in a graph or not).
  *   out             handle referring to both buffers (not to d_w_bf16 nor to the mask).
  */
 CRISP_API crisp_status_t crisp_encode(const uint16_t *d_w_bf16, int64_t ld_w, crisp_mask_t mask,

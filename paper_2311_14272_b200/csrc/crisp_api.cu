@@ -102,8 +102,6 @@ crisp_handle_s *new_handle(const uint16_t *d_w_bf16, int64_t ld_w, const crisp_m
     h->halo = nullptr;
     h->last = crisp_launch_info_t{-1, 0, 0, 1, 0, 0, 0, 0, 1};
     h->last_resident = 0;
-    h->stream = nullptr;
-    h->settled = 0;
     *L = crisp::EncodeLayer{};
     L->g = g;
     L->w = d_w_bf16; L->ld = ld_w;
@@ -423,7 +421,7 @@ crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ld
     if (ncols <= 0 || ldx < ncols || ldy < ncols) return CRISP_BAD_SHAPE;
     if (!aligned(d_x_bf16, 2) || !aligned(d_y, y_dtype ? 4 : 2)) return CRISP_INVALID_ARG;
     if ((ncols + 63) / 64 > 0x7FFFFFFFll) return CRISP_UNSUPPORTED;
-    const uint64_t encodes = crisp::encode_launches.load(std::memory_order_relaxed);
+    const uint64_t moment = crisp::encodes.now();
     int path = h->forced_path >= 0 ? h->forced_path : h->exec_kind;
     if (h->g.kkeep == 0 || !crisp::tc_operands_ok(d_x_bf16, ldx, d_y, ldy, y_dtype, ncols)) path = CRISP_PATH_DIRECT;
     cudaError_t e = cudaErrorNotSupported;
@@ -434,7 +432,7 @@ crisp_status_t crisp_spmm(crisp_handle_t h, const uint16_t *d_x_bf16, int64_t ld
     } else if (path == CRISP_PATH_DIRECT) {
         e = crisp::launch_spmm_direct(h->g, h->d_blk_col, h->d_vals, h->d_idx, d_x_bf16, ldx, ncols,
                                       d_y, ldy, y_dtype, h->epilogue, (cudaStream_t)stream);
-        if (e == cudaSuccess) crisp::note_launch(h, crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0}, 0, (cudaStream_t)stream, encodes);
+        if (e == cudaSuccess) crisp::note_launch(h, crisp_launch_info_t{CRISP_PATH_DIRECT, 0, 0, 1, 0, 0, 0, 0}, 0, (cudaStream_t)stream, moment);
     } else {
         e = crisp::launch_spmm_tc(h, path, d_x_bf16, ldx, ncols, d_y, ldy, y_dtype, nullptr,
                                   (cudaStream_t)stream);

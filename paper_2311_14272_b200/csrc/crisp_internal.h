@@ -4,10 +4,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "crisp.h"
+#include "settled.h"
 
 namespace crisp {
 
@@ -64,8 +64,8 @@ struct Batch {
 // is every buffer of the caller too: the weights may come from crisp_decode) with plain loads, behind the wait.  The
 // read-only path (__ldg, const __restrict__) is for data that stays as it is for the kernel's whole life: its loads may be
 // moved above the wait and need not see what the wait makes visible.  (Plain loads take the same time.)
-// What weights_settled() allows ahead of the wait, a handle's walk lists and weight tiles, is read from L2 (__ldcg, and TMA): an SM's L1 may hold a line from
-// before the encode.
+// What a product may read ahead of the wait where its handle is settled (settled.h), walk lists and weight tiles, comes from L2 (__ldcg, and TMA): an
+// SM's L1 may hold a line from before the encode.
 __device__ __forceinline__ void wait_for_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // The kernels of the mask / encode / decode chain begin with this.  The next kernel may begin as this one's last CTAs end; asked for at the
@@ -175,8 +175,7 @@ struct crisp_handle_s {
     // written under this lock, and a launch is made from copies.
     std::mutex plan_lock;
     crisp_launch_info_t last;               // what the last product on this handle launched
-    void *stream;                           // where that was (nullptr too where there was none: see settled)
-    uint64_t settled;                       // encode launches of the process before it, plus one; 0: there was none, or it was captured
+    crisp::Settled settled;                 // and whether the next one may read the weights early
     int64_t last_resident;                  // and the bytes of weight tiles it kept in shared memory
 };
 
@@ -265,14 +264,20 @@ int64_t conv_box(int n, int row, const ConvGeom &cv, int *tw, int *th, int *tb);
 // spmm_halo.cu: convolutions whose taps share one load of the activation
 cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, int y_dtype, const ConvGeom &cv, int device,
                              cudaStream_t st, bool *done);
-// After the launch of a product: for crisp_last_launch, and for weights_settled(); encodes: encode_launches before it.
-void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes, cudaStream_t st, uint64_t encodes);
-// Whether a product may read the handle's weight tiles and walk lists before the kernel in front of it in the stream has finished (lock held).  That
-// kernel must not be the one that writes them: true where a product of this handle went before in the same stream and nothing has been
-// encoded since.  The kernel in front then either is that product or came after it, began when that product had waited for all that came before, and
-// everything up to the encode had finished by then.  (A product in another stream, or one that was captured, says nothing about the kernel in front.)
-bool weights_settled(const crisp_handle_s *h, cudaStream_t st, uint64_t encodes);
-extern std::atomic<uint64_t> encode_launches;                // of the process (encode_kernels.cu)
+extern EncodeCount encodes;                                   // (encode_kernels.cu)
+// After the launch of a product: for crisp_last_launch, and for h->settled; moment: encodes.now() before it.
+void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes, cudaStream_t st, uint64_t moment);
+// Launches a product whose parameters p say whether it reads the weights early.  An encode that another host thread has called meanwhile may
+// have come between the decision and the launch: the product is then made once more, behind everything (its results are the same buffer).
+template <typename Params, typename Launch>
+cudaError_t launch_product(Params &p, uint64_t moment, const Launch &launch) {
+    cudaError_t e = launch();
+    if (e == cudaSuccess && p.early && encodes.now() != moment) {
+        p.early = 0;
+        e = launch();
+    }
+    return e;
+}
 // conv == nullptr: d_x is the [k, ncols] matrix.  Otherwise d_x is the activation and ncols = batch*ho*wo.
 // `h->plan` is reused when the operands, shape and epilogue are those of the previous call; `h->last` is filled in.
 cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols,

@@ -524,16 +524,39 @@ cudaError_t encode_batch(const EncodeLayer *layers, int n, cudaStream_t st) {
 
 }  // namespace
 
-std::atomic<uint64_t> encode_launches{0};
+EncodeCount encodes;
+
+namespace {
+
+// If the stream is being captured: the encode counts as one that may happen at any time, from here on until the graph and all that is made from it (it holds a
+// reference to the object for each, and until launches under way have finished) are gone.
+void count_graph(cudaStream_t st) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamGetCaptureInfo(st, &capture, nullptr, &graph) == cudaSuccess && capture == cudaStreamCaptureStatusNone) return;
+    encodes.graph_made();
+    cudaUserObject_t object;
+    if (capture != cudaStreamCaptureStatusActive || !graph ||
+        cudaUserObjectCreate(&object, &encodes, [](void *count) { static_cast<EncodeCount *>(count)->graph_gone(); }, 1u, (unsigned)cudaUserObjectNoDestructorSync) != cudaSuccess)
+        return;                                              // (it counts for good)
+    if (cudaGraphRetainUserObject(graph, object, 1u, (unsigned)cudaGraphUserObjectMove) != cudaSuccess) {
+        encodes.graph_made();                                // (for the reference that is given up)
+        cudaUserObjectRelease(object, 1u);
+    }
+}
+
+}  // namespace
 
 cudaError_t launch_encode(const EncodeLayer *layers, int n, cudaStream_t st) {
-    encode_launches.fetch_add(1, std::memory_order_relaxed);
-    if (n == 1) return encode_batch<1>(layers, 1, st);
-    for (int at = 0; at < n; at += kBatchLayers) {
-        cudaError_t e = encode_batch<kBatchLayers>(layers + at, n - at < kBatchLayers ? n - at : kBatchLayers, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    count_graph(st);
+    encodes.begin();
+    cudaError_t e = cudaSuccess;
+    if (n == 1) e = encode_batch<1>(layers, 1, st);
+    else
+        for (int at = 0; at < n && e == cudaSuccess; at += kBatchLayers)
+            e = encode_batch<kBatchLayers>(layers + at, n - at < kBatchLayers ? n - at : kBatchLayers, st);
+    encodes.end();
+    return e;
 }
 
 cudaError_t launch_decode(const Geometry &g, const int32_t *d_blk_col, const uint16_t *d_vals,

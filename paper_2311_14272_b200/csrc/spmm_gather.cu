@@ -683,7 +683,7 @@ cudaError_t launch_spmm_gather(crisp_handle_s *h, const uint16_t *d_x, int64_t l
     int device = 0;
     cudaError_t e = cudaGetDevice(&device);
     if (e != cudaSuccess) return e;
-    const uint64_t encodes = encode_launches.load(std::memory_order_relaxed);
+    const uint64_t moment = encodes.now();
     const Geometry &g = h->g;
     const bool sparse = h->exec_kind == CRISP_PATH_SPARSE;
     const TcImageLayout L = tc_image_layout(g, h->exec_kind);
@@ -760,7 +760,7 @@ cudaError_t launch_spmm_gather(crisp_handle_s *h, const uint16_t *d_x, int64_t l
     }
     const int grid = p.split > 1 ? p.num_tiles * p.split : (p.num_tiles < sms ? p.num_tiles : sms);
     e = launch_clusters(kern, (unsigned)grid, (unsigned)kThreads, smem, st, (unsigned)p.split, image, rows, p);
-    if (e == cudaSuccess) note_launch(h, crisp_launch_info_t{CRISP_PATH_DIRECT, kCols, 2, 1, kEpiWarps, (int)stages, grid, 0, 1}, 0, st, encodes);
+    if (e == cudaSuccess) note_launch(h, crisp_launch_info_t{CRISP_PATH_DIRECT, kCols, 2, 1, kEpiWarps, (int)stages, grid, 0, 1}, 0, st, moment);
     return e;
 }
 

@@ -54,7 +54,7 @@ struct HaloParams {
     int wo, ho, batch;
     uint32_t a_bytes, entry_bytes, x_bytes, x_stage, x_stages, w_stages;       // (a stage of weights: kGroup entries)
     int resident;
-    int early;                           // weight tiles and walks may be read before the kernel in front has finished (weights_settled)
+    int early;                           // weight tiles and walks may be read before the kernel in front has finished (settled.h)
     uint16_t *y;
     int64_t ldy;
     // From this channel on (a multiple of 32) results are stored pixel by pixel: all where TMA cannot address the pixels (pitch or base not a
@@ -549,7 +549,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
                              cudaStream_t st, bool *done) {
     *done = false;
     if (y_dtype != 0 || !cv.nhwc_out || h->nt_override > 0 || h->group_override > 0) return cudaSuccess;
-    const uint64_t encodes = encode_launches.load(std::memory_order_relaxed);
+    const uint64_t moment = encodes.now();
     HaloLaunch launch;
     {
         std::lock_guard<std::mutex> hold(h->plan_lock);
@@ -573,7 +573,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
             if (fresh.refused) return cudaSuccess;
         }
         launch = plan->launch;
-        launch.p.early = weights_settled(h, st, encodes);
+        launch.p.early = h->settled.holds(st, moment);
     }
     *done = true;
     static std::atomic<bool> configured[16][64];
@@ -589,8 +589,10 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
     p.bias = h->epilogue.bias; p.relu = h->epilogue.relu;
     p.wait_limit = h->wait_limit_cycles ? h->wait_limit_cycles : kWaitLimitCycles;
     p.skip_fill = h->debug_skip_stage;
-    const cudaError_t e = launch_chained(launch.kern, (unsigned)launch.grid, (unsigned)kThreads, launch.smem, st, launch.mx, launch.my, launch.ma, p);
-    if (e == cudaSuccess) note_launch(h, launch.info, launch.resident_bytes, st, encodes);
+    const cudaError_t e = launch_product(p, moment, [&] {
+        return launch_chained(launch.kern, (unsigned)launch.grid, (unsigned)kThreads, launch.smem, st, launch.mx, launch.my, launch.ma, p);
+    });
+    if (e == cudaSuccess) note_launch(h, launch.info, launch.resident_bytes, st, moment);
     return e;
 }
 

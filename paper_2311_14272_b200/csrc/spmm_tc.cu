@@ -72,7 +72,7 @@ struct TcParams {
     int a_map;                  // map_a views the image as rows of 256 bytes: weight tiles come in as tiled loads
     int x_map_3d;               // map_x views X as [ncols/64][k][64]: one load fetches all NT boxes
     uint32_t resident_bytes;    // kResident: the weight tiles of the one walk there is, kept in front of the ring
-    int early;                  // weight tiles and walk lists may be read before the kernel in front has finished (weights_settled)
+    int early;                  // weight tiles and walk lists may be read before the kernel in front has finished (settled.h)
 };
 
 constexpr uint32_t kWideStageBytes = 2048;                      // epilogue staging tile: 16 rows x 128 bytes
@@ -1061,19 +1061,14 @@ struct TcPlan {
 
 void tc_plan_destroy(TcPlan *plan) { delete plan; }
 
-void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes, cudaStream_t st, uint64_t encodes) {
+void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes, cudaStream_t st, uint64_t moment) {
     std::lock_guard<std::mutex> hold(h->plan_lock);
     h->last = info;
     h->last_resident = resident_bytes;
-    if (h->settled == encodes + 1 && h->stream == st) return;
+    if (h->settled.holds(st, moment)) return;
     // (what is captured has not run; one name of a stream stands for another stream in every thread)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    const bool ran = st != cudaStreamPerThread && cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
-    h->stream = st;
-    h->settled = ran ? encodes + 1 : 0;
-}
-bool weights_settled(const crisp_handle_s *h, cudaStream_t st, uint64_t encodes) {
-    return h->settled == encodes + 1 && h->stream == st;
+    h->settled.note(st, moment, st != cudaStreamPerThread && cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone);
 }
 
 int64_t conv_box(int n, int row, const ConvGeom &cv, int *tw, int *th, int *tb) {
@@ -1328,7 +1323,7 @@ cudaError_t make_plan(const crisp_handle_s *h, int kind, const uint16_t *d_x, in
 
 cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols,
                            void *d_y, int64_t ldy, int y_dtype, const ConvGeom *conv, cudaStream_t st) {
-    const uint64_t encodes = encode_launches.load(std::memory_order_relaxed);
+    const uint64_t moment = encodes.now();
     int device = 0;
     cudaError_t e = cudaGetDevice(&device);
     if (e != cudaSuccess) return e;
@@ -1369,11 +1364,13 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
             if (conv) plan->conv = *conv;
         }
         launch = plan->launch;
-        launch.p.early = launch.p.walk_cache && weights_settled(h, st, encodes);      // (lists that are read in place are read behind the wait)
+        launch.p.early = launch.p.walk_cache && h->settled.holds(st, moment);      // (lists that are read in place are read behind the wait)
     }
-    e = launch_chained(launch.variant.kern, (unsigned)launch.grid, (unsigned)launch.variant.threads, launch.smem, st, launch.mx, launch.my,
-                       launch.ma, launch.p);
-    if (e == cudaSuccess) note_launch(h, launch.info, launch.p.resident_bytes, st, encodes);
+    e = launch_product(launch.p, moment, [&] {
+        return launch_chained(launch.variant.kern, (unsigned)launch.grid, (unsigned)launch.variant.threads, launch.smem, st, launch.mx, launch.my,
+                              launch.ma, launch.p);
+    });
+    if (e == cudaSuccess) note_launch(h, launch.info, launch.p.resident_bytes, st, moment);
     return e;
 }
 

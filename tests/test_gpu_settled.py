@@ -1,5 +1,6 @@
 """Products whose weight tiles and walk lists are read before the kernel in front of them has finished: never where that kernel is the one that
-encodes them, in eager order, through handles that share buffers, across streams and in graphs."""
+encodes them, in eager order, through handles that share buffers, across streams and in graphs, of products and of encodes.  The rule by itself is
+tested in test_settled.py.  (The kernel for odd pitches, "odd" here, never reads early; its products settle the handle like the others.)"""
 import ctypes as C
 
 import pytest
@@ -127,4 +128,89 @@ def test_streams_and_graphs():
             graph.replay()
             torch.cuda.synchronize()
             assert torch.equal(y, ref)
+    L.close()
+
+
+@pytest.mark.parametrize("kind", ["tma", "wide", "odd", "conv"])
+@pytest.mark.parametrize("kept_handle", [False, True])
+def test_replayed_encodes(kind, kept_handle):
+    """A graph encodes again at every replay, into the buffers of the handle that was captured, or of one that was there before; products right in
+    front of the replay and right behind it."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    g = torch.Generator(device="cuda").manual_seed(13)
+    rows, k, x, call = _case(kind, torch, g)
+    L = _layer(B, torch, rows, k, 2, 4, 64, 64, g)
+    ws = [torch.randn(rows, k, generator=g, device="cuda").bfloat16() for _ in range(6)]
+    refs = []
+    for w in ws:
+        L.encode(w)
+        torch.cuda.synchronize()
+        refs.append(call(L, x))
+        torch.cuda.synchronize()
+    assert not torch.equal(refs[0], refs[1])
+    w = ws[-1].clone()
+    other = 0
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        if kept_handle:
+            other = B.crisp_encode(w, k, L.mask, L.canonical_buf, L.exec_buf)
+        else:
+            L.encode(w)
+    busy = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    outs = []
+    for rep in range(3):
+        for _ in range(4):
+            busy.zero_()
+        for i, new in enumerate(ws):
+            w.copy_(new)
+            graph.replay()
+            outs.append((i, [call(L, x) for _ in range(1 + i % 3)]))
+    torch.cuda.synchronize()
+    for i, out in outs:
+        assert all(torch.equal(refs[i], o) for o in out)
+    del graph
+    L.encode(ws[0])                                       # (and without the graph as before)
+    assert all(torch.equal(refs[0], call(L, x)) for _ in range(3))
+    B.crisp_destroy(other)
+    L.close()
+
+
+@pytest.mark.parametrize("kind", ["tma", "conv"])
+def test_products_captured_in_a_stream_where_one_went_before(kind):
+    """Such a product is captured as one that reads early; it is replayed behind an encode, first in its graph and behind another kernel."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    g = torch.Generator(device="cuda").manual_seed(17)
+    rows, k, x, call = _case(kind, torch, g)
+    L = _layer(B, torch, rows, k, 2, 4, 64, 64, g)
+    ws = [torch.randn(rows, k, generator=g, device="cuda").bfloat16() for _ in range(6)]
+    refs = []
+    for w in ws:
+        L.encode(w)
+        torch.cuda.synchronize()
+        refs.append(call(L, x))
+        torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    h = B.crisp_encode(ws[0], k, L.mask, L.canonical_buf, L.exec_buf)      # (later encodes fill the buffers of the handle whose products are captured)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        assert torch.equal(call(L, x), refs[0])
+    with torch.cuda.graph(graph, stream=stream):
+        first, second = call(L, x), call(L, x)
+    busy = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    for rep in range(3):
+        for i, w in enumerate(ws):
+            busy.zero_()
+            B.crisp_destroy(h)
+            h = B.crisp_encode(w, k, L.mask, L.canonical_buf, L.exec_buf)
+            graph.replay()
+            a, b = first.clone(), second.clone()
+            eager = call(L, x)
+            assert torch.equal(a, refs[i]) and torch.equal(b, refs[i]) and torch.equal(eager, refs[i])
+    B.crisp_destroy(h)
     L.close()
