@@ -675,6 +675,20 @@ class HybridLayer:
             pass
 
 
+def _holds_rows(t, rows, k):
+    """Whether `rows` rows of k elements lie at the tensor's address, its first stride apart: a matrix of at least that size whose columns are
+    consecutive, or more dimensions where those behind the first are dense in any order (a convolution's weights, channels last or not)."""
+    shape, strides = t.shape, t.stride()
+    if not shape or shape[0] < rows or 0 in shape:
+        return False
+    run = 1
+    for step, size in sorted((step, size) for step, size in zip(strides[1:], shape[1:]) if size != 1):
+        if step != run:
+            return k == 1
+        run *= size
+    return run >= k
+
+
 class PruningNetwork:
     """One pruning iteration of Algorithm 1 over all layers of a network, without the fine-tuning that follows it:
 
@@ -714,6 +728,7 @@ class PruningNetwork:
         for L, w, gs, acc, s in zip(self.layers, weights, grads, self.acc, self.sal):
             rows, k = L.desc.rows, L.desc.k
             for i, g in enumerate(gs):
+                self._check_gradient(g, L)
                 crisp_saliency_accumulate(g, 0 if g.dtype == self.torch.bfloat16 else 1, g.stride(0), rows, k, acc, k, i == 0,
                                           stream)
             crisp_saliency_finish_max(acc, k, w, w.stride(0), rows, k, len(gs), s, k, L.workspace, stream)
@@ -723,9 +738,20 @@ class PruningNetwork:
             count += 1
         return count
 
+    def _check_gradient(self, g, layer):
+        """The library gets an address and a pitch: what is no bf16 or fp32 matrix of the layer's size on a GPU would be read beyond its end, or as
+        something else.  (What only has a tensor's methods answers for itself.)"""
+        torch = self.torch
+        if isinstance(g, torch.Tensor):
+            assert g.is_cuda and g.dtype in (torch.bfloat16, torch.float32) and _holds_rows(g, layer.desc.rows, layer.desc.k), \
+                "a gradient is a bf16 or fp32 CUDA tensor of its layer's shape"
+
     def _table(self, arr, layers, weights, grads):
         """Fills in the table of the layers: one host array each for what there is per gradient (returned; the entries point into them),
         and one struct per layer."""
+        for L, gs in zip(layers, grads):
+            for g in gs:
+                self._check_gradient(g, L)
         flat = [g for gs in grads for g in gs]
         ptrs = array("Q", [g.data_ptr() for g in flat])
         lds = array("q", [g.stride()[0] for g in flat])
@@ -760,7 +786,8 @@ class PruningNetwork:
             gradients = [gs if type(gs) in (list, tuple) else list(gs) for gs in grads[:count]]
             table = _network.table(layers, weights, gradients, self.sal, C.addressof(arr))
         if table is None:
-            assert all(w.is_cuda and w.element_size() == 2 and w.stride()[1] == 1 for w in weights)
+            assert all(w.is_cuda and w.element_size() == 2 and w.stride()[1] == 1 and (not isinstance(w, torch.Tensor) or _holds_rows(w, L.desc.rows, L.desc.k))
+                       for w, L in zip(weights, layers))
             if not at_once:
                 count = self._score_in_turn(weights, grads, stream)
                 arr, layers = (PruneLayer * count)(), layers[:count]

@@ -31,7 +31,7 @@ struct Ref {                             // an owned reference
     Ref &operator=(const Ref &) = delete;
 };
 
-// A plain tensor (or parameter) on a GPU, or nullptr.
+// A plain tensor (or parameter) of two dimensions on a GPU, or nullptr.
 const at::Tensor *plain(PyObject *o) {
     if (!THPVariable_CheckExact(o)) return nullptr;
     const at::Tensor &t = THPVariable_Unpack(o);
@@ -48,6 +48,10 @@ bool buffer(PyObject *owner, PyObject *name, void **out, int64_t *numel) {
         if (numel) *numel = t.numel();
     }
     return true;
+}
+// Whether it holds the layer's rows of consecutive elements.
+bool holds(const at::Tensor &t, const crisp_layer_desc_t &d) {
+    return t.size(0) >= d.rows && t.size(1) >= d.k && (t.stride(1) == 1 || d.k == 1);
 }
 bool descriptor(PyObject *layer, crisp_layer_desc_t *copy, double *keep_ratio) {        // reads it, or sets its keep ratio
     Ref o(PyObject_GetAttr(layer, names.desc));
@@ -99,7 +103,7 @@ PyObject *table(PyObject *, PyObject *const *args, Py_ssize_t n) {
         if (!descriptor(layer, &P.desc, nullptr) || !buffer(layer, names.mask_buf, &P.d_mask_buf, nullptr) ||
             !buffer(layer, names.workspace, &P.d_workspace, nullptr))
             return nullptr;
-        if (!P.d_mask_buf || !P.d_workspace) Py_RETURN_NONE;
+        if (!P.d_mask_buf || !P.d_workspace || !holds(*w, P.desc)) Py_RETURN_NONE;
         P.d_w_bf16 = static_cast<const uint16_t *>(w->data_ptr()); P.ld_w = w->stride(0);
         P.d_saliency = static_cast<float *>(s->data_ptr()); P.ld_s = s->stride(0);
         P.d_grads = ptrs; P.ld_grads = lds; P.grad_dtypes = dtypes;
@@ -107,7 +111,7 @@ PyObject *table(PyObject *, PyObject *const *args, Py_ssize_t n) {
         PyObject **items = PySequence_Fast_ITEMS(gs);
         for (int32_t h = 0; h < P.samples; ++h) {
             const at::Tensor *g = plain(items[h]);
-            if (!g) Py_RETURN_NONE;
+            if (!g || (g->scalar_type() != at::kBFloat16 && g->scalar_type() != at::kFloat) || !holds(*g, P.desc)) Py_RETURN_NONE;
             *ptrs++ = g->data_ptr(); *lds++ = g->stride(0);
             *dtypes++ = g->scalar_type() == at::kBFloat16 ? 0 : 1;
         }

@@ -78,9 +78,51 @@ def test_wrong_weights_are_refused_as_before():
     for bad in (weights[0].float(), weights[0].t().contiguous().t(), weights[0].cpu()):
         with pytest.raises(AssertionError):
             net.step([bad] + weights[1:], grads, 0.7)
+    short = weights[0][:-1], weights[0][:, :-1]
+    for bad in short:
+        with pytest.raises(AssertionError):
+            net.step([bad] + weights[1:], grads, 0.7)
     with pytest.raises(TypeError):
         B._network.table([], [])
     L = net.layers[0]
     with pytest.raises(B.CrispError):                     # nothing encoded yet
         L.decode()
     net.close()
+
+
+@pytest.mark.parametrize("native", [True, False])
+@pytest.mark.parametrize("in_turn", [False, True])
+def test_gradients_of_another_kind_are_refused(native, in_turn, monkeypatch):
+    """Before anything is launched that would read them."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    weights, grads = _inputs(torch, 8, 2)
+    net = B.PruningNetwork(SHAPES, 2, 4, 32, 32)
+    if not native:
+        monkeypatch.setattr(B, "_network", False)
+    g = grads[1][1]
+    for bad in (g.half(), g.double(), g.t().contiguous().t(), g[:-1], g[:, :-1], g.cpu(), torch.cat([g, g], 1)[:, ::2]):
+        given = [grads[0], [grads[1][0], bad], grads[2]]
+        with pytest.raises(AssertionError):
+            net.step(weights, (list(gs) for gs in given) if in_turn else given, 0.7)
+    net.step(weights, grads, 0.7)
+    net.close()
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_larger_gradients_and_those_of_convolutions(native, monkeypatch):
+    """The layer's rows and columns of a larger matrix, and dense tensors of more dimensions, count as they lie."""
+    import torch
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    weights, grads = _inputs(torch, 9, 2)
+    if not native:
+        monkeypatch.setattr(B, "_network", False)
+    forms = [lambda g: torch.nn.functional.pad(g, (0, 3, 0, 2)), lambda g: g.reshape(g.shape[0], -1, 2, 2),
+             lambda g: g.reshape(g.shape[0], 2, 2, -1).permute(0, 3, 1, 2)]
+    want = _run(B, torch, weights, grads)
+    for form in forms:
+        got = _run(B, torch, weights, [[form(g) for g in gs] for gs in grads])
+        for a, b in zip(want, got):
+            assert a[0] == b[0] and all(torch.equal(x, y) for x, y in zip(a[1], b[1]))
