@@ -423,6 +423,7 @@ struct HaloPlan {
     int64_t ldy;
     ConvGeom conv;
     int device;
+    bool plain;                          // results pixel by pixel (plain_from), which the choice of a tile depends on
     bool refused;
     HaloLaunch launch;
 };
@@ -440,6 +441,11 @@ bool make_map_nhwc(CUtensorMap *map, const void *base, uint64_t c, uint64_t pitc
 
 enum class Choice { kTaken, kRefused, kNoMaps };
 
+// From which channel on results are stored pixel by pixel (see HaloParams).
+int plain_channels(int rows, const void *d_y, int64_t ldy) {
+    return ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0 ? 0 : rows % 8 != 0 ? rows / 32 * 32 : rows;
+}
+
 // Whether convolutions of this shape go through the kernel above, and the plan of this one if so.
 Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_t ldy, const ConvGeom &cv, int device,
                HaloLaunch *plan) {
@@ -449,15 +455,19 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
     const TcImageLayout L = tc_image_layout(g, h->exec_kind);
     const int sms = sm_count_of(device);
     HaloParams p = {};
+    p.plain_from = plain_channels(g.rows, d_y, ldy);
+    const bool plain = p.plain_from < g.rows;
     // Cycles of a launch in its longest CTA, by what was measured.  An entry of the walk takes as long as shared memory needs to feed its
     // MMAs and take in its weight tile, at least the 330 that issuing it takes; a box of the activation a cycle for each pixel of 128
-    // bytes; a tile 300 more, and 800 where its accumulator has to be drained before the next one begins; the gather in spmm_tc.cu
-    // 700 for an entry of 256 pixels, 500 for one of 128.
+    // bytes; a tile 300 more, and where its accumulator has to be drained before the next one begins 800, or 1800 with results that are stored pixel by
+    // pixel, which takes longer than the next tile's MMAs; the gather in spmm_tc.cu 700 for an entry of 256 pixels, 500 for one of 128.
     // Both sides of the lines it draws (us, 3x3, replayed from a graph): 56 x 56 x 16 images, 256 -> 256 channels, 19 entries: 224 pixels in 4
     // waves of tiles 25.9, 256 in 3 waves 24.1, the gather in 3 waves 26.7; 3:4 dense tiles 30.4, 28.0, 29.7; 56 x 56 x 4, 384 -> 384,
     // 11 entries: 224 in 2 waves 12.1, 256 in one 9.2, gather 9.9; 14 x 14 x 32, 256 -> 256: 128 pixels 8.8, gather 10.2; 7 x 7 x 8, 512 -> 512:
     // 64 pixels 15.0, gather 17.1; 1x1, 64 -> 64, 112 x 112 x 16: 11.8 and 14.1; 512 -> 512, 7 x 7 x 3: 6.4 and 6.3.  (The 800: 224 and 256 pixels, 128 -> 128, 224 x 224 x 3
-    // 30.5 and 26.8, x 4 38.1 and 34.9, which 1800 left with 224; 256 -> 112, 1x1, 224 x 224 x 2 10.2 and 11.7, 64 -> 509, 1x1 50.3 and 56.1, which 300 would take to 256.)
+    // 30.5 and 26.8, x 4 38.1 and 34.9, which 1800 left with 224; 256 -> 112, 1x1, 224 x 224 x 2 10.2 and 11.7, 64 -> 509, 1x1 50.3 and 56.1, which 300 would take to 256.  The 1800: 224 and 256 pixels, 224 x 224, all channels
+    // pixel by pixel, 128 -> 477 53.3 and 58.1, 256 -> 408 52.8 and 58.2, 256 -> 171, 1x1 29.5 and 28.8; the last ones only, 128 -> 477 53.6 and 57.4, 64 -> 243 29.0 and 27.9; 0.97 of
+    // the time with 224 in the mean of 50 random shapes that the 800 would take to 256, 0.88 to 1.15.)
     const int cpt = cv.channels / g.bk, boxes = L.wcap < cpt ? L.wcap : cpt;
     auto waves = [&](int64_t tiles) { return (tiles * L.nst + sms - 1) / sms; };
     int n = 0;
@@ -468,7 +478,7 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
             if (pw > 256 || ph > 256 || (int64_t)pw * ph * tb * 128 > 56 * 1024 || (ph * tb * pw) * 8 > 0xFFFF) continue;
             const int64_t count = (int64_t)((cv.wo + 7) / 8) * ((cv.ho + th - 1) / th) * ((cv.batch + tb - 1) / tb);
             const int fill = cand + (sparse ? 144 : 256), entry = fill > 330 ? fill : 330;
-            const int64_t cost = waves(count) * (L.wcap * entry + boxes * pw * ph * tb + (cand == 256 && sparse ? 800 : 300)) + 2500;
+            const int64_t cost = waves(count) * (L.wcap * entry + boxes * pw * ph * tb + (cand == 256 && sparse ? plain ? 1800 : 800 : 300)) + 2500;
             if (n && cost >= best) continue;
             best = cost; n = cand; tiles = count * L.nst;
             p.th = th; p.tb = tb; p.pw = pw;
@@ -522,7 +532,6 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
     if (p.w_stages < 2) return Choice::kRefused;
     p.resident = L.nst == 1 && (uint32_t)L.wcap <= p.w_stages * kGroup;
     p.y = reinterpret_cast<uint16_t *>(d_y); p.ldy = ldy;
-    p.plain_from = ldy % 8 != 0 || reinterpret_cast<uintptr_t>(d_y) % 16 != 0 ? 0 : g.rows % 8 != 0 ? g.rows / 32 * 32 : g.rows;
     plan->smem = fixed + (size_t)p.x_stages * p.x_stage + (size_t)p.w_stages * w_stage;
     plan->grid = (int)(tiles < sms ? tiles : sms);
     if (!make_map_image(&plan->ma, h->d_exec + L.image_off, (uint64_t)L.stack * L.nst * L.wcap * L.entry_bytes, L.entry_bytes) ||
@@ -530,7 +539,6 @@ Choice plan_halo(const crisp_handle_s *h, const uint16_t *d_x, void *d_y, int64_
         (p.plain_from > 0 && !make_map_nhwc(&plan->my, d_y, g.rows, ldy, cv.wo, cv.ho, cv.batch, 32, 8, p.tb, 4 / p.tb)))
         return Choice::kNoMaps;
     plan->p = p;
-    const bool plain = p.plain_from < g.rows;
     plan->which = (n == 256 ? 12 : n == 224 ? 8 : n == 128 ? 4 : 0) + (sparse ? 2 : 0) + (plain ? 1 : 0);
 #define CRISP_HALO_KERNELS(N) spmm_halo_kernel<N, false, false>, spmm_halo_kernel<N, false, true>, spmm_halo_kernel<N, true, false>, spmm_halo_kernel<N, true, true>
     static const HaloKernel kernels[16] = {CRISP_HALO_KERNELS(64), CRISP_HALO_KERNELS(128), CRISP_HALO_KERNELS(224), CRISP_HALO_KERNELS(256)};
@@ -554,7 +562,8 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
     {
         std::lock_guard<std::mutex> hold(h->plan_lock);
         HaloPlan *plan = h->halo;
-        const bool same = plan && plan->device == device && same_conv(plan->conv, cv);
+        const bool plain = plain_channels(h->g.rows, d_y, ldy) < h->g.rows;
+        const bool same = plan && plan->device == device && plan->plain == plain && same_conv(plan->conv, cv);
         if (same && plan->refused) return cudaSuccess;
         if (!same || plan->x != d_x || plan->y != d_y || plan->ldy != ldy) {
             const cudaError_t e = ensure_context(device);    // (a plan encodes tensor maps)
@@ -562,7 +571,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
             HaloPlan fresh = {};
             const Choice choice = plan_halo(h, d_x, d_y, ldy, cv, device, &fresh.launch);
             if (choice == Choice::kNoMaps) return cudaSuccess;
-            fresh.x = d_x; fresh.y = d_y; fresh.ldy = ldy; fresh.conv = cv; fresh.device = device;
+            fresh.x = d_x; fresh.y = d_y; fresh.ldy = ldy; fresh.conv = cv; fresh.device = device; fresh.plain = plain;
             fresh.refused = choice == Choice::kRefused;
             if (!plan) {
                 plan = new (std::nothrow) HaloPlan;

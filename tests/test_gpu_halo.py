@@ -133,3 +133,30 @@ def test_a_wait_that_runs_out_is_reported():
     torch.cuda.synchronize()
     assert L.device_status() == 0 and torch.equal(y, want)
     L.close()
+
+
+@pytest.mark.parametrize("s_out,c,b,side,keep", [(168, 128, 28, 56, 0.5), (368, 64, 1, 224, 0.75)])
+def test_results_stored_pixel_by_pixel_keep_two_accumulators(s_out, c, b, side, keep):
+    """On one handle in turn: where TMA stores the results 256 pixels are the better tile, where they leave pixel by pixel 224, whatever was
+    asked for before."""
+    import torch
+    import torch.nn.functional as F
+    from paper_2311_14272_b200 import binding as B
+    B.load()
+    g = torch.Generator(device="cuda").manual_seed(s_out)
+    L = B.HybridLayer(s_out, 9 * c, 2, 4, 64, 64, keep)
+    L.build_mask(torch.rand(s_out, 9 * c, generator=g, device="cuda")).encode(torch.randn(s_out, 9 * c, generator=g, device="cuda").bfloat16())
+    x = torch.randn(b, side, side, c, generator=g, device="cuda").bfloat16()
+    # two orders of a sum of 9 c products differ by at most 2 * 9 c * 2^-23 * sum |w x|, their bf16 roundings by at most 2^-7 of the value
+    mags = F.conv2d(x.float().abs().permute(0, 3, 1, 2), L.decode().float().abs().view(s_out, 3, 3, c).permute(0, 3, 1, 2), padding=1).permute(0, 2, 3, 1)
+    first = None
+    for pitch, tile in [(s_out, 256), (s_out + 4, 224), (s_out + 8, 256), (s_out + 1, 224), (s_out, 256)]:
+        y = torch.full((b, side, side, pitch), 7.0, dtype=torch.bfloat16, device="cuda")
+        L.spmm_conv(x, 3, 3, 1, y=y, nhwc_out=True)
+        assert L.last_launch()["tile_cols"] == tile
+        got = y[..., :s_out].float()
+        assert bool((y[..., s_out:] == 7).all())
+        if first is None:
+            first = got
+        assert bool(((got - first).abs() <= 2.0 ** -7 * first.abs() + 18 * c * 2.0 ** -23 * mags).all())
+    L.close()
