@@ -8,6 +8,8 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import re
+import sys
 from array import array
 from typing import Optional
 
@@ -73,15 +75,20 @@ _network = None                                           # what goes over all t
 
 
 def _bind_network():
-    """csrc/network.cpp for the library that is loaded, or False in a tree where it could not be built (it needs torch's headers)."""
+    """csrc/network.cpp for the library that is loaded, or False in a tree where it could not be built (it needs torch's headers) or was built for
+    another torch or Python."""
     global _network
     lib = load()
     if _network is not False:
-        import torch                                      # noqa: F401  (the module's libraries)
+        import torch                                      # (the module's libraries)
+        release = ".".join(re.findall(r"\d+", torch.__version__)[:3])
         try:
             from . import _network as module
-            module.bind(C.cast(lib.crisp_decode, C.c_void_p).value)
-            _network = module
+            if getattr(module, "built_for", None) == "%s %d.%d" % (release, *sys.version_info[:2]):
+                module.bind(C.cast(lib.crisp_decode, C.c_void_p).value)
+                _network = module
+            else:
+                _network = False
         except ImportError:
             _network = False
     return _network

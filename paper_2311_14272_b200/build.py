@@ -34,19 +34,54 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _stale() -> bool:
-    built = [LIB] + ([CALLS] if HAVE_PYTHON_H else []) + ([NETWORK] if HAVE_PYTHON_H and torch_dir() else [])
+def _older(built, deps) -> bool:
     if not all(os.path.exists(f) for f in built):
         return True
     t = min(os.path.getmtime(f) for f in built)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.cpp")) \
-        + glob.glob(os.path.join(ROOT, "include", "*.h")) + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _stale() -> bool:
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(CSRC, "calls.cpp")] \
+        + glob.glob(os.path.join(ROOT, "include", "*.h")) + [os.path.abspath(__file__)]
+    return _older([LIB] + ([CALLS] if HAVE_PYTHON_H else []), deps)
+
+
+def build_network(force: bool = False) -> bool:
+    """Builds csrc/network.cpp where torch's headers are and its version of them compiles; whether there is a module then.  The library works
+    without it (the binding has the same in Python), so a compiler's error takes the module away and is not raised."""
+    where = torch_dir()
+    if not HAVE_PYTHON_H or not where:
+        print("no headers of Python or torch: a pruning iteration's table is made in Python", file=sys.stderr)
+        return False
+    source, include = os.path.join(CSRC, "network.cpp"), os.path.join(where, "include")
+    api = os.path.join(include, "torch", "csrc", "api", "include")
+    deps = [source, os.path.join(ROOT, "include", "crisp.h"), os.path.abspath(__file__), os.path.join(include, "torch", "csrc", "autograd", "python_variable.h")]
+    if not force and not _older([NETWORK], deps):            # (another torch brings newer headers)
+        return True
+    tmp = NETWORK + f".{os.getpid()}.tmp"
+    try:
+        subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                               "-I", PYTHON_INCLUDE, "-I", os.path.join(ROOT, "include"), "-isystem", include, "-isystem", api, "-o", tmp,
+                               source, "-L", os.path.join(where, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"])
+        os.replace(tmp, NETWORK)
+        return True
+    except (subprocess.CalledProcessError, OSError) as e:
+        print(f"{source} does not compile against {where} ({e}): a pruning iteration's table is made in Python", file=sys.stderr)
+        for f in (tmp, NETWORK):
+            if os.path.exists(f):
+                os.remove(f)
+        return False
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
-        return LIB
+    if force or _stale():
+        _build_library(verbose)
+    build_network(force)
+    return LIB
+
+
+def _build_library(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = LIB + f".{os.getpid()}.tmp"
     cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + \
@@ -55,23 +90,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.replace(tmp, LIB)
     if not HAVE_PYTHON_H:
         print(f"no Python.h in {PYTHON_INCLUDE}: the hot calls go through ctypes", file=sys.stderr)
-        return LIB
+        return
     tmp = CALLS + f".{os.getpid()}.tmp"
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
                            "-I", PYTHON_INCLUDE, "-I", os.path.join(ROOT, "include"), "-o", tmp,
                            os.path.join(CSRC, "calls.cpp")])
     os.replace(tmp, CALLS)
-    where = torch_dir()
-    if not where:
-        print("no headers of torch: a pruning iteration's table is made in Python", file=sys.stderr)
-        return LIB
-    tmp = NETWORK + f".{os.getpid()}.tmp"
-    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-                           "-I", PYTHON_INCLUDE, "-I", os.path.join(ROOT, "include"), "-isystem", os.path.join(where, "include"),
-                           "-isystem", os.path.join(where, "include", "torch", "csrc", "api", "include"), "-o", tmp,
-                           os.path.join(CSRC, "network.cpp"), "-L", os.path.join(where, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"])
-    os.replace(tmp, NETWORK)
-    return LIB
 
 
 if __name__ == "__main__":

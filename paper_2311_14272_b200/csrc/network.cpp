@@ -8,6 +8,7 @@
 #include <ATen/ops/empty_strided.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/version.h>
 
 #include <cstdint>
 #include <cstring>
@@ -204,5 +205,14 @@ PyMODINIT_FUNC PyInit__network(void) {
     names = {PyUnicode_InternFromString("desc"), PyUnicode_InternFromString("mask_buf"), PyUnicode_InternFromString("workspace"),
              PyUnicode_InternFromString("canonical_buf"), PyUnicode_InternFromString("exec_buf"), PyUnicode_InternFromString("mask"),
              PyUnicode_InternFromString("handle"), PyUnicode_InternFromString("kkeep")};
-    return PyModule_Create(&module);
+    PyObject *m = PyModule_Create(&module);
+    // what the binding compares: the layout of torch's tensors and of Python's objects is that of the headers
+#define CRISP_TEXT2(x) #x
+#define CRISP_TEXT(x) CRISP_TEXT2(x)
+    if (m && PyModule_AddStringConstant(m, "built_for", CRISP_TEXT(TORCH_VERSION_MAJOR) "." CRISP_TEXT(TORCH_VERSION_MINOR) "." CRISP_TEXT(TORCH_VERSION_PATCH)
+                                        " " CRISP_TEXT(PY_MAJOR_VERSION) "." CRISP_TEXT(PY_MINOR_VERSION)) != 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
 }
