@@ -66,17 +66,43 @@ def test_synthetic_scores_match_oracle(env, seed):
         assert np.array_equal(got, want), (frac, got, want)
 
 
-def test_rank_sums_beyond_64_bits_and_wide_scale_gaps(env):
+@pytest.mark.parametrize("rows", [600, 900])                  # 1800 scores: a CTA has the layer in shared memory; 2700: sums in global memory
+def test_rank_sums_beyond_64_bits_and_wide_scale_gaps(env, rows):
     B, torch = env
-    big = np.full((600, 3), (1 << 55) - 1, dtype=np.uint64)
+    big = np.full((rows, 3), (1 << 55) - 1, dtype=np.uint64)
     big[:, 1] -= 1
     big[:, 2] -= 5
     small = np.array([[3, 1, 2]], dtype=np.uint64)
     for exps in ([0, 70], [0, -3], [100, -100], [-100, 100], [0, 64]):
         layers, _keep = synthetic(B, torch, [big, small], exps, [64, 64], [0, 0])
-        for frac in (0.0, 1 / 1803, 0.2, 0.34, 0.67, 0.9, 1.0):
+        for frac in (0.0, 1 / (3 * rows + 3), 0.2, 0.34, 0.67, 0.9, 1.0):
             want = oracle.global_rank([big, small], exps, [64, 64], frac)
             assert np.array_equal(gpu_rank(B, torch, layers, frac), want), (exps, frac)
+
+
+# Both sides of the lines between the two ways of forming the rank-column sums: 64 layers, 2560 scores a layer, 2^19 comparisons a layer.
+LINES = {
+    "64_layers": [(3, 5)] * 64, "65_layers": [(3, 5)] * 65, "200_layers": [(2, 3)] * 200,
+    "2560_scores": [(40, 64)], "2561_scores": [(13, 197)], "2560_scores_in_a_column": [(2560, 1)], "2561_scores_in_a_column": [(2561, 1)],
+    "compares_at_the_line": [(2, 512)], "compares_beyond": [(2, 513)], "one_row_below": [(1, 724)], "one_row_beyond": [(1, 725)],
+    "one_large_among_small": [(3, 5), (64, 128), (1, 1), (7, 33)], "64_at_the_line": [(40, 64)] * 64,
+}
+
+
+@pytest.mark.parametrize("name", sorted(LINES))
+def test_lines_between_the_two_ways(env, name):
+    B, torch = env
+    rng = np.random.default_rng(len(name))
+    shapes = LINES[name]
+    for hi in (3, 1 << 55):                                   # ties everywhere; sums beyond 32 bits
+        scores = [rng.integers(0, hi, size=s, dtype=np.uint64) for s in shapes]
+        exps = [int(e) for e in rng.integers(-2, 3, len(shapes))]
+        elems = [1024 * int(e) for e in rng.integers(1, 5, len(shapes))]
+        mk = [int(rng.integers(0, min(s[1], 2) + 1)) for s in shapes]
+        layers, _keep = synthetic(B, torch, scores, exps, elems, mk)
+        for frac in (0.0, 0.3, 0.5, 0.9, 1.0):
+            want = oracle.global_rank(scores, exps, elems, frac, min_keep=mk)
+            assert np.array_equal(gpu_rank(B, torch, layers, frac), want), frac
 
 
 def test_degenerate_inputs(env):
