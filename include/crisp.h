@@ -269,9 +269,9 @@ CRISP_API crisp_status_t crisp_saliency_finish_max(const float *d_acc, int64_t l
  *
  * layers (host array) is read before the call returns.  d_workspace: crisp_global_rank_sizes
  * bytes, 256-byte aligned, scratch.  d_kkeep: device, int32 [n_layers], written on `stream`.
- * nblk <= 4096 per layer (CRISP_UNSUPPORTED beyond).  No device memory is allocated; the layer table is
- * staged through a small temporary host array, so the call is refused (CRISP_UNSUPPORTED) while
- * `stream` is being captured into a graph.
+ * nblk <= 4096 per layer (CRISP_UNSUPPORTED beyond).  No device memory is allocated; the layer table of
+ * large networks is staged through a small temporary host array, so the call is refused (CRISP_UNSUPPORTED)
+ * while `stream` is being captured into a graph, whatever the network.
  */
 typedef struct {
     const unsigned long long *d_scores;  /* device, [nrt, nblk] block scores                      */

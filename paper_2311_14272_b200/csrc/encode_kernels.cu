@@ -285,8 +285,8 @@ encode_kernel(const __grid_constant__ Batch<EncodeLayer, CAP> batch) {
 // V = 8 N / M consecutive ones of their block and their offsets V consecutive fields, so a lane reads both with a load or
 // two and shifts every value to its place in registers.  Which slot of the row tile holds a block column is looked up once
 // per CTA.  Measured (4096 x 4096, 2:4, keep 0.5; 33 MB out, 19 MB in): 9.8 us, against 25 us + 6 us for a memset
-// and a kernel that scattered 2-byte values one by one with three integer divisions each.  What is left is mostly the way of 33 MB into L2 (a fill of as
-// much takes 10.8); several slabs of 32 rows a CTA, the next one's loads ahead, gained nothing.
+// and a kernel that scattered 2-byte values one by one with three integer divisions each.  (A fill of as much takes
+// 10.8: writing is most of it.)  Several slabs of 32 rows a CTA, the next one's loads ahead, gained nothing.
 // With one or two values a group a byte permute puts a pair of values into a word of the result, and what it does follows from the group's offset
 // fields: a table of selectors in shared memory, 2 bytes for a word of two elements.  (Placing value by value with 64-bit shifts, as from three values a group on, took 160
 // instructions a lane and row, two thirds of the issue slots, and 11.3 us.  That form is kept there as it was.)

@@ -157,6 +157,9 @@ __device__ __forceinline__ void floor_parts2(uint64_t v, uint64_t &r, uint64_t &
 // Measured (us, 4096 x 4096, 2:4, S of 64 MiB): the pass over S and this kernel 17.0 + 3.8, where a memset, a pass for bits and maximum and a second one
 // for the scores took 1.8 + 16.2 + 11.4; mask, encoding and decoding in a row 59.3 -> 47.2.  The mask phase alone, in a row: 28.8 -> 18.5, 4:8 in blocks of 32 x 32
 // 41.1 -> 39.8.  Where no record stands (elements spread over 20 binades evenly) this kernel is a second pass over S: 28.8 -> 31.5 and 41.1 -> 52.6.
+// Where all elements count (score mode 1, n = m) the small ones decide: 2 % of the records of normal S do not stand, 36 % of those of products of two normals; calls
+// with 64 x 64 blocks in a row, 4:4 35.6 -> 30.7 and 35.2 -> 36.8, 8:8 42.4 -> 39.9 and 42.5 -> 46.2, mode 1 of 2:4 33.9 -> 29.7 and 33.9 -> 35.9; smaller
+// layers gain in all of them (256 x 2304, 4:4, 12.5 -> 12.4 for products).
 template <int CAP>
 __global__ void __launch_bounds__(kM1Threads)
 block_score_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
@@ -322,8 +325,8 @@ block_select_kernel(const __grid_constant__ Batch<ScoreLayer, CAP> batch) {
 // The whole projection of a small layer in one launch: a cluster of up to eight CTAs, each with whole row tiles, so that all that
 // crosses between them is the layer maximum.  Group bits and the maximum in a first pass over S, scores in a second (out of L1 and L2)
 // summed in shared memory, then the selection: what the kernels above compute, from the same definitions.  What bounds it is instructions on
-// one SM (some 250 for eight elements), and for the smallest layers the two passes' round trips.  A memset and three kernels in its place
-// take the device 10 to 15 us and the host about as long.
+// one SM (some 250 for eight elements), and for the smallest layers the two passes' round trips.  Three kernels in its place take the device 5.5 to
+// 10 us and the host more.
 constexpr int kSmallThreads = 1024, kSmallMaxBlocks = 512, kSmallCluster = 8;
 template <int M>
 __global__ void __launch_bounds__(kSmallThreads)
@@ -462,10 +465,13 @@ mask_small_kernel(const float *s, int64_t ld, Geometry g, bool vec_ok, bool max_
         cluster_wait();
     }
 }
-// Layers that it takes: up to 2^14 elements a CTA.  Mask phase replayed from a graph, and mask, encoding and decoding called in a row, us, this kernel and
-// the others: 256 x 256 (2^13 a CTA) 6.3 and 10.4, 14.3 and 19; 128 x 256 (2^14) 8.0 and 10.4, 15.6 and 19; 25 x 489 (2^14, one CTA) 9.2
-// and 13.1, 19.5 and 21; 256 x 512 in four CTAs (2^15) 12.1 and 10.5, 19.9 and 19.  A CTA takes its row tiles one after the other, so of two at most (mask
-// phase: two, 435 x 35 9.0 and 13.2, 464 x 218 12.2 and 12.6; four, 1949 x 46 15.3 and 13.2; six, 1497 x 58 19.0 and 12.4).
+// Layers that it takes: up to 2^14 elements a CTA, in two row tiles at most (a CTA takes them one after the other).  The line was drawn when the others were a memset
+// and three kernels with two passes over S; since they are three with one, it lies on the high side.  Mask phase replayed from a graph, and mask, encoding and
+// decoding called in a row, us, this kernel and the others, 2:4.  One row tile a CTA: 16 x 32 (2^10 elements) 3.7 and 6.8, 12.1 and 15.9; 64 x 64 (2^11)
+// 5.1 and 5.5, 12.0 and 15.8; 17 x 140 (2^13.3) 5.5 and 8.2, 12.5 and 15.8; 25 x 489 (2^14) 8.8 and 9.6, 17.0 and 18.3; 128 x 256 (2^14) 8.0 and
+// 5.8, 14.7 and 15.7; 374 x 248, 3:4 (2^14) 8.8 and 7.5, 16.3 and 16.1.  Two: 435 x 35 (2^12) 8.7 and 7.8, 16.4 and 16.1; 464 x 218 (2^13.8) 11.6 and
+// 9.6, 21.7 and 20.0; 941 x 103, 4:8 (2^14) 12.1 and 8.8, 20.9 and 18.0.  Beyond: 256 x 512 in four CTAs (2^15) 12.4 and 6.6, 19.5 and 15.6; four row
+// tiles, 1949 x 46 15.5 and 8.3, 24.0 and 17.1.
 constexpr int64_t kSmallPerCta = 1 << 14;
 int small_ctas(const Geometry &g) {
     const int ctas = g.nrt < kSmallCluster ? g.nrt : kSmallCluster;

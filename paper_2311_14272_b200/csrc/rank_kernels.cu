@@ -280,8 +280,8 @@ CRISP_API crisp_status_t crisp_global_rank(int32_t n_layers, const crisp_rank_la
     if (!d_workspace || !d_kkeep || reinterpret_cast<uintptr_t>(d_workspace) % crisp::kAlign) return CRISP_INVALID_ARG;
     if (!(prune_fraction >= 0.0 && prune_fraction <= 1.0)) return CRISP_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    // The layer table is staged from a temporary host array, so the call cannot be part of a stream capture
-    // (the graph would keep a pointer to memory that is gone when it is replayed).
+    // A table that does not fit a kernel parameter is staged from a temporary host array, so the call cannot be part of a stream capture
+    // (the graph would keep a pointer to memory that is gone when it is replayed); smaller ones neither, so that no size decides it.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return CRISP_CUDA_ERROR;
     if (cap != cudaStreamCaptureStatusNone) return CRISP_UNSUPPORTED;

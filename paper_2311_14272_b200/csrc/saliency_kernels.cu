@@ -102,7 +102,8 @@ saliency_finish_kernel(const float *__restrict__ acc, int64_t ld_a, const uint16
 // rows, and a warp 512 consecutive bytes of each row (32 x 32 elements a warp: 64 us on the first below, twice the requests).  Bound by HBM; what a small network waits
 // for is latency, so items are CTAs of their own, all layers share the launch and a sample is asked for before the last one is added.
 // Measured (us, this kernel and the score kernel; 13 layers of VGG-16, 14.7 M weights, four bf16 samples, 206 MB): 52.2 + 3.4, before the
-// records 51.1 + 14.8; 35 layers of MobileNetV2 13.0 + 3.2, 15.0 + 5.8.  Four rows a lane 56.5 and 17.1, two CTAs an SM 53.6 and 15.9.
+// records 51.1 + 14.8; 35 layers of MobileNetV2 13.0 + 3.2, 15.0 + 5.8.  Four rows a lane 56.5 and 17.1, two CTAs an SM 53.6 and 15.9
+// (the 40 registers of three spill 64 to 112 bytes, all forms).
 constexpr int kSalChunk = 256, kSalWords = kSalChunk / 32;                     // k-elements of a work item: 32 lanes x 8
 constexpr int kSalLaneRows = 2, kSalItemThreads = kM1Rows / kSalLaneRows * 32;
 struct SaliencyLayer {
