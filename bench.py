@@ -479,7 +479,7 @@ def measure_global_rank(torch, B, dev, with_oracle, iters=12):
                 ts.append(a.elapsed_time(b))
         rec = {"network": name, "layers": len(layers), "rank_positions": int(sum(L.nblk - 1 for L in layers)),
                "block_scores": int(sum(L.nrt * L.nblk for L in layers)), "prune_fraction": 0.6,
-               "global_rank_us": float(np.mean(ts)) * 1e3, "launches": 3,
+               "global_rank_us": float(np.mean(ts)) * 1e3, "launches": 2,
                "kkeep": kk.cpu().numpy().tolist()}
         if with_oracle:
             import oracle
@@ -530,10 +530,10 @@ def measure_iteration(torch, B, dev, with_oracle, samples=4, iters=9):
         weights = sum(r * k for r, k in shapes)
         rec = {"network": name, "layers": len(shapes), "weights": int(weights), "samples": samples, "kappa": kappa,
                "iteration_us": float(np.median(ts)), "iteration_us_min": float(np.min(ts)),
-               # clear, saliency + bits, scores, three for the ranking, selection, encode: all layers at once
-               "launches": 8, "kkeep": [int(c) for c in kk],
-               # gradients and W in, S out and in again, kept half of W in, values + offsets + image out
-               "algorithmic_bytes": int(weights * (samples * 2 + 2 + 4 + 4 + 2 + 2))}
+               # clear, saliency + bits, scores, two for the ranking, selection, encode: all layers at once
+               "launches": 7, "kkeep": [int(c) for c in kk],
+               # gradients and W in, S out, kept half of W in, values + offsets + image out
+               "algorithmic_bytes": int(weights * (samples * 2 + 2 + 4 + 2 + 2))}
         rec["achieved_gbs"] = rec["algorithmic_bytes"] / (rec["iteration_us"] * 1e-6) / 1e9
         if with_oracle:
             import oracle
