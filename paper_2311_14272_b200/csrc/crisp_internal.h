@@ -267,17 +267,6 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
 extern EncodeCount encodes;                                   // (encode_kernels.cu)
 // After the launch of a product: for crisp_last_launch, and for h->settled; moment: encodes.now() before it.
 void note_launch(crisp_handle_s *h, const crisp_launch_info_t &info, int64_t resident_bytes, cudaStream_t st, uint64_t moment);
-// Launches a product whose parameters p say whether it reads the weights early.  An encode that another host thread has called meanwhile may
-// have come between the decision and the launch: the product is then made once more, behind everything (its results are the same buffer).
-template <typename Params, typename Launch>
-cudaError_t launch_product(Params &p, uint64_t moment, const Launch &launch) {
-    cudaError_t e = launch();
-    if (e == cudaSuccess && p.early && encodes.now() != moment) {
-        p.early = 0;
-        e = launch();
-    }
-    return e;
-}
 // conv == nullptr: d_x is the [k, ncols] matrix.  Otherwise d_x is the activation and ncols = batch*ho*wo.
 // `h->plan` is reused when the operands, shape and epilogue are those of the previous call; `h->last` is filled in.
 cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int64_t ldx, int64_t ncols,

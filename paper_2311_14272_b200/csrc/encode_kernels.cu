@@ -533,10 +533,11 @@ namespace {
 void count_graph(cudaStream_t st) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaGraph_t graph = nullptr;
-    if (cudaStreamGetCaptureInfo(st, &capture, nullptr, &graph) == cudaSuccess && capture == cudaStreamCaptureStatusNone) return;
+    const cudaError_t asked = cudaStreamGetCaptureInfo(st, &capture, nullptr, &graph);
+    if (asked == cudaSuccess && capture != cudaStreamCaptureStatusActive) return;      // (one that has failed makes no graph)
     encodes.graph_made();
     cudaUserObject_t object;
-    if (capture != cudaStreamCaptureStatusActive || !graph ||
+    if (asked != cudaSuccess || !graph ||
         cudaUserObjectCreate(&object, &encodes, [](void *count) { static_cast<EncodeCount *>(count)->graph_gone(); }, 1u, (unsigned)cudaUserObjectNoDestructorSync) != cudaSuccess)
         return;                                              // (it counts for good)
     if (cudaGraphRetainUserObject(graph, object, 1u, (unsigned)cudaGraphUserObjectMove) != cudaSuccess) {

@@ -43,4 +43,17 @@ private:
     uint64_t at_ = 0;
 };
 
+// Launches a product whose parameters p say whether it reads early, decided at `moment`.  An encode that another host thread has called meanwhile may have
+// come between the decision and the launch: the product is then made once more, behind everything (its results are the same buffer).
+// launch() returns 0 where it succeeded.
+template <typename Params, typename Launch>
+auto launch_product(const EncodeCount &encodes, Params &p, uint64_t moment, const Launch &launch) {
+    auto error = launch();
+    if (error == 0 && p.early && encodes.now() != moment) {
+        p.early = 0;
+        error = launch();
+    }
+    return error;
+}
+
 }  // namespace crisp

@@ -598,7 +598,7 @@ cudaError_t launch_spmm_halo(crisp_handle_s *h, const uint16_t *d_x, void *d_y, 
     p.bias = h->epilogue.bias; p.relu = h->epilogue.relu;
     p.wait_limit = h->wait_limit_cycles ? h->wait_limit_cycles : kWaitLimitCycles;
     p.skip_fill = h->debug_skip_stage;
-    const cudaError_t e = launch_product(p, moment, [&] {
+    const cudaError_t e = launch_product(encodes, p, moment, [&] {
         return launch_chained(launch.kern, (unsigned)launch.grid, (unsigned)kThreads, launch.smem, st, launch.mx, launch.my, launch.ma, p);
     });
     if (e == cudaSuccess) note_launch(h, launch.info, launch.resident_bytes, st, moment);

@@ -1366,7 +1366,7 @@ cudaError_t launch_spmm_tc(crisp_handle_s *h, int kind, const uint16_t *d_x, int
         launch = plan->launch;
         launch.p.early = launch.p.walk_cache && h->settled.holds(st, moment);      // (lists that are read in place are read behind the wait)
     }
-    e = launch_product(launch.p, moment, [&] {
+    e = launch_product(encodes, launch.p, moment, [&] {
         return launch_chained(launch.variant.kern, (unsigned)launch.grid, (unsigned)launch.variant.threads, launch.smem, st, launch.mx, launch.my,
                               launch.ma, launch.p);
     });

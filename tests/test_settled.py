@@ -29,6 +29,17 @@ CASES = {
 }
 
 
+# (whether it decided to read early, what happens while it is launched, error and number of launches)
+LAUNCHES = {
+    "alone": (1, "", "0 1"),
+    "encoded_meanwhile": (1, "count.begin(); count.end();", "0 2"),
+    "being_encoded": (1, "count.begin();", "0 2"),
+    "captured_meanwhile": (1, "count.graph_made();", "0 2"),
+    "encoded_meanwhile_but_not_early": (0, "count.begin(); count.end();", "0 1"),
+    "failed": (1, "count.begin(); return 3;", "3 1"),
+}
+
+
 @pytest.fixture(scope="module")
 def program(tmp_path_factory):
     d = tmp_path_factory.mktemp("settled")
@@ -37,6 +48,11 @@ def program(tmp_path_factory):
         '  auto encode = [&] { count.begin(); count.end(); }; auto product = [&](const void *st) { handle.note(st, count.now(), true); };\n'
         '  (void)encode; (void)product; %s\n  puts(handle.holds(%s, count.now()) ? "early" : "waits"); return 0; }\n'
         % (name, case[0], case[1] if len(case) == 3 else "a") for name, case in CASES.items())
+    # launches of a product that decided at a moment whether it reads early: what happens during the first one, and how often it is launched
+    for name, (early, during, launches) in LAUNCHES.items():
+        bodies += ('if (!strcmp(name, "%s")) { EncodeCount count; struct { int early; } p = {%d}; int n = 0; const uint64_t at = count.now();\n'
+                   '  int e = launch_product(count, p, at, [&] { if (!n++) { %s } else if (p.early) return 7; return 0; });\n'
+                   '  printf("%%d %%d\\n", e, n); return 0; }\n' % (name, early, during))
     src = d / "settled.cpp"
     src.write_text('#include <cstdio>\n#include <cstring>\n#include "settled.h"\nusing namespace crisp;\n'
                    "int main(int, char **argv) {\nconst char *name = argv[1];\n" + bodies + "return 1; }\n")
@@ -48,3 +64,9 @@ def program(tmp_path_factory):
 def test_rule(program, name):
     out = subprocess.run([program, name], capture_output=True, text=True, check=True).stdout.strip()
     assert out == ("early" if CASES[name][-1] else "waits")
+
+
+@pytest.mark.parametrize("name", sorted(LAUNCHES))
+def test_an_encode_that_comes_between(program, name):
+    """The decision and the launch are not one step: behind an encode of another thread the product is made once more, and not early."""
+    assert subprocess.run([program, name], capture_output=True, text=True, check=True).stdout.strip() == LAUNCHES[name][-1]
